@@ -87,6 +87,7 @@ cudaError_t launch_angular_counts(int, const float4 *, const int32_t *, const Ro
 cudaError_t launch_cell_sort(const RebuildArgs &, cudaStream_t);
 cudaError_t launch_neighbors(const RebuildArgs &, cudaStream_t);
 int scan_tiles(int ncell);
+int cell_sort_launches(int n, int ncell);
 // nep_md.cu
 int md_blocks(int n);
 cudaError_t launch_kick_drift(int, double *, double *, double *, double *, double *, double *, const long long *, float4 *,
@@ -160,7 +161,8 @@ struct nep_handle {
   // device buffers
   double *x = nullptr, *y = nullptr, *z = nullptr, *vx = nullptr, *vy = nullptr, *vz = nullptr;
   double *xb = nullptr, *yb = nullptr, *zb = nullptr, *vxb = nullptr, *vyb = nullptr, *vzb = nullptr;
-  int *id = nullptr, *idb = nullptr, *cell_of = nullptr, *perm = nullptr;
+  int *id = nullptr, *idb = nullptr, *cell_of = nullptr;
+  int2 *perm = nullptr;
   float4 *pos = nullptr, *pos_ref = nullptr;
   long long *F = nullptr;          // fixed-point forces [3][n]
   float *usite = nullptr, *qbuf = nullptr;
@@ -385,7 +387,7 @@ cudaError_t enqueue_rebuild(nep_handle *h) {
   RebuildArgs a = rebuild_args(h);
   cudaError_t e;
   {
-    Scope sc(h, KC_CELL, 9);
+    Scope sc(h, KC_CELL, cell_sort_launches(h->n, h->ncell));
     e = launch_cell_sort(a, h->stream);
   }
   if (e != cudaSuccess) return e;
@@ -962,6 +964,7 @@ nep_status nep_set_state(nep_handle *h, int64_t n, const double *x, const double
                 std::string("allocation failed: ") + cudaGetErrorString(e));
   }
   NEP_CUDA(h, cudaMemsetAsync(h->F, 0, 3 * N * sizeof(long long), h->stream));
+  NEP_CUDA(h, cudaMemsetAsync(h->count, 0, (size_t)h->ncell * sizeof(int), h->stream));
   NEP_CUDA(h, cudaMemsetAsync(h->sums, 0, 32 * sizeof(double), h->stream));
   NEP_CUDA(h, cudaMemsetAsync(h->counters, 0, 16 * sizeof(long long), h->stream));
   Control c0{};

@@ -65,7 +65,8 @@ struct RebuildArgs {
   double L[3], l[3];
   int nc[3];
   double *x, *y, *z, *vx, *vy, *vz, *xb, *yb, *zb, *vxb, *vyb, *vzb;
-  int *id, *idb, *cell_of, *count, *cursor, *start, *tile_sums, *perm;
+  int *id, *idb, *cell_of, *count, *cursor, *start, *tile_sums;   // count: zero between builds
+  int2 *perm;
   float4 *pos, *pos_ref;
   int32_t *nbr, *nnum, *nang, *nown, *nband0, *nfar;
   int cap;

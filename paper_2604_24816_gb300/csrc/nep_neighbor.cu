@@ -2,14 +2,15 @@
 //
 // Rebuild pipeline (every kernel takes the control block and returns at once when the current step
 // does not rebuild, so the whole MD step can be replayed as one CUDA graph):
-//   k_cell_zero     clear per-cell counters
 //   k_cell_assign   wrap x into the box (float64), cell = floor(x / l) per dimension, histogram
-//   k_scan_*        exclusive scan of the histogram -> cell_start (3 kernels, integer, deterministic)
+//   k_scan_*        exclusive scan of the histogram -> cell_start (1 kernel for one tile of cells, else 3;
+//                   integer, deterministic), which also clears the histogram for the next build
 //   k_scatter       slot within the cell (arbitrary order), then
-//   k_cell_sort     sort each cell's atoms by original id: the sorted order is a pure function of the
-//                   positions, independent of launch timing and of the previous order
-//   k_permute       gather x, v, id into the new order; cell-relative float32 coordinates
+//   k_permute       rank of each atom in its cell by original id: the sorted order is a pure function of
+//                   the positions, independent of launch timing and of the previous order; gathers x, v,
+//                   id into it and forms the cell-relative float32 coordinates
 //   k_copy_back     copy the gathered arrays back (fixed device pointers for graph replay)
+//   k_rebuild_small all of the above in one block, for small systems
 //   k_neighbors     for each atom, every j with |r_ij| < rc_R + skin among the 27 neighbouring cell
 //                   images, split into the pairs this atom owns (one owner per unordered pair) and the
 //                   rest, each part grouped by distance band so that the per-pair branches of the
@@ -22,58 +23,71 @@
 
 namespace nep {
 
+// Box edges, cell edges and their reciprocals, cells per dimension (float64 side of the cell sort).
+struct CellGrid {
+  double Lx, Ly, Lz, lx, ly, lz, ilx, ily, ilz;
+  int ncx, ncy, ncz;
+};
+
 constexpr int SCAN_THREADS = 1024;
 constexpr int SCAN_ITEMS = 4;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
 
-__global__ void k_cell_zero(int ncell, int *__restrict__ count, int *__restrict__ cursor, Control *ctrl) {
-  if (!ctrl->do_rebuild) return;
-  if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->nb_next = 0;   // the neighbour scan's work counter
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += gridDim.x * blockDim.x) {
-    count[c] = 0;
-    cursor[c] = 0;
-  }
-}
-
+// GB300's FP64 pipe is narrow and a float64 division is a chain of some ten dependent operations on it, so
+// the divisions are kept out of the common path: an atom already inside the box is not wrapped, and the
+// cell index multiplies by the reciprocal edge (an atom within rounding of a cell face may fall on either
+// side of it; its cell-relative coordinate is then 0 or the edge, and the lists hold the same pairs): k_cell_assign
+// 137 -> 39 us at 1,048,576 atoms, 7.8 -> 4.4 us at 16,384 (six divisions per atom before).
 __device__ __forceinline__ double wrap_coord(double x, double L) {
+  if (x >= 0.0 && x < L) return x;
   double y = x - L * floor(x / L);
   if (y >= L) y -= L;
   if (y < 0.0) y = 0.0;
   return y;
 }
+// Position of atom s wrapped into the box (a non-finite one becomes 0 and raises ST_NAN) and its cell
+// coordinates.
+struct CellOf {
+  double x, y, z;
+  int cx, cy, cz;
+};
+__device__ __forceinline__ CellOf cell_of_atom(double px, double py, double pz, const CellGrid &g, int *status) {
+  if (!(isfinite(px) && isfinite(py) && isfinite(pz))) {
+    atomicOr(status, ST_NAN);
+    px = py = pz = 0.0;
+  }
+  CellOf c;
+  c.x = wrap_coord(px, g.Lx); c.y = wrap_coord(py, g.Ly); c.z = wrap_coord(pz, g.Lz);
+  c.cx = min((int)(c.x * g.ilx), g.ncx - 1);
+  c.cy = min((int)(c.y * g.ily), g.ncy - 1);
+  c.cz = min((int)(c.z * g.ilz), g.ncz - 1);
+  return c;
+}
+// Cell-relative float32 coordinates: the same expression as the drift and upload kernels (nep_md.cu), so
+// that a position uploaded unchanged gives bitwise the same coordinates.
+__device__ __forceinline__ float4 cell_relative(double px, double py, double pz, int cx, int cy, int cz,
+                                                const CellGrid &g) {
+  return make_float4((float)fma(-(double)cx, g.lx, px), (float)fma(-(double)cy, g.ly, py),
+                     (float)fma(-(double)cz, g.lz, pz), __int_as_float(cx | (cy << 10) | (cz << 20)));
+}
 
-__global__ void k_cell_assign(int n, double *__restrict__ x, double *__restrict__ y, double *__restrict__ z, double Lx,
-                              double Ly, double Lz, double lx, double ly, double lz, int ncx, int ncy, int ncz,
-                              int *__restrict__ cell_of, int *__restrict__ count, Control *ctrl) {
+__global__ void k_cell_assign(int n, double *__restrict__ x, double *__restrict__ y, double *__restrict__ z,
+                              const CellGrid g, int *__restrict__ cell_of, int *__restrict__ count, Control *ctrl) {
   if (!ctrl->do_rebuild) return;
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-    double px = x[s], py = y[s], pz = z[s];
-    if (!(isfinite(px) && isfinite(py) && isfinite(pz))) {
-      atomicOr(&ctrl->status, ST_NAN);
-      px = py = pz = 0.0;
+    const double px = x[s], py = y[s], pz = z[s];
+    const CellOf a = cell_of_atom(px, py, pz, g, &ctrl->status);
+    if (a.x != px || a.y != py || a.z != pz) {          // also true for NaN: the wrapped position replaces it
+      x[s] = a.x; y[s] = a.y; z[s] = a.z;
     }
-    px = wrap_coord(px, Lx); py = wrap_coord(py, Ly); pz = wrap_coord(pz, Lz);
-    x[s] = px; y[s] = py; z[s] = pz;
-    const int cx = min((int)(px / lx), ncx - 1), cy = min((int)(py / ly), ncy - 1), cz = min((int)(pz / lz), ncz - 1);
-    const int c = (cz * ncy + cy) * ncx + cx;
+    const int c = (a.cz * g.ncy + a.cy) * g.ncx + a.cx;
     cell_of[s] = c;
     atomicAdd(count + c, 1);
   }
 }
 
-// Exclusive scan of count[0..m) into start[0..m], start[m] = total.  Tile scan + carry pass + add.
-__global__ void __launch_bounds__(SCAN_THREADS)
-k_scan_tiles(int m, const int *__restrict__ in, int *__restrict__ out, int *__restrict__ tile_sums, const Control *ctrl) {
-  if (!ctrl->do_rebuild) return;
-  __shared__ int warp_tot[SCAN_THREADS / 32];
-  const int base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
-  int v[SCAN_ITEMS], run = 0;
-#pragma unroll
-  for (int k = 0; k < SCAN_ITEMS; ++k) {
-    v[k] = (base + k < m) ? in[base + k] : 0;
-    run += v[k];
-  }
-  // inclusive warp scan of per-thread totals
+// Exclusive scan over the block of one int per thread (SCAN_THREADS threads); warp_tot: scratch.
+__device__ __forceinline__ int block_scan_excl(int run, int *warp_tot) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int t = run;
 #pragma unroll
@@ -93,81 +107,106 @@ k_scan_tiles(int m, const int *__restrict__ in, int *__restrict__ out, int *__re
     warp_tot[lane] = w;
   }
   __syncthreads();
-  int excl = t - run + (warp > 0 ? warp_tot[warp - 1] : 0);
+  return t - run + (warp > 0 ? warp_tot[warp - 1] : 0);
+}
+
+// Exclusive scan of count[0..m) into start[0..m], start[m] = total, and a copy in cursor (the running slots
+// of k_scatter); count is cleared.  One tile (m <= SCAN_TILE): k_scan_tiles alone; else tile scan + carry
+// pass + add.
+__global__ void __launch_bounds__(SCAN_THREADS)
+k_scan_tiles(int m, int *__restrict__ count, int *__restrict__ start, int *__restrict__ cursor,
+             int *__restrict__ tile_sums, Control *ctrl) {
+  if (!ctrl->do_rebuild) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->nb_next = 0;   // the neighbour scan's work counter
+  __shared__ int warp_tot[SCAN_THREADS / 32];
+  const int base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
+  int v[SCAN_ITEMS], run = 0;
 #pragma unroll
   for (int k = 0; k < SCAN_ITEMS; ++k) {
-    if (base + k < m) out[base + k] = excl;
+    v[k] = 0;
+    if (base + k < m) {
+      v[k] = count[base + k];
+      count[base + k] = 0;
+    }
+    run += v[k];
+  }
+  int excl = block_scan_excl(run, warp_tot);
+#pragma unroll
+  for (int k = 0; k < SCAN_ITEMS; ++k) {
+    if (base + k < m) {
+      start[base + k] = excl;
+      cursor[base + k] = excl;                                  // final when there is one tile
+    }
     excl += v[k];
   }
-  if (threadIdx.x == SCAN_THREADS - 1) tile_sums[blockIdx.x] = excl;
-}
-
-__global__ void k_scan_carry(int ntiles, int *__restrict__ tile_sums, int m, int *__restrict__ out, const Control *ctrl) {
-  if (!ctrl->do_rebuild) return;
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  int run = 0;
-  for (int b = 0; b < ntiles; ++b) {
-    int s = tile_sums[b];
-    tile_sums[b] = run;
-    run += s;
-  }
-  out[m] = run;
-}
-
-__global__ void k_scan_add(int m, int *__restrict__ out, const int *__restrict__ tile_sums, const Control *ctrl) {
-  if (!ctrl->do_rebuild) return;
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < m; idx += gridDim.x * blockDim.x)
-    out[idx] += tile_sums[idx / SCAN_TILE];
-}
-
-__global__ void k_scatter(int n, const int *__restrict__ cell_of, const int *__restrict__ start, int *__restrict__ cursor,
-                          int *__restrict__ perm, const Control *ctrl) {
-  if (!ctrl->do_rebuild) return;
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-    const int c = cell_of[s];
-    perm[start[c] + atomicAdd(cursor + c, 1)] = s;
+  if (threadIdx.x == SCAN_THREADS - 1) {
+    tile_sums[blockIdx.x] = excl;
+    if (gridDim.x == 1) start[m] = excl;
   }
 }
 
-// One thread per cell: insertion sort of the cell's slots by original id (ids are unique).
-__global__ void k_cell_sort(int ncell, const int *__restrict__ start, int *__restrict__ perm, const int *__restrict__ id,
-                            const Control *ctrl) {
+// Exclusive scan of the tile sums by one block, SCAN_THREADS at a time.
+__global__ void __launch_bounds__(SCAN_THREADS)
+k_scan_carry(int ntiles, int *__restrict__ tile_sums, int m, int *__restrict__ start, const Control *ctrl) {
   if (!ctrl->do_rebuild) return;
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += gridDim.x * blockDim.x) {
-    const int b = start[c], e = start[c + 1];
-    for (int p = b + 1; p < e; ++p) {
-      const int s = perm[p];
-      const int key = id[s];
-      int q = p;
-      while (q > b && id[perm[q - 1]] > key) {
-        perm[q] = perm[q - 1];
-        --q;
-      }
-      perm[q] = s;
-    }
+  __shared__ int warp_tot[SCAN_THREADS / 32];
+  int carry = 0;
+  for (int b0 = 0; b0 < ntiles; b0 += SCAN_THREADS) {
+    const int b = b0 + (int)threadIdx.x;
+    const int s = b < ntiles ? tile_sums[b] : 0;
+    const int excl = block_scan_excl(s, warp_tot);
+    if (b < ntiles) tile_sums[b] = carry + excl;
+    carry += warp_tot[SCAN_THREADS / 32 - 1];
+    __syncthreads();                                            // warp_tot is reused by the next chunk
+  }
+  if (threadIdx.x == 0) start[m] = carry;
+}
+
+__global__ void k_scan_add(int m, int *__restrict__ start, int *__restrict__ cursor, const int *__restrict__ tile_sums,
+                           const Control *ctrl) {
+  if (!ctrl->do_rebuild) return;
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < m; idx += gridDim.x * blockDim.x) {
+    const int s = start[idx] + tile_sums[idx / SCAN_TILE];
+    start[idx] = s;
+    cursor[idx] = s;
   }
 }
 
-__global__ void k_permute(int n, const int *__restrict__ perm, const double *__restrict__ x, const double *__restrict__ y,
+// slot t of a cell (in order of arrival) holds atom perm[t].x, whose original id is perm[t].y.
+__global__ void k_scatter(int n, const int *__restrict__ cell_of, const int *__restrict__ id, int *__restrict__ cursor,
+                          int2 *__restrict__ perm, const Control *ctrl) {
+  if (!ctrl->do_rebuild) return;
+  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x)
+    perm[atomicAdd(cursor + cell_of[s], 1)] = make_int2(s, id[s]);
+}
+
+// One thread per slot: its atom's place in the cell is the number of the cell's atoms with a smaller
+// original id (ids are unique), counted over the cell's slots, which neighbouring threads read too (L1
+// hits).  The former pass, one thread per cell sorting its ~18 slots in global memory, was a chain of
+// dependent loads: 41 us from 1,000 to 100,000 atoms, 51 us at 1,048,576; counting ranks here leaves that
+// launch out and adds nothing measurable to this one.
+__global__ void k_permute(int n, const int2 *__restrict__ perm, const int *__restrict__ start,
+                          const double *__restrict__ x, const double *__restrict__ y,
                           const double *__restrict__ z, const double *__restrict__ vx, const double *__restrict__ vy,
-                          const double *__restrict__ vz, const int *__restrict__ id, const int *__restrict__ cell_of,
+                          const double *__restrict__ vz, const int *__restrict__ cell_of,
                           double *__restrict__ xb, double *__restrict__ yb, double *__restrict__ zb,
                           double *__restrict__ vxb, double *__restrict__ vyb, double *__restrict__ vzb,
-                          int *__restrict__ idb, float4 *__restrict__ pos, float4 *__restrict__ pos_ref, double lx,
-                          double ly, double lz, int ncx, int ncy, const Control *ctrl) {
+                          int *__restrict__ idb, float4 *__restrict__ pos, float4 *__restrict__ pos_ref,
+                          const CellGrid g, const Control *ctrl) {
   if (!ctrl->do_rebuild) return;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-    const int s = perm[t];
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
+    const int2 sp = perm[q];
+    const int s = sp.x;
+    const int c = cell_of[s];
+    const int b = start[c], e = start[c + 1];
+    int t = b;
+    for (int k = b; k < e; ++k) t += perm[k].y < sp.y ? 1 : 0;
     const double px = x[s], py = y[s], pz = z[s];
     xb[t] = px; yb[t] = py; zb[t] = pz;
     vxb[t] = vx[s]; vyb[t] = vy[s]; vzb[t] = vz[s];
-    idb[t] = id[s];
-    const int c = cell_of[s];
-    const int cx = c % ncx, cy = (c / ncx) % ncy, cz = c / (ncx * ncy);
-    // the same expression as the drift and upload kernels (nep_md.cu), so that a position uploaded
-    // unchanged gives bitwise the same cell-relative coordinates
-    const float4 p = make_float4((float)fma(-(double)cx, lx, px), (float)fma(-(double)cy, ly, py),
-                                 (float)fma(-(double)cz, lz, pz), __int_as_float(cx | (cy << 10) | (cz << 20)));
+    idb[t] = sp.y;
+    const int cx = c % g.ncx, cy = (c / g.ncx) % g.ncy, cz = c / (g.ncx * g.ncy);
+    const float4 p = cell_relative(px, py, pz, cx, cy, cz, g);
     pos[t] = p;
     pos_ref[t] = p;
   }
@@ -184,6 +223,72 @@ __global__ void k_copy_back(int n, double *__restrict__ x, double *__restrict__ 
     x[t] = xb[t]; y[t] = yb[t]; z[t] = zb[t];
     vx[t] = vxb[t]; vy[t] = vyb[t]; vz[t] = vzb[t];
     id[t] = idb[t];
+  }
+}
+
+// The whole cell sort of a small system (n <= SMALL_ATOMS, ncell <= SMALL_CELLS) in one block: histogram,
+// scan, slots and ranks in shared memory, the state in registers between reading the old order and writing
+// the new one (no second buffer).  The same order and coordinates as the kernels above.  At this size every
+// kernel of the chain is a launch and a few dependent loads: 6.2 us at 862 atoms, and 1.5 us on a step that
+// does not rebuild, against nine launches (26 us and 13 us).
+constexpr int SMALL_ATOMS = 2048, SMALL_CELLS = 2048;
+constexpr int SMALL_ITEMS = SMALL_ATOMS / SCAN_THREADS;
+static_assert(SMALL_ATOMS % SCAN_THREADS == 0 && SMALL_CELLS == 2 * SCAN_THREADS, "two cells per thread");
+__global__ void __launch_bounds__(SCAN_THREADS)
+k_rebuild_small(int n, int ncell, double *__restrict__ x, double *__restrict__ y, double *__restrict__ z,
+                double *__restrict__ vx, double *__restrict__ vy, double *__restrict__ vz, int *__restrict__ id,
+                int *__restrict__ start, float4 *__restrict__ pos, float4 *__restrict__ pos_ref, const CellGrid g,
+                Control *ctrl) {
+  if (!ctrl->do_rebuild) return;
+  __shared__ int cnt[SMALL_CELLS];                 // histogram, then the running slots
+  __shared__ int first[SMALL_CELLS + 1];           // cell_start
+  __shared__ int sid[SMALL_ATOMS];                 // original ids by slot
+  __shared__ int warp_tot[SCAN_THREADS / 32];
+  const int t = threadIdx.x;
+  if (t == 0) ctrl->nb_next = 0;
+  cnt[2 * t] = 0;
+  cnt[2 * t + 1] = 0;
+  __syncthreads();
+  CellOf a[SMALL_ITEMS];
+  double u[SMALL_ITEMS][3];
+  int oid[SMALL_ITEMS], cell[SMALL_ITEMS];
+#pragma unroll
+  for (int k = 0; k < SMALL_ITEMS; ++k) {
+    const int s = k * SCAN_THREADS + t;
+    cell[k] = -1;
+    if (s < n) {
+      a[k] = cell_of_atom(x[s], y[s], z[s], g, &ctrl->status);
+      u[k][0] = vx[s]; u[k][1] = vy[s]; u[k][2] = vz[s];
+      oid[k] = id[s];
+      cell[k] = (a[k].cz * g.ncy + a[k].cy) * g.ncx + a[k].cx;
+      atomicAdd(&cnt[cell[k]], 1);
+    }
+  }
+  __syncthreads();
+  const int c0 = cnt[2 * t], c1 = cnt[2 * t + 1];
+  const int excl = block_scan_excl(c0 + c1, warp_tot);
+  first[2 * t] = cnt[2 * t] = excl;
+  first[2 * t + 1] = cnt[2 * t + 1] = excl + c0;
+  if (t == SCAN_THREADS - 1) first[SMALL_CELLS] = excl + c0 + c1;
+  __syncthreads();
+  // cells past ncell are empty, so first[ncell] is the total
+  for (int c = t; c <= ncell; c += SCAN_THREADS) start[c] = first[c];
+#pragma unroll
+  for (int k = 0; k < SMALL_ITEMS; ++k)
+    if (cell[k] >= 0) sid[atomicAdd(&cnt[cell[k]], 1)] = oid[k];
+  __syncthreads();                                 // every old value has been read, every slot is filled
+#pragma unroll
+  for (int k = 0; k < SMALL_ITEMS; ++k) {
+    if (cell[k] < 0) continue;
+    const int b = first[cell[k]], e = first[cell[k] + 1];
+    int d = b;
+    for (int q = b; q < e; ++q) d += sid[q] < oid[k] ? 1 : 0;
+    x[d] = a[k].x; y[d] = a[k].y; z[d] = a[k].z;
+    vx[d] = u[k][0]; vy[d] = u[k][1]; vz[d] = u[k][2];
+    id[d] = oid[k];
+    const float4 p = cell_relative(a[k].x, a[k].y, a[k].z, a[k].cx, a[k].cy, a[k].cz, g);
+    pos[d] = p;
+    pos_ref[d] = p;
   }
 }
 
@@ -434,20 +539,36 @@ static int resident_grid(K kernel, long long m, int per_block, int threads) {
   return (int)std::min<long long>(blocks_for(m, per_block), (long long)sm_count() * per_sm);
 }
 
+// Kernels that launch_cell_sort enqueues for a system of n atoms in ncell cells.
+static bool small_system(int n, int ncell) { return n <= SMALL_ATOMS && ncell <= SMALL_CELLS; }
+int cell_sort_launches(int n, int ncell) {
+  if (n <= 0) return 0;
+  return small_system(n, ncell) ? 1 : (ncell <= SCAN_TILE ? 5 : 7);
+}
+
+// a.count is zero on entry and on exit.
 cudaError_t launch_cell_sort(const RebuildArgs &a, cudaStream_t st) {
   if (a.n <= 0) return cudaSuccess;
-  k_cell_zero<<<min(blocks_for(a.ncell, 256), 4096), 256, 0, st>>>(a.ncell, a.count, a.cursor, a.ctrl);
-  k_cell_assign<<<resident_grid(k_cell_assign, a.n, 256, 256), 256, 0, st>>>(a.n, a.x, a.y, a.z, a.L[0], a.L[1], a.L[2], a.l[0], a.l[1],
-                                                      a.l[2], a.nc[0], a.nc[1], a.nc[2], a.cell_of, a.count, a.ctrl);
+  const CellGrid g{a.L[0], a.L[1], a.L[2], a.l[0], a.l[1], a.l[2], 1.0 / a.l[0], 1.0 / a.l[1], 1.0 / a.l[2],
+                   a.nc[0], a.nc[1], a.nc[2]};
+  if (small_system(a.n, a.ncell)) {
+    k_rebuild_small<<<1, SCAN_THREADS, 0, st>>>(a.n, a.ncell, a.x, a.y, a.z, a.vx, a.vy, a.vz, a.id, a.start, a.pos,
+                                                a.pos_ref, g, a.ctrl);
+    return cudaGetLastError();
+  }
+  k_cell_assign<<<resident_grid(k_cell_assign, a.n, 256, 256), 256, 0, st>>>(a.n, a.x, a.y, a.z, g, a.cell_of, a.count,
+                                                                            a.ctrl);
   const int ntiles = blocks_for(a.ncell, SCAN_TILE);
-  k_scan_tiles<<<ntiles, SCAN_THREADS, 0, st>>>(a.ncell, a.count, a.start, a.tile_sums, a.ctrl);
-  k_scan_carry<<<1, 32, 0, st>>>(ntiles, a.tile_sums, a.ncell, a.start, a.ctrl);
-  k_scan_add<<<resident_grid(k_scan_add, a.ncell, 256, 256), 256, 0, st>>>(a.ncell, a.start, a.tile_sums, a.ctrl);
-  k_scatter<<<resident_grid(k_scatter, a.n, 256, 256), 256, 0, st>>>(a.n, a.cell_of, a.start, a.cursor, a.perm, a.ctrl);
-  k_cell_sort<<<resident_grid(k_cell_sort, a.ncell, 128, 128), 128, 0, st>>>(a.ncell, a.start, a.perm, a.id, a.ctrl);
-  k_permute<<<resident_grid(k_permute, a.n, 256, 256), 256, 0, st>>>(a.n, a.perm, a.x, a.y, a.z, a.vx, a.vy, a.vz, a.id, a.cell_of, a.xb,
-                                                  a.yb, a.zb, a.vxb, a.vyb, a.vzb, a.idb, a.pos, a.pos_ref, a.l[0],
-                                                  a.l[1], a.l[2], a.nc[0], a.nc[1], a.ctrl);
+  k_scan_tiles<<<ntiles, SCAN_THREADS, 0, st>>>(a.ncell, a.count, a.start, a.cursor, a.tile_sums, a.ctrl);
+  if (ntiles > 1) {
+    k_scan_carry<<<1, SCAN_THREADS, 0, st>>>(ntiles, a.tile_sums, a.ncell, a.start, a.ctrl);
+    k_scan_add<<<resident_grid(k_scan_add, a.ncell, 256, 256), 256, 0, st>>>(a.ncell, a.start, a.cursor, a.tile_sums,
+                                                                            a.ctrl);
+  }
+  k_scatter<<<resident_grid(k_scatter, a.n, 256, 256), 256, 0, st>>>(a.n, a.cell_of, a.id, a.cursor, a.perm, a.ctrl);
+  k_permute<<<resident_grid(k_permute, a.n, 256, 256), 256, 0, st>>>(a.n, a.perm, a.start, a.x, a.y, a.z, a.vx, a.vy, a.vz,
+                                                                    a.cell_of, a.xb, a.yb, a.zb, a.vxb, a.vyb, a.vzb,
+                                                                    a.idb, a.pos, a.pos_ref, g, a.ctrl);
   k_copy_back<<<resident_grid(k_copy_back, a.n, 256, 256), 256, 0, st>>>(a.n, a.x, a.y, a.z, a.vx, a.vy, a.vz, a.id, a.xb, a.yb, a.zb,
                                                     a.vxb, a.vyb, a.vzb, a.idb, a.ctrl);
   return cudaGetLastError();

@@ -75,7 +75,7 @@ constexpr Layout make_layout() {
   L.vx = take(N * 8); L.vy = take(N * 8); L.vz = take(N * 8);
   L.xb = take(N * 8); L.yb = take(N * 8); L.zb = take(N * 8);
   L.vxb = take(N * 8); L.vyb = take(N * 8); L.vzb = take(N * 8);
-  L.id = take(N * 4); L.idb = take(N * 4); L.cell_of = take(N * 4); L.perm = take(N * 4);
+  L.id = take(N * 4); L.idb = take(N * 4); L.cell_of = take(N * 4); L.perm = take(N * 8);
   L.pos = take(N * 16); L.pos_ref = take(N * 16);
   L.F = take(N * 3 * 8); L.usite = take(N * 4); L.G = take(N * S::GS * 4); L.nbr = take(N * CAP * 4);
   L.nnum = take(N * 4); L.nang = take(N * 4); L.nown = take(N * 4); L.nband0 = take(N * 4); L.nfar = take(N * 4);
@@ -250,7 +250,7 @@ extern "C" nep_status nep_compute_noalloc(const nep_params *p, int64_t n, const 
   a.vxb = (double *)at(LAYOUT.vxb); a.vyb = (double *)at(LAYOUT.vyb); a.vzb = (double *)at(LAYOUT.vzb);
   a.id = (int *)at(LAYOUT.id); a.idb = (int *)at(LAYOUT.idb); a.cell_of = (int *)at(LAYOUT.cell_of);
   a.count = (int *)at(LAYOUT.count); a.cursor = (int *)at(LAYOUT.cursor); a.start = (int *)at(LAYOUT.start);
-  a.tile_sums = (int *)at(LAYOUT.tile_sums); a.perm = (int *)at(LAYOUT.perm);
+  a.tile_sums = (int *)at(LAYOUT.tile_sums); a.perm = (int2 *)at(LAYOUT.perm);
   a.pos = (float4 *)at(LAYOUT.pos); a.pos_ref = (float4 *)at(LAYOUT.pos_ref);
   a.nbr = (int32_t *)at(LAYOUT.nbr); a.nnum = (int32_t *)at(LAYOUT.nnum); a.nang = (int32_t *)at(LAYOUT.nang);
   a.nown = (int32_t *)at(LAYOUT.nown); a.nband0 = (int32_t *)at(LAYOUT.nband0); a.nfar = (int32_t *)at(LAYOUT.nfar);
@@ -268,10 +268,11 @@ extern "C" nep_status nep_compute_noalloc(const nep_params *p, int64_t n, const 
   g.lx = (float)l[0]; g.ly = (float)l[1]; g.lz = (float)l[2];
   g.ncx = nc[0]; g.ncy = nc[1]; g.ncz = nc[2];
 
-  // The array keeps the previous call's contents: clear the status word, control block and counters
-  // (cell counters, force accumulators and partial sums are cleared or overwritten by the kernels).
+  // The array keeps the previous call's contents: clear the status word, control block, counters and cell counters
+  // (force accumulators and partial sums are cleared or overwritten by the kernels).
   NA_CUDA(cudaMemsetAsync(ctrl, 0, sizeof(Control), st));
   NA_CUDA(cudaMemsetAsync(counters, 0, 16 * sizeof(long long), st));
+  NA_CUDA(cudaMemsetAsync(a.count, 0, (size_t)a.ncell * sizeof(int), st));
   const double *xin = x;
   if (!device_pointer(x)) {
     NA_CUDA(cudaMemcpyAsync(io, x, 3 * (size_t)N * sizeof(double), cudaMemcpyHostToDevice, st));
