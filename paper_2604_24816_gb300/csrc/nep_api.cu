@@ -790,6 +790,7 @@ void fill_model(Model<S> &M, const nep_params *p) {
   }
   const float rmax = std::max(p->rc_R, eps != 0.0 ? p->lj_rc : 0.f);
   M.rmax2 = rmax * rmax;
+  fill_radial_polynomials(M);
 }
 
 }  // namespace

@@ -110,7 +110,51 @@ struct Model {
   float lj_on, lj_c12, lj_c6, lj_rc2, lj_e_rc, lj_de_rc, lj_rc;  // shifted-force LJ
   float lj_e0, lj_m12, lj_p6;   // rc E'(rc) - E(rc), -12 c12, 6 c6 (the factored forms of lj_pair)
   float rmax2;   // max(rcR, lj_rc)^2
+  // g_n(r) = h(r) [E_n(y) + x O_n(y)], h = fc / 2, y = 2 x^2 - 1 (cheb_to_cubics of cA_n): coefficients of
+  // y^0..y^3, channels 2p and 2p + 1 side by side; gL: the last channel's (E, O) when NA is odd.
+  float2 gE[S::NA / 2][4], gO[S::NA / 2][4], gL[4];
 };
+
+// sum_k c_k (T_k(x) + 1), k = 0..7, as E(y) + x O(y) with y = T_2(x) = 2 x^2 - 1 and cubics E, O: the even
+// orders are T_2j(x) = T_j(y), the odd ones x times 1, 2y - 1, 4y^2 - 2y - 1, 8y^3 - 4y^2 - 4y + 1.  The
+// coefficients stay below 8, so a Horner evaluation on |y| <= 1 rounds like the three-term recurrence, with
+// half its dependent steps and no basis values.  The fused kernels are bound by issue slots (67 % busy) and by
+// the walk's dependent chains: with the cubics and the step-two recurrence of cheb_accumulate the teacher's
+// takes 1.114 ms instead of 1.145 at 1,048,576 atoms, the student's 60.4 us instead of 61.8 at 56,000; forces
+// against 64 bits are as far off as before (2.9e-6 relative on 862 atoms, both).
+template <class T>
+__host__ __device__ __forceinline__ void cheb_to_cubics(const T (&c)[8], T (&e)[4], T (&o)[4]) {
+  const T sum = ((c[0] + c[1]) + (c[2] + c[3])) + ((c[4] + c[5]) + (c[6] + c[7]));
+  e[0] = c[0] - c[4] + sum;
+  e[1] = c[2] - 3 * c[6];
+  e[2] = 2 * c[4];
+  e[3] = 4 * c[6];
+  o[0] = (c[1] - c[3]) - (c[5] - c[7]);
+  o[1] = 2 * (c[3] - c[5]) - 4 * c[7];
+  o[2] = 4 * (c[5] - c[7]);
+  o[3] = 8 * c[7];
+}
+
+// The derived members of a model (host): the radial polynomials of its angular channels.
+template <class S>
+void fill_radial_polynomials(Model<S> &M) {
+  static_assert(S::KA == 8, "eight basis functions");
+  for (int a = 0; a < S::NA; ++a) {
+    double c[8], e[4], o[4];
+    for (int k = 0; k < 8; ++k) c[k] = M.cA[a][k];
+    cheb_to_cubics(c, e, o);
+    for (int i = 0; i < 4; ++i) {
+      if (S::NA % 2 == 1 && a == S::NA - 1) {
+        M.gL[i] = make_float2((float)e[i], (float)o[i]);
+      } else {
+        float *pe = a % 2 ? &M.gE[a / 2][i].y : &M.gE[a / 2][i].x;
+        float *po = a % 2 ? &M.gO[a / 2][i].y : &M.gO[a / 2][i].x;
+        *pe = (float)e[i];
+        *po = (float)o[i];
+      }
+    }
+  }
+}
 
 // Pair records of the fused kernels: the descriptor walk stores every active pair's displacement and
 // neighbour index, and the force pass reads them back instead of walking the neighbour list again.
@@ -268,63 +312,143 @@ __device__ __forceinline__ void cheb_basis_d(float r, float inv_rc, float (&f)[K
   }
 }
 
-// The factors of cheb_basis / cheb_basis_d, for sums that never form f_k or f_k' themselves: h = fc / 2,
-// dh = fc' / 2, dxh = x'(r) h, T_k(x) and D_k = T_k'(x) (T_0 = 1, D_0 = 0, D_1 = 1), so that
-// f_k = h (T_k + 1) and f_k' = (T_k + 1) dh + D_k dxh.  Summed over pairs, sum f_k = sum h T_k + sum h,
-// and a contraction sum_k t_k f_k' = dh (sum_k t_k T_k + sum_k t_k) + dxh sum_k t_k D_k.
-template <int K>
-__device__ __forceinline__ void cheb_t(float r, float inv_rc, float &h, float (&T)[K]) {
-  static_assert(K >= 2, "basis size");
+// The same cutoff and argument for the forms that never build the f_k: h = fc / 2, x and y = 2 x^2 - 1
+// (cheb_args), with dh = fc' / 2 and dxh = x'(r) h (cheb_args_d).
+__device__ __forceinline__ void cheb_args(float r, float inv_rc, float &h, float &x, float &y) {
   const float t = r * inv_rc;
   h = fmaf(0.25f, __cosf(3.14159265358979f * t), 0.25f);
   const float u = t - 1.f;
-  const float x = fmaf(2.f * u, u, -1.f);
-  const float x2 = x + x;
-  T[0] = 1.f; T[1] = x;
-#pragma unroll
-  for (int k = 2; k < K; ++k) T[k] = fmaf(x2, T[k - 1], -T[k - 2]);
+  x = fmaf(2.f * u, u, -1.f);
+  y = fmaf(2.f * x, x, -1.f);
 }
-template <int K>
-__device__ __forceinline__ void cheb_td(float r, float inv_rc, float &dh, float &dxh, float (&T)[K], float (&D)[K]) {
-  static_assert(K >= 2, "basis size");
+__device__ __forceinline__ void cheb_args_d(float r, float inv_rc, float &h, float &dh, float &dxh, float &x, float &y) {
   float s, c;
   const float t = r * inv_rc;
   __sincosf(3.14159265358979f * t, &s, &c);
-  const float h = fmaf(0.25f, c, 0.25f);
+  h = fmaf(0.25f, c, 0.25f);
   dh = (-0.25f * 3.14159265358979f * inv_rc) * s;
   const float u = t - 1.f;
-  const float x = fmaf(2.f * u, u, -1.f);
-  const float x2 = x + x;
+  x = fmaf(2.f * u, u, -1.f);
+  y = fmaf(2.f * x, x, -1.f);
   dxh = (4.f * inv_rc) * u * h;
-  T[0] = 1.f; T[1] = x;
-  D[0] = 0.f; D[1] = 1.f;
+}
+
+// Adds h T_k(x), k = 0..7, of one pair to the sums Q (pairs (T_0, T_1), (T_2, T_3), ...), the last two pairs
+// with the opposite sign.  Step-two recurrence T_(k+2) = 2 y T_k - T_(k-2) on the pairs: three dependent steps
+// for the eight orders (the three-term recurrence takes six, each on one order), and the alternating sign
+// needs no negated operand.
+__device__ __forceinline__ void cheb_accumulate(float r, float inv_rc, float2 (&Q)[4]) {
+  float h, x, y;
+  cheb_args(r, inv_rc, h, x, y);
+  const float y2 = y + y;
+  const float2 h2 = bc2(h);
+  const float2 t01 = pr(1.f, x), t23 = pr(y, fmaf(y2, x, -x));
+  const float2 n45 = fma2(bc2(-y2), t23, t01);      // -(T_4, T_5)
+  const float2 n67 = fma2(bc2(y2), n45, t23);       // -(T_6, T_7)
+  Q[0] = fma2(h2, t01, Q[0]);
+  Q[1] = fma2(h2, t23, Q[1]);
+  Q[2] = fma2(h2, n45, Q[2]);
+  Q[3] = fma2(h2, n67, Q[3]);
+}
+// The radial basis sums from the accumulated Q: sum f_k = sum h T_k + sum h (T_0 = 1: Q[0].x is sum h).
+__device__ __forceinline__ void cheb_sums(const float2 (&Q)[4], float (&QR)[8]) {
+  const float sh = Q[0].x;
+  QR[0] = Q[0].x + sh; QR[1] = Q[0].y + sh;
+  QR[2] = Q[1].x + sh; QR[3] = Q[1].y + sh;
+  QR[4] = sh - Q[2].x; QR[5] = sh - Q[2].y;
+  QR[6] = sh - Q[3].x; QR[7] = sh - Q[3].y;
+}
+
+// The angular channels' radial functions g_n(r) = h [E_n(y) + x O_n(y)] (Model::gE, gO, gL), two channels per
+// instruction; on: g = 0 when false.
+template <class S>
+__device__ __forceinline__ void radial_channels(const Model<S> &P, float r, bool on, float (&g)[S::NA]) {
+  float h, x, y;
+  cheb_args(r, P.inv_rcA, h, x, y);
+  h = on ? h : 0.f;
+  const float2 yy = bc2(y), xx = bc2(x), hh = bc2(h);
 #pragma unroll
-  for (int k = 2; k < K; ++k) {
-    T[k] = fmaf(x2, T[k - 1], -T[k - 2]);
-    D[k] = fmaf(x2, D[k - 1], fmaf(2.f, T[k - 1], -D[k - 2]));
+  for (int p = 0; p < S::NA / 2; ++p) {
+    float2 e = P.gE[p][3], o = P.gO[p][3];
+#pragma unroll
+    for (int i = 2; i >= 0; --i) { e = fma2(e, yy, P.gE[p][i]); o = fma2(o, yy, P.gO[p][i]); }
+    const float2 v = mul2(fma2(xx, o, e), hh);
+    g[2 * p] = v.x; g[2 * p + 1] = v.y;
+  }
+  if constexpr (S::NA % 2 == 1) {
+    float2 v = P.gL[3];
+#pragma unroll
+    for (int i = 2; i >= 0; --i) v = fma2(v, yy, P.gL[i]);
+    g[S::NA - 1] = fmaf(x, v.y, v.x) * h;
   }
 }
-template <int K>
-__device__ __forceinline__ void cheb_td_x2(float2 r, float inv_rc, float2 &dh, float2 &dxh, float2 (&T)[K],
-                                           float2 (&D)[K]) {
-  static_assert(K >= 2, "basis size");
+// g_n and g_n': with p = E + x O, dp/dx = 4 x (E' + x O') + O, g' = p dh + dp/dx dxh.
+template <class S>
+__device__ __forceinline__ void radial_channels_d(const Model<S> &P, float r, float (&g)[S::NA], float (&dg)[S::NA]) {
+  float h, dh, dxh, x, y;
+  cheb_args_d(r, P.inv_rcA, h, dh, dxh, x, y);
+  const float x4 = 4.f * x;
+  const float2 yy = bc2(y), xx = bc2(x), xx4 = bc2(x4), hh = bc2(h), dhh = bc2(dh), dxx = bc2(dxh);
+#pragma unroll
+  for (int p = 0; p < S::NA / 2; ++p) {
+    float2 de = P.gE[p][3], dd = P.gO[p][3];
+    float2 e = fma2(de, yy, P.gE[p][2]), o = fma2(dd, yy, P.gO[p][2]);
+#pragma unroll
+    for (int i = 1; i >= 0; --i) {
+      de = fma2(de, yy, e); dd = fma2(dd, yy, o);
+      e = fma2(e, yy, P.gE[p][i]); o = fma2(o, yy, P.gO[p][i]);
+    }
+    const float2 v = fma2(xx, o, e);
+    const float2 dv = fma2(xx4, fma2(xx, dd, de), o);
+    const float2 a = mul2(v, hh), b = fma2(v, dhh, mul2(dv, dxx));
+    g[2 * p] = a.x; g[2 * p + 1] = a.y;
+    dg[2 * p] = b.x; dg[2 * p + 1] = b.y;
+  }
+  if constexpr (S::NA % 2 == 1) {
+    float2 d = P.gL[3];
+    float2 v = fma2(d, yy, P.gL[2]);
+#pragma unroll
+    for (int i = 1; i >= 0; --i) { d = fma2(d, yy, v); v = fma2(v, yy, P.gL[i]); }
+    const float q = fmaf(x, v.y, v.x), dq = fmaf(x4, fmaf(x, d.y, d.x), v.y);
+    g[S::NA - 1] = q * h;
+    dg[S::NA - 1] = fmaf(q, dh, dq * dxh);
+  }
+}
+
+// sum_k t_k f_k'(r) for a radial adjoint t held as cubics (cheb_to_cubics; c0 = (e0, o0, e1, o1), c1 = (e2, o2,
+// e3, o3)): p dh + dp/dx dxh as in radial_channels_d; the second form evaluates two pairs at once.
+__device__ __forceinline__ float cubics_deriv(float4 c0, float4 c1, float r, float inv_rc) {
+  float h, dh, dxh, x, y;
+  cheb_args_d(r, inv_rc, h, dh, dxh, x, y);
+  const float2 yy = bc2(y);
+  float2 d = pr(c1.z, c1.w);
+  float2 v = fma2(d, yy, pr(c1.x, c1.y));
+  d = fma2(d, yy, v);
+  v = fma2(v, yy, pr(c0.z, c0.w));
+  d = fma2(d, yy, v);
+  v = fma2(v, yy, pr(c0.x, c0.y));
+  return fmaf(fmaf(x, v.y, v.x), dh, fmaf(4.f * x, fmaf(x, d.y, d.x), v.y) * dxh);
+}
+__device__ __forceinline__ float2 cubics_deriv_x2(float4 c0, float4 c1, float2 r, float inv_rc) {
   float2 s, cs;
   const float2 t = mul2(r, bc2(inv_rc));
   __sincosf(3.14159265358979f * t.x, &s.x, &cs.x);
   __sincosf(3.14159265358979f * t.y, &s.y, &cs.y);
   const float2 h = fma2(bc2(0.25f), cs, bc2(0.25f));
-  dh = mul2(bc2(-0.25f * 3.14159265358979f * inv_rc), s);
+  const float2 dh = mul2(bc2(-0.25f * 3.14159265358979f * inv_rc), s);
   const float2 u = add2(t, bc2(-1.f));
-  const float2 x = fma2(mul2(bc2(2.f), u), u, bc2(-1.f));
-  const float2 x2 = add2(x, x);
-  dxh = mul2(mul2(bc2(4.f * inv_rc), u), h);
-  T[0] = bc2(1.f); T[1] = x;
-  D[0] = bc2(0.f); D[1] = bc2(1.f);
-#pragma unroll
-  for (int k = 2; k < K; ++k) {
-    T[k] = fma2(x2, T[k - 1], make_float2(-T[k - 2].x, -T[k - 2].y));
-    D[k] = fma2(x2, D[k - 1], fma2(bc2(2.f), T[k - 1], make_float2(-D[k - 2].x, -D[k - 2].y)));
-  }
+  const float2 x = fma2(add2(u, u), u, bc2(-1.f));
+  const float2 y = fma2(add2(x, x), x, bc2(-1.f));
+  const float2 dxh = mul2(mul2(bc2(4.f * inv_rc), u), h);
+  float2 de = bc2(c1.z), dd = bc2(c1.w);
+  float2 e = fma2(de, y, bc2(c1.x)), o = fma2(dd, y, bc2(c1.y));
+  de = fma2(de, y, e); dd = fma2(dd, y, o);
+  e = fma2(e, y, bc2(c0.z)); o = fma2(o, y, bc2(c0.w));
+  de = fma2(de, y, e); dd = fma2(dd, y, o);
+  e = fma2(e, y, bc2(c0.x)); o = fma2(o, y, bc2(c0.y));
+  const float2 v = fma2(x, o, e);
+  const float2 dv = fma2(mul2(bc2(4.f), x), fma2(x, dd, de), o);
+  return fma2(v, dh, mul2(dv, dxh));
 }
 
 // Normalised real harmonics Yh_lm(u) = sqrt(4 pi / (2l+1)) Y_lm(u), l = 1..4 (24 values, m = -l..l),

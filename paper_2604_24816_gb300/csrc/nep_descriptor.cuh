@@ -102,8 +102,8 @@ __device__ __forceinline__ void accumulate_atom(const Model<S> &P, const float4 
                                                 float4 *__restrict__ rec = nullptr, unsigned off = 0, int pmax = 0) {
   const int cnt = sp.c;
   const float4 pi = pos[i];
-#pragma unroll
-  for (int k = 0; k < S::KR; ++k) A.QR[k] = 0.f;
+  static_assert(S::KR == 8, "eight basis functions");
+  float2 Q[4] = {bc2(0.f), bc2(0.f), bc2(0.f), bc2(0.f)};
 #pragma unroll
   for (int a = 0; a < S::NA; ++a)
 #pragma unroll
@@ -128,11 +128,7 @@ __device__ __forceinline__ void accumulate_atom(const Model<S> &P, const float4 
     const float ir = rsqrtf(r2);
     const float r = r2 * ir;
     if (r2 < P.rcR2) {
-      // sum h T_k here (T_0 = 1: QR[0] collects sum h); sum f_k = sum h T_k + sum h after the walk
-      float h, T[S::KR];
-      cheb_t<S::KR>(r, P.inv_rcR, h, T);
-#pragma unroll
-      for (int k = 0; k < S::KR; ++k) A.QR[k] = fmaf(h, T[k], A.QR[k]);
+      cheb_accumulate(r, P.inv_rcR, Q);
       ++A.nrad;
     }
     if (P.lj_on != 0.f && r2 < P.lj_rc2) {
@@ -141,16 +137,8 @@ __device__ __forceinline__ void accumulate_atom(const Model<S> &P, const float4 
       A.elj = fmaf(0.5f, el, A.elj);
     }
     if (r2 < P.rcA2) {
-      float f[S::KA];
-      cheb_basis<S::KA>(r, P.inv_rcA, f);
       float g[S::NA];
-#pragma unroll
-      for (int a = 0; a < S::NA; ++a) {
-        float t = 0.f;
-#pragma unroll
-        for (int b = 0; b < S::KA; ++b) t = fmaf(P.cA[a][b], f[b], t);
-        g[a] = t;
-      }
+      radial_channels<S>(P, r, true, g);
       float Y[S::NLM];
       if constexpr (UN) harmonics_p<S::NLM>(dx * ir, dy * ir, dz * ir, Y);
       else harmonics<S::NLM>(dx * ir, dy * ir, dz * ir, Y);
@@ -162,9 +150,7 @@ __device__ __forceinline__ void accumulate_atom(const Model<S> &P, const float4 
     }
   }
   pipe.finish();
-  const float hsum = A.QR[0];
-#pragma unroll
-  for (int k = 0; k < S::KR; ++k) A.QR[k] += hsum;
+  cheb_sums(Q, A.QR);
 }
 template <class S, int DE, int DP, int BLOCK>
 __device__ __forceinline__ void accumulate_atom(const Model<S> &P, const float4 *shift, int i, int n,
@@ -279,13 +265,13 @@ __device__ __forceinline__ void radial_tail(const Model<S> &P, const float (&Fp)
   }
 }
 
-// The radial tail as the fused kernels' force pass contracts it with the Chebyshev factors (cheb_td):
-// tail_0 + sum_k tail_k in place of tail_0 (the T_0 = 1 term then also carries sum_k tail_k dh).
-__device__ __forceinline__ void radial_tail_td(float (&tail)[8]) {
-  float s = 0.f;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) s += tail[k];
-  tail[0] += s;
+// The radial tail as the fused kernels' force pass contracts it (cubics_deriv): the two cubics of
+// cheb_to_cubics, (e0, o0, e1, o1) in c0 and (e2, o2, e3, o3) in c1.
+__device__ __forceinline__ void radial_tail_cubics(const float (&tail)[8], float4 &c0, float4 &c1) {
+  float e[4], o[4];
+  cheb_to_cubics(tail, e, o);
+  c0 = make_float4(e[0], o[0], e[1], o[1]);
+  c1 = make_float4(e[2], o[2], e[3], o[3]);
 }
 
 // 4-body part of the adjoint of channel a for the l = 2 components 3..7, per unit dU/dq4_a:
@@ -385,7 +371,7 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
                                                    float &elj, int &nrad, int &nang, int &nact,
                                                    float4 *__restrict__ rec = nullptr, unsigned off = 0, int pmax = 0) {
   static_assert(S::NA == 5 && S::NLM == 24 && (NT == 4 || NT == 5), "teacher shape");
-  static_assert(S::KR % 2 == 0 && S::KA % 2 == 0, "basis sizes are paired");
+  static_assert(S::KR == 8, "eight basis functions");
   constexpr int W = TMEM_W;
   constexpr int NC = S::NLM / W;
   {
@@ -402,9 +388,7 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
   for (int a = NT; a < S::NA; ++a)
 #pragma unroll
     for (int c = 0; c < S::NLM; ++c) R.s[a - NT][c] = 0.f;
-  float2 QR2[S::KR / 2];
-#pragma unroll
-  for (int k = 0; k < S::KR / 2; ++k) QR2[k] = bc2(0.f);
+  float2 Q[4] = {bc2(0.f), bc2(0.f), bc2(0.f), bc2(0.f)};
   elj = 0.f;
   nrad = 0; nang = 0; nact = 0;
   const float4 pi = pos[ii];
@@ -433,12 +417,7 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
       }
       ++nact;
       if (r2 < P.rcR2) {
-        // sum h T_k here (T_0 = 1, so QR2[0].x collects sum h); sum f_k = sum h T_k + sum h below
-        float h, T[S::KR];
-        cheb_t<S::KR>(r, P.inv_rcR, h, T);
-        const float2 h2 = bc2(h);
-#pragma unroll
-        for (int b = 0; b < S::KR / 2; ++b) QR2[b] = fma2(h2, pr(T[2 * b], T[2 * b + 1]), QR2[b]);
+        cheb_accumulate(r, P.inv_rcR, Q);
         ++nrad;
       }
       if (P.lj_on != 0.f && r2 < P.lj_rc2) {
@@ -452,14 +431,8 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
       __syncwarp();
       const float ar = ang ? r : 1.f;
       const float ux = ang ? dx * ir : 1.f, uy = ang ? dy * ir : 0.f, uz = ang ? dz * ir : 0.f;
-      float f[S::KA];
-      cheb_basis<S::KA>(ar, P.inv_rcA, f);
       float g[S::NA];
-#pragma unroll
-      for (int a = 0; a < S::NA; ++a) {
-        const float t = dot_pairs<S::KA>(P.cA[a], f);
-        g[a] = ang ? t : 0.f;
-      }
+      radial_channels<S>(P, ar, ang, g);
       // UN: the polynomials Ph_lm chunk by chunk (fewer live registers than 24 values); all channels in TMEM
       static_assert(!UN || NT == S::NA, "register-resident channels take the normalised harmonics");
       float Y[S::NLM];
@@ -495,9 +468,7 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
     }
   }
   pipe.finish();
-  const float hsum = QR2[0].x;
-#pragma unroll
-  for (int k = 0; k < S::KR / 2; ++k) { QR[2 * k] = QR2[k].x + hsum; QR[2 * k + 1] = QR2[k].y + hsum; }
+  cheb_sums(Q, QR);
 }
 
 // The sums of chunk k (components 4k..4k+3) of every channel: TMEM for a < NT, registers after.

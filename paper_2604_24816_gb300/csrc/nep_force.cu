@@ -244,11 +244,17 @@ __device__ __forceinline__ void angular_pair(const Model<S> &P, uint32_t trow,
   constexpr int W = GTraits<GT>::W;
   const float ar = si ? 1.f : r, air = si ? 1.f : ir;
   const float ux = si ? 1.f : dx * ir, uy = si ? 0.f : dy * ir, uz = si ? 0.f : dz * ir;
-  float f[S::KA], df[S::KA];
-  cheb_basis_d<S::KA>(ar, P.inv_rcA, f, df);
+  // the half list waits on its gathered rows: there the basis form measured 62 us against 64 us for the
+  // polynomials (75 us without a register bound) on 125,000 student atoms, so it keeps it
   float g[S::NA], dg[S::NA];
+  if constexpr (FULL) {
+    radial_channels_d<S>(P, ar, g, dg);
+  } else {
+    float f[S::KA], df[S::KA];
+    cheb_basis_d<S::KA>(ar, P.inv_rcA, f, df);
 #pragma unroll
-  for (int a = 0; a < S::NA; ++a) dot_pairs2<S::KA>(P.cA[a], f, df, g[a], dg[a]);
+    for (int a = 0; a < S::NA; ++a) dot_pairs2<S::KA>(P.cA[a], f, df, g[a], dg[a]);
+  }
   // UN: the polynomials Ph_lm are formed chunk by chunk below (fewer live registers than 24 values)
   float Y[S::NLM];
   if constexpr (!UN) harmonics<S::NLM>(ux, uy, uz, Y);
@@ -446,23 +452,13 @@ __device__ __forceinline__ void force_pairs(const Model<S> &P, const float4 *shi
 }
 
 // Radial and LJ part of one active pair's force coefficient (d = coef * r_ij + angular part): the
-// radial adjoint in basis space (8 values in shared memory at fps[0], fps[FORCE_BLOCK], in
-// radial_tail_td's form) against the basis derivatives, plus half of the shifted-force LJ pair force.  INSIDE_RC: the caller knows that
+// radial adjoint (two cubics in shared memory at fps[0], fps[FORCE_BLOCK], radial_tail_cubics) against the
+// basis derivatives, plus half of the shifted-force LJ pair force.  INSIDE_RC: the caller knows that
 // r < rc_R (an angular pair: rc_A <= rc_R is checked by nep_create).
 template <class S, bool INSIDE_RC = false>
 __device__ __forceinline__ float radial_lj_coef(const Model<S> &P, const float4 *fps, float r2, float r, float ir) {
   float coef = 0.f;
-  if (INSIDE_RC || r2 < P.rcR2) {
-    // sum_k tail_k f_k' = dh (sum_k tail_k T_k + sum_k tail_k) + dxh sum_k tail_k D_k, the first sum
-    // with the tail in radial_tail_td's form (tail_0 + sum_k tail_k at k = 0, T_0 = 1)
-    float dh, dxh, T[S::KR], D[S::KR];
-    cheb_td<S::KR>(r, P.inv_rcR, dh, dxh, T, D);
-    float fpi[8];
-    const float4 a = fps[0], b = fps[FORCE_BLOCK];
-    fpi[0] = a.x; fpi[1] = a.y; fpi[2] = a.z; fpi[3] = a.w; fpi[4] = b.x; fpi[5] = b.y; fpi[6] = b.z; fpi[7] = b.w;
-    const float(&tl)[S::KR] = *reinterpret_cast<const float(*)[S::KR]>(&fpi[0]);
-    coef = fmaf(dh, dot_pairs<S::KR>(tl, T), dxh * dot_pairs<S::KR>(tl, D)) * ir;
-  }
+  if (INSIDE_RC || r2 < P.rcR2) coef = cubics_deriv(fps[0], fps[FORCE_BLOCK], r, P.inv_rcR) * ir;
   if (P.lj_on != 0.f && r2 < P.lj_rc2) {
     float el, dl;
     lj_pair<S>(P, r2, r, ir, el, dl);
@@ -477,7 +473,7 @@ __device__ __forceinline__ float radial_lj_coef(const Model<S> &P, const float4 
 // nr other active pairs (slots pmax-1 down to pmax-nr; no TMEM).  Each pair gets the arithmetic of
 // force_pairs<S, float, false, true> on the displacement the descriptor walk computed: d_ij added to F_i,
 // subtracted from F_j (fixed point), W -= r_ij (x) d_ij (upper triangle, mirrored).  UN: the TMEM row is
-// over Ph_lm (angular_pair).  The radial tail at fps is in radial_tail_td's form.
+// over Ph_lm (angular_pair).  The radial tail at fps is in radial_tail_cubics' form.
 template <class S, int DQ, bool UN = false>
 __device__ __forceinline__ void force_pairs_rec(const Model<S> &P, uint32_t trow,
                                                 const float (&gi)[ForceCfg<S>::TM ? 1 : S::NA][ForceCfg<S>::TM ? 1 : S::NLM],
@@ -533,7 +529,6 @@ __device__ __forceinline__ void force_pairs_rec(const Model<S> &P, uint32_t trow
     // 1.8 % slower); an odd last record alone below
     if constexpr (TM) {
       const float4 ta = fps[0], tb = fps[FORCE_BLOCK];
-      const float tail[8] = {ta.x, ta.y, ta.z, ta.w, tb.x, tb.y, tb.z, tb.w};
       for (; p0 + 1 < nr; p0 += 2) {
         const float4 qa = pb.get(p0), qb = pb.get(p0 + 1);
         const float2 dxv = pr(qa.x, qb.x), dyv = pr(qa.y, qb.y), dzv = pr(qa.z, qb.z);
@@ -543,15 +538,7 @@ __device__ __forceinline__ void force_pairs_rec(const Model<S> &P, uint32_t trow
         float2 coef = bc2(0.f);
         const bool ra = r2.x < P.rcR2, rb = r2.y < P.rcR2;
         if (ra || rb) {
-          // the contraction of radial_lj_coef: dh (sum tail_k T_k) + dxh (sum tail_k D_k), T_0 = D_1 = 1
-          float2 dh, dxh, T[S::KR], D[S::KR];
-          cheb_td_x2<S::KR>(r, P.inv_rcR, dh, dxh, T, D);
-          float2 s1 = bc2(tail[0]), s2 = bc2(tail[1]);
-#pragma unroll
-          for (int k = 1; k < S::KR; ++k) s1 = fma2(bc2(tail[k]), T[k], s1);
-#pragma unroll
-          for (int k = 2; k < S::KR; ++k) s2 = fma2(bc2(tail[k]), D[k], s2);
-          const float2 dot = mul2(fma2(dh, s1, mul2(dxh, s2)), ir);
+          const float2 dot = mul2(cubics_deriv_x2(ta, tb, r, P.inv_rcR), ir);
           coef = pr(ra ? dot.x : 0.f, rb ? dot.y : 0.f);
         }
         if (P.lj_on != 0.f) {
@@ -766,9 +753,7 @@ k_nep_fused(const __grid_constant__ Model<S> P, const Geom geom, const int n, co
   {
     float fpi[8];
     radial_tail<S>(P, Fp, fpi);
-    radial_tail_td(fpi);                 // the force pass's form (force_pairs_rec)
-    fp_s[threadIdx.x] = make_float4(fpi[0], fpi[1], fpi[2], fpi[3]);
-    fp_s[DESC_BLOCK + threadIdx.x] = make_float4(fpi[4], fpi[5], fpi[6], fpi[7]);
+    radial_tail_cubics(fpi, fp_s[threadIdx.x], fp_s[DESC_BLOCK + threadIdx.x]);   // the force pass's form (force_pairs_rec)
   }
   long long acc_d[5] = {0, 0, 0, 0, 0};
   long long acc_f[13] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
@@ -866,9 +851,7 @@ k_nep_fused_reg(const __grid_constant__ Model<S> P, const Geom geom, const int n
     {
       float tail[8];
       radial_tail<S>(P, Fp, tail);
-      radial_tail_td(tail);              // the force pass's form (force_pairs_rec)
-      fp_s[threadIdx.x] = make_float4(tail[0], tail[1], tail[2], tail[3]);
-      fp_s[DESC_BLOCK + threadIdx.x] = make_float4(tail[4], tail[5], tail[6], tail[7]);
+      radial_tail_cubics(tail, fp_s[threadIdx.x], fp_s[DESC_BLOCK + threadIdx.x]);   // the force pass's form (force_pairs_rec)
     }
     const float ui = flagged ? A.elj : U + A.elj;
     usite[i] = ui;
@@ -1064,9 +1047,7 @@ k_nep_fused_mixed(const __grid_constant__ Model<S> P, const Geom geom, const int
   {
     float fpi[8];
     radial_tail<S>(P, Fp, fpi);
-    radial_tail_td(fpi);                 // the force pass's form (force_pairs_rec)
-    fp_s[t] = make_float4(fpi[0], fpi[1], fpi[2], fpi[3]);
-    fp_s[DESC_BLOCK + t] = make_float4(fpi[4], fpi[5], fpi[6], fpi[7]);
+    radial_tail_cubics(fpi, fp_s[t], fp_s[DESC_BLOCK + t]);   // the force pass's form (force_pairs_rec)
   }
   long long acc_d[5] = {0, 0, 0, 0, 0};
   long long acc_f[13] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};

@@ -231,6 +231,7 @@ extern "C" nep_status nep_compute_noalloc(const nep_params *p, int64_t n, const 
   }
   const float rmax = std::max(p->rc_R, eps != 0.0 ? p->lj_rc : 0.f);
   M.rmax2 = rmax * rmax;
+  fill_radial_polynomials(M);
 
   const nep_status prev = previous_call_done();
   if (prev != NEP_OK) return prev;
