@@ -220,12 +220,31 @@ __device__ __forceinline__ void fill_shift_table(float4 *tab, const Geom &g) {
 // Packed float2 arithmetic: two FP32 operations per instruction on the sm_100 family (FFMA2, FADD2,
 // FMUL2), each rounded as its scalar counterpart.  The hot loops pair independent operations so that
 // they issue half as many FP32 instructions.
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 bc2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 pr(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ float hsum(float2 a) { return a.x + a.y; }
+// (The host forms serve the host-side checks.)
+__host__ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+#ifdef __CUDA_ARCH__
+  return __ffma2_rn(a, b, c);
+#else
+  return make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
+#endif
+}
+__host__ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
+#ifdef __CUDA_ARCH__
+  return __fadd2_rn(a, b);
+#else
+  return make_float2(a.x + b.x, a.y + b.y);
+#endif
+}
+__host__ __device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+#ifdef __CUDA_ARCH__
+  return __fmul2_rn(a, b);
+#else
+  return make_float2(a.x * b.x, a.y * b.y);
+#endif
+}
+__host__ __device__ __forceinline__ float2 bc2(float a) { return make_float2(a, a); }
+__host__ __device__ __forceinline__ float2 pr(float a, float b) { return make_float2(a, b); }
+__host__ __device__ __forceinline__ float hsum(float2 a) { return a.x + a.y; }
 
 // sum_k c[k] f[k] (K even) as K/2 paired multiply-adds (even and odd k accumulated apart) and one add.
 template <int K>
@@ -542,9 +561,8 @@ __host__ __device__ constexpr int harmonic_grad_mask(int lm) {
 }
 
 // The same harmonics without their constant factors: Yh_lm = hnorm(lm) Ph_lm, with Ph_lm (harmonics_p)
-// a polynomial with small integer coefficients.  A sum or an adjoint row kept over Ph instead of Yh
-// (s'_nlm = s_nlm / hnorm(lm), G'_nlm = hnorm(lm) G_nlm) gives the same products G s and G dYh/du with
-// the per-pair constant multiplies moved to one multiply per atom and component.
+// a polynomial with small integer coefficients: an independent form that the host-side checks compare the
+// kernels' harmonics with (the fused kernels use the solid harmonics of nep_solid.cuh).
 __host__ __device__ constexpr float hnorm(int lm) {
   constexpr float s3 = 1.7320508075688772f, s5 = 2.2360679774997896f, s6 = 2.449489742783178f;
   constexpr float s10 = 3.1622776601683795f, s15 = 3.872983346207417f, s35 = 5.916079783099616f;
@@ -593,8 +611,7 @@ __host__ __device__ __forceinline__ void harmonics_p(float x, float y, float z, 
   }
 }
 
-// Ph_lm alone (lm a compile-time constant after unrolling), for loops that form the components chunk by
-// chunk instead of holding all 24.
+// Ph_lm alone (lm a compile-time constant after unrolling).
 __host__ __device__ __forceinline__ float harmonic_p(int lm, float x, float y, float z) {
   const float x2 = x * x, y2 = y * y, z2 = z * z;
   const float xy = x * y, d = x2 - y2, e = x2 + y2;
@@ -680,17 +697,10 @@ __device__ __forceinline__ void harmonic_grad_acc(int lm, float x, float y, floa
 
 // The same for the two components lm0, lm0 + 1 with weights b = (b_lm0, b_lm0+1), accumulated into the
 // component pairs g[d] (even and odd lm apart): paired multiply-adds where both are non-zero.
-// UN: the gradients of the polynomials Ph (harmonic_grad_p), for weights taken over Ph.
-template <bool UN = false>
 __device__ __forceinline__ void harmonic_grad_acc2(int lm0, float x, float y, float z, float2 b, float2 (&g)[3]) {
   float a0[3], a1[3];
-  if constexpr (UN) {
-    harmonic_grad_p(lm0, x, y, z, a0);
-    harmonic_grad_p(lm0 + 1, x, y, z, a1);
-  } else {
-    harmonic_grad(lm0, x, y, z, a0);
-    harmonic_grad(lm0 + 1, x, y, z, a1);
-  }
+  harmonic_grad(lm0, x, y, z, a0);
+  harmonic_grad(lm0 + 1, x, y, z, a1);
   const int m0 = harmonic_grad_mask(lm0), m1 = harmonic_grad_mask(lm0 + 1);
 #pragma unroll
   for (int d = 0; d < 3; ++d) {

@@ -8,6 +8,7 @@
 #include <cuda_fp16.h>
 
 #include "nep_common.cuh"
+#include "nep_solid.cuh"
 #include "nep_tc.cuh"
 
 namespace nep {
@@ -94,8 +95,8 @@ struct AtomSums {
 // Walk atom i's full neighbour row and accumulate q_n, s_nlm and the LJ energy.  REC: every active pair
 // is also recorded as (dx, dy, dz, j) at rec[off + slot * BLOCK], angular pairs from slot 0 up and the
 // other active pairs from slot pmax - 1 down (the layout of accumulate_atom_tm's records).
-// UN: the sums over the polynomials Ph_lm without their constant factors (s' = s / hnorm, harmonics_p).
-template <class S, int DE, int DP, int BLOCK, bool REC = false, bool UN = false>
+// SOLID: the sums over the solid harmonics (s' = s / solid_norm, in the order of nep_solid.cuh).
+template <class S, int DE, int DP, int BLOCK, bool REC = false, bool SOLID = false>
 __device__ __forceinline__ void accumulate_atom(const Model<S> &P, const float4 *shift, int i, int n,
                                                 const float4 *__restrict__ pos, const int32_t *__restrict__ nbr,
                                                 RowSpan sp, uint32_t *ring_e, float4 *ring_p, AtomSums<S> &A,
@@ -140,8 +141,17 @@ __device__ __forceinline__ void accumulate_atom(const Model<S> &P, const float4 
       float g[S::NA];
       radial_channels<S>(P, r, true, g);
       float Y[S::NLM];
-      if constexpr (UN) harmonics_p<S::NLM>(dx * ir, dy * ir, dz * ir, Y);
-      else harmonics<S::NLM>(dx * ir, dy * ir, dz * ir, Y);
+      if constexpr (SOLID) {
+        const Solid<S::NLM> H(dx * ir, dy * ir, dz * ir);
+#pragma unroll
+        for (int k = 0; k < S::NLM / 4; ++k) {
+          float2 y01, y23;
+          H.chunk(k, y01, y23);
+          Y[4 * k] = y01.x; Y[4 * k + 1] = y01.y; Y[4 * k + 2] = y23.x; Y[4 * k + 3] = y23.y;
+        }
+      } else {
+        harmonics<S::NLM>(dx * ir, dy * ir, dz * ir, Y);
+      }
 #pragma unroll
       for (int a = 0; a < S::NA; ++a)
 #pragma unroll
@@ -186,8 +196,8 @@ __device__ __forceinline__ void fourbody_tensors(const float (&s2)[S::NA][5], Fo
 }
 
 // Descriptors [q_n | q_nl (n-major, l = 1..LMAX) | q4_n = tr(T_n^3) = 3 det T_n (teacher shape only)].
-// UN: A holds s'_nlm (accumulate_atom<.., UN>), scaled by hnorm(lm) here.
-template <class S, bool UN = false>
+// SOLID: A holds s' (accumulate_atom<.., SOLID>), scaled by solid_norm here.
+template <class S, bool SOLID = false>
 __device__ __forceinline__ void descriptors_of(const Model<S> &P, const AtomSums<S> &A, float (&q)[S::NDES],
                                                FourBody<S> &T) {
 #pragma unroll
@@ -200,22 +210,21 @@ __device__ __forceinline__ void descriptors_of(const Model<S> &P, const AtomSums
 #pragma unroll
   for (int a = 0; a < S::NA; ++a) {
 #pragma unroll
-    for (int l = 1; l <= S::LMAX; ++l) {
-      float t = 0.f;
+    for (int l = 1; l <= S::LMAX; ++l) q[S::NR + a * S::LMAX + (l - 1)] = 0.f;
 #pragma unroll
-      for (int c = l * l - 1; c < (l + 1) * (l + 1) - 1; ++c) {
-        const float sc = UN ? hnorm(c) * A.s[a][c] : A.s[a][c];
-        t = fmaf(sc, sc, t);
-      }
-      q[S::NR + a * S::LMAX + (l - 1)] = t;
+    for (int c = 0; c < S::NLM; ++c) {
+      const float sc = SOLID ? solid_norm(S::NLM, c) * A.s[a][c] : A.s[a][c];
+      float &ql = q[S::NR + a * S::LMAX + (SOLID ? solid_l(S::NLM, c) : lm_l(c)) - 1];
+      ql = fmaf(sc, sc, ql);
     }
   }
   if constexpr (S::FOURBODY) {
+    static_assert(!SOLID, "the register-resident solid-harmonic rows have no 4-body term");
     float s2[S::NA][5];
 #pragma unroll
     for (int a = 0; a < S::NA; ++a)
 #pragma unroll
-      for (int m = 0; m < 5; ++m) s2[a][m] = UN ? hnorm(3 + m) * A.s[a][3 + m] : A.s[a][3 + m];
+      for (int m = 0; m < 5; ++m) s2[a][m] = A.s[a][3 + m];
     fourbody_tensors<S>(s2, T, q);
   }
 }
@@ -294,21 +303,22 @@ __device__ __forceinline__ void fourbody_adjoint(int a, const FourBody<S> &T, fl
 
 // Adjoint of channel a: gl[c] = dU/ds_{a,c} = 2 Fp_{a,l(c)} s_{a,c} (+ 4-body gradient for l = 2:
 // d tr(T^3)/d s_m = 3 (T^2) : dT/ds_m).
-// UN: A holds s'_nlm and the row is G'_nlm = hnorm(lm) G_nlm (adjoint_chunk).
-template <class S, bool UN = false>
+// SOLID: A holds s' and the row is G' = solid_norm G, over the solid harmonics (adjoint_chunk).
+template <class S, bool SOLID = false>
 __device__ __forceinline__ void adjoint_channel(int a, const AtomSums<S> &A, const FourBody<S> &T,
                                                 const float (&Fp)[S::NDES], float (&gl)[S::NLM]) {
 #pragma unroll
   for (int c = 0; c < S::NLM; ++c) {
-    const float h = UN ? hnorm(c) : 1.f;
-    gl[c] = (2.f * h * h) * Fp[S::NR + a * S::LMAX + lm_l(c) - 1] * A.s[a][c];
+    const float h = SOLID ? solid_norm(S::NLM, c) : 1.f;
+    gl[c] = (2.f * h * h) * Fp[S::NR + a * S::LMAX + (SOLID ? solid_l(S::NLM, c) : lm_l(c)) - 1] * A.s[a][c];
   }
   if constexpr (S::FOURBODY) {
+    static_assert(!SOLID, "the register-resident solid-harmonic rows have no 4-body term");
     const float f4 = Fp[S::NR + S::NA * S::LMAX + a];
     float g4[5];
     fourbody_adjoint<S>(a, T, g4);
 #pragma unroll
-    for (int m = 0; m < 5; ++m) gl[3 + m] = fmaf(UN ? hnorm(3 + m) * f4 : f4, g4[m], gl[3 + m]);
+    for (int m = 0; m < 5; ++m) gl[3 + m] = fmaf(f4, g4[m], gl[3 + m]);
   }
 }
 
@@ -363,7 +373,7 @@ __device__ __forceinline__ void tm_store(uint32_t trow, int k, const float (&v)[
 // thread's column of a [pmax][BLOCK] array): angular pairs (r < rc_A) from
 // slot 0 up in walk order, the other active pairs from slot pmax - 1 down (pmax >= the row length, so
 // the two never meet).
-template <class S, int NT, int DE, int DP, int BLOCK, bool REC = false, bool UN = false>
+template <class S, int NT, int DE, int DP, int BLOCK, bool REC = false, bool SOLID = false>
 __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const float4 *shift, uint32_t trow, int ii,
                                                    int n, const float4 *__restrict__ pos,
                                                    const int32_t *__restrict__ nbr, RowSpan sp, uint32_t *ring_e,
@@ -433,18 +443,18 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
       const float ux = ang ? dx * ir : 1.f, uy = ang ? dy * ir : 0.f, uz = ang ? dz * ir : 0.f;
       float g[S::NA];
       radial_channels<S>(P, ar, ang, g);
-      // UN: the polynomials Ph_lm chunk by chunk (fewer live registers than 24 values); all channels in TMEM
-      static_assert(!UN || NT == S::NA, "register-resident channels take the normalised harmonics");
+      // SOLID: the components chunk by chunk (fewer live registers than 24 values); all channels in TMEM
+      static_assert(!SOLID || NT == S::NA, "register-resident channels take the normalised harmonics");
+      const Solid<S::NLM> H(ux, uy, uz);
       float Y[S::NLM];
-      if constexpr (!UN) harmonics<S::NLM>(ux, uy, uz, Y);
+      if constexpr (!SOLID) harmonics<S::NLM>(ux, uy, uz, Y);
 #pragma unroll
       for (int k = 0; k < NC; ++k) {
         float sv[S::NA][W];
         tm_load<S, NT>(trow, k, sv);
         float2 y01, y23;
-        if constexpr (UN) {
-          y01 = pr(harmonic_p(W * k, ux, uy, uz), harmonic_p(W * k + 1, ux, uy, uz));
-          y23 = pr(harmonic_p(W * k + 2, ux, uy, uz), harmonic_p(W * k + 3, ux, uy, uz));
+        if constexpr (SOLID) {
+          H.chunk(k, y01, y23);
         } else {
           y01 = pr(Y[W * k], Y[W * k + 1]);
           y23 = pr(Y[W * k + 2], Y[W * k + 3]);
@@ -483,8 +493,8 @@ __device__ __forceinline__ void sums_chunk(uint32_t trow, int k, const RegSums<S
 
 // Descriptors from the radial basis sums and the sums s_nlm (q_nl = sum_m s_nlm^2, 4-body from the
 // l = 2 sums), as descriptors_of.
-// UN: sums over Ph_lm (accumulate_atom_tm), scaled by hnorm(lm) here.
-template <class S, int NT, bool UN = false>
+// SOLID: sums over the solid harmonics (accumulate_atom_tm), scaled by solid_norm here.
+template <class S, int NT, bool SOLID = false>
 __device__ __forceinline__ void descriptors_tm(const Model<S> &P, uint32_t trow, const float (&QR)[S::KR],
                                                const RegSums<S, NT> &R, float (&q)[S::NDES], FourBody<S> &T) {
   constexpr int W = TMEM_W;
@@ -507,33 +517,36 @@ __device__ __forceinline__ void descriptors_tm(const Model<S> &P, uint32_t trow,
 #pragma unroll
       for (int cc = 0; cc < W; ++cc) {
         const int lm = W * k + cc;
-        if constexpr (UN) sv[a][cc] *= hnorm(lm);
-        float &ql = q[S::NR + a * S::LMAX + lm_l(lm) - 1];
+        if constexpr (SOLID) sv[a][cc] *= solid_norm(S::NLM, lm);
+        float &ql = q[S::NR + a * S::LMAX + (SOLID ? solid_l(S::NLM, lm) : lm_l(lm)) - 1];
         ql = fmaf(sv[a][cc], sv[a][cc], ql);
-        if (lm >= 3 && lm < 8) s2[a][lm - 3] = sv[a][cc];
+        const int m2 = SOLID ? solid_quadrupole(S::NLM, lm) : (lm >= 3 && lm < 8 ? lm - 3 : -1);
+        if (m2 >= 0) s2[a][m2 < 0 ? 0 : m2] = sv[a][cc];
       }
   }
   fourbody_tensors<S>(s2, T, q);
 }
 
 // 4-body adjoint factors g4[a] = 3 (T_a^2) : dT_a/ds_m of every channel, with the tensors T_a rebuilt
-// from the l = 2 sums (components 3..7: chunk 0 holds component 3, chunk 1 components 4..7), so that
-// T need not stay live across the network.
-template <class S, int NT, bool UN = false>
+// from the l = 2 sums (chunks 0 and 1, and the zonal component of chunk 5 with SOLID), so that T need not
+// stay live across the network.
+template <class S, int NT, bool SOLID = false>
 __device__ __forceinline__ void fourbody_adjoint_tm(uint32_t trow, const RegSums<S, NT> &R, float (&g4)[S::NA][5]) {
   static_assert(S::FOURBODY && S::NLM == 24, "teacher shape");
-  float c0[S::NA][TMEM_W], c1[S::NA][TMEM_W];
-  sums_chunk<S, NT>(trow, 0, R, c0);
-  sums_chunk<S, NT>(trow, 1, R, c1);
   float s2[S::NA][5];
 #pragma unroll
-  for (int a = 0; a < S::NA; ++a) {
-    s2[a][0] = c0[a][3];
+  for (int k = 0; k < S::NLM / TMEM_W; ++k) {
+    if (!(k < 2 || (SOLID && k == 5))) continue;
+    float sv[S::NA][TMEM_W];
+    sums_chunk<S, NT>(trow, k, R, sv);
 #pragma unroll
-    for (int m = 1; m < 5; ++m) s2[a][m] = c1[a][m - 1];
-    if constexpr (UN) {
+    for (int cc = 0; cc < TMEM_W; ++cc) {
+      const int lm = TMEM_W * k + cc;
+      const int m2 = SOLID ? solid_quadrupole(S::NLM, lm) : (lm >= 3 && lm < 8 ? lm - 3 : -1);
+      if (m2 >= 0) {
 #pragma unroll
-      for (int m = 0; m < 5; ++m) s2[a][m] *= hnorm(3 + m);
+        for (int a = 0; a < S::NA; ++a) s2[a][m2 < 0 ? 0 : m2] = SOLID ? solid_norm(S::NLM, lm) * sv[a][cc] : sv[a][cc];
+      }
     }
   }
   FourBody<S> T;
@@ -545,18 +558,19 @@ __device__ __forceinline__ void fourbody_adjoint_tm(uint32_t trow, const RegSums
 
 // The adjoint of components c..c+3 of channel a, gl = 2 Fp_{a,l} s + (4-body terms for l = 2), as
 // adjoint_channel; g4 = fourbody_adjoint of channel a.
-// UN: sv holds s'_nlm (sums over Ph_lm) and the row is G'_nlm = hnorm(lm) G_nlm, the weights of Ph_lm:
-// G' = 2 hnorm^2 Fp s' + hnorm f4 g4.
-template <class S, bool UN = false>
+// SOLID: sv holds s' (sums over the solid harmonics) and the row is G' = norm G, the weights of the solid
+// harmonics: G' = 2 norm^2 Fp s' + norm f4 g4.
+template <class S, bool SOLID = false>
 __device__ __forceinline__ void adjoint_chunk(int a, int c, const float (&sv)[TMEM_W], const float (&g4)[5],
                                               const float (&Fp)[S::NDES], float (&gl)[TMEM_W]) {
 #pragma unroll
   for (int cc = 0; cc < TMEM_W; ++cc) {
     const int lm = c + cc;
-    const float h = UN ? hnorm(lm) : 1.f;
-    gl[cc] = (2.f * h * h) * Fp[S::NR + a * S::LMAX + lm_l(lm) - 1] * sv[cc];
-    if (S::FOURBODY && lm >= 3 && lm < 8)
-      gl[cc] = fmaf(UN ? h * Fp[S::NR + S::NA * S::LMAX + a] : Fp[S::NR + S::NA * S::LMAX + a], g4[lm - 3], gl[cc]);
+    const float h = SOLID ? solid_norm(S::NLM, lm) : 1.f;
+    gl[cc] = (2.f * h * h) * Fp[S::NR + a * S::LMAX + (SOLID ? solid_l(S::NLM, lm) : lm_l(lm)) - 1] * sv[cc];
+    const int m2 = SOLID ? solid_quadrupole(S::NLM, lm) : (lm >= 3 && lm < 8 ? lm - 3 : -1);
+    if (S::FOURBODY && m2 >= 0)
+      gl[cc] = fmaf(h * Fp[S::NR + S::NA * S::LMAX + a], g4[m2 < 0 ? 0 : m2], gl[cc]);
   }
 }
 

@@ -233,9 +233,9 @@ struct ForceCfg {
 // H = G^i (FULL; in TMEM at trow for the teacher shape, else in gi) or G^i + (-1)^l G^j (half list, G^j
 // gathered from Gj).  Returns sum_lm (A_lm - l B_lm / r) Yh_lm (al, even and odd lm apart) and
 // sum_lm B_lm grad P_lm(u) (gv), A_lm = sum_n H_nlm g_n'(r), B_lm = sum_n H_nlm g_n(r).  si: a stand-in
-// pair (r = 1 along x) for lanes that only take part in the warp-collective TMEM loads.  UN: the row
-// holds G'_nlm = hnorm(lm) G_nlm, the weights of the polynomials Ph_lm (harmonics_p).
-template <class S, class GT, bool FULL, bool UN = false>
+// pair (r = 1 along x) for lanes that only take part in the warp-collective TMEM loads.  (The separate force
+// kernels; the fused ones use angular_pair_solid.)
+template <class S, class GT, bool FULL>
 __device__ __forceinline__ void angular_pair(const Model<S> &P, uint32_t trow,
                                              const float (&gi)[ForceCfg<S>::TM ? 1 : S::NA][ForceCfg<S>::TM ? 1 : S::NLM],
                                              const GT *__restrict__ Gj, bool si, float r, float ir, float dx, float dy,
@@ -255,9 +255,8 @@ __device__ __forceinline__ void angular_pair(const Model<S> &P, uint32_t trow,
 #pragma unroll
     for (int a = 0; a < S::NA; ++a) dot_pairs2<S::KA>(P.cA[a], f, df, g[a], dg[a]);
   }
-  // UN: the polynomials Ph_lm are formed chunk by chunk below (fewer live registers than 24 values)
   float Y[S::NLM];
-  if constexpr (!UN) harmonics<S::NLM>(ux, uy, uz, Y);
+  harmonics<S::NLM>(ux, uy, uz, Y);
   const float2 air2 = bc2(air);
   // d/dd [g_n(r) Yh_lm(u)] = (g_n' - l g_n / r) Yh_lm u + (g_n / r) grad P_lm(u); per component
   // A_lm = sum_n H_nlm g_n', B_lm = sum_n H_nlm g_n, in pairs of consecutive components (lm, lm + 1)
@@ -309,16 +308,88 @@ __device__ __forceinline__ void angular_pair(const Model<S> &P, uint32_t trow,
     }
     const float2 nl01 = mul2(pr(-(float)lm_l(lm0), -(float)lm_l(lm0 + 1)), air2);
     const float2 nl23 = mul2(pr(-(float)lm_l(lm0 + 2), -(float)lm_l(lm0 + 3)), air2);
-    if constexpr (UN) {
-      al = fma2(fma2(nl01, bv01, av01), pr(harmonic_p(lm0, ux, uy, uz), harmonic_p(lm0 + 1, ux, uy, uz)), al);
-      al = fma2(fma2(nl23, bv23, av23), pr(harmonic_p(lm0 + 2, ux, uy, uz), harmonic_p(lm0 + 3, ux, uy, uz)), al);
-    } else {
-      al = fma2(fma2(nl01, bv01, av01), pr(Y[lm0], Y[lm0 + 1]), al);
-      al = fma2(fma2(nl23, bv23, av23), pr(Y[lm0 + 2], Y[lm0 + 3]), al);
-    }
-    harmonic_grad_acc2<UN>(lm0, ux, uy, uz, bv01, gv);
-    harmonic_grad_acc2<UN>(lm0 + 2, ux, uy, uz, bv23, gv);
+    al = fma2(fma2(nl01, bv01, av01), pr(Y[lm0], Y[lm0 + 1]), al);
+    al = fma2(fma2(nl23, bv23, av23), pr(Y[lm0 + 2], Y[lm0 + 3]), al);
+    harmonic_grad_acc2(lm0, ux, uy, uz, bv01, gv);
+    harmonic_grad_acc2(lm0 + 2, ux, uy, uz, bv23, gv);
   }
+}
+
+// The adjoint row of an atom as angular_pair_solid reads it, four components of every channel at a time.
+template <class S>
+struct RowTmem {
+  uint32_t trow;
+  __device__ __forceinline__ void load(int k, float (&h)[S::NA][4]) const { tm_load<S, S::NA>(trow, k, h); }
+};
+template <class S>
+struct RowReg {
+  const float (&g)[S::NA][S::NLM];
+  __device__ __forceinline__ void load(int k, float (&h)[S::NA][4]) const {
+#pragma unroll
+    for (int a = 0; a < S::NA; ++a)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) h[a][c] = g[a][4 * k + c];
+  }
+};
+
+// The same force part for a row over the solid harmonics (G' = solid_norm G): with f_lm = R_lm(u), homogeneous
+// of degree l in u, d/dd [g(r) f(u)] = g' f u + (g / r) (grad f - u (u . grad f)), so no factor l appears:
+// al = sum_lm A_lm R_lm and gv = sum_lm B_lm grad R_lm (SolidGrad) give the force (al - u . gv / r) u + gv / r.
+// The zonal weights come first (their chunk is the row's last), since each degree's gradient needs its own.
+template <class S, class Row>
+__device__ __forceinline__ void angular_pair_solid(const Model<S> &P, const Row &row, bool si, float r, float ir,
+                                                   float dx, float dy, float dz, float &coef, float &vx, float &vy,
+                                                   float &vz) {
+  constexpr int NP = solid_pairs(S::NLM), NC = S::NLM / 4;
+  const float ar = si ? 1.f : r;
+  const float ux = si ? 1.f : dx * ir, uy = si ? 0.f : dy * ir, uz = si ? 0.f : dz * ir;
+  float g[S::NA], dg[S::NA];
+  radial_channels_d<S>(P, ar, g, dg);
+  const Solid<S::NLM> H(ux, uy, uz);
+  SolidGrad G;
+  float2 al = bc2(0.f), b[NP];
+  float b0[S::LMAX + 1];
+#pragma unroll
+  for (int kk = 0; kk < NC; ++kk) {
+    const int k = kk == 0 ? NC - 1 : kk - 1;
+    float h[S::NA][4];
+    row.load(k, h);
+    float2 a01 = mul2(pr(h[0][0], h[0][1]), bc2(dg[0])), a23 = mul2(pr(h[0][2], h[0][3]), bc2(dg[0]));
+    float2 b01 = mul2(pr(h[0][0], h[0][1]), bc2(g[0])), b23 = mul2(pr(h[0][2], h[0][3]), bc2(g[0]));
+#pragma unroll
+    for (int a = 1; a < S::NA; ++a) {
+      const float2 h01 = pr(h[a][0], h[a][1]), h23 = pr(h[a][2], h[a][3]);
+      const float2 dg2 = bc2(dg[a]), g2 = bc2(g[a]);
+      a01 = fma2(h01, dg2, a01);
+      a23 = fma2(h23, dg2, a23);
+      b01 = fma2(h01, g2, b01);
+      b23 = fma2(h23, g2, b23);
+    }
+    float2 y01, y23;
+    H.chunk(k, y01, y23);
+    al = fma2(a01, y01, al);
+    al = fma2(a23, y23, al);
+    if (2 * k < NP) b[2 * k < NP ? 2 * k : 0] = b01;
+    else { b0[4 * k - 2 * NP + 1] = b01.x; b0[4 * k - 2 * NP + 2] = b01.y; }
+    if (2 * k + 1 < NP) b[2 * k + 1 < NP ? 2 * k + 1 : 0] = b23;
+    else { b0[4 * k - 2 * NP + 3] = b23.x; b0[4 * k - 2 * NP + 4] = b23.y; }
+    // the degrees whose pairs are complete after this chunk
+    if constexpr (S::NLM == 24) {
+      if (k == 0) G.template add<1>(H, b, b0[1]);
+      if (k == 1) G.template add<2>(H, b + 1, b0[2]);
+      if (k == 2) G.template add<3>(H, b + 3, b0[3]);
+      if (k == 4) G.template add<4>(H, b + 6, b0[4]);
+    } else {
+      if (k == 0) {
+        G.template add<1>(H, b, b0[1]);
+        G.template add<2>(H, b + 1, b0[2]);
+      }
+    }
+  }
+  float gx, gy, gz;
+  G.get(gx, gy, gz);
+  coef = (hsum(al) - ir * fmaf(ux, gx, fmaf(uy, gy, uz * gz))) * ir;
+  vx = gx * ir; vy = gy * ir; vz = gz * ir;
 }
 
 // The pair loop of the force kernel (see k_force), for atom i whose adjoint row is already in place:
@@ -472,12 +543,10 @@ __device__ __forceinline__ float radial_lj_coef(const Model<S> &P, const float4 
 // loop runs to the warp's largest na and lanes past their own count compute a stand-in pair), then the
 // nr other active pairs (slots pmax-1 down to pmax-nr; no TMEM).  Each pair gets the arithmetic of
 // force_pairs<S, float, false, true> on the displacement the descriptor walk computed: d_ij added to F_i,
-// subtracted from F_j (fixed point), W -= r_ij (x) d_ij (upper triangle, mirrored).  UN: the TMEM row is
-// over Ph_lm (angular_pair).  The radial tail at fps is in radial_tail_cubics' form.
-template <class S, int DQ, bool UN = false>
-__device__ __forceinline__ void force_pairs_rec(const Model<S> &P, uint32_t trow,
-                                                const float (&gi)[ForceCfg<S>::TM ? 1 : S::NA][ForceCfg<S>::TM ? 1 : S::NLM],
-                                                const float4 *fps, int i, bool live,
+// subtracted from F_j (fixed point), W -= r_ij (x) d_ij (upper triangle, mirrored).  The row is over the
+// solid harmonics (angular_pair_solid), the radial tail at fps in radial_tail_cubics' form.
+template <class S, int DQ, class Row>
+__device__ __forceinline__ void force_pairs_rec(const Model<S> &P, const Row &row, const float4 *fps, int i, bool live,
                                                 int n, const float4 *rec, unsigned off, int pmax, int na, int nr,
                                                 float4 *ring,
                                                 unsigned long long *__restrict__ Ffix, int *__restrict__ status,
@@ -510,13 +579,9 @@ __device__ __forceinline__ void force_pairs_rec(const Model<S> &P, uint32_t trow
       const float r = r2 * ir;
       float coef = valid ? radial_lj_coef<S, true>(P, fps, r2, r, ir) : 0.f;
       if constexpr (TM) __syncwarp();
-      float2 al, gv[3];
-      angular_pair<S, float, true, UN>(P, trow, gi, static_cast<const float *>(nullptr), !valid, r, ir, q.x, q.y, q.z,
-                                       al, gv);
-      if (valid) {
-        coef = fmaf(hsum(al), ir, coef);
-        apply(q.x, q.y, q.z, __float_as_int(q.w), coef, hsum(gv[0]) * ir, hsum(gv[1]) * ir, hsum(gv[2]) * ir);
-      }
+      float ca, vx, vy, vz;
+      angular_pair_solid<S>(P, row, !valid, r, ir, q.x, q.y, q.z, ca, vx, vy, vz);
+      if (valid) apply(q.x, q.y, q.z, __float_as_int(q.w), coef + ca, vx, vy, vz);
     }
     pa.finish();
   }
@@ -775,8 +840,7 @@ k_nep_fused(const __grid_constant__ Model<S> P, const Geom geom, const int n, co
   warp_sum_stage<5>(acc_d, wsum_d[threadIdx.x >> 5]);
 
   // forces: every active pair of the row with the own adjoint row, from the pair records
-  const float gi[1][1] = {{0.f}};
-  force_pairs_rec<S, PIPE_DP, true>(P, trow, gi, fp_s + threadIdx.x, i, live, n, pc.rec, rec_off, pc.pmax, nang,
+  force_pairs_rec<S, PIPE_DP>(P, RowTmem<S>{trow}, fp_s + threadIdx.x, i, live, n, pc.rec, rec_off, pc.pmax, nang,
                                     nact - nang, ring_p, Ffix, status, acc_f);
   tc_fence_before();
   __syncthreads();
@@ -862,7 +926,7 @@ k_nep_fused_reg(const __grid_constant__ Model<S> P, const Geom geom, const int n
     acc_d[3] = A.cnt;
     acc_d[4] = A.nact;
     acc_f[9] = A.cnt; acc_f[10] = A.nact; acc_f[11] = A.nrad; acc_f[12] = A.nang;
-    force_pairs_rec<S, PIPE_DP, true>(P, 0u, gi, fp_s + threadIdx.x, i, true, n, pc.rec, rec_off, pc.pmax, A.nang,
+    force_pairs_rec<S, PIPE_DP>(P, RowReg<S>{gi}, fp_s + threadIdx.x, i, true, n, pc.rec, rec_off, pc.pmax, A.nang,
                                 A.nact - A.nang, ring_p, Ffix, status, acc_f);
   }
   __syncthreads();
@@ -1064,8 +1128,7 @@ k_nep_fused_mixed(const __grid_constant__ Model<S> P, const Geom geom, const int
   }
   __shared__ long long wsum_d[DESC_BLOCK / 32][5];
   warp_sum_stage<5>(acc_d, wsum_d[t >> 5]);
-  const float gi[1][1] = {{0.f}};
-  force_pairs_rec<S, PIPE_DP, true>(P, trow, gi, fp_s + t, i, live, n, pc.rec, rec_off, pc.pmax, nang, nact - nang, ring_p,
+  force_pairs_rec<S, PIPE_DP>(P, RowTmem<S>{trow}, fp_s + t, i, live, n, pc.rec, rec_off, pc.pmax, nang, nact - nang, ring_p,
                               Ffix, status, acc_f);
   tc_fence_before();
   __syncthreads();
