@@ -249,9 +249,9 @@ nep_status nep_angular_p90(nep_handle *h, int *p90, int *cpb);
  * nep_set_state allocate).  It evaluates the float32 teacher shape only (params as for nep_create with
  * precision NEP_FP32; another shape or precision returns NEP_ERR_UNSUPPORTED; max_neighbors and
  * rebuild_every are ignored, the list capacity is 128), on up to NEP_NOALLOC_MAX_ATOMS atoms in boxes of
- * up to NEP_NOALLOC_MAX_CELLS neighbour cells, with the separate descriptor and full-row force kernels
- * (not the fused kernel of nep_compute, whose pair records would need more scratch), and keeps every
- * intermediate buffer in one fixed file-scope device array (about 11 MB, held by every GPU that loads
+ * up to NEP_NOALLOC_MAX_CELLS neighbour cells, with the kernels that nep_compute takes for small systems
+ * (several lanes per atom, no per-atom rows in memory), and keeps every
+ * intermediate buffer in one fixed file-scope device array (about 7 MB, held by every GPU that loads
  * the library until the process exits); it calls no cudaMalloc, cudaFree or other allocating routine.
  * x: [n][3] positions, E: scalar, F: [n][3] float64 in the caller's order, virial: [9]; each pointer
  * host or device, E/F/virial may be NULL.  cuda_stream: the stream to run on (NULL = the legacy default

@@ -46,9 +46,6 @@ cudaError_t launch_fused_reg(const Model<S> &, const Geom &, int, const float4 *
                              const PairCache &, cudaStream_t);
 cudaError_t pair_cache_sm_bound(int *nsm);
 size_t pair_cache_region_elems(int pmax);
-#ifndef NEP_FUSED
-#define NEP_FUSED 1
-#endif
 int descriptor_blocks(int n);
 int force_blocks(int n);
 // nep_mixed.cu
@@ -57,14 +54,16 @@ cudaError_t launch_descriptor_mixed(const Model<S> &, const Geom &, int, const f
                                     const RowExt &, __half *, float *, float *, long long *, long long *, int *,
                                     const Fallback &, cudaStream_t);
 int mixed_descriptor_blocks(int n);
+// nep_wide.cu
+int wide_lanes(int n);
+template <class S, class MT>
+cudaError_t launch_wide(int, const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
+                        float *, float *, long long *, long long *, long long *, int *, const Fallback &, int *,
+                        cudaStream_t);
 template <class S>
-cudaError_t launch_fallback_descriptor(const Model<S> &, const Geom &, int, const float4 *, const int32_t *,
-                                       const int32_t *, const int *, const int *, int, float *, float *, long long *,
-                                       long long *, int *, cudaStream_t);
-template <class S>
-cudaError_t launch_fallback_force(const Model<S> &, const Geom &, int, const float4 *, const int32_t *,
-                                  const int32_t *, const int *, const int *, int, const float *, long long *,
-                                  long long *, int *, cudaStream_t);
+cudaError_t launch_wide_list(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
+                             const int *, const int *, int, float *, long long *, long long *, long long *,
+                             long long *, int *, cudaStream_t);
 cudaError_t launch_fallback_flags(const int *, const int *, int, const int *, int *, cudaStream_t);
 // nep_force.cu / nep_ablation.cu: kernel variants for ablation
 template <class S>
@@ -176,7 +175,8 @@ struct nep_handle {
   double *io = nullptr;            // staging 2 x [n][3] float64 for host transfers
   int32_t *io_i = nullptr;         // staging for neighbour output
   size_t io_i_elems = 0;
-  int nb_d = 0, nb_f = 0, nb_k = 0;
+  int nb_d = 0, nb_f = 0, nb_k = 0;   // rows of partial sums of the last evaluation
+  int wide = 0;                    // lanes per atom of the wide kernels, 0: one thread per atom
 
   // host mirrors (pinned)
   double *h_sums = nullptr;
@@ -205,7 +205,6 @@ struct nep_handle {
   double fb_frac = 1.0 / 16.0;
   int fb_cap = 0;
   int *fb_list = nullptr, *fb_count = nullptr;
-  float *fb_G = nullptr;
 
   // buffers of the ablation variants (allocated on first use)
   float *abl_f = nullptr, *abl_s = nullptr;
@@ -277,7 +276,7 @@ void free_system(nep_handle *h) {
   dfree(h->nbr); dfree(h->nnum); dfree(h->nang); dfree(h->nown); dfree(h->nband0); dfree(h->nfar);
   dfree(h->count); dfree(h->cursor); dfree(h->start); dfree(h->tile_sums);
   dfree(h->part_d); dfree(h->part_f); dfree(h->part_k); dfree(h->io); dfree(h->io_i);
-  dfree(h->fb_list); dfree(h->fb_count); dfree(h->fb_G);
+  dfree(h->fb_list); dfree(h->fb_count);
   dfree(h->abl_f); dfree(h->abl_s); dfree(h->abl_cnt);
   dfree(h->pc_rec); dfree(h->pc_mask); dfree(h->inv);
   h->pc_nsm = 0;
@@ -395,28 +394,18 @@ cudaError_t enqueue_rebuild(nep_handle *h) {
   return launch_neighbors(a, h->stream);
 }
 
+// The teacher on the flagged atoms of a student's evaluation (after the student's kernels).
+cudaError_t enqueue_fallback(nep_handle *h, const Geom &g) {
+  Scope sc(h, KC_FB, 1);
+  return launch_wide_list<CuShape>(h->fb_model, g, h->n, h->pos, h->nbr, rows_of(h), h->fb_list, h->fb_count, h->fb_cap,
+                                   h->usite, h->F, h->part_d, h->part_f, h->counters, &h->ctrl->status, h->stream);
+}
+
 // Descriptors + network + forces; partial sums reduced with KE partials pk (may be null).
 template <class S>
 cudaError_t forces_of(nep_handle *h, const Model<S> &M, float *qout) {
+  constexpr bool teacher = std::is_same<S, CuShape>::value;
   const Geom g = geom_of(h);
-  if constexpr (std::is_same<S, CuShape>::value && NEP_FUSED) {
-    if (!h->fb_on) {
-      // the teacher: descriptors, network and forces in one kernel (forces zeroed first); the network in
-      // float32, or as two tensor-core GEMMs with bf16 / f16 operands in the mixed-precision forms
-      Scope sc(h, KC_FORCE, 1);
-      cudaError_t e = cudaMemsetAsync(h->F, 0, 3 * (size_t)h->n * sizeof(long long), h->stream);
-      if (e != cudaSuccess) return e;
-      const PairCache pc{h->pc_rec, h->pc_mask, h->pc_nsm, h->cap, h->pc_slots};
-      if (h->precision == NEP_FP32)
-        return launch_fused<CuShape>(M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F, h->part_d,
-                                     h->part_f, &h->ctrl->status, pc, h->stream);
-      if (h->precision == NEP_MIX_BF16)
-        return launch_fused_mixed<CuShape, __nv_bfloat16>(M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F,
-                                                          h->part_d, h->part_f, &h->ctrl->status, pc, h->stream);
-      return launch_fused_mixed<CuShape, __half>(M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F,
-                                                 h->part_d, h->part_f, &h->ctrl->status, pc, h->stream);
-    }
-  }
   Fallback fb{};
   fb.on = h->fb_on ? 1 : 0;
   if (fb.on) {
@@ -425,64 +414,61 @@ cudaError_t forces_of(nep_handle *h, const Model<S> &M, float *qout) {
   }
   cudaError_t e;
   if (fb.on && (e = cudaMemsetAsync(h->fb_count, 0, sizeof(int), h->stream)) != cudaSuccess) return e;
-  if constexpr (std::is_same<S, StudentShape>::value && NEP_FUSED) {
-    if (h->precision == NEP_FP32) {
-      // the student in float32: descriptors, network and full-row forces in one kernel (forces zeroed
-      // first), then the teacher on the flagged atoms
-      {
-        Scope sc(h, KC_FORCE, 1);
-        if ((e = cudaMemsetAsync(h->F, 0, 3 * (size_t)h->n * sizeof(long long), h->stream)) != cudaSuccess) return e;
+  if (h->wide > 0 || teacher || h->precision == NEP_FP32) {
+    // descriptors, network and full-row forces in one kernel (forces zeroed first), then the teacher on the
+    // flagged atoms; the network in float32, or with bf16 / f16 operands in the mixed-precision forms
+    {
+      Scope sc(h, KC_FORCE, 1);
+      if ((e = cudaMemsetAsync(h->F, 0, 3 * (size_t)h->n * sizeof(long long), h->stream)) != cudaSuccess) return e;
+      if (h->wide > 0) {
+        int blocks = 0;
+        if (h->precision == NEP_FP32)
+          e = launch_wide<S, float>(h->wide, M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F, h->part_d,
+                                    h->part_f, &h->ctrl->status, fb, &blocks, h->stream);
+        else if (h->precision == NEP_MIX_BF16)
+          e = launch_wide<S, __nv_bfloat16>(h->wide, M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F,
+                                            h->part_d, h->part_f, &h->ctrl->status, fb, &blocks, h->stream);
+        else
+          e = launch_wide<S, __half>(h->wide, M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F, h->part_d,
+                                     h->part_f, &h->ctrl->status, fb, &blocks, h->stream);
+        h->nb_d = h->nb_f = blocks;
+      } else {
         const PairCache pc{h->pc_rec, h->pc_mask, h->pc_nsm, h->cap, h->pc_slots};
-        e = launch_fused_reg<StudentShape>(M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F, h->part_d,
-                                           h->part_f, &h->ctrl->status, fb, pc, h->stream);
+        if constexpr (teacher) {
+          if (h->precision == NEP_FP32)
+            e = launch_fused<CuShape>(M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F, h->part_d,
+                                      h->part_f, &h->ctrl->status, pc, h->stream);
+          else if (h->precision == NEP_MIX_BF16)
+            e = launch_fused_mixed<CuShape, __nv_bfloat16>(M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout,
+                                                           h->F, h->part_d, h->part_f, &h->ctrl->status, pc, h->stream);
+          else
+            e = launch_fused_mixed<CuShape, __half>(M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F,
+                                                    h->part_d, h->part_f, &h->ctrl->status, pc, h->stream);
+        } else {
+          e = launch_fused_reg<StudentShape>(M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F, h->part_d,
+                                             h->part_f, &h->ctrl->status, fb, pc, h->stream);
+        }
       }
-      if (e == cudaSuccess && fb.on) {
-        Scope sc(h, KC_FB, 2);
-        e = launch_fallback_descriptor<CuShape>(h->fb_model, g, h->n, h->pos, h->nbr, h->nnum, h->fb_list,
-                                                h->fb_count, h->fb_cap, h->fb_G, h->usite, h->part_d, h->counters,
-                                                &h->ctrl->status, h->stream);
-        if (e == cudaSuccess)
-          e = launch_fallback_force<CuShape>(h->fb_model, g, h->n, h->pos, h->nbr, h->nnum, h->fb_list, h->fb_count,
-                                             h->fb_cap, h->fb_G, h->F, h->part_f, &h->ctrl->status, h->stream);
-      }
-      return e;
     }
+    return e == cudaSuccess && fb.on ? enqueue_fallback(h, g) : e;
   }
+  // the student's mixed form: tensor-core descriptor kernel, then the half-list force kernel over float16 rows
   {
     Scope sc(h, KC_DESC, 1);
-    if (h->precision == NEP_FP32)
-      e = launch_descriptor<S>(M, g, h->n, h->pos, h->nbr, rows_of(h), static_cast<float *>(h->G), h->usite, qout, h->F,
-                               h->part_d, &h->ctrl->status, fb, h->stream);
-    else if (h->precision == NEP_MIX_BF16)
+    if (h->precision == NEP_MIX_BF16)
       e = launch_descriptor_mixed<S, __nv_bfloat16>(M, g, h->n, h->pos, h->nbr, rows_of(h), static_cast<__half *>(h->G),
-                                                     h->usite, qout, h->F, h->part_d, &h->ctrl->status, fb, h->stream);
+                                                    h->usite, qout, h->F, h->part_d, &h->ctrl->status, fb, h->stream);
     else
       e = launch_descriptor_mixed<S, __half>(M, g, h->n, h->pos, h->nbr, rows_of(h), static_cast<__half *>(h->G),
-                                              h->usite, qout, h->F, h->part_d, &h->ctrl->status, fb, h->stream);
+                                             h->usite, qout, h->F, h->part_d, &h->ctrl->status, fb, h->stream);
   }
   if (e != cudaSuccess) return e;
-  if (fb.on) {
-    Scope sc(h, KC_FB, 1);
-    e = launch_fallback_descriptor<CuShape>(h->fb_model, g, h->n, h->pos, h->nbr, h->nnum, h->fb_list, h->fb_count,
-                                            h->fb_cap, h->fb_G, h->usite, h->part_d, h->counters, &h->ctrl->status,
-                                            h->stream);
-    if (e != cudaSuccess) return e;
-  }
   {
     Scope sc(h, KC_FORCE, 1);
-    if (h->precision == NEP_FP32)
-      e = launch_force<S, float>(M, g, h->n, h->pos, h->nbr, rows_of(h), static_cast<const float *>(h->G),
-                                 h->F, h->part_f, &h->ctrl->status, h->stream);
-    else
-      e = launch_force<S, __half>(M, g, h->n, h->pos, h->nbr, rows_of(h), static_cast<const __half *>(h->G),
-                                  h->F, h->part_f, &h->ctrl->status, h->stream);
+    e = launch_force<S, __half>(M, g, h->n, h->pos, h->nbr, rows_of(h), static_cast<const __half *>(h->G), h->F,
+                                h->part_f, &h->ctrl->status, h->stream);
   }
-  if (e == cudaSuccess && fb.on) {
-    Scope sc(h, KC_FB, 1);
-    e = launch_fallback_force<CuShape>(h->fb_model, g, h->n, h->pos, h->nbr, h->nnum, h->fb_list, h->fb_count,
-                                       h->fb_cap, h->fb_G, h->F, h->part_f, &h->ctrl->status, h->stream);
-  }
-  return e;
+  return e == cudaSuccess && fb.on ? enqueue_fallback(h, g) : e;
 }
 
 cudaError_t enqueue_forces(nep_handle *h, float *qout) {
@@ -728,14 +714,13 @@ nep_status upload_state_sorted(nep_handle *h, const double *x, const double *v) 
   return NEP_OK;
 }
 
-// Fallback buffers for the current system: flagged-atom list, its length, teacher adjoint rows.
+// Fallback buffers for the current system: flagged-atom list and its length.
 cudaError_t alloc_fallback(nep_handle *h) {
-  dfree(h->fb_list); dfree(h->fb_count); dfree(h->fb_G);
+  dfree(h->fb_list); dfree(h->fb_count);
   const size_t N = (size_t)std::max(h->n, 1);
   h->fb_cap = (int)std::min<double>((double)N, std::max(1.0, std::ceil((double)N * h->fb_frac)));
   cudaError_t e = dalloc(h->fb_list, (size_t)h->fb_cap);
   if (e == cudaSuccess) e = dalloc(h->fb_count, 1);
-  if (e == cudaSuccess) e = dalloc(h->fb_G, (size_t)h->fb_cap * CuShape::GS);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->fb_count, 0, sizeof(int), h->stream);
   return e;
 }
@@ -929,6 +914,7 @@ nep_status nep_set_state(nep_handle *h, int64_t n, const double *x, const double
   h->ncell = (int)ncell;
   h->nb_d = h->precision == NEP_FP32 ? descriptor_blocks(h->n) : mixed_descriptor_blocks(h->n);
   h->nb_f = force_blocks(h->n);
+  h->wide = wide_lanes(h->n);
   h->nb_k = md_blocks(h->n);
   const size_t N = (size_t)std::max(h->n, 1);
   cudaError_t e = cudaSuccess;
@@ -943,10 +929,12 @@ nep_status nep_set_state(nep_handle *h, int64_t n, const double *x, const double
   A(dalloc(h->nband0, N)); A(dalloc(h->nfar, N));
   A(dalloc(h->count, (size_t)h->ncell)); A(dalloc(h->cursor, (size_t)h->ncell)); A(dalloc(h->start, (size_t)h->ncell + 1));
   A(dalloc(h->tile_sums, (size_t)scan_tiles(h->ncell) + 1));
-  A(dalloc(h->part_d, (size_t)h->nb_d * 5 + 1)); A(dalloc(h->part_f, (size_t)h->nb_f * 13 + 1));
+  const size_t nb_w = h->wide > 0 ? WIDE_MAX_BLOCKS : 0;
+  A(dalloc(h->part_d, std::max((size_t)h->nb_d, nb_w) * 5 + 1));
+  A(dalloc(h->part_f, std::max((size_t)h->nb_f, nb_w) * 13 + 1));
   A(dalloc(h->part_k, (size_t)h->nb_k + 1)); A(dalloc(h->io, 6 * N));
   if (h->fb_on) A(alloc_fallback(h));
-  if (e == cudaSuccess && (h->shape == 0 || h->precision == NEP_FP32)) {
+  if (e == cudaSuccess && h->wide == 0 && (h->shape == 0 || h->precision == NEP_FP32)) {
     // pair records of the fused kernels: pc_slots regions per SM index, list capacity records per atom
     h->pc_slots = h->shape == 0 ? PC_SLOTS : PC_SLOTS_REG;
     A(pair_cache_sm_bound(&h->pc_nsm));

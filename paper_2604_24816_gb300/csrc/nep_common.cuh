@@ -199,6 +199,9 @@ __device__ __forceinline__ int acquire_record_slot(const PairCache &pc) {
   return slot;
 }
 
+// Rows of per-block partial sums that a wide kernel (nep_wide.cu) writes at most.
+constexpr int WIDE_MAX_BLOCKS = 152 * 8;
+
 // Cell geometry of the current neighbour list.
 struct Geom {
   float lx, ly, lz;      // cell edge lengths (float)

@@ -162,13 +162,6 @@ __device__ __forceinline__ void accumulate_atom(const Model<S> &P, const float4 
   pipe.finish();
   cheb_sums(Q, A.QR);
 }
-template <class S, int DE, int DP, int BLOCK>
-__device__ __forceinline__ void accumulate_atom(const Model<S> &P, const float4 *shift, int i, int n,
-                                                const float4 *__restrict__ pos, const int32_t *__restrict__ nbr,
-                                                int cnt, uint32_t *ring_e, float4 *ring_p, AtomSums<S> &A) {
-  accumulate_atom<S, DE, DP, BLOCK>(P, shift, i, n, pos, nbr, RowSpan{cnt, cnt, 0}, ring_e, ring_p, A);
-}
-
 // Traceless 4-body tensors T_n rebuilt from the l = 2 sums (components 3..7 = m -2..2).
 template <class S>
 struct FourBody {

@@ -3,9 +3,8 @@
 // Some callers cannot allocate GPU memory at the point where they need forces: a plugin running
 // inside another program's memory pool or allocator budget, or an embedded runtime that forbids
 // cudaMalloc after start-up.  For them this entry point evaluates E, F and the virial of a small system
-// of the float32 teacher shape with the separate descriptor and full-row force kernels, but every
-// intermediate buffer (cell lists, neighbour lists, adjoint rows, partial sums, status word) lives in
-// one file-scope __device__ array of fixed size, created when the library is loaded and kept by every
+// of the float32 teacher shape with the kernels that nep_compute takes for small systems (nep_wide.cu), but
+// every intermediate buffer (cell lists, neighbour lists, partial sums, status word) lives in one file-scope __device__ array of fixed size, created when the library is loaded and kept by every
 // GPU that loads it until the process exits.
 //
 // The device address of that array is looked up once per device with cudaGetSymbolAddress (in host
@@ -29,15 +28,11 @@
 #include "nep_gb300.h"
 
 namespace nep {
-template <class S>
-cudaError_t launch_descriptor(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
-                              float *, float *, float *, long long *, long long *, int *, const Fallback &,
-                              cudaStream_t);
-template <class S, class GT>
-cudaError_t launch_force(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
-                         const GT *, long long *, long long *, int *, cudaStream_t);
-int descriptor_blocks(int n);
-int force_blocks(int n);
+int wide_lanes(int n);
+template <class S, class MT>
+cudaError_t launch_wide(int, const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
+                        float *, float *, long long *, long long *, long long *, int *, const Fallback &, int *,
+                        cudaStream_t);
 cudaError_t launch_cell_sort(const RebuildArgs &, cudaStream_t);
 cudaError_t launch_neighbors(const RebuildArgs &, cudaStream_t);
 int scan_tiles(int ncell);
@@ -62,7 +57,7 @@ constexpr size_t up256(size_t b) { return (b + 255) / 256 * 256; }
 
 // Byte offsets of the pieces inside the scratch array.
 struct Layout {
-  size_t x, y, z, vx, vy, vz, xb, yb, zb, vxb, vyb, vzb, id, idb, cell_of, perm, pos, pos_ref, F, usite, G, nbr,
+  size_t x, y, z, vx, vy, vz, xb, yb, zb, vxb, vyb, vzb, id, idb, cell_of, perm, pos, pos_ref, F, usite, nbr,
       nnum, nang, nown, nband0, nfar, count, cursor, start, tile_sums, part_d, part_f, sums, counters, ctrl, io, total;
 };
 
@@ -77,11 +72,11 @@ constexpr Layout make_layout() {
   L.vxb = take(N * 8); L.vyb = take(N * 8); L.vzb = take(N * 8);
   L.id = take(N * 4); L.idb = take(N * 4); L.cell_of = take(N * 4); L.perm = take(N * 8);
   L.pos = take(N * 16); L.pos_ref = take(N * 16);
-  L.F = take(N * 3 * 8); L.usite = take(N * 4); L.G = take(N * S::GS * 4); L.nbr = take(N * CAP * 4);
+  L.F = take(N * 3 * 8); L.usite = take(N * 4); L.nbr = take(N * CAP * 4);
   L.nnum = take(N * 4); L.nang = take(N * 4); L.nown = take(N * 4); L.nband0 = take(N * 4); L.nfar = take(N * 4);
   L.count = take((size_t)NC_MAX * 4); L.cursor = take((size_t)NC_MAX * 4); L.start = take(((size_t)NC_MAX + 1) * 4);
   L.tile_sums = take(((size_t)NC_MAX / 4096 + 2) * 4);
-  L.part_d = take(((size_t)N / 64 + 2) * 5 * 8); L.part_f = take(((size_t)N / 64 + 2) * 13 * 8);
+  L.part_d = take((size_t)WIDE_MAX_BLOCKS * 5 * 8); L.part_f = take((size_t)WIDE_MAX_BLOCKS * 13 * 8);
   L.sums = take(32 * 8); L.counters = take(16 * 8); L.ctrl = take(sizeof(Control)); L.io = take(N * 3 * 8);
   L.total = o;
   return L;
@@ -89,7 +84,7 @@ constexpr Layout make_layout() {
 
 constexpr Layout LAYOUT = make_layout();
 
-// The scratch memory of nep_compute_noalloc (about 11 MB for 8,192 atoms).
+// The scratch memory of nep_compute_noalloc (about 7 MB for 8,192 atoms).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[LAYOUT.total];
 
 constexpr int MAX_DEVICES = 64;
@@ -284,11 +279,11 @@ extern "C" nep_status nep_compute_noalloc(const nep_params *p, int64_t n, const 
   NA_CUDA(launch_cell_sort(a, st));
   NA_CUDA(launch_neighbors(a, st));
   const RowExt rows{a.nnum, a.nown, a.nband0, a.nfar, nullptr};   // one evaluation: the whole rows
-  NA_CUDA(launch_descriptor<S>(M, g, N, a.pos, a.nbr, rows, (float *)at(LAYOUT.G), (float *)at(LAYOUT.usite),
-                               nullptr, Ffix, pd, &ctrl->status, Fallback{}, st));
-  NA_CUDA((launch_force<S, float>(M, g, N, a.pos, a.nbr, rows, (const float *)at(LAYOUT.G), Ffix, pf, &ctrl->status,
-                                  st)));
-  NA_CUDA(launch_finalize(pd, descriptor_blocks(N), pf, force_blocks(N), nullptr, 0, sums, counters, st));
+  int blocks = 0;
+  NA_CUDA(cudaMemsetAsync(Ffix, 0, 3 * (size_t)N * sizeof(long long), st));
+  NA_CUDA((launch_wide<S, float>(std::max(8, wide_lanes(N)), M, g, N, a.pos, a.nbr, rows, (float *)at(LAYOUT.usite),
+                                 nullptr, Ffix, pd, pf, &ctrl->status, Fallback{}, &blocks, st)));
+  NA_CUDA(launch_finalize(pd, blocks, pf, blocks, nullptr, 0, sums, counters, st));
   const bool f_dev = F && device_pointer(F);
   const bool e_dev = E && device_pointer(E);
   const bool w_dev = virial && device_pointer(virial);

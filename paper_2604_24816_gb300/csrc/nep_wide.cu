@@ -1,0 +1,591 @@
+// nep_wide.cu -- descriptors, network and forces with G lanes per atom (sm_103a).
+//
+// The fused kernels of nep_force.cu give each atom one thread, which walks its row alone: 45 us from one block
+// to one block per SM, whatever the atom count, since a warp then issues one instruction every three cycles.
+// Systems that leave the chip empty that way (and the few atoms that a student's fallback hands to the
+// teacher) take k_nep_wide: a group of G = 8, 16 or 32 lanes shares an atom.
+//   walk      the lanes stride over the neighbour row; entries inside the cutoff are compacted by ballot into
+//             the group's shared memory (angular pairs from the front, the others from the back), radial
+//             basis sums and LJ energy in registers, combined by shuffles;
+//   sums      G angular pairs at a time: each lane writes one pair's channel functions g_n and solid harmonics
+//             to shared memory, then owns NLM / G components and adds all channels over the staged pairs;
+//   network   descriptors, neurons and their backward products distributed over the lanes (W0 in shared
+//             memory, rows padded to an odd length so that both rows and columns are read without conflicts);
+//   forces    the lanes stride over the compacted entries again, each evaluating whole pairs with the adjoint
+//             row read from shared memory, and scatter d_ij as the fused kernels do.
+// Everything of an atom stays inside its warp, so no block barrier is needed after the tables are staged.  The
+// sums of a row are taken in a fixed order (lane, then shuffle tree), so results are reproducible bit for bit.
+// MT = __nv_bfloat16 / __half rounds the network's operands (scaled descriptors, W0, backward factors) to that
+// type before the float32 products, as the tensor-core form does with its GEMM operands, and takes its tanh from
+// the special-function unit as well.
+#include <algorithm>
+#include <type_traits>
+
+#include "nep_pair.cuh"
+
+namespace nep {
+namespace {
+
+constexpr int WIDE_BLOCK = 128;
+constexpr int WIDE_WARPS = WIDE_BLOCK / 32;
+constexpr int WIDE_CAP = 128;          // entries per atom: the largest list capacity
+
+template <class MT>
+__device__ __forceinline__ float round_to(float x) {
+  if constexpr (std::is_same<MT, float>::value) return x;
+  else if constexpr (std::is_same<MT, __half>::value) return __half2float(__float2half_rn(x));
+  else return __bfloat162float(__float2bfloat16_rn(x));
+}
+
+// The model tables the lanes index (read from shared memory; the constant bank serves one address at a time).
+template <class S>
+struct WideNet {
+  static constexpr int LD = S::NDES | 1;
+  float W0[S::NNEU * LD];
+  float cR[S::NR * S::KR];
+  float qs[S::NDES], b0[S::NNEU], w1[S::NNEU], norm[S::NLM];
+};
+
+// One atom's workspace.
+template <class S>
+struct __align__(16) WideAtom {
+  uint32_t ent[WIDE_CAP];              // active list entries: angular from the front, others from the back
+  float row[S::NA][S::NLM];            // s', then the adjoint row (16-byte rows: NLM is a multiple of 4)
+  float Q[8];                          // radial sums, then the radial adjoint
+  float q[32], t[32];                  // scaled descriptors then dU/dq; backward factors
+  float g4[S::FOURBODY ? S::NA : 1][5];
+};
+
+template <class S>
+struct RowShared {
+  const float *g;
+  __device__ __forceinline__ void load(int k, float (&h)[S::NA][4]) const {
+#pragma unroll
+    for (int a = 0; a < S::NA; ++a) {
+      const float4 v = *reinterpret_cast<const float4 *>(g + a * S::NLM + 4 * k);
+      h[a][0] = v.x; h[a][1] = v.y; h[a][2] = v.z; h[a][3] = v.w;
+    }
+  }
+};
+
+template <int G>
+__device__ __forceinline__ float group_sum(float v) {
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Sums of the 8 values over the group: lane gl ends with value gl / (G / 8).
+template <int G>
+__device__ __forceinline__ float group_sum8(const float (&v)[8], int gl) {
+  float a[4], b[2];
+  const bool h0 = (gl & (G / 2)) != 0, h1 = (gl & (G / 4)) != 0, h2 = (gl & (G / 8)) != 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float keep = h0 ? v[4 + k] : v[k], give = h0 ? v[k] : v[4 + k];
+    a[k] = keep + __shfl_xor_sync(0xffffffffu, give, G / 2);
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float keep = h1 ? a[2 + k] : a[k], give = h1 ? a[k] : a[2 + k];
+    b[k] = keep + __shfl_xor_sync(0xffffffffu, give, G / 4);
+  }
+  const float keep = h2 ? b[1] : b[0], give = h2 ? b[0] : b[1];
+  float c = keep + __shfl_xor_sync(0xffffffffu, give, G / 8);
+#pragma unroll
+  for (int o = G / 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  return c;
+}
+
+template <class S, int G>
+struct __align__(16) WideShared {
+  float4 shift[27];
+  WideAtom<S> ws[WIDE_WARPS * (32 / G)];
+  WideNet<S> net;
+  // one staged pair per lane; with rows of an odd length the lanes write their own rows, and the lanes of a
+  // group read consecutive values of one row, G rows apart from the next group's, without bank conflicts
+  static constexpr int STP = (S::NA + S::NLM) | 1;
+  float stage[WIDE_WARPS][32 * STP];
+};
+
+template <class S, class MT, int G, bool LIST>
+__device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P, const Geom &geom, const int n,
+                                          const int m, const int32_t *__restrict__ list, const float4 *__restrict__ pos,
+                                          const int32_t *__restrict__ nbr, const RowExt &X, float *__restrict__ usite,
+                                          float *__restrict__ qout, unsigned long long *__restrict__ Ffix,
+                                          long long *__restrict__ part_d, long long *__restrict__ part_f,
+                                          int *__restrict__ status, const Fallback &fb) {
+  constexpr bool MIX = !std::is_same<MT, float>::value;
+  constexpr int NG = 32 / G;                           // atoms per warp
+  constexpr int LD = WideNet<S>::LD;
+  constexpr int STP = WideShared<S, G>::STP;
+  constexpr int CPL = (S::NLM + G - 1) / G;            // components per lane
+  constexpr int NP2 = 2 * solid_pairs(S::NLM);
+  float4 *shift = M.shift;
+  WideNet<S> &net = M.net;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int gl = lane % G, grp = lane / G;
+  int base = ((int)blockIdx.x * WIDE_WARPS + warp) * NG;
+  // a block without flagged atoms has nothing to add (block-uniform; in LIST no block writes a row of its own)
+  if (LIST && (int)blockIdx.x * WIDE_WARPS * NG >= m) return;
+  const bool skip = skip_far(X);
+  // an atom's row extent, first two entries per lane and first neighbour: loaded before the tables are staged
+  // and at the end of the previous atom, so that the chain extent -> entry -> position starts early
+  bool live;
+  int i;
+  RowSpan sp;
+  float4 pi, pj;
+  uint32_t e, e1;
+  auto entry = [&](int k) -> uint32_t {                // the k-th walked entry of atom i
+    return k < sp.c ? (uint32_t)nbr[(size_t)(k < sp.c1 ? k : k + sp.gap) * n + i] : 0u;
+  };
+  auto load_atom = [&]() {
+    live = base + grp < m;
+    i = live ? (LIST ? list[base + grp] : base + grp) : 0;
+    sp = live ? full_row(X, i, skip) : RowSpan{0, 0, 0};
+    pi = pos[i];
+    e = entry(gl);
+    e1 = entry(gl + G);
+    pj = pos[e & J_MASK];
+  };
+  load_atom();
+  fill_shift_table(shift, geom);
+  for (int t = threadIdx.x; t < S::NNEU * S::NDES; t += WIDE_BLOCK)
+    net.W0[(t / S::NDES) * LD + t % S::NDES] = round_to<MT>(P.W0[t / S::NDES][t % S::NDES]);
+  for (int t = threadIdx.x; t < S::NR * S::KR; t += WIDE_BLOCK) net.cR[t] = P.cR[t / S::KR][t % S::KR];
+  for (int t = threadIdx.x; t < S::NDES; t += WIDE_BLOCK) net.qs[t] = P.qs[t];
+  for (int t = threadIdx.x; t < S::NNEU; t += WIDE_BLOCK) { net.b0[t] = P.b0[t]; net.w1[t] = P.w1[t]; }
+  for (int t = threadIdx.x; t < S::NLM; t += WIDE_BLOCK) {
+    float v = 0.f;
+#pragma unroll
+    for (int c = 0; c < S::NLM; ++c)
+      if (t == c) v = solid_norm(S::NLM, c);
+    net.norm[t] = v;
+  }
+  __syncthreads();
+  const unsigned gmask = (G == 32 ? 0xffffffffu : ((1u << G) - 1u)), below = (1u << gl) - 1u;
+  WideAtom<S> &A = M.ws[warp * NG + grp];
+  float *st = M.stage[warp] + lane * STP;              // this lane's staged pair
+  const float *sg = M.stage[warp] + grp * G * STP;     // the group's
+  long long acc_d[5] = {0, 0, 0, 0, 0}, acc_f[13] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  const int per_pass = (int)gridDim.x * WIDE_WARPS * NG;
+  for (; base < m; base += per_pass) {                 // warp-uniform
+    auto offset_of = [&](uint32_t e, float4 pj, float &dx, float &dy, float &dz) {
+      const float4 o = shift[e >> J_BITS];
+      dx = pj.x - pi.x + o.x; dy = pj.y - pi.y + o.y; dz = pj.z - pi.z + o.z;
+      return dx * dx + dy * dy + dz * dz;
+    };
+
+    // walk: entries one step further ahead than positions
+    float2 Q[4] = {bc2(0.f), bc2(0.f), bc2(0.f), bc2(0.f)};
+    float elj = 0.f;
+    int na = 0, no = 0, nrad = 0;
+    const int trip = __reduce_max_sync(0xffffffffu, (sp.c + G - 1) / G);
+    for (int it = 0; it < trip; ++it) {
+      const int k = it * G + gl;
+      const uint32_t e2 = entry(k + 2 * G);
+      const float4 p1 = pos[e1 & J_MASK];
+      float dx, dy, dz;
+      const float r2 = offset_of(e, pj, dx, dy, dz);
+      const bool act = k < sp.c && r2 < P.rmax2, ang = act && r2 < P.rcA2;
+      const unsigned ba = (__ballot_sync(0xffffffffu, ang) >> (grp * G)) & gmask;
+      const unsigned bo = (__ballot_sync(0xffffffffu, act && !ang) >> (grp * G)) & gmask;
+      if (act) A.ent[ang ? na + __popc(ba & below) : WIDE_CAP - 1 - (no + __popc(bo & below))] = e;
+      na += __popc(ba);
+      no += __popc(bo);
+      if (act) {
+        const float ir = rsqrtf(r2), r = r2 * ir;
+        if (r2 < P.rcR2) {
+          cheb_accumulate(r, P.inv_rcR, Q);
+          ++nrad;
+        }
+        if (!LIST && P.lj_on != 0.f && r2 < P.lj_rc2) {
+          float el, dl;
+          lj_pair<S>(P, r2, r, ir, el, dl);
+          elj = fmaf(0.5f, el, elj);
+        }
+      }
+      e = e1; e1 = e2; pj = p1;
+    }
+    {
+      float v[8];
+      cheb_sums(Q, v);                                 // linear: the lanes' sums add up to the atom's
+      const float t = group_sum8<G>(v, gl);
+      if ((gl & (G / 8 - 1)) == 0) A.Q[gl / (G / 8)] = t;
+    }
+    elj = group_sum<G>(elj);
+    __syncwarp();
+
+    // angular sums, G pairs at a time
+    float s[S::NA][CPL];
+#pragma unroll
+    for (int a = 0; a < S::NA; ++a)
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) s[a][c] = 0.f;
+    const int chunks = __reduce_max_sync(0xffffffffu, (na + G - 1) / G);
+    for (int ch = 0; ch < chunks; ++ch) {
+      const int p = ch * G + gl;
+      const bool has = p < na;
+      float r = 1.f, ux = 1.f, uy = 0.f, uz = 0.f;
+      if (has) {
+        const uint32_t ep = A.ent[p];
+        float dx, dy, dz;
+        const float r2 = offset_of(ep, pos[ep & J_MASK], dx, dy, dz);
+        const float ir = rsqrtf(r2);
+        r = r2 * ir; ux = dx * ir; uy = dy * ir; uz = dz * ir;
+      }
+      float g[S::NA];
+      radial_channels<S>(P, r, has, g);                // zero without a pair
+      const Solid<S::NLM> H(ux, uy, uz);
+#pragma unroll
+      for (int a = 0; a < S::NA; ++a) st[a] = g[a];
+#pragma unroll
+      for (int k = 0; k < S::NLM / 4; ++k) {
+        float2 y01, y23;
+        H.chunk(k, y01, y23);
+        st[S::NA + 4 * k] = y01.x; st[S::NA + 4 * k + 1] = y01.y;
+        st[S::NA + 4 * k + 2] = y23.x; st[S::NA + 4 * k + 3] = y23.y;
+      }
+      __syncwarp();
+      const int cnt = __reduce_max_sync(0xffffffffu, min(G, na - ch * G));
+#pragma unroll 2
+      for (int q = 0; q < cnt; ++q) {
+        const float *sq = sg + q * STP;
+        float y[CPL];
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) y[c] = gl + c * G < S::NLM ? sq[S::NA + gl + c * G] : 0.f;
+#pragma unroll
+        for (int a = 0; a < S::NA; ++a) {
+          const float ga = sq[a];
+#pragma unroll
+          for (int c = 0; c < CPL; ++c) s[a][c] = fmaf(ga, y[c], s[a][c]);
+        }
+      }
+      __syncwarp();                                    // read before the next chunk's pairs replace them
+    }
+#pragma unroll
+    for (int c = 0; c < CPL; ++c)
+      if (gl + c * G < S::NLM) {
+#pragma unroll
+        for (int a = 0; a < S::NA; ++a) A.row[a][gl + c * G] = s[a][c];
+      }
+    __syncwarp();
+
+    // descriptors [q_n | q_nl | q4_n], one per lane and turn
+    bool out = false;
+    for (int d = gl; d < S::NDES; d += G) {
+      float q;
+      if (d < S::NR) {
+        q = 0.f;
+#pragma unroll
+        for (int k = 0; k < S::KR; ++k) q = fmaf(net.cR[d * S::KR + k], A.Q[k], q);
+      } else if (d < S::NR + S::NA * S::LMAX) {
+        const int a = (d - S::NR) / S::LMAX, l = (d - S::NR) % S::LMAX + 1;
+        const float z = net.norm[NP2 + l - 1] * A.row[a][NP2 + l - 1];
+        q = z * z;
+        for (int c = l * (l - 1); c < l * (l + 1); ++c) {
+          const float v = net.norm[c] * A.row[a][c];
+          q = fmaf(v, v, q);
+        }
+      } else {
+        q = 0.f;
+        if constexpr (S::FOURBODY) {
+          // one channel's tensor: fourbody_tensors / fourbody_adjoint of a one-channel shape
+          using One = Shape<1, 1, 8, 8, 4, true, 1>;
+          const int a = d - S::NR - S::NA * S::LMAX;
+          float s2[1][5], q1[One::NDES], g1[5];
+#pragma unroll
+          for (int p = 0; p < S::NLM; ++p) {
+            const int m2 = solid_quadrupole(S::NLM, p);
+            if (m2 >= 0) s2[0][m2 < 0 ? 0 : m2] = solid_norm(S::NLM, p) * A.row[a][p];
+          }
+          FourBody<One> T;
+          fourbody_tensors<One>(s2, T, q1);
+          q = q1[One::NR + One::NA * One::LMAX];
+          fourbody_adjoint<One>(0, T, g1);
+#pragma unroll
+          for (int k = 0; k < 5; ++k) A.g4[a][k] = g1[k];
+        }
+      }
+      if (!LIST && live && qout != nullptr) qout[(size_t)i * S::NDES + d] = q;
+      const float qt = q * net.qs[d];
+      if constexpr (S::NDES <= 16) {
+        if (!LIST && fb.on) out |= (qt < fb.lo[d]) | (qt > fb.hi[d]);
+      }
+      A.q[d] = round_to<MT>(qt);
+    }
+    bool flagged = false;
+    if constexpr (!LIST && S::NDES <= 16) {
+      const unsigned any = __ballot_sync(0xffffffffu, out);   // by every lane, also those past the last atom
+      flagged = live && fb.on && ((any >> (grp * G)) & gmask) != 0u;
+      if (flagged && gl == 0) flag_atom(fb, i, status);
+    }
+    __syncwarp();
+
+    // network: neurons, then their backward products
+    float U = 0.f;
+    for (int mu = gl; mu < S::NNEU; mu += G) {
+      const float *w = net.W0 + mu * LD;
+      float z0 = -net.b0[mu], z1 = 0.f;
+#pragma unroll
+      for (int v = 0; v + 1 < S::NDES; v += 2) {
+        z0 = fmaf(w[v], A.q[v], z0);
+        z1 = fmaf(w[v + 1], A.q[v + 1], z1);
+      }
+      if (S::NDES & 1) z0 = fmaf(w[S::NDES - 1], A.q[S::NDES - 1], z0);
+      const float z = z0 + z1;
+      const float h = MIX ? tanh_sfu(z) : tanhf(z);
+      U = fmaf(net.w1[mu], h, U);
+      A.t[mu] = round_to<MT>(net.w1[mu] * (1.f - h * h));
+    }
+    U = group_sum<G>(U) - P.b1;
+    __syncwarp();                                      // t is complete, q has been read
+    for (int v = gl; v < S::NDES; v += G) {
+      const float *w = net.W0 + v;
+      float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+      for (int mu = 0; mu + 1 < S::NNEU; mu += 2) {
+        d0 = fmaf(A.t[mu], w[mu * LD], d0);
+        d1 = fmaf(A.t[mu + 1], w[(mu + 1) * LD], d1);
+      }
+      if (S::NNEU & 1) d0 = fmaf(A.t[S::NNEU - 1], w[(S::NNEU - 1) * LD], d0);
+      A.q[v] = flagged ? 0.f : (d0 + d1) * net.qs[v];  // dU/dq
+    }
+    __syncwarp();
+
+    // adjoint row G' = 2 norm^2 Fp s' + norm f4 g4 over the sums, radial adjoint over the radial sums
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) {
+      const int p = gl + c * G;
+      if (p < S::NLM) {
+        const int l = p < NP2 ? (p < 2 ? 1 : (p < 6 ? 2 : (p < 12 ? 3 : 4))) : p - NP2 + 1;
+        const float h = net.norm[p], hh = 2.f * h * h;
+        int m2 = -1;
+#pragma unroll
+        for (int u = 0; u < S::NLM; ++u)
+          if (u == p) m2 = solid_quadrupole(S::NLM, u);
+#pragma unroll
+        for (int a = 0; a < S::NA; ++a) {
+          float gl_ = hh * A.q[S::NR + a * S::LMAX + l - 1] * s[a][c];
+          if constexpr (S::FOURBODY) {
+            if (m2 >= 0) gl_ = fmaf(h * A.q[S::NR + S::NA * S::LMAX + a], A.g4[a][m2], gl_);
+          }
+          A.row[a][p] = gl_;
+        }
+      }
+    }
+    for (int k = gl; k < 8; k += G) {
+      float t = 0.f;
+#pragma unroll
+      for (int a = 0; a < S::NR; ++a) t = fmaf(A.q[a], net.cR[a * S::KR + k], t);
+      A.Q[k] = t;
+    }
+    __syncwarp();
+    float4 c0, c1;
+    {
+      float tail[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) tail[k] = A.Q[k];
+      radial_tail_cubics(tail, c0, c1);
+    }
+    if (live && gl == 0) {
+      const float ui = LIST ? U : (flagged ? elj : U + elj);
+      if (LIST) usite[i] += U;                         // the student's kernel left the LJ energy there
+      else usite[i] = ui;
+      if (!isfinite(ui)) atomicOr(status, ST_NAN);
+      acc_d[0] += to_fix32(ui);
+      acc_d[2] += na;
+      acc_d[3] += sp.c;
+      acc_d[4] += na + no;
+    }
+    acc_d[1] += nrad;
+
+    // forces: the compacted entries, angular ones first
+    const RowShared<S> row{&A.row[0][0]};
+    float fx = 0.f, fy = 0.f, fz = 0.f;
+    float wxx = 0.f, wxy = 0.f, wxz = 0.f, wyy = 0.f, wyz = 0.f, wzz = 0.f;
+    const int nact = na + no;
+    const int ftrip = __reduce_max_sync(0xffffffffu, (nact + G - 1) / G);
+    auto active = [&](int p) -> uint32_t {
+      return p < nact ? A.ent[p < na ? p : WIDE_CAP - 1 - (p - na)] : 0u;
+    };
+    e = active(gl);
+    pj = pos[e & J_MASK];
+    for (int it = 0; it < ftrip; ++it) {
+      const int p = it * G + gl;
+      const uint32_t en = active(p + G);
+      const float4 pn = pos[en & J_MASK];
+      const bool valid = p < nact, ang = p < na;
+      float dx = 1.f, dy = 0.f, dz = 0.f, r2 = 1.f;
+      if (valid) r2 = offset_of(e, pj, dx, dy, dz);
+      const float ir = rsqrtf(r2), r = r2 * ir;
+      float coef = valid ? radial_lj_coef<S, false, !LIST>(P, c0, c1, r2, r, ir) : 0.f;
+      float vx = 0.f, vy = 0.f, vz = 0.f;
+      if (ang) {
+        float ca;
+        angular_pair_solid<S>(P, row, false, r, ir, dx, dy, dz, ca, vx, vy, vz);
+        coef += ca;
+      }
+      if (valid) {
+        const int j = (int)(e & J_MASK);
+        const float Dx = fmaf(coef, dx, vx), Dy = fmaf(coef, dy, vy), Dz = fmaf(coef, dz, vz);
+        fx += Dx; fy += Dy; fz += Dz;
+        long long ox, oy, oz;
+        to_fix32x3(-Dx, -Dy, -Dz, ox, oy, oz);
+        red_add(Ffix + j, ox);
+        red_add(Ffix + (size_t)n + j, oy);
+        red_add(Ffix + 2 * (size_t)n + j, oz);
+        wxx = fmaf(dx, Dx, wxx); wxy = fmaf(dx, Dy, wxy); wxz = fmaf(dx, Dz, wxz);
+        wyy = fmaf(dy, Dy, wyy); wyz = fmaf(dy, Dz, wyz); wzz = fmaf(dz, Dz, wzz);
+      }
+      e = en; pj = pn;
+    }
+    fx = group_sum<G>(fx); fy = group_sum<G>(fy); fz = group_sum<G>(fz);
+    if (live && gl == 0) {
+      red_add(Ffix + i, to_fix32(fx));
+      red_add(Ffix + (size_t)n + i, to_fix32(fy));
+      red_add(Ffix + 2 * (size_t)n + i, to_fix32(fz));
+      if (!(isfinite(fx) && isfinite(fy) && isfinite(fz))) atomicOr(status, ST_NAN);
+    }
+    // W = -sum of r_ij (x) d_ij, upper triangle (symmetric: U_i is rotation invariant)
+    acc_f[0] -= to_fix32(wxx); acc_f[1] -= to_fix32(wxy); acc_f[2] -= to_fix32(wxz);
+    acc_f[4] -= to_fix32(wyy); acc_f[5] -= to_fix32(wyz); acc_f[8] -= to_fix32(wzz);
+    base += per_pass;
+    if (base < m) load_atom();                         // warp-uniform
+    base -= per_pass;
+    __syncwarp();                                      // the workspace is the warp's next atoms'
+  }
+  acc_f[3] = acc_f[1]; acc_f[6] = acc_f[2]; acc_f[7] = acc_f[5];
+  if constexpr (LIST) {
+    // added to the sums of the student's kernels (integers: any order gives the same result)
+    __shared__ long long red[WIDE_WARPS][10];
+    long long v[10] = {acc_d[0], acc_f[0], acc_f[1], acc_f[2], acc_f[3], acc_f[4], acc_f[5], acc_f[6], acc_f[7], acc_f[8]};
+    warp_sum_stage<10>(v, red[warp]);
+    __syncthreads();
+    if (threadIdx.x < 10) {
+      long long t = 0;
+      for (int w = 0; w < WIDE_WARPS; ++w) t += red[w][threadIdx.x];
+      if (t != 0)
+        atomicAdd(reinterpret_cast<unsigned long long *>(threadIdx.x == 0 ? part_d : part_f + threadIdx.x - 1),
+                  (unsigned long long)t);
+    }
+  } else {
+    // the force pass visits the walk's active pairs
+    acc_f[9] = acc_d[3]; acc_f[10] = acc_d[4]; acc_f[11] = acc_d[1]; acc_f[12] = acc_d[2];
+    block_sum_store<5, WIDE_WARPS>(acc_d, part_d);
+    block_sum_store<13, WIDE_WARPS>(acc_f, part_f);
+  }
+}
+
+// One evaluation of all n atoms.
+template <class S, class MT, int G>
+__global__ void __launch_bounds__(WIDE_BLOCK, 4)
+k_nep_wide(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
+           const int32_t *__restrict__ nbr, const RowExt X, float *__restrict__ usite, float *__restrict__ qout,
+           unsigned long long *__restrict__ Ffix, long long *__restrict__ part_d, long long *__restrict__ part_f,
+           int *__restrict__ status, const __grid_constant__ Fallback fb) {
+  __shared__ WideShared<S, G> M;
+  wide_body<S, MT, G, false>(M, P, geom, n, n, nullptr, pos, nbr, X, usite, qout, Ffix, part_d, part_f, status, fb);
+}
+
+// The fallback model on the first min(*count, cap) atoms of list: only its network's part is added to usite, to
+// the forces and to the partial sums (the pair term is the student's).  Few flagged atoms take a warp each, many
+// a quarter of one: at 131,072 atoms 20 us against 28 for 1,311 flagged ones, 39 against 33 for 8,192 (of
+// 16,384), 426 against 264 for all (eager times, with 6 us of launch).  The two kernels of one thread per flagged
+// atom that this replaces took 66 us from one to 16,384 flagged atoms (their serial row walk), 321 for 131,072 and
+// 2.02 ms for 1,048,576, where this takes 2.1.
+constexpr int LIST_WARP_MAX = 4096;
+template <class S>
+__global__ void __launch_bounds__(WIDE_BLOCK, 4)
+k_nep_wide_list(const __grid_constant__ Model<S> P, const Geom geom, const int n, const int32_t *__restrict__ list,
+                const int *__restrict__ count, const int cap, const float4 *__restrict__ pos,
+                const int32_t *__restrict__ nbr, const RowExt X, float *__restrict__ usite,
+                unsigned long long *__restrict__ Ffix, long long *__restrict__ part_d, long long *__restrict__ part_f,
+                long long *__restrict__ counters, int *__restrict__ status) {
+  __shared__ __align__(16) unsigned char raw[sizeof(WideShared<S, 8>)];
+  static_assert(sizeof(WideShared<S, 8>) >= sizeof(WideShared<S, 32>), "one buffer for both splits");
+  const int m = min(*count, cap);
+  if (blockIdx.x == 0 && threadIdx.x == 0)
+    atomicAdd(reinterpret_cast<unsigned long long *>(counters + 9), (unsigned long long)m);
+  if (m == 0) return;
+  const Fallback none{};
+  if (m <= LIST_WARP_MAX)
+    wide_body<S, float, 32, true>(reinterpret_cast<WideShared<S, 32> &>(raw), P, geom, n, m, list, pos, nbr, X, usite,
+                                  nullptr, Ffix, part_d, part_f, status, none);
+  else
+    wide_body<S, float, 8, true>(reinterpret_cast<WideShared<S, 8> &>(raw), P, geom, n, m, list, pos, nbr, X, usite,
+                                 nullptr, Ffix, part_d, part_f, status, none);
+}
+
+// Blocks that fit on the device at once (at most WIDE_MAX_BLOCKS), or fewer for few atoms; the kernels loop.
+template <class K>
+int wide_grid(K kernel, int atoms, int lanes) {
+  int d = 0, sms = 0, per = 0;
+  if (cudaGetDevice(&d) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, WIDE_BLOCK, 0) != cudaSuccess || sms * per <= 0) {
+    cudaGetLastError();
+    sms = 152;
+    per = 1;
+  }
+  const long long need = ((long long)atoms * lanes + WIDE_BLOCK - 1) / WIDE_BLOCK;
+  return (int)std::max(1ll, std::min(need, (long long)std::min(sms * per, WIDE_MAX_BLOCKS)));
+}
+
+}  // namespace
+
+// Lanes per atom for a system of n atoms, 0: one thread per atom (the fused kernels of nep_force.cu).  Measured
+// per evaluation (eager, with the launch's own 7 us) for the teacher: at 256 atoms 50 us with one thread per atom,
+// 25 / 19 / 17 us with 8 / 16 / 32 lanes; at 2,048 51, 26 / 22 / 23; at 4,000 50, 28 / 28 / 30; at 10,976 53,
+// 45 / 46 / 50; at 16,384 53 (MD step 72.5), 54 (70.9) / 57 / 67; at 32,000 66, 83 / 93 / 112, where the wide
+// form's extra work (1.6 x the instructions per atom) is no longer hidden.  The student (40 us with one thread
+// per atom up to 16,384 atoms; 15 at 256 with 32 lanes, 20 at 4,000 with 16, 36 at 16,384 with 8) and the
+// mixed forms cross at the same sizes.
+int wide_lanes(int n) { return n <= 1024 ? 32 : (n <= 4096 ? 16 : (n <= 16384 ? 8 : 0)); }
+
+// One force evaluation with G = wide_lanes(n) lanes per atom; Ffix must be zero.  *blocks = partial-sum rows
+// written (at most WIDE_MAX_BLOCKS).
+template <class S, class MT>
+cudaError_t launch_wide(int lanes, const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
+                        const RowExt &X, float *usite, float *qout, long long *Ffix, long long *part_d,
+                        long long *part_f, int *status, const Fallback &fb, int *blocks, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  auto run = [&](auto kernel, int g_lanes) {
+    *blocks = wide_grid(kernel, n, g_lanes);
+    kernel<<<*blocks, WIDE_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, usite, qout,
+                                           reinterpret_cast<unsigned long long *>(Ffix), part_d, part_f, status, fb);
+  };
+  if (lanes == 32) run(k_nep_wide<S, MT, 32>, 32);
+  else if (lanes == 16) run(k_nep_wide<S, MT, 16>, 16);
+  else run(k_nep_wide<S, MT, 8>, 8);
+  return cudaGetLastError();
+}
+
+// The fallback model on the flagged atoms (list, count on the device): its site energies are added to usite and
+// to part_d[0], its forces to Ffix, its virial to part_f[0..8], the atom count to counters[9].
+template <class S>
+cudaError_t launch_wide_list(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
+                             const RowExt &X, const int *list, const int *count, int cap, float *usite, long long *Ffix,
+                             long long *part_d, long long *part_f, long long *counters, int *status, cudaStream_t st) {
+  if (n <= 0 || cap <= 0) return cudaSuccess;
+  k_nep_wide_list<S><<<wide_grid(k_nep_wide_list<S>, cap, 32), WIDE_BLOCK, 0, st>>>(
+      P, g, n, list, count, cap, pos, nbr, X, usite, reinterpret_cast<unsigned long long *>(Ffix), part_d, part_f,
+      counters, status);
+  return cudaGetLastError();
+}
+template cudaError_t launch_wide_list<CuShape>(const Model<CuShape> &, const Geom &, int, const float4 *, const int32_t *,
+                                               const RowExt &, const int *, const int *, int, float *, long long *,
+                                               long long *, long long *, long long *, int *, cudaStream_t);
+
+#define NEP_INSTANTIATE(SH, MT)                                                                                     \
+  template cudaError_t launch_wide<SH, MT>(int, const Model<SH> &, const Geom &, int, const float4 *, const int32_t *, \
+                                           const RowExt &, float *, float *, long long *, long long *, long long *,   \
+                                           int *, const Fallback &, int *, cudaStream_t);
+NEP_INSTANTIATE(CuShape, float)
+NEP_INSTANTIATE(CuShape, __nv_bfloat16)
+NEP_INSTANTIATE(CuShape, __half)
+NEP_INSTANTIATE(StudentShape, float)
+NEP_INSTANTIATE(StudentShape, __nv_bfloat16)
+NEP_INSTANTIATE(StudentShape, __half)
+#undef NEP_INSTANTIATE
+
+}  // namespace nep
