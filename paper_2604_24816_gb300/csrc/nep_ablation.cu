@@ -29,7 +29,7 @@ template <class S, int NT>
 __global__ void __launch_bounds__(TB, 2)
 k_descriptor_tiled(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
                    const int32_t *__restrict__ nbr, const RowExt X, float *__restrict__ G,
-                   float *__restrict__ usite, long long *__restrict__ Ffix, long long *__restrict__ part,
+                   float *__restrict__ usite, long long *__restrict__ Ffix, const EvalSums sums,
                    int *__restrict__ status, float *__restrict__ sbuf) {
   __shared__ float4 shift[27];
   __shared__ uint32_t ring_e[T_DE * TB];
@@ -204,7 +204,7 @@ k_descriptor_tiled(const __grid_constant__ Model<S> P, const Geom geom, const in
     acc[3] = cnt;
     acc[4] = nact;
   }
-  block_sum_store<5>(acc, part);
+  eval_add_d<TB / 32>(sums, acc);
 }
 
 // The angular part of one pair's force with the centre's adjoint row in shared memory (Gs: [NA][NLM]
@@ -267,7 +267,7 @@ template <class S, int CPB>
 __global__ void __launch_bounds__(TB, 2)
 k_force_cpb(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
             const int32_t *__restrict__ nbr, const RowExt X, const float *__restrict__ G,
-            unsigned long long *__restrict__ Ffix, long long *__restrict__ part, int *__restrict__ status) {
+            unsigned long long *__restrict__ Ffix, const EvalSums sums, int *__restrict__ status) {
   static_assert(CPB >= 1 && CPB <= 3 && S::GS % 4 == 0, "1 to 3 centres per warp");
   constexpr int NW = TB / 32;
   __shared__ float4 shift[27];
@@ -378,7 +378,7 @@ k_force_cpb(const __grid_constant__ Model<S> P, const Geom geom, const int n, co
   acc[3] = acc[1]; acc[4] = -to_fix32(wyy); acc[5] = -to_fix32(wyz);
   acc[6] = acc[2]; acc[7] = acc[5]; acc[8] = -to_fix32(wzz);
   acc[9] = cnt_list; acc[10] = cnt_act; acc[11] = cnt_rad; acc[12] = cnt_ang;
-  block_sum_store<13, NW>(acc, part);
+  eval_add_f<NW>(sums, acc);
 }
 
 // Angular pairs (r < rc_A) of every atom's walked row.
@@ -416,10 +416,10 @@ __global__ void k_store_float3(int n, const int *__restrict__ id, const float *_
 
 template <class S, int NT>
 cudaError_t launch_descriptor_tiled(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
-                                    const RowExt &X, float *G, float *usite, long long *Ffix, long long *part,
+                                    const RowExt &X, float *G, float *usite, long long *Ffix, const EvalSums &sums,
                                     int *status, float *sbuf, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_descriptor_tiled<S, NT><<<(n + TB - 1) / TB, TB, 0, st>>>(P, g, n, pos, nbr, X, G, usite, Ffix, part, status,
+  k_descriptor_tiled<S, NT><<<(n + TB - 1) / TB, TB, 0, st>>>(P, g, n, pos, nbr, X, G, usite, Ffix, sums, status,
                                                                sbuf);
   return cudaGetLastError();
 }
@@ -429,24 +429,22 @@ cudaError_t launch_store_float3(int n, const int *id, const float *Ff, double *o
   return cudaGetLastError();
 }
 
-int tiled_descriptor_blocks(int n) { return (n + TB - 1) / TB; }
-
 template <class S>
 cudaError_t launch_force_cpb(int cpb, const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
-                             const RowExt &X, const float *G, long long *Ffix, long long *part, int *status,
+                             const RowExt &X, const float *G, long long *Ffix, const EvalSums &sums, int *status,
                              cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int grid = (n + TB - 1) / TB;
   unsigned long long *F = reinterpret_cast<unsigned long long *>(Ffix);
-  if (cpb == 1) k_force_cpb<S, 1><<<grid, TB, 0, st>>>(P, g, n, pos, nbr, X, G, F, part, status);
-  else if (cpb == 2) k_force_cpb<S, 2><<<grid, TB, 0, st>>>(P, g, n, pos, nbr, X, G, F, part, status);
-  else if (cpb == 3) k_force_cpb<S, 3><<<grid, TB, 0, st>>>(P, g, n, pos, nbr, X, G, F, part, status);
+  if (cpb == 1) k_force_cpb<S, 1><<<grid, TB, 0, st>>>(P, g, n, pos, nbr, X, G, F, sums, status);
+  else if (cpb == 2) k_force_cpb<S, 2><<<grid, TB, 0, st>>>(P, g, n, pos, nbr, X, G, F, sums, status);
+  else if (cpb == 3) k_force_cpb<S, 3><<<grid, TB, 0, st>>>(P, g, n, pos, nbr, X, G, F, sums, status);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 template cudaError_t launch_force_cpb<CuShape>(int, const Model<CuShape> &, const Geom &, int, const float4 *,
-                                               const int32_t *, const RowExt &, const float *, long long *, long long *,
-                                               int *, cudaStream_t);
+                                               const int32_t *, const RowExt &, const float *, long long *,
+                                               const EvalSums &, int *, cudaStream_t);
 
 cudaError_t launch_angular_counts(int n, const float4 *pos, const int32_t *nbr, const RowExt &X, const Geom &g,
                                   float rcA2, int *out, cudaStream_t st) {
@@ -456,9 +454,9 @@ cudaError_t launch_angular_counts(int n, const float4 *pos, const int32_t *nbr, 
 
 template cudaError_t launch_descriptor_tiled<CuShape, 1>(const Model<CuShape> &, const Geom &, int, const float4 *,
                                                          const int32_t *, const RowExt &, float *, float *,
-                                                         long long *, long long *, int *, float *, cudaStream_t);
+                                                         long long *, const EvalSums &, int *, float *, cudaStream_t);
 template cudaError_t launch_descriptor_tiled<CuShape, 3>(const Model<CuShape> &, const Geom &, int, const float4 *,
                                                          const int32_t *, const RowExt &, float *, float *,
-                                                         long long *, long long *, int *, float *, cudaStream_t);
+                                                         long long *, const EvalSums &, int *, float *, cudaStream_t);
 
 }  // namespace nep

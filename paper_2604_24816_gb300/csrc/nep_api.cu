@@ -1,10 +1,10 @@
 // nep_api.cu -- the C ABI declared in include/nep_gb300.h: handle, device buffers, step sequencing.
 //
-// One MD step enqueues: kick+drift -> step control -> rebuild chain (kernels return at once unless
-// the control kernel asked for a rebuild) -> descriptors+network -> forces -> kick -> reductions.
-// Because the rebuild decision is taken on the device, a step has a fixed launch sequence: it is
-// captured once as a CUDA graph and replayed, with no host synchronisation inside an md_verlet_step
-// call.  With timing enabled the same sequence is launched eagerly with CUDA events around each
+// One MD step enqueues: kick+drift (which clears the forces) -> rebuild decision and chain (kernels return at
+// once unless a rebuild was decided) -> descriptors, network and forces (whose last block publishes the energy and
+// virial); the closing half kick belongs to the next step or the end of the call.  Because the rebuild decision is
+// taken on the device, a step has a fixed launch sequence: steps are captured as a CUDA graph and replayed, with no
+// host synchronisation inside an md_verlet_step call.  With timing enabled the same sequence is launched eagerly with CUDA events around each
 // kernel class.  The only host waits are bounded polls of a stream event (NEP_ERR_TIMEOUT).
 #include <cuda_runtime.h>
 
@@ -21,6 +21,7 @@
 
 #include "nep_gb300.h"
 #include "nep_common.cuh"
+#include "nep_control.cuh"
 #include "nep_descriptor.cuh"
 #include "nep_tc.cuh"
 
@@ -28,81 +29,73 @@ namespace nep {
 // nep_force.cu
 template <class S>
 cudaError_t launch_descriptor(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
-                              float *, float *, float *, long long *, long long *, int *, const Fallback &,
+                              float *, float *, float *, long long *, const EvalSums &, int *, const Fallback &,
                               cudaStream_t);
 template <class S, class GT>
 cudaError_t launch_force(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
-                         const GT *, long long *, long long *, int *, cudaStream_t);
+                         const GT *, long long *, const EvalSums &, int *, cudaStream_t);
 template <class S>
 cudaError_t launch_fused(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &, float *,
-                         float *, long long *, long long *, long long *, int *, const PairCache &, cudaStream_t);
+                         float *, long long *, const EvalSums &, int *, const PairCache &, cudaStream_t);
 template <class S, class MT>
 cudaError_t launch_fused_mixed(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
-                               float *, float *, long long *, long long *, long long *, int *, const PairCache &,
-                               cudaStream_t);
+                               float *, float *, long long *, const EvalSums &, int *, const PairCache &, cudaStream_t);
 template <class S>
 cudaError_t launch_fused_reg(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
-                             float *, float *, long long *, long long *, long long *, int *, const Fallback &,
+                             float *, float *, long long *, const EvalSums &, int *, const Fallback &,
                              const PairCache &, cudaStream_t);
 cudaError_t pair_cache_sm_bound(int *nsm);
 size_t pair_cache_region_elems(int pmax);
-int descriptor_blocks(int n);
-int force_blocks(int n);
 // nep_mixed.cu
 template <class S, class MT>
 cudaError_t launch_descriptor_mixed(const Model<S> &, const Geom &, int, const float4 *, const int32_t *,
-                                    const RowExt &, __half *, float *, float *, long long *, long long *, int *,
+                                    const RowExt &, __half *, float *, float *, long long *, const EvalSums &, int *,
                                     const Fallback &, cudaStream_t);
-int mixed_descriptor_blocks(int n);
 // nep_wide.cu
 int wide_lanes(int n);
 template <class S, class MT>
 cudaError_t launch_wide(int, const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
-                        float *, float *, long long *, long long *, long long *, int *, const Fallback &, int *,
-                        cudaStream_t);
+                        float *, float *, long long *, const EvalSums &, int *, const Fallback &, cudaStream_t);
 template <class S>
 cudaError_t launch_wide_list(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
-                             const int *, const int *, int, float *, long long *, long long *, long long *,
-                             long long *, int *, cudaStream_t);
+                             const int *, const int *, int, float *, long long *, const EvalSums &, int *,
+                             cudaStream_t);
 cudaError_t launch_fallback_flags(const int *, const int *, int, const int *, int *, cudaStream_t);
 // nep_force.cu / nep_ablation.cu: kernel variants for ablation
 template <class S>
 cudaError_t launch_force_float_scatter(const Model<S> &, const Geom &, int, const float4 *, const int32_t *,
-                                       const RowExt &, const float *, float *, long long *, int *, cudaStream_t);
+                                       const RowExt &, const float *, float *, const EvalSums &, int *, cudaStream_t);
 template <class S>
 cudaError_t launch_force_half_list(const Model<S> &, const Geom &, int, const float4 *, const int32_t *,
-                                   const RowExt &, const float *, long long *, long long *, int *, cudaStream_t);
+                                   const RowExt &, const float *, long long *, const EvalSums &, int *, cudaStream_t);
 template <class S, int NT>
 cudaError_t launch_descriptor_tiled(const Model<S> &, const Geom &, int, const float4 *, const int32_t *,
-                                    const RowExt &, float *, float *, long long *, long long *, int *, float *,
+                                    const RowExt &, float *, float *, long long *, const EvalSums &, int *, float *,
                                     cudaStream_t);
 cudaError_t launch_store_float3(int, const int *, const float *, double *, cudaStream_t);
 template <class S>
 cudaError_t launch_force_cpb(int, const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
-                             const float *, long long *, long long *, int *, cudaStream_t);
+                             const float *, long long *, const EvalSums &, int *, cudaStream_t);
 cudaError_t launch_angular_counts(int, const float4 *, const int32_t *, const RowExt &, const Geom &, float, int *,
                                   cudaStream_t);
 // nep_neighbor.cu
-cudaError_t launch_cell_sort(const RebuildArgs &, cudaStream_t);
+cudaError_t launch_cell_sort(const RebuildArgs &, int, cudaStream_t);
+bool cell_sort_decides(int n, int ncell);
 cudaError_t launch_neighbors(const RebuildArgs &, cudaStream_t);
 int scan_tiles(int ncell);
 int cell_sort_launches(int n, int ncell);
 // nep_md.cu
-int md_blocks(int n);
-cudaError_t launch_kick_drift(int, double *, double *, double *, double *, double *, double *, const long long *, float4 *,
+cudaError_t launch_kick_drift(int, double *, double *, double *, double *, double *, double *, long long *, float4 *,
                               const float4 *, double, double, const double *, float, Control *, cudaStream_t);
-cudaError_t launch_control(Control *, bool, cudaStream_t);
+cudaError_t launch_control(Control *, int, cudaStream_t);
 cudaError_t launch_control_cond(Control *, cudaGraphConditionalHandle, cudaStream_t);
-cudaError_t launch_control_check(Control *, cudaStream_t);
 cudaError_t launch_inverse_order(int, const int *, int *, cudaStream_t);
 cudaError_t launch_load_state_sorted(int, const double *, const double *, const int *, double *, double *, double *,
                                      double *, double *, double *, float4 *, const float4 *, const double *,
                                      const double *, float, Control *, cudaStream_t);
-cudaError_t launch_kick(int, double *, double *, double *, const long long *, double, double, long long *, Control *,
+cudaError_t launch_kick(int, double *, double *, double *, const long long *, double, double, const EvalSums &, Control *,
                         cudaStream_t);
-cudaError_t launch_kinetic(int, const double *, const double *, const double *, double, long long *, cudaStream_t);
-cudaError_t launch_finalize(const long long *, int, const long long *, int, const long long *, int, double *,
-                            long long *, cudaStream_t);
+cudaError_t launch_kinetic(int, const double *, const double *, const double *, double, const EvalSums &, cudaStream_t);
 cudaError_t launch_load_state(int, const double *, const double *, double *, double *, double *, double *, double *,
                               double *, int *, int *, cudaStream_t);
 cudaError_t launch_store_vec(int, const int *, const double *, const double *, const double *, const double *, int,
@@ -129,6 +122,28 @@ enum KClass {
 struct Timer {
   int cls;
   cudaEvent_t a, b;
+};
+
+// A captured sequence of MD steps.
+struct StepGraph {
+  cudaGraphExec_t exec = nullptr;
+  double dt = 0.0;
+  int steps = 0;
+  long long launches = 0;          // our kernel launches in it, outside a conditional rebuild chain
+  void destroy() {
+    if (exec) cudaGraphExecDestroy(exec);
+    exec = nullptr;
+  }
+};
+
+// What the host reads after a call, contiguous so that one copy brings it (three copies of 1.3 us each, with the
+// gaps between them, before); then the running totals (EvalSums).
+struct DeviceReport {
+  Control ctrl;
+  double sums[32];
+  long long counters[16];
+  long long acc[N_SUMS];
+  unsigned done;
 };
 
 }  // namespace
@@ -168,27 +183,22 @@ struct nep_handle {
   void *G = nullptr;               // adjoint rows: float32 (plain) or float16 (mixed) [n][GS]
   int32_t *nbr = nullptr, *nnum = nullptr, *nang = nullptr, *nown = nullptr, *nband0 = nullptr, *nfar = nullptr;
   int *count = nullptr, *cursor = nullptr, *start = nullptr, *tile_sums = nullptr;
-  long long *part_d = nullptr, *part_f = nullptr, *part_k = nullptr;   // per-block int64 partial sums
+  DeviceReport *rep = nullptr;     // control block, sums and counters, read back together
+  Control *ctrl = nullptr;         // its parts
   double *sums = nullptr;
   long long *counters = nullptr;   // pair counts (descriptor, force) and evaluations
-  Control *ctrl = nullptr;
   double *io = nullptr;            // staging 2 x [n][3] float64 for host transfers
   int32_t *io_i = nullptr;         // staging for neighbour output
   size_t io_i_elems = 0;
-  int nb_d = 0, nb_f = 0, nb_k = 0;   // rows of partial sums of the last evaluation
   int wide = 0;                    // lanes per atom of the wide kernels, 0: one thread per atom
 
-  // host mirrors (pinned)
-  double *h_sums = nullptr;
-  Control *h_ctrl = nullptr;
-  long long *h_counters = nullptr;
+  // host mirror (pinned)
+  DeviceReport *h_rep = nullptr;
   cudaEvent_t done = nullptr;
 
-  // graph of one MD step
-  cudaGraphExec_t graph = nullptr;
-  double graph_dt = 0.0;
-  long long graph_launches = 0;   // our kernel launches in one captured step, outside the rebuild chain
-  long long graph_rebuild_launches = 0;   // those of the rebuild chain (run on rebuild steps only)
+  // graphs of MD steps: one step, and several
+  StepGraph graph1, graphk;
+  long long graph_rebuild_launches = 0;   // kernel launches of a conditional rebuild chain (run on rebuild steps only)
 
   // timing
   bool timing = false;
@@ -268,14 +278,15 @@ void dfree(T *&p) {
 }
 
 void free_system(nep_handle *h) {
-  if (h->graph) { cudaGraphExecDestroy(h->graph); h->graph = nullptr; }
+  h->graph1.destroy();
+  h->graphk.destroy();
   dfree(h->x); dfree(h->y); dfree(h->z); dfree(h->vx); dfree(h->vy); dfree(h->vz);
   dfree(h->xb); dfree(h->yb); dfree(h->zb); dfree(h->vxb); dfree(h->vyb); dfree(h->vzb);
   dfree(h->id); dfree(h->idb); dfree(h->cell_of); dfree(h->perm);
   dfree(h->pos); dfree(h->pos_ref); dfree(h->F); dfree(h->usite); dfree(h->G); dfree(h->qbuf);
   dfree(h->nbr); dfree(h->nnum); dfree(h->nang); dfree(h->nown); dfree(h->nband0); dfree(h->nfar);
   dfree(h->count); dfree(h->cursor); dfree(h->start); dfree(h->tile_sums);
-  dfree(h->part_d); dfree(h->part_f); dfree(h->part_k); dfree(h->io); dfree(h->io_i);
+  dfree(h->io); dfree(h->io_i);
   dfree(h->fb_list); dfree(h->fb_count);
   dfree(h->abl_f); dfree(h->abl_s); dfree(h->abl_cnt);
   dfree(h->pc_rec); dfree(h->pc_mask); dfree(h->inv);
@@ -353,6 +364,14 @@ float far_dmax2(float skin) {
   return d > 0.f ? d * d : -1.f;
 }
 
+// A new system's control block (the handle's rebuild policy), no sums, no counts.
+cudaError_t reset_report(nep_handle *h) {
+  *h->h_rep = DeviceReport{};
+  h->h_rep->ctrl.rebuild_every = h->rebuild_every;
+  h->h_rep->ctrl.far_dmax2 = far_dmax2(h->skin);
+  return cudaMemcpyAsync(h->rep, h->h_rep, sizeof(DeviceReport), cudaMemcpyHostToDevice, h->stream);
+}
+
 RebuildArgs rebuild_args(nep_handle *h) {
   RebuildArgs a;
   a.n = h->n; a.ncell = h->ncell;
@@ -381,29 +400,42 @@ Geom geom_of(nep_handle *h) {
   return g;
 }
 
-// Rebuild chain (cell sort + neighbour list); kernels act only if ctrl->do_rebuild is set.
-cudaError_t enqueue_rebuild(nep_handle *h) {
+// Rebuild chain (cell sort + neighbour list), after the decision of kind `decide` (nep_control.cuh): taken by the
+// sort's own kernel for small systems, by a control kernel otherwise.  The kernels act only if ctrl->do_rebuild is
+// set.
+cudaError_t enqueue_rebuild(nep_handle *h, int decide) {
   RebuildArgs a = rebuild_args(h);
   cudaError_t e;
+  if (decide != DECIDE_DONE && !cell_sort_decides(h->n, h->ncell)) {
+    Scope sc(h, KC_CELL, 1);
+    if ((e = launch_control(h->ctrl, decide, h->stream)) != cudaSuccess) return e;
+    decide = DECIDE_DONE;
+  }
   {
     Scope sc(h, KC_CELL, cell_sort_launches(h->n, h->ncell));
-    e = launch_cell_sort(a, h->stream);
+    e = launch_cell_sort(a, decide, h->stream);
   }
   if (e != cudaSuccess) return e;
   Scope sc(h, KC_NEIGH, 1);
   return launch_neighbors(a, h->stream);
 }
 
+// The running totals of an evaluation; last: the kernel that gets them ends it.
+EvalSums eval_sums(nep_handle *h, bool last) {
+  return EvalSums{h->rep->acc, &h->rep->done, h->sums, h->counters, last ? 1 : 0};
+}
+
 // The teacher on the flagged atoms of a student's evaluation (after the student's kernels).
 cudaError_t enqueue_fallback(nep_handle *h, const Geom &g) {
   Scope sc(h, KC_FB, 1);
   return launch_wide_list<CuShape>(h->fb_model, g, h->n, h->pos, h->nbr, rows_of(h), h->fb_list, h->fb_count, h->fb_cap,
-                                   h->usite, h->F, h->part_d, h->part_f, h->counters, &h->ctrl->status, h->stream);
+                                   h->usite, h->F, eval_sums(h, true), &h->ctrl->status, h->stream);
 }
 
-// Descriptors + network + forces; partial sums reduced with KE partials pk (may be null).
+// Descriptors + network + forces, energy, virial and counters.  zeroed: the forces are already clear (the drift
+// kernel of an MD step clears them).
 template <class S>
-cudaError_t forces_of(nep_handle *h, const Model<S> &M, float *qout) {
+cudaError_t forces_of(nep_handle *h, const Model<S> &M, float *qout, bool zeroed) {
   constexpr bool teacher = std::is_same<S, CuShape>::value;
   const Geom g = geom_of(h);
   Fallback fb{};
@@ -415,75 +447,82 @@ cudaError_t forces_of(nep_handle *h, const Model<S> &M, float *qout) {
   cudaError_t e;
   if (fb.on && (e = cudaMemsetAsync(h->fb_count, 0, sizeof(int), h->stream)) != cudaSuccess) return e;
   if (h->wide > 0 || teacher || h->precision == NEP_FP32) {
-    // descriptors, network and full-row forces in one kernel (forces zeroed first), then the teacher on the
-    // flagged atoms; the network in float32, or with bf16 / f16 operands in the mixed-precision forms
+    // descriptors, network and full-row forces in one kernel, then the teacher on the flagged atoms; the network
+    // in float32, or with bf16 / f16 operands in the mixed-precision forms
     {
       Scope sc(h, KC_FORCE, 1);
-      if ((e = cudaMemsetAsync(h->F, 0, 3 * (size_t)h->n * sizeof(long long), h->stream)) != cudaSuccess) return e;
+      if (!zeroed &&
+          (e = cudaMemsetAsync(h->F, 0, 3 * (size_t)h->n * sizeof(long long), h->stream)) != cudaSuccess)
+        return e;
+      const EvalSums es = eval_sums(h, !fb.on);
+      int *status = &h->ctrl->status;
+      const RowExt rows = rows_of(h);
       if (h->wide > 0) {
-        int blocks = 0;
         if (h->precision == NEP_FP32)
-          e = launch_wide<S, float>(h->wide, M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F, h->part_d,
-                                    h->part_f, &h->ctrl->status, fb, &blocks, h->stream);
+          e = launch_wide<S, float>(h->wide, M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status, fb,
+                                    h->stream);
         else if (h->precision == NEP_MIX_BF16)
-          e = launch_wide<S, __nv_bfloat16>(h->wide, M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F,
-                                            h->part_d, h->part_f, &h->ctrl->status, fb, &blocks, h->stream);
+          e = launch_wide<S, __nv_bfloat16>(h->wide, M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status,
+                                            fb, h->stream);
         else
-          e = launch_wide<S, __half>(h->wide, M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F, h->part_d,
-                                     h->part_f, &h->ctrl->status, fb, &blocks, h->stream);
-        h->nb_d = h->nb_f = blocks;
+          e = launch_wide<S, __half>(h->wide, M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status, fb,
+                                     h->stream);
       } else {
         const PairCache pc{h->pc_rec, h->pc_mask, h->pc_nsm, h->cap, h->pc_slots};
         if constexpr (teacher) {
           if (h->precision == NEP_FP32)
-            e = launch_fused<CuShape>(M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F, h->part_d,
-                                      h->part_f, &h->ctrl->status, pc, h->stream);
+            e = launch_fused<CuShape>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status, pc, h->stream);
           else if (h->precision == NEP_MIX_BF16)
-            e = launch_fused_mixed<CuShape, __nv_bfloat16>(M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout,
-                                                           h->F, h->part_d, h->part_f, &h->ctrl->status, pc, h->stream);
+            e = launch_fused_mixed<CuShape, __nv_bfloat16>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es,
+                                                           status, pc, h->stream);
           else
-            e = launch_fused_mixed<CuShape, __half>(M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F,
-                                                    h->part_d, h->part_f, &h->ctrl->status, pc, h->stream);
+            e = launch_fused_mixed<CuShape, __half>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status,
+                                                    pc, h->stream);
         } else {
-          e = launch_fused_reg<StudentShape>(M, g, h->n, h->pos, h->nbr, rows_of(h), h->usite, qout, h->F, h->part_d,
-                                             h->part_f, &h->ctrl->status, fb, pc, h->stream);
+          e = launch_fused_reg<StudentShape>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status, fb, pc,
+                                             h->stream);
         }
       }
     }
     return e == cudaSuccess && fb.on ? enqueue_fallback(h, g) : e;
   }
-  // the student's mixed form: tensor-core descriptor kernel, then the half-list force kernel over float16 rows
-  {
-    Scope sc(h, KC_DESC, 1);
-    if (h->precision == NEP_MIX_BF16)
-      e = launch_descriptor_mixed<S, __nv_bfloat16>(M, g, h->n, h->pos, h->nbr, rows_of(h), static_cast<__half *>(h->G),
-                                                    h->usite, qout, h->F, h->part_d, &h->ctrl->status, fb, h->stream);
-    else
-      e = launch_descriptor_mixed<S, __half>(M, g, h->n, h->pos, h->nbr, rows_of(h), static_cast<__half *>(h->G),
-                                             h->usite, qout, h->F, h->part_d, &h->ctrl->status, fb, h->stream);
+  if constexpr (teacher) {
+    return cudaErrorInvalidValue;          // not reached: the teacher took the branch above
+  } else {
+    // the student's mixed form: tensor-core descriptor kernel (which clears the forces), then the half-list force
+    // kernel over float16 rows
+    {
+      Scope sc(h, KC_DESC, 1);
+      const EvalSums es = eval_sums(h, false);
+      if (h->precision == NEP_MIX_BF16)
+        e = launch_descriptor_mixed<S, __nv_bfloat16>(M, g, h->n, h->pos, h->nbr, rows_of(h), static_cast<__half *>(h->G),
+                                                      h->usite, qout, h->F, es, &h->ctrl->status, fb, h->stream);
+      else
+        e = launch_descriptor_mixed<S, __half>(M, g, h->n, h->pos, h->nbr, rows_of(h), static_cast<__half *>(h->G),
+                                               h->usite, qout, h->F, es, &h->ctrl->status, fb, h->stream);
+    }
+    if (e != cudaSuccess) return e;
+    {
+      Scope sc(h, KC_FORCE, 1);
+      e = launch_force<S, __half>(M, g, h->n, h->pos, h->nbr, rows_of(h), static_cast<const __half *>(h->G), h->F,
+                                  eval_sums(h, !fb.on), &h->ctrl->status, h->stream);
+    }
+    return e == cudaSuccess && fb.on ? enqueue_fallback(h, g) : e;
   }
-  if (e != cudaSuccess) return e;
-  {
-    Scope sc(h, KC_FORCE, 1);
-    e = launch_force<S, __half>(M, g, h->n, h->pos, h->nbr, rows_of(h), static_cast<const __half *>(h->G), h->F,
-                                h->part_f, &h->ctrl->status, h->stream);
-  }
-  return e == cudaSuccess && fb.on ? enqueue_fallback(h, g) : e;
 }
 
-cudaError_t enqueue_forces(nep_handle *h, float *qout) {
-  return h->shape == 0 ? forces_of<CuShape>(h, h->model_t, qout) : forces_of<StudentShape>(h, h->model_s, qout);
+cudaError_t enqueue_forces(nep_handle *h, float *qout, bool zeroed = false) {
+  return h->shape == 0 ? forces_of<CuShape>(h, h->model_t, qout, zeroed)
+                       : forces_of<StudentShape>(h, h->model_s, qout, zeroed);
 }
 
-cudaError_t enqueue_finalize(nep_handle *h, bool with_kinetic) {
-  Scope sc(h, KC_RED, 1);
-  return launch_finalize(h->part_d, h->nb_d, h->part_f, h->nb_f, with_kinetic ? h->part_k : nullptr, h->nb_k, h->sums,
-                         h->counters, h->stream);
+cudaError_t enqueue_kinetic(nep_handle *h) {
+  Scope sc(h, KC_OTHER, 1);
+  return launch_kinetic(h->n, h->vx, h->vy, h->vz, h->mass, eval_sums(h, true), h->stream);
 }
 
-// One velocity-Verlet step.
 // One MD step.  Launched eagerly (capture = false) the rebuild chain's kernels run every step and
-// return at once unless the control kernel decided to rebuild.  Under stream capture (capture = true)
+// return at once unless the decision is to rebuild.  Under stream capture (capture = true)
 // the chain is the body of a conditional graph node whose condition the control kernel sets, so a
 // step without a rebuild launches none of its kernels; the chain is captured from the auxiliary stream
 // into the node's body graph.
@@ -491,6 +530,15 @@ cudaError_t enqueue_step(nep_handle *h, double dt, bool capture = false) {
   const double kick = 0.5 * dt * ACC_CONV / h->mass;
   const float hs = 0.5f * h->skin;
   cudaError_t e;
+  cudaStreamCaptureStatus cs;
+  cudaGraph_t graph = nullptr;
+  const cudaGraphNode_t *deps = nullptr;
+  size_t nd = 0;
+  cudaGraphConditionalHandle cond{};
+  if (capture) {
+    if ((e = cudaStreamGetCaptureInfo(h->stream, &cs, nullptr, &graph, &deps, nullptr, &nd)) != cudaSuccess) return e;
+    if ((e = cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault)) != cudaSuccess) return e;
+  }
   {
     Scope sc(h, KC_DRIFT, 1);
     e = launch_kick_drift(h->n, h->x, h->y, h->z, h->vx, h->vy, h->vz, h->F, h->pos, h->pos_ref, kick, dt, h->l,
@@ -498,20 +546,8 @@ cudaError_t enqueue_step(nep_handle *h, double dt, bool capture = false) {
   }
   if (e != cudaSuccess) return e;
   if (!capture) {
-    {
-      Scope sc(h, KC_CELL, 1);
-      e = launch_control(h->ctrl, false, h->stream);
-    }
-    if (e != cudaSuccess) return e;
-    if ((e = enqueue_rebuild(h)) != cudaSuccess) return e;
+    if ((e = enqueue_rebuild(h, DECIDE_STEP)) != cudaSuccess) return e;
   } else {
-    cudaStreamCaptureStatus cs;
-    cudaGraph_t graph = nullptr;
-    const cudaGraphNode_t *deps = nullptr;
-    size_t nd = 0;
-    if ((e = cudaStreamGetCaptureInfo(h->stream, &cs, nullptr, &graph, &deps, nullptr, &nd)) != cudaSuccess) return e;
-    cudaGraphConditionalHandle cond;
-    if ((e = cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault)) != cudaSuccess) return e;
     {
       Scope sc(h, KC_CELL, 1);
       e = launch_control_cond(h->ctrl, cond, h->stream);
@@ -536,7 +572,7 @@ cudaError_t enqueue_step(nep_handle *h, double dt, bool capture = false) {
     const long long before = h->launch_total;
     cudaStream_t main = h->stream;
     h->stream = h->aux;                       // the chain's launches go to the body graph
-    const cudaError_t eb = enqueue_rebuild(h);
+    const cudaError_t eb = enqueue_rebuild(h, DECIDE_DONE);
     h->stream = main;
     cudaGraph_t captured = nullptr;
     const cudaError_t ee = cudaStreamEndCapture(h->aux, &captured);
@@ -545,37 +581,26 @@ cudaError_t enqueue_step(nep_handle *h, double dt, bool capture = false) {
     if (eb != cudaSuccess) return eb;
     if (ee != cudaSuccess) return ee;
   }
-  if ((e = enqueue_forces(h, nullptr)) != cudaSuccess) return e;
-  // the energy, virial and pair counts of this evaluation (the kinetic energy is the one of the last
+  // the energy, virial and pair counts are published by the evaluation (the kinetic energy is the one of the last
   // closing kick, refreshed by enqueue_step_end); the closing half kick is left to the next step's
   // opening kick, which applies both at once
-  Scope sc(h, KC_RED, 1);
-  return launch_finalize(h->part_d, h->nb_d, h->part_f, h->nb_f, nullptr, h->nb_k, h->sums, h->counters, h->stream);
+  return enqueue_forces(h, nullptr, true);
 }
 
-// The closing half kick of the last step of md_verlet_step, its kinetic energy, and the sums again
-// with it (no counters: the evaluation was counted by its own step).
+// The closing half kick of the last step of md_verlet_step, and its kinetic energy.
 cudaError_t enqueue_step_end(nep_handle *h, double dt) {
   const double kick = 0.5 * dt * ACC_CONV / h->mass;
-  cudaError_t e;
-  {
-    Scope sc(h, KC_KICK, 1);
-    e = launch_kick(h->n, h->vx, h->vy, h->vz, h->F, kick, h->mass, h->part_k, h->ctrl, h->stream);
-  }
-  if (e != cudaSuccess) return e;
-  Scope sc(h, KC_RED, 1);
-  return launch_finalize(h->part_d, h->nb_d, h->part_f, h->nb_f, h->part_k, h->nb_k, h->sums, nullptr, h->stream);
+  Scope sc(h, KC_KICK, 1);
+  return launch_kick(h->n, h->vx, h->vy, h->vz, h->F, kick, h->mass, eval_sums(h, true), h->ctrl, h->stream);
 }
 
 // Read back the control block and translate device-detected conditions into a status.
 nep_status check_device_status(nep_handle *h) {
-  NEP_CUDA(h, cudaMemcpyAsync(h->h_ctrl, h->ctrl, sizeof(Control), cudaMemcpyDeviceToHost, h->stream));
-  NEP_CUDA(h, cudaMemcpyAsync(h->h_sums, h->sums, 32 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  NEP_CUDA(h, cudaMemcpyAsync(h->h_counters, h->counters, 16 * sizeof(long long), cudaMemcpyDeviceToHost, h->stream));
+  NEP_CUDA(h, cudaMemcpyAsync(h->h_rep, h->rep, offsetof(DeviceReport, acc), cudaMemcpyDeviceToHost, h->stream));
   nep_status s = wait_stream(h);
   if (s != NEP_OK) return s;
   if (h->timing) collect_timers(h);
-  const int st = h->h_ctrl->status;
+  const int st = h->h_rep->ctrl.status;
   if (st & ST_OVERFLOW)
     return fail(h, NEP_ERR_NEIGH_OVERFLOW, "an atom has more neighbours within rc_R + skin than max_neighbors");
   if (st & ST_NAN) return fail(h, NEP_ERR_NAN, "non-finite position, energy or force");
@@ -589,21 +614,13 @@ nep_status check_device_status(nep_handle *h) {
 nep_status ensure_nlist(nep_handle *h) {
   if (h->have_nlist && h->recheck) {
     // an upload kept the list: rebuild (on the device) only if an atom moved more than skin/2
-    {
-      Scope sc(h, KC_CELL, 1);
-      NEP_CUDA(h, launch_control_check(h->ctrl, h->stream));
-    }
-    NEP_CUDA(h, enqueue_rebuild(h));
+    NEP_CUDA(h, enqueue_rebuild(h, DECIDE_CHECK));
     h->recheck = false;
     return NEP_OK;
   }
   if (h->have_nlist) return NEP_OK;
   h->recheck = false;
-  {
-    Scope sc(h, KC_CELL, 1);
-    NEP_CUDA(h, launch_control(h->ctrl, true, h->stream));
-  }
-  NEP_CUDA(h, enqueue_rebuild(h));
+  NEP_CUDA(h, enqueue_rebuild(h, DECIDE_FORCE));
   h->have_nlist = true;
   h->have_forces = false;
   return NEP_OK;
@@ -613,30 +630,34 @@ nep_status compute_internal(nep_handle *h, float *qout) {
   nep_status s = ensure_nlist(h);
   if (s != NEP_OK) return s;
   NEP_CUDA(h, enqueue_forces(h, qout));
-  {
-    Scope sc(h, KC_OTHER, 1);
-    NEP_CUDA(h, launch_kinetic(h->n, h->vx, h->vy, h->vz, h->mass, h->part_k, h->stream));
-  }
-  NEP_CUDA(h, enqueue_finalize(h, true));
+  NEP_CUDA(h, enqueue_kinetic(h));
   h->have_forces = true;
   return NEP_OK;
 }
 
-nep_status build_graph(nep_handle *h, double dt) {
-  if (h->graph) { cudaGraphExecDestroy(h->graph); h->graph = nullptr; }
+// Steps that a replayed graph holds at most.
+constexpr int GRAPH_STEPS = 16;
+
+// Captures `steps` MD steps: with the rebuild chain behind a conditional node, or (small systems, whose chain is
+// two kernels that take the decision themselves) as plain kernels.
+nep_status build_graph(nep_handle *h, StepGraph &sg, double dt, int steps) {
+  sg.destroy();
   cudaGraph_t g = nullptr;
   const long long before = h->launch_total;
+  const bool conditional = !cell_sort_decides(h->n, h->ncell);
   NEP_CUDA(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-  cudaError_t e = enqueue_step(h, dt, true);
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < steps && e == cudaSuccess; ++k) e = enqueue_step(h, dt, conditional);
   cudaError_t e2 = cudaStreamEndCapture(h->stream, &g);
-  h->graph_launches = h->launch_total - before;   // kernels of one captured step, without the rebuild chain
+  sg.launches = h->launch_total - before;
   h->launch_total = before;
   if (e != cudaSuccess) { if (g) cudaGraphDestroy(g); return cuda_fail(h, e, "capture step"); }
   if (e2 != cudaSuccess) return cuda_fail(h, e2, "cudaStreamEndCapture");
-  e = cudaGraphInstantiate(&h->graph, g, 0);
+  e = cudaGraphInstantiate(&sg.exec, g, 0);
   cudaGraphDestroy(g);
-  if (e != cudaSuccess) { h->graph = nullptr; return cuda_fail(h, e, "cudaGraphInstantiate"); }
-  h->graph_dt = dt;
+  if (e != cudaSuccess) { sg.exec = nullptr; return cuda_fail(h, e, "cudaGraphInstantiate"); }
+  sg.dt = dt;
+  sg.steps = steps;
   return NEP_OK;
 }
 
@@ -697,20 +718,12 @@ nep_status upload_state_sorted(nep_handle *h, const double *x, const double *v) 
   }
   h->recheck = true;
   nep_status s = check_device_status(h);
-  if (s != NEP_OK || h->h_ctrl->changed || !had_forces) return s;
+  if (s != NEP_OK || h->h_rep->ctrl.changed || !had_forces) return s;
   // positions unchanged: keep the list state and the forces; refresh the kinetic energy sum (the
   // evaluation counters are not touched: no force evaluation ran)
   h->recheck = had_recheck;
   h->have_forces = true;
-  {
-    Scope sc(h, KC_OTHER, 1);
-    NEP_CUDA(h, launch_kinetic(h->n, h->vx, h->vy, h->vz, h->mass, h->part_k, h->stream));
-  }
-  {
-    Scope sc(h, KC_RED, 1);
-    NEP_CUDA(h, launch_finalize(h->part_d, h->nb_d, h->part_f, h->nb_f, h->part_k, h->nb_k, h->sums, nullptr,
-                                h->stream));
-  }
+  NEP_CUDA(h, enqueue_kinetic(h));
   return NEP_OK;
 }
 
@@ -841,20 +854,18 @@ nep_status nep_create(const nep_params *p, void *cuda_stream, nep_handle **out) 
     h->own_stream = true;
   }
   if ((e = cudaEventCreateWithFlags(&h->done, cudaEventDisableTiming)) != cudaSuccess ||
-      (e = dalloc(h->sums, 32)) != cudaSuccess || (e = dalloc(h->counters, 16)) != cudaSuccess ||
-      (e = dalloc(h->ctrl, 1)) != cudaSuccess || (e = cudaMallocHost((void **)&h->h_sums, 32 * sizeof(double))) != cudaSuccess ||
-      (e = cudaMallocHost((void **)&h->h_ctrl, sizeof(Control))) != cudaSuccess ||
-      (e = cudaMallocHost((void **)&h->h_counters, 16 * sizeof(long long))) != cudaSuccess) {
+      (e = dalloc(h->rep, 1)) != cudaSuccess ||
+      (e = cudaMallocHost((void **)&h->h_rep, sizeof(DeviceReport))) != cudaSuccess) {
     nep_destroy(h);
     return NEP_ERR_CUDA;
   }
-  cudaMemsetAsync(h->sums, 0, 32 * sizeof(double), h->stream);
-  cudaMemsetAsync(h->counters, 0, 16 * sizeof(long long), h->stream);
-  Control c0{};
-  c0.rebuild_every = h->rebuild_every;
-  c0.far_dmax2 = far_dmax2(h->skin);
-  cudaMemcpyAsync(h->ctrl, &c0, sizeof(Control), cudaMemcpyHostToDevice, h->stream);
-  if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) { nep_destroy(h); return NEP_ERR_CUDA; }
+  h->ctrl = &h->rep->ctrl;
+  h->sums = h->rep->sums;
+  h->counters = h->rep->counters;
+  if ((e = reset_report(h)) != cudaSuccess || (e = cudaStreamSynchronize(h->stream)) != cudaSuccess) {
+    nep_destroy(h);
+    return NEP_ERR_CUDA;
+  }
   *out = h;
   return NEP_OK;
 }
@@ -863,10 +874,8 @@ nep_status nep_destroy(nep_handle *h) {
   if (!h) return NEP_OK;
   if (h->stream) cudaStreamSynchronize(h->stream);
   free_system(h);
-  dfree(h->sums); dfree(h->counters); dfree(h->ctrl);
-  if (h->h_sums) cudaFreeHost(h->h_sums);
-  if (h->h_ctrl) cudaFreeHost(h->h_ctrl);
-  if (h->h_counters) cudaFreeHost(h->h_counters);
+  dfree(h->rep);
+  if (h->h_rep) cudaFreeHost(h->h_rep);
   for (auto &t : h->timers) { cudaEventDestroy(t.a); cudaEventDestroy(t.b); }
   if (h->done) cudaEventDestroy(h->done);
   for (cudaEvent_t ev : h->aux_ev)
@@ -912,10 +921,7 @@ nep_status nep_set_state(nep_handle *h, int64_t n, const double *x, const double
   }
   if (ncell > (int64_t)1 << 30) return fail(h, NEP_ERR_ARG, "too many cells");
   h->ncell = (int)ncell;
-  h->nb_d = h->precision == NEP_FP32 ? descriptor_blocks(h->n) : mixed_descriptor_blocks(h->n);
-  h->nb_f = force_blocks(h->n);
   h->wide = wide_lanes(h->n);
-  h->nb_k = md_blocks(h->n);
   const size_t N = (size_t)std::max(h->n, 1);
   cudaError_t e = cudaSuccess;
   auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
@@ -929,10 +935,7 @@ nep_status nep_set_state(nep_handle *h, int64_t n, const double *x, const double
   A(dalloc(h->nband0, N)); A(dalloc(h->nfar, N));
   A(dalloc(h->count, (size_t)h->ncell)); A(dalloc(h->cursor, (size_t)h->ncell)); A(dalloc(h->start, (size_t)h->ncell + 1));
   A(dalloc(h->tile_sums, (size_t)scan_tiles(h->ncell) + 1));
-  const size_t nb_w = h->wide > 0 ? WIDE_MAX_BLOCKS : 0;
-  A(dalloc(h->part_d, std::max((size_t)h->nb_d, nb_w) * 5 + 1));
-  A(dalloc(h->part_f, std::max((size_t)h->nb_f, nb_w) * 13 + 1));
-  A(dalloc(h->part_k, (size_t)h->nb_k + 1)); A(dalloc(h->io, 6 * N));
+  A(dalloc(h->io, 6 * N));
   if (h->fb_on) A(alloc_fallback(h));
   if (e == cudaSuccess && h->wide == 0 && (h->shape == 0 || h->precision == NEP_FP32)) {
     // pair records of the fused kernels: pc_slots regions per SM index, list capacity records per atom
@@ -954,12 +957,7 @@ nep_status nep_set_state(nep_handle *h, int64_t n, const double *x, const double
   }
   NEP_CUDA(h, cudaMemsetAsync(h->F, 0, 3 * N * sizeof(long long), h->stream));
   NEP_CUDA(h, cudaMemsetAsync(h->count, 0, (size_t)h->ncell * sizeof(int), h->stream));
-  NEP_CUDA(h, cudaMemsetAsync(h->sums, 0, 32 * sizeof(double), h->stream));
-  NEP_CUDA(h, cudaMemsetAsync(h->counters, 0, 16 * sizeof(long long), h->stream));
-  Control c0{};
-  c0.rebuild_every = h->rebuild_every;
-  c0.far_dmax2 = far_dmax2(h->skin);
-  NEP_CUDA(h, cudaMemcpyAsync(h->ctrl, &c0, sizeof(Control), cudaMemcpyHostToDevice, h->stream));
+  NEP_CUDA(h, reset_report(h));
   return upload_state(h, x, v);
 }
 
@@ -992,8 +990,8 @@ nep_status nep_compute(nep_handle *h, double *E, double *F, double *virial) {
   }
   s = check_device_status(h);
   if (s != NEP_OK) return s;
-  if (E) *E = h->h_sums[0];
-  if (virial) for (int k = 0; k < 9; ++k) virial[k] = h->h_sums[1 + k];
+  if (E) *E = h->h_rep->sums[0];
+  if (virial) for (int k = 0; k < 9; ++k) virial[k] = h->h_rep->sums[1 + k];
   return NEP_OK;
 }
 
@@ -1007,23 +1005,44 @@ nep_status md_verlet_step(nep_handle *h, double dt_fs, int n_steps) {
     if (s == NEP_OK && !h->timing) s = check_device_status(h);   // the host copy of the rebuild count
     if (s != NEP_OK) return s;
   }
-  if (h->timing) {
-    for (int k = 0; k < n_steps; ++k) NEP_CUDA(h, enqueue_step(h, dt_fs));
-    NEP_CUDA(h, enqueue_step_end(h, dt_fs));
-  } else {
-    if (!h->graph || h->graph_dt != dt_fs) {
-      nep_status s = build_graph(h, dt_fs);
+  const long long rebuilds_before = h->h_rep->ctrl.rebuilds;
+  int left = n_steps;
+  if (!h->timing) {
+    // A graph of several steps (as many as the first such call has, at most GRAPH_STEPS) saves the 5 us between
+    // replays and, for small systems, the 2 us between launches: ten steps of 256 atoms take 254 us, against 347
+    // launch by launch and 361 from a one-step graph with a conditional node (8 us per step).  Larger systems'
+    // graphs hold a conditional chain per step, whose capture costs a call of 10 steps 80 us; they are built when
+    // a second call comes (56,000 student atoms: 1,043 -> 998 us per call).
+    const bool conditional = !cell_sort_decides(h->n, h->ncell);
+    if (left >= 4 && (!h->graphk.exec || h->graphk.dt != dt_fs) &&
+        (!conditional || (h->graph1.exec && h->graph1.dt == dt_fs))) {
+      nep_status s = build_graph(h, h->graphk, dt_fs, std::min(left, GRAPH_STEPS));
       if (s != NEP_OK) return s;
     }
-    const long long rebuilds_before = h->h_ctrl->rebuilds;
-    for (int k = 0; k < n_steps; ++k) NEP_CUDA(h, cudaGraphLaunch(h->graph, h->stream));
-    NEP_CUDA(h, enqueue_step_end(h, dt_fs));
-    nep_status s = check_device_status(h);
-    // the rebuild chain's kernels ran on the rebuild steps only
-    h->launch_total += h->graph_launches * n_steps + h->graph_rebuild_launches * (h->h_ctrl->rebuilds - rebuilds_before);
-    return s;
+    const bool several = h->graphk.exec && h->graphk.dt == dt_fs;
+    for (; several && left >= h->graphk.steps; left -= h->graphk.steps) {
+      NEP_CUDA(h, cudaGraphLaunch(h->graphk.exec, h->stream));
+      h->launch_total += h->graphk.launches;
+    }
+    // the remaining steps: small systems launch by launch, larger ones from a graph with the conditional chain
+    if (left > 0 && conditional) {
+      if (!h->graph1.exec || h->graph1.dt != dt_fs) {
+        nep_status s = build_graph(h, h->graph1, dt_fs, 1);
+        if (s != NEP_OK) return s;
+      }
+      for (; left > 0; --left) {
+        NEP_CUDA(h, cudaGraphLaunch(h->graph1.exec, h->stream));
+        h->launch_total += h->graph1.launches;
+      }
+    }
   }
-  return check_device_status(h);
+  for (; left > 0; --left) NEP_CUDA(h, enqueue_step(h, dt_fs));
+  NEP_CUDA(h, enqueue_step_end(h, dt_fs));
+  nep_status s = check_device_status(h);
+  // a conditional rebuild chain's kernels ran on the rebuild steps only
+  if (!h->timing && !cell_sort_decides(h->n, h->ncell))
+    h->launch_total += h->graph_rebuild_launches * (h->h_rep->ctrl.rebuilds - rebuilds_before);
+  return s;
 }
 
 nep_status nep_get_state(nep_handle *h, double *x, double *v) {
@@ -1074,15 +1093,15 @@ nep_status nep_get_thermo(nep_handle *h, double out[8]) {
   if (!h->have_state) return fail(h, NEP_ERR_STATE, "nep_set_state has not been called");
   nep_status s = check_device_status(h);
   if (s != NEP_OK) return s;
-  const double pe = h->h_sums[0], ke = h->h_sums[10];
+  const double pe = h->h_rep->sums[0], ke = h->h_rep->sums[10];
   const double V = h->L[0] * h->L[1] * h->L[2];
-  const double trW = h->h_sums[1] + h->h_sums[5] + h->h_sums[9];
+  const double trW = h->h_rep->sums[1] + h->h_rep->sums[5] + h->h_rep->sums[9];
   out[0] = pe;
   out[1] = ke;
   out[2] = h->n > 1 ? 2.0 * ke / ((3.0 * h->n - 3.0) * KB_EV) : 0.0;
   out[3] = (2.0 * ke + trW) / (3.0 * V);
-  out[4] = h->h_sums[1]; out[5] = h->h_sums[5]; out[6] = h->h_sums[9];
-  out[7] = (double)h->h_ctrl->rebuilds;
+  out[4] = h->h_rep->sums[1]; out[5] = h->h_rep->sums[5]; out[6] = h->h_rep->sums[9];
+  out[7] = (double)h->h_rep->ctrl.rebuilds;
   return NEP_OK;
 }
 
@@ -1167,12 +1186,12 @@ nep_status nep_get_counters(nep_handle *h, int64_t out[13]) {
   if (!h || !out) return NEP_ERR_ARG;
   nep_status s = check_device_status(h);
   if (s != NEP_OK && s != NEP_ERR_NEIGH_OVERFLOW && s != NEP_ERR_NAN) return s;
-  const long long *c = h->h_counters;
+  const long long *c = h->h_rep->counters;
   out[0] = c[0];                // descriptor: radial pairs
   out[1] = c[1];                // descriptor: angular pairs
   out[2] = c[8];                // force evaluations
-  out[3] = h->h_ctrl->rebuilds;
-  out[4] = h->h_ctrl->steps;
+  out[3] = h->h_rep->ctrl.rebuilds;
+  out[4] = h->h_rep->ctrl.steps;
   out[5] = h->launch_total;
   out[6] = c[2];                // descriptor: list entries
   out[7] = c[3];                // descriptor: active pairs
@@ -1189,7 +1208,8 @@ nep_status nep_set_fallback(nep_handle *h, const nep_params *teacher, const floa
   if (!h) return NEP_ERR_ARG;
   if (teacher == nullptr) {
     h->fb_on = false;
-    if (h->graph) { cudaGraphExecDestroy(h->graph); h->graph = nullptr; }
+    h->graph1.destroy();
+    h->graphk.destroy();
     return NEP_OK;
   }
   if (h->shape != 1) return fail(h, NEP_ERR_UNSUPPORTED, "the fallback is for a student-shaped model");
@@ -1211,7 +1231,8 @@ nep_status nep_set_fallback(nep_handle *h, const nep_params *teacher, const floa
   }
   h->fb_frac = max_fraction > 0.0 ? max_fraction : 1.0 / 16.0;
   h->fb_on = true;
-  if (h->graph) { cudaGraphExecDestroy(h->graph); h->graph = nullptr; }
+  h->graph1.destroy();
+  h->graphk.destroy();
   h->have_forces = false;
   if (h->have_state) {
     cudaError_t e = alloc_fallback(h);
@@ -1271,24 +1292,24 @@ nep_status nep_run_variant(nep_handle *h, int variant, double *ms, double *F) {
       if (!h->abl_f) e = dalloc(h->abl_f, 3 * N);
       if (e == cudaSuccess)
         e = launch_descriptor<CuShape>(h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->usite, nullptr, h->F,
-                                       h->part_d, &h->ctrl->status, Fallback{}, h->stream);
+                                       EvalSums{}, &h->ctrl->status, Fallback{}, h->stream);
       if (e == cudaSuccess) e = cudaMemsetAsync(h->abl_f, 0, 3 * N * sizeof(float), h->stream);
       if (e == cudaSuccess) e = cudaEventRecord(a, h->stream);
       if (e == cudaSuccess)
         e = launch_force_float_scatter<CuShape>(h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->abl_f,
-                                                h->part_f, &h->ctrl->status, h->stream);
+                                                EvalSums{}, &h->ctrl->status, h->stream);
       if (e == cudaSuccess) e = cudaEventRecord(b, h->stream);
       if (e == cudaSuccess) e = launch_store_float3(h->n, h->id, h->abl_f, h->io, h->stream);
     } else if (variant == NEP_VARIANT_HALF_LIST || variant == NEP_VARIANT_SEPARATE_FORCE) {
       e = launch_descriptor<CuShape>(h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->usite, nullptr, h->F,
-                                     h->part_d, &h->ctrl->status, Fallback{}, h->stream);
+                                     EvalSums{}, &h->ctrl->status, Fallback{}, h->stream);
       if (e == cudaSuccess) e = cudaEventRecord(a, h->stream);
       if (e == cudaSuccess && variant == NEP_VARIANT_HALF_LIST)
         e = launch_force_half_list<CuShape>(h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->F,
-                                            h->part_f, &h->ctrl->status, h->stream);
+                                            EvalSums{}, &h->ctrl->status, h->stream);
       if (e == cudaSuccess && variant == NEP_VARIANT_SEPARATE_FORCE)
         e = launch_force<CuShape, float>(h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->F,
-                                         h->part_f, &h->ctrl->status, h->stream);
+                                         EvalSums{}, &h->ctrl->status, h->stream);
       if (e == cudaSuccess) e = cudaEventRecord(b, h->stream);
       if (e == cudaSuccess) e = launch_store_force(h->n, h->id, h->F, h->io, h->stream);
     } else if (variant >= NEP_VARIANT_CPB1 && variant <= NEP_VARIANT_CPB_AUTO) {
@@ -1302,10 +1323,10 @@ nep_status nep_run_variant(nep_handle *h, int variant, double *ms, double *F) {
         }
       }
       e = launch_descriptor<CuShape>(h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->usite, nullptr, h->F,
-                                     h->part_d, &h->ctrl->status, Fallback{}, h->stream);
+                                     EvalSums{}, &h->ctrl->status, Fallback{}, h->stream);
       if (e == cudaSuccess) e = cudaEventRecord(a, h->stream);
       if (e == cudaSuccess)
-        e = launch_force_cpb<CuShape>(cpb, h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->F, h->part_f,
+        e = launch_force_cpb<CuShape>(cpb, h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->F, EvalSums{},
                                       &h->ctrl->status, h->stream);
       if (e == cudaSuccess) e = cudaEventRecord(b, h->stream);
       if (e == cudaSuccess) e = launch_store_force(h->n, h->id, h->F, h->io, h->stream);
@@ -1313,11 +1334,11 @@ nep_status nep_run_variant(nep_handle *h, int variant, double *ms, double *F) {
       e = cudaEventRecord(a, h->stream);
       if (e == cudaSuccess)
         e = launch_descriptor<CuShape>(h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->usite, nullptr, h->F,
-                                       h->part_d, &h->ctrl->status, Fallback{}, h->stream);
+                                       EvalSums{}, &h->ctrl->status, Fallback{}, h->stream);
       if (e == cudaSuccess) e = cudaEventRecord(b, h->stream);
       if (e == cudaSuccess)
         e = launch_force<CuShape, float>(h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->F,
-                                         h->part_f, &h->ctrl->status, h->stream);
+                                         EvalSums{}, &h->ctrl->status, h->stream);
       if (e == cudaSuccess) e = launch_store_force(h->n, h->id, h->F, h->io, h->stream);
     } else {
       if (!h->abl_s) e = dalloc(h->abl_s, (size_t)CuShape::NA * CuShape::NLM * N);
@@ -1325,14 +1346,14 @@ nep_status nep_run_variant(nep_handle *h, int variant, double *ms, double *F) {
       if (e == cudaSuccess) {
         if (variant == NEP_VARIANT_TILE1)
           e = launch_descriptor_tiled<CuShape, 1>(h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->usite, h->F,
-                                                  h->part_d, &h->ctrl->status, h->abl_s, h->stream);
+                                                  EvalSums{}, &h->ctrl->status, h->abl_s, h->stream);
         else
           e = launch_descriptor_tiled<CuShape, 3>(h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->usite, h->F,
-                                                  h->part_d, &h->ctrl->status, h->abl_s, h->stream);
+                                                  EvalSums{}, &h->ctrl->status, h->abl_s, h->stream);
       }
       if (e == cudaSuccess) e = cudaEventRecord(b, h->stream);
       if (e == cudaSuccess)
-        e = launch_force<CuShape, float>(h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->F, h->part_f,
+        e = launch_force<CuShape, float>(h->model_t, g, h->n, h->pos, h->nbr, rows_of(h), G, h->F, EvalSums{},
                                          &h->ctrl->status, h->stream);
       if (e == cudaSuccess) e = launch_store_force(h->n, h->id, h->F, h->io, h->stream);
     }

@@ -199,9 +199,6 @@ __device__ __forceinline__ int acquire_record_slot(const PairCache &pc) {
   return slot;
 }
 
-// Rows of per-block partial sums that a wide kernel (nep_wide.cu) writes at most.
-constexpr int WIDE_MAX_BLOCKS = 152 * 8;
-
 // Cell geometry of the current neighbour list.
 struct Geom {
   float lx, ly, lz;      // cell edge lengths (float)
@@ -792,40 +789,52 @@ __device__ __forceinline__ void to_fix32x3(float x, float y, float z, long long 
   }
 }
 
-// Block-wide sum of NV int64 values into out[blockIdx.x * NV + v].  Integer addition is associative,
-// so the result does not depend on the reduction order.  NW bounds the warps per block (the size of
-// the shared scratch).
-template <int NV, int NW = 32>
-__device__ __forceinline__ void block_sum_store(long long (&v)[NV], long long *out) {
-  static_assert(NW >= 1 && NW <= 32, "1..32 warps");
-  __shared__ long long red[NW][NV];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) red[warp][k] = v[k];
-  }
-  __syncthreads();
-  if (warp == 0) {
-    const int nw = blockDim.x >> 5;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      long long t = lane < nw && lane < NW ? red[lane][k] : 0ll;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-      if (lane == 0) out[(size_t)blockIdx.x * NV + k] = t;
-    }
-  }
+// 64-bit integer add to global memory whose result nobody reads (the fixed-point force scatter, the running
+// sums): a reduction, which returns nothing, so no register waits for the memory system (atomicAdd on a
+// generic pointer becomes a value-returning atomic).  Integer addition is associative, so the sums do
+// not depend on the order in which the additions arrive.
+__device__ __forceinline__ void red_add(unsigned long long *p, long long v) {
+  asm volatile("red.global.add.u64 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "l"(v));
 }
 
-// block_sum_store in two halves, so that no block barrier is needed where the values become known:
-// warp_sum_stage adds the warp's NV int64 values (lane 0 writes them to dst[0..NV-1]); after a later
-// block barrier, block_store_staged adds the staged sums of the block's warps into
-// out[blockIdx.x * NV + v].  Integer sums: the result does not depend on the order.
+// Energy, virial and counters of an evaluation.  Every block adds its integer (fixed-point) sums to the running
+// totals acc, and the last block of the evaluation's last kernel turns them into sums and counters and clears
+// acc: no array of per-block rows and no reduction kernel (which took 2.4 us per step up to 16,384 atoms, 6.4 at
+// 1,048,576 and 36 at 8,388,608; 18 reductions per block disappear beside the block's own work).  Integer sums:
+// the result does not depend on the order of the blocks.
+// Index v: 0 E, 1..9 W, 10 kinetic energy, 11..14 {radial pairs, angular pairs, list entries, active pairs} of the
+// descriptor walk, 15..18 {list entries, active, radial, angular pairs} of the force pass.
+// counters[v - 11] += total for v >= 11, counters[8] += 1 per evaluation.
+constexpr int N_SUMS = 19;
+struct EvalSums {
+  long long *acc;        // [N_SUMS] running totals (zero between evaluations); nullptr: nothing is summed
+  unsigned *done;        // blocks of the publishing kernel that have added theirs (zero between kernels)
+  double *sums;
+  long long *counters;
+  int publish;           // this kernel is the evaluation's last
+};
+// The totals of index v, published by one thread.
+__device__ __forceinline__ void publish_sum(const EvalSums &E, int v) {
+  const long long tot = (long long)atomicExch(reinterpret_cast<unsigned long long *>(E.acc + v), 0ull);
+  E.sums[v] = v <= 10 ? (double)tot * FIX_INV : (double)tot;       // energies/virial are fixed point
+  if (v >= 11) E.counters[v - 11] += tot;
+  if (v == 0) E.counters[8] += 1;
+}
+// Whether the calling warp's block is the last of the grid to get here (after its additions); resets the count.
+__device__ __forceinline__ bool last_block(unsigned *done) {
+  __threadfence();
+  __syncwarp();
+  unsigned k = 0;
+  if ((threadIdx.x & 31) == 0) k = atomicAdd(done, 1u);
+  const bool last = __shfl_sync(0xffffffffu, k, 0) == gridDim.x - 1;
+  if (last) {
+    __threadfence();
+    if ((threadIdx.x & 31) == 0) *done = 0u;
+  }
+  return last;
+}
+
+// The warp's sums of NV int64 values, written by lane 0 to dst[0..NV-1].
 template <int NV>
 __device__ __forceinline__ void warp_sum_stage(long long (&v)[NV], long long *dst) {
 #pragma unroll
@@ -838,16 +847,43 @@ __device__ __forceinline__ void warp_sum_stage(long long (&v)[NV], long long *ds
     for (int k = 0; k < NV; ++k) dst[k] = v[k];
   }
 }
-template <int NV, int NW>
-__device__ __forceinline__ void block_store_staged(const long long (*src)[NV], long long *out) {
-  if (threadIdx.x < NV) {
-    long long t = 0;
-    const int nw = min(NW, (int)(blockDim.x >> 5));
-    for (int w = 0; w < nw; ++w) t += src[w][threadIdx.x];
-    out[(size_t)blockIdx.x * NV + threadIdx.x] = t;
+// After a block barrier that follows warp_sum_stage: the block's staged sums of NW warps, d = {E, radial pairs,
+// angular pairs, list entries, active pairs} and f = {W[9], list entries, active, radial, angular pairs} (either may
+// be nullptr), added to the running totals.
+template <int NW>
+__device__ __forceinline__ void eval_add(const EvalSums &E, const long long (*d)[5], const long long (*f)[13]) {
+  const int t = threadIdx.x;
+  if (t >= 32 || E.acc == nullptr) return;
+  long long v = 0;
+  int idx = 0;
+  if (t < 5) {
+    idx = t == 0 ? 0 : 10 + t;
+    if (d != nullptr)
+      for (int w = 0; w < NW; ++w) v += d[w][t];
+  } else if (t < 18) {
+    const int k = t - 5;
+    idx = k < 9 ? 1 + k : 6 + k;
+    if (f != nullptr)
+      for (int w = 0; w < NW; ++w) v += f[w][k];
   }
+  if (v != 0) red_add(reinterpret_cast<unsigned long long *>(E.acc + idx), v);
+  if (E.publish && last_block(E.done) && t < 18) publish_sum(E, idx);
 }
-
+// Stages and adds one of the two groups at the end of a kernel (block barrier inside).
+template <int NW>
+__device__ __forceinline__ void eval_add_d(const EvalSums &E, long long (&v)[5]) {
+  __shared__ long long w[NW][5];
+  warp_sum_stage<5>(v, w[threadIdx.x >> 5]);
+  __syncthreads();
+  eval_add<NW>(E, w, nullptr);
+}
+template <int NW>
+__device__ __forceinline__ void eval_add_f(const EvalSums &E, long long (&v)[13]) {
+  __shared__ long long w[NW][13];
+  warp_sum_stage<13>(v, w[threadIdx.x >> 5]);
+  __syncthreads();
+  eval_add<NW>(E, nullptr, w);
+}
 
 // ---------------------------------------------------------------------------------------------------
 // Asynchronous per-thread neighbour pipeline (cp.async into shared memory).  The walk over an atom's
@@ -953,14 +989,6 @@ struct NbrPipe {
 
   __device__ __forceinline__ void finish() { cp_async_wait<0>(); }
 };
-
-// 64-bit integer add to global memory whose result nobody reads (the fixed-point force scatter): a
-// reduction, which returns nothing, so no register waits for the memory system (atomicAdd on a
-// generic pointer becomes a value-returning atomic).  Integer addition is associative, so the sums do
-// not depend on the order in which the additions arrive.
-__device__ __forceinline__ void red_add(unsigned long long *p, long long v) {
-  asm volatile("red.global.add.u64 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "l"(v));
-}
 
 // cp.async ring of pair records (16 bytes each, L2 only): record k of this thread is src[k * stride];
 // DQ records in flight, as NbrPipe's positions.

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(DESC_BLOCK, NEP_DESC_MINB)
 k_descriptor(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
              const int32_t *__restrict__ nbr, const RowExt X, float *__restrict__ G,
              float *__restrict__ usite, float *__restrict__ qout, long long *__restrict__ Ffix,
-             long long *__restrict__ part, int *__restrict__ status, const __grid_constant__ Fallback fb) {
+             const EvalSums sums, int *__restrict__ status, const __grid_constant__ Fallback fb) {
   __shared__ float4 shift[27];
   __shared__ uint32_t ring_e[PIPE_DE * DESC_BLOCK];
   __shared__ float4 ring_p[PIPE_DP * DESC_BLOCK];
@@ -116,7 +116,7 @@ k_descriptor(const __grid_constant__ Model<S> P, const Geom geom, const int n, c
     acc[3] = A.cnt;
     acc[4] = A.nact;
   }
-  block_sum_store<5, DESC_BLOCK / 32>(acc, part);
+  eval_add_d<DESC_BLOCK / 32>(sums, acc);
 }
 
 // Teacher-shape descriptor kernel with the 120 angular sums s_nlm accumulated in tensor memory (TMEM)
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(DESC_BLOCK, NEP_DESC_MINB_TM)
 k_descriptor_tm(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
                 const int32_t *__restrict__ nbr, const RowExt X, float *__restrict__ G,
                 float *__restrict__ usite, float *__restrict__ qout, long long *__restrict__ Ffix,
-                long long *__restrict__ part, int *__restrict__ status, const __grid_constant__ Fallback fb) {
+                const EvalSums sums, int *__restrict__ status, const __grid_constant__ Fallback fb) {
   static_assert(S::NA == 5 && S::NLM == 24 && S::FOURBODY && DESC_BLOCK == 128, "teacher shape, 4 warps");
   constexpr int W = TMEM_W;
   constexpr uint32_t TCOLS = 128;
@@ -206,7 +206,7 @@ k_descriptor_tm(const __grid_constant__ Model<S> P, const Geom geom, const int n
     tc_fence_after();
     tmem_dealloc(tmem_base, TCOLS);
   }
-  block_sum_store<5, DESC_BLOCK / 32>(acc, part);
+  eval_add_d<DESC_BLOCK / 32>(sums, acc);
 }
 
 // Adjoint row G_i of the force kernel: in registers for small shapes; for the teacher shape (120
@@ -562,7 +562,7 @@ template <class S, class GT, bool FS = false, bool FULL = false>
 __global__ void __launch_bounds__(FORCE_BLOCK, FULL && ForceCfg<S>::TM ? NEP_FORCE_MINB_FULL : ForceCfg<S>::MINB)
 k_force(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
         const int32_t *__restrict__ nbr, const RowExt X, const GT *__restrict__ G,
-        unsigned long long *__restrict__ Ffix, long long *__restrict__ part,
+        unsigned long long *__restrict__ Ffix, const EvalSums sums,
         int *__restrict__ status, float *__restrict__ Ff = nullptr) {
   constexpr bool TM = ForceCfg<S>::TM;
   constexpr int W = GTraits<GT>::W;
@@ -639,7 +639,7 @@ k_force(const __grid_constant__ Model<S> P, const Geom geom, const int n, const 
       tmem_dealloc(tmem_base, ForceCfg<S>::TCOLS);
     }
   }
-  block_sum_store<13, FORCE_BLOCK / 32>(acc, part);
+  eval_add_f<FORCE_BLOCK / 32>(sums, acc);
 }
 
 // Descriptors, network and forces of the float32 teacher in one kernel.  The full-row force form reads
@@ -657,8 +657,8 @@ template <class S>
 __global__ void __launch_bounds__(DESC_BLOCK, NEP_FUSED_MINB)
 k_nep_fused(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
             const int32_t *__restrict__ nbr, const RowExt X, float *__restrict__ usite,
-            float *__restrict__ qout, unsigned long long *__restrict__ Ffix, long long *__restrict__ part_d,
-            long long *__restrict__ part_f, int *__restrict__ status, const PairCache pc) {
+            float *__restrict__ qout, unsigned long long *__restrict__ Ffix, const EvalSums sums,
+            int *__restrict__ status, const PairCache pc) {
   static_assert(ForceCfg<S>::TM && DESC_BLOCK == 128 && FORCE_BLOCK == 128, "teacher shape, 4 warps");
   constexpr int W = TMEM_W;
   constexpr uint32_t TCOLS = 128;
@@ -744,12 +744,13 @@ k_nep_fused(const __grid_constant__ Model<S> P, const Geom geom, const int n, co
   }
   // the energy and counters: summed over the warp now (fewer live registers in the force pass), over
   // the block after the closing barrier
-  __shared__ long long wsum_d[DESC_BLOCK / 32][5];
+  __shared__ long long wsum_d[DESC_BLOCK / 32][5], wsum_f[DESC_BLOCK / 32][13];
   warp_sum_stage<5>(acc_d, wsum_d[threadIdx.x >> 5]);
 
   // forces: every active pair of the row with the own adjoint row, from the pair records
   force_pairs_rec<S, PIPE_DP>(P, RowTmem<S>{trow}, fp_s + threadIdx.x, i, live, n, pc.rec, rec_off, pc.pmax, nang,
                                     nact - nang, ring_p, Ffix, status, acc_f);
+  warp_sum_stage<13>(acc_f, wsum_f[threadIdx.x >> 5]);
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x < 32) {
@@ -760,8 +761,7 @@ k_nep_fused(const __grid_constant__ Model<S> P, const Geom geom, const int n, co
     __threadfence();          // this block's record reads are complete (cp.async waited, barrier above)
     atomicAnd(pc.slot_mask + slot / pc.slots, ~(1u << (slot % pc.slots)));
   }
-  block_store_staged<5, DESC_BLOCK / 32>(wsum_d, part_d);
-  block_sum_store<13, DESC_BLOCK / 32>(acc_f, part_f);
+  eval_add<DESC_BLOCK / 32>(sums, wsum_d, wsum_f);
 }
 
 // The fused kernel for shapes whose per-atom row fits in registers (the distilled student: 4 x 8
@@ -780,8 +780,8 @@ template <class S>
 __global__ void __launch_bounds__(DESC_BLOCK, NEP_FUSED_REG_MINB)
 k_nep_fused_reg(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
                 const int32_t *__restrict__ nbr, const RowExt X, float *__restrict__ usite,
-                float *__restrict__ qout, unsigned long long *__restrict__ Ffix, long long *__restrict__ part_d,
-                long long *__restrict__ part_f, int *__restrict__ status, const __grid_constant__ Fallback fb,
+                float *__restrict__ qout, unsigned long long *__restrict__ Ffix, const EvalSums sums,
+            int *__restrict__ status, const __grid_constant__ Fallback fb,
                 const PairCache pc) {
   static_assert(!ForceCfg<S>::TM && DESC_BLOCK == FORCE_BLOCK, "register-resident rows");
   __shared__ float4 shift[27];
@@ -837,13 +837,15 @@ k_nep_fused_reg(const __grid_constant__ Model<S> P, const Geom geom, const int n
     force_pairs_rec<S, PIPE_DP>(P, RowReg<S>{gi}, fp_s + threadIdx.x, i, true, n, pc.rec, rec_off, pc.pmax, A.nang,
                                 A.nact - A.nang, ring_p, Ffix, status, acc_f);
   }
+  __shared__ long long wsum_d[DESC_BLOCK / 32][5], wsum_f[DESC_BLOCK / 32][13];
+  warp_sum_stage<5>(acc_d, wsum_d[threadIdx.x >> 5]);
+  warp_sum_stage<13>(acc_f, wsum_f[threadIdx.x >> 5]);
   __syncthreads();
   if (threadIdx.x == 0 && slot >= 0) {
     __threadfence();          // this block's record reads are complete (cp.async waited, barrier above)
     atomicAnd(pc.slot_mask + slot / pc.slots, ~(1u << (slot % pc.slots)));
   }
-  block_sum_store<5, DESC_BLOCK / 32>(acc_d, part_d);
-  block_sum_store<13, DESC_BLOCK / 32>(acc_f, part_f);
+  eval_add<DESC_BLOCK / 32>(sums, wsum_d, wsum_f);
 }
 
 // Mixed-precision form of the fused kernel: the same descriptor walk (pair records), float32 adjoint
@@ -867,8 +869,8 @@ template <class S, class MT>
 __global__ void __launch_bounds__(DESC_BLOCK, NEP_FUSED_MINB)
 k_nep_fused_mixed(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
                   const int32_t *__restrict__ nbr, const RowExt X, float *__restrict__ usite,
-                  float *__restrict__ qout, unsigned long long *__restrict__ Ffix, long long *__restrict__ part_d,
-                  long long *__restrict__ part_f, int *__restrict__ status, const PairCache pc) {
+                  float *__restrict__ qout, unsigned long long *__restrict__ Ffix, const EvalSums sums,
+            int *__restrict__ status, const PairCache pc) {
   static_assert(ForceCfg<S>::TM && DESC_BLOCK == 128 && S::NDES <= FM_K && S::NNEU <= FM_N, "teacher shape");
   constexpr int NT = 4;
   constexpr int W = TMEM_W;
@@ -1034,10 +1036,11 @@ k_nep_fused_mixed(const __grid_constant__ Model<S> P, const Geom geom, const int
     acc_d[4] = nact;
     acc_f[9] = cnt; acc_f[10] = nact; acc_f[11] = nrad; acc_f[12] = nang;
   }
-  __shared__ long long wsum_d[DESC_BLOCK / 32][5];
+  __shared__ long long wsum_d[DESC_BLOCK / 32][5], wsum_f[DESC_BLOCK / 32][13];
   warp_sum_stage<5>(acc_d, wsum_d[t >> 5]);
   force_pairs_rec<S, PIPE_DP>(P, RowTmem<S>{trow}, fp_s + t, i, live, n, pc.rec, rec_off, pc.pmax, nang, nact - nang, ring_p,
                               Ffix, status, acc_f);
+  warp_sum_stage<13>(acc_f, wsum_f[threadIdx.x >> 5]);
   tc_fence_before();
   __syncthreads();
   if (t < 32) {
@@ -1048,8 +1051,7 @@ k_nep_fused_mixed(const __grid_constant__ Model<S> P, const Geom geom, const int
     __threadfence();
     atomicAnd(pc.slot_mask + slot / pc.slots, ~(1u << (slot % pc.slots)));
   }
-  block_store_staged<5, DESC_BLOCK / 32>(wsum_d, part_d);
-  block_sum_store<13, DESC_BLOCK / 32>(acc_f, part_f);
+  eval_add<DESC_BLOCK / 32>(sums, wsum_d, wsum_f);
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -1060,14 +1062,14 @@ k_nep_fused_mixed(const __grid_constant__ Model<S> P, const Geom geom, const int
 #endif
 template <class S>
 cudaError_t launch_descriptor(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
-                              const RowExt &X, float *G, float *usite, float *qout, long long *Ffix,
-                              long long *part, int *status, const Fallback &fb, cudaStream_t st) {
+                              const RowExt &X, float *G, float *usite, float *qout, long long *Ffix, const EvalSums &sums,
+                         int *status, const Fallback &fb, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int grid = (n + DESC_BLOCK - 1) / DESC_BLOCK;
   if constexpr (ForceCfg<S>::TM && NEP_DESC_TM)
-    k_descriptor_tm<S><<<grid, DESC_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, G, usite, qout, Ffix, part, status, fb);
+    k_descriptor_tm<S><<<grid, DESC_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, G, usite, qout, Ffix, sums, status, fb);
   else
-    k_descriptor<S><<<grid, DESC_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, G, usite, qout, Ffix, part, status, fb);
+    k_descriptor<S><<<grid, DESC_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, G, usite, qout, Ffix, sums, status, fb);
   return cudaGetLastError();
 }
 
@@ -1083,12 +1085,13 @@ constexpr bool force_full_row() {
 template <class S, class GT>
 cudaError_t launch_force(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
                          const RowExt &X, const GT *G,
-                         long long *Ffix, long long *part, int *status, cudaStream_t st) {
+                         long long *Ffix, const EvalSums &sums,
+                         int *status, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int grid = (n + FORCE_BLOCK - 1) / FORCE_BLOCK;
   constexpr bool full = force_full_row<S, GT>();
   k_force<S, GT, false, full><<<grid, FORCE_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, G,
-                                                           reinterpret_cast<unsigned long long *>(Ffix), part, status);
+                                                           reinterpret_cast<unsigned long long *>(Ffix), sums, status);
   return cudaGetLastError();
 }
 
@@ -1096,56 +1099,56 @@ cudaError_t launch_force(const Model<S> &P, const Geom &g, int n, const float4 *
 // owner, gathering the neighbour's adjoint row), instead of the full-row form.
 template <class S>
 cudaError_t launch_force_half_list(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
-                                   const RowExt &X, const float *G, long long *Ffix,
-                                   long long *part, int *status, cudaStream_t st) {
+                                   const RowExt &X, const float *G, long long *Ffix, const EvalSums &sums,
+                         int *status, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int grid = (n + FORCE_BLOCK - 1) / FORCE_BLOCK;
   k_force<S, float, false, false><<<grid, FORCE_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, G,
-                                                               reinterpret_cast<unsigned long long *>(Ffix), part,
+                                                               reinterpret_cast<unsigned long long *>(Ffix), sums,
                                                                status);
   return cudaGetLastError();
 }
 template cudaError_t launch_force_half_list<CuShape>(const Model<CuShape> &, const Geom &, int, const float4 *,
                                                      const int32_t *, const RowExt &, const float *, long long *,
-                                                     long long *, int *, cudaStream_t);
+                                                     const EvalSums &, int *, cudaStream_t);
 
 // Ablation: the production (full-row) force kernel with float atomicAdd scatter into Ff [3][n] (zeroed
 // by the caller) instead of fixed-point integer atomics.
 template <class S>
 cudaError_t launch_force_float_scatter(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
                                        const RowExt &X, const float *G, float *Ff,
-                                       long long *part, int *status, cudaStream_t st) {
+                                       const EvalSums &sums, int *status, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int grid = (n + FORCE_BLOCK - 1) / FORCE_BLOCK;
-  k_force<S, float, true, true><<<grid, FORCE_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, G, nullptr, part,
+  k_force<S, float, true, true><<<grid, FORCE_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, G, nullptr, sums,
                                                              status, Ff);
   return cudaGetLastError();
 }
 template cudaError_t launch_force_float_scatter<CuShape>(const Model<CuShape> &, const Geom &, int, const float4 *,
                                                          const int32_t *, const RowExt &, const float *, float *,
-                                                         long long *, int *, cudaStream_t);
+                                                         const EvalSums &, int *, cudaStream_t);
 
 // Fused descriptor + force evaluation of the float32 teacher (k_nep_fused); Ffix must be zero.
 template <class S>
 cudaError_t launch_fused(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
-                         const RowExt &X, float *usite, float *qout, long long *Ffix, long long *part_d,
-                         long long *part_f, int *status, const PairCache &pc, cudaStream_t st) {
+                         const RowExt &X, float *usite, float *qout, long long *Ffix, const EvalSums &sums,
+                         int *status, const PairCache &pc, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int grid = (n + DESC_BLOCK - 1) / DESC_BLOCK;
   k_nep_fused<S><<<grid, DESC_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, usite, qout,
-                                              reinterpret_cast<unsigned long long *>(Ffix), part_d, part_f, status, pc);
+                                              reinterpret_cast<unsigned long long *>(Ffix), sums, status, pc);
   return cudaGetLastError();
 }
 template cudaError_t launch_fused<CuShape>(const Model<CuShape> &, const Geom &, int, const float4 *, const int32_t *,
-                                           const RowExt &, float *, float *, long long *, long long *, long long *,
+                                           const RowExt &, float *, float *, long long *, const EvalSums &,
                                            int *, const PairCache &, cudaStream_t);
 
 // Fused evaluation of a register-resident shape (k_nep_fused_reg); Ffix must be zero.  Fails with
 // cudaErrorInvalidConfiguration if more blocks than PC_SLOTS_REG could be resident on an SM.
 template <class S>
 cudaError_t launch_fused_reg(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
-                             const RowExt &X, float *usite, float *qout, long long *Ffix, long long *part_d,
-                             long long *part_f, int *status, const Fallback &fb, const PairCache &pc,
+                             const RowExt &X, float *usite, float *qout, long long *Ffix, const EvalSums &sums,
+                         int *status, const Fallback &fb, const PairCache &pc,
                              cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   int per_sm = 0;
@@ -1154,34 +1157,34 @@ cudaError_t launch_fused_reg(const Model<S> &P, const Geom &g, int n, const floa
   if (per_sm > pc.slots) return cudaErrorInvalidConfiguration;
   const int grid = (n + DESC_BLOCK - 1) / DESC_BLOCK;
   k_nep_fused_reg<S><<<grid, DESC_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, usite, qout,
-                                                  reinterpret_cast<unsigned long long *>(Ffix), part_d, part_f,
+                                                  reinterpret_cast<unsigned long long *>(Ffix), sums,
                                                   status, fb, pc);
   return cudaGetLastError();
 }
 template cudaError_t launch_fused_reg<StudentShape>(const Model<StudentShape> &, const Geom &, int, const float4 *,
                                                     const int32_t *, const RowExt &, float *, float *, long long *,
-                                                    long long *, long long *, int *, const Fallback &,
+                                                    const EvalSums &, int *, const Fallback &,
                                                     const PairCache &, cudaStream_t);
 
 // Mixed-precision fused evaluation of the teacher (k_nep_fused_mixed); Ffix must be zero.
 template <class S, class MT>
 cudaError_t launch_fused_mixed(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
-                               const RowExt &X, float *usite, float *qout, long long *Ffix, long long *part_d,
-                               long long *part_f, int *status, const PairCache &pc, cudaStream_t st) {
+                               const RowExt &X, float *usite, float *qout, long long *Ffix, const EvalSums &sums,
+                         int *status, const PairCache &pc, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int grid = (n + DESC_BLOCK - 1) / DESC_BLOCK;
   k_nep_fused_mixed<S, MT><<<grid, DESC_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, usite, qout,
-                                                        reinterpret_cast<unsigned long long *>(Ffix), part_d, part_f,
+                                                        reinterpret_cast<unsigned long long *>(Ffix), sums,
                                                         status, pc);
   return cudaGetLastError();
 }
 template cudaError_t launch_fused_mixed<CuShape, __nv_bfloat16>(const Model<CuShape> &, const Geom &, int,
                                                                 const float4 *, const int32_t *, const RowExt &,
-                                                                float *, float *, long long *, long long *,
-                                                                long long *, int *, const PairCache &, cudaStream_t);
+                                                                float *, float *, long long *, const EvalSums &,
+                                                                int *, const PairCache &, cudaStream_t);
 template cudaError_t launch_fused_mixed<CuShape, __half>(const Model<CuShape> &, const Geom &, int, const float4 *,
                                                          const int32_t *, const RowExt &, float *, float *,
-                                                         long long *, long long *, long long *, int *,
+                                                         long long *, const EvalSums &, int *,
                                                          const PairCache &, cudaStream_t);
 
 // Records per SM bound of the pair cache: %nsmid of the current device (synchronous).
@@ -1199,19 +1202,16 @@ cudaError_t pair_cache_sm_bound(int *nsm) {
 // Pair records per region: one float4 per record, DESC_BLOCK threads.
 size_t pair_cache_region_elems(int pmax) { return (size_t)pmax * DESC_BLOCK; }
 
-int descriptor_blocks(int n) { return (n + DESC_BLOCK - 1) / DESC_BLOCK; }
-int force_blocks(int n) { return (n + FORCE_BLOCK - 1) / FORCE_BLOCK; }
-
 #define NEP_INSTANTIATE(SH)                                                                                    \
   template cudaError_t launch_descriptor<SH>(const Model<SH> &, const Geom &, int, const float4 *, const int32_t *,   \
-                                             const RowExt &, float *, float *, float *, long long *, long long *,    \
+                                             const RowExt &, float *, float *, float *, long long *, const EvalSums &, \
                                              int *, const Fallback &, cudaStream_t);                                  \
   template cudaError_t launch_force<SH, float>(const Model<SH> &, const Geom &, int, const float4 *, const int32_t *, \
-                                               const RowExt &, const float *, long long *, long long *, int *,         \
+                                               const RowExt &, const float *, long long *, const EvalSums &, int *,    \
                                                cudaStream_t);                                                         \
   template cudaError_t launch_force<SH, __half>(const Model<SH> &, const Geom &, int, const float4 *,                 \
                                                 const int32_t *, const RowExt &, const __half *, long long *,         \
-                                                long long *, int *, cudaStream_t);
+                                                const EvalSums &, int *, cudaStream_t);
 NEP_INSTANTIATE(CuShape)
 NEP_INSTANTIATE(StudentShape)
 #undef NEP_INSTANTIATE

@@ -6,6 +6,7 @@
 // atom whose cell-relative coordinate moved more than skin/2 since the last rebuild; the control
 // kernel then asks the next rebuild chain to run.
 #include "nep_common.cuh"
+#include "nep_control.cuh"
 
 #include <cfloat>
 
@@ -26,9 +27,11 @@ __device__ __forceinline__ void note_displacement(bool moved, float dd, Control 
   }
 }
 
+// Opening kick and drift; the forces are read and cleared for the coming evaluation (the memset they would need
+// costs 5 us at 1,048,576 atoms; here the stores hide behind the FP64 arithmetic).
 __global__ void k_kick_drift(int n, double *__restrict__ x, double *__restrict__ y, double *__restrict__ z,
                              double *__restrict__ vx, double *__restrict__ vy, double *__restrict__ vz,
-                             const long long *__restrict__ F, float4 *__restrict__ pos,
+                             long long *__restrict__ F, float4 *__restrict__ pos,
                              const float4 *__restrict__ pos_ref, double kick, double dt, double lx, double ly,
                              double lz, float half_skin2, Control *ctrl) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -63,76 +66,41 @@ __global__ void k_kick_drift(int n, double *__restrict__ x, double *__restrict__
     const float d2 = ddx * ddx + ddy * ddy + ddz * ddz;
     moved = !(d2 <= half_skin2);       // also true for NaN
     dd = d2 <= 1.0e30f ? d2 : 1.0e30f;
+    F[i] = 0; F[(size_t)n + i] = 0; F[2 * (size_t)n + i] = 0;
   }
   note_displacement(moved, dd, ctrl);
 }
 
-// Decide whether this step rebuilds the neighbour list.
-// After the rebuild decision: may the row walks of this evaluation leave the far bands out (no atom
-// moved far enough since the build to bring a far-band pair inside rc_R)?
-__device__ __forceinline__ void decide_far(Control *ctrl) {
-  if (ctrl->do_rebuild) ctrl->dmax2 = 0.f;
-  ctrl->skip_far = ctrl->dmax2 < ctrl->far_dmax2 ? 1 : 0;
-}
-
-__device__ __forceinline__ int step_control(Control *ctrl) {
-  ctrl->steps += 1;
-  ctrl->steps_since += 1;
-  int rb = ctrl->moved | ctrl->force_rebuild;
-  if (ctrl->rebuild_every > 0 && ctrl->steps_since >= ctrl->rebuild_every) rb = 1;
-  ctrl->do_rebuild = rb;
-  if (rb) {
-    ctrl->moved = 0;
-    ctrl->force_rebuild = 0;
-    ctrl->steps_since = 0;
-    ctrl->rebuilds += 1;
-  }
-  decide_far(ctrl);
-  ctrl->pending = 1;    // this step's closing half kick: done by the next step's opening kick or the final one
-  return rb;
-}
-__global__ void k_control(Control *ctrl) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  step_control(ctrl);
-}
-// The same in a captured MD step, where the rebuild chain is the body of a conditional graph node:
-// the decision also sets that node's condition, so that a step without a rebuild launches none of the
+// The step's rebuild decision (step_control) in a kernel of its own: with a condition, in a captured MD step whose
+// rebuild chain is the body of a conditional graph node, so that a step without a rebuild launches none of the
 // chain's kernels.
 __global__ void k_control_cond(Control *ctrl, cudaGraphConditionalHandle cond) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  cudaGraphSetConditional(cond, step_control(ctrl) ? 1u : 0u);
+  cudaGraphSetConditional(cond, decide_rebuild(ctrl, DECIDE_STEP) ? 1u : 0u);
+}
+__global__ void k_control_as(Control *ctrl, int decide) {
+  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  decide_rebuild(ctrl, decide);
 }
 
-// Outside MD steps, after an upload that kept the list: rebuild only if an atom moved more than
-// skin/2 (or a rebuild was requested); the step counters are not touched.
-__global__ void k_control_check(Control *ctrl) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const int rb = ctrl->moved | ctrl->force_rebuild;
-  ctrl->do_rebuild = rb;
-  if (rb) {
-    ctrl->moved = 0;
-    ctrl->force_rebuild = 0;
-    ctrl->steps_since = 0;
-    ctrl->rebuilds += 1;
+// The block's kinetic energy into the running total; the last block publishes it.
+constexpr int MD_BLOCK = 256;
+__device__ __forceinline__ void add_kinetic(const EvalSums &E, long long (&v)[1]) {
+  __shared__ long long w[MD_BLOCK / 32][1];
+  warp_sum_stage<1>(v, w[threadIdx.x >> 5]);
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  if (threadIdx.x == 0) {
+    long long t = 0;
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += w[k][0];
+    if (t != 0) red_add(reinterpret_cast<unsigned long long *>(E.acc + 10), t);
   }
-  decide_far(ctrl);
+  if (last_block(E.done) && threadIdx.x == 0) publish_sum(E, 10);
 }
 
-// Rebuild unconditionally (outside MD steps).
-__global__ void k_control_force(Control *ctrl) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  ctrl->do_rebuild = 1;
-  ctrl->moved = 0;
-  ctrl->force_rebuild = 0;
-  ctrl->steps_since = 0;
-  ctrl->rebuilds += 1;
-  decide_far(ctrl);
-}
-
-// The closing half kick of md_verlet_step's last step, with the kinetic-energy partials.
+// The closing half kick of md_verlet_step's last step, with the kinetic energy.
 __global__ void k_kick(int n, double *__restrict__ vx, double *__restrict__ vy, double *__restrict__ vz,
-                       const long long *__restrict__ F, double kick, double mass, long long *__restrict__ part,
-                       Control *ctrl) {
+                       const long long *__restrict__ F, double kick, double mass, const EvalSums sums, Control *ctrl) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) ctrl->pending = 0;
   long long acc[1] = {0};
@@ -144,60 +112,16 @@ __global__ void k_kick(int n, double *__restrict__ vx, double *__restrict__ vy, 
     vx[i] = ux; vy[i] = uy; vz[i] = uz;
     acc[0] = __double2ll_rn(0.5 * mass * KE_CONV * (ux * ux + uy * uy + uz * uz) * 4294967296.0);
   }
-  block_sum_store<1>(acc, part);
+  add_kinetic(sums, acc);
 }
 
 // Kinetic energy only (no kick): for thermo outside MD steps.
 __global__ void k_kinetic(int n, const double *__restrict__ vx, const double *__restrict__ vy,
-                          const double *__restrict__ vz, double mass, long long *__restrict__ part) {
+                          const double *__restrict__ vz, double mass, const EvalSums sums) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   long long acc[1] = {0};
   if (i < n) acc[0] = __double2ll_rn(0.5 * mass * KE_CONV * (vx[i] * vx[i] + vy[i] * vy[i] + vz[i] * vz[i]) * 4294967296.0);
-  block_sum_store<1>(acc, part);
-}
-
-// Reduction of the per-block int64 partials (fixed point for energies and virial), one block per
-// reduced quantity v:
-//   pd (stride 5):  {site energy, radial pairs, angular pairs, list entries, active pairs} (descriptor)
-//   pf (stride 13): {virial W[9], owned list entries, owned active, owned radial, owned angular} (force)
-//   pk (stride 1):  kinetic energy
-// sums[v]: 0 E, 1..9 W, 10 KE, 11..14 descriptor counts, 15..18 force counts;
-// counters[v - 11] += sums[v] for v >= 11, counters[8] += 1 per evaluation.
-constexpr int N_SUMS = 19;
-
-constexpr int FIN_THREADS = 1024;   // one block per sum; the partials are 8-byte integers, so the
-                                    // order of the additions does not change the result
-__global__ void __launch_bounds__(FIN_THREADS)
-k_finalize(const long long *__restrict__ pd, int nbd, const long long *__restrict__ pf, int nbf,
-           const long long *__restrict__ pk, int nbk, double *__restrict__ sums, long long *__restrict__ counters) {
-  static_assert(FIN_THREADS == 1024, "32 warp sums, reduced by one warp");
-  __shared__ long long red[FIN_THREADS / 32];
-  const int v = blockIdx.x;
-  const long long *src;
-  int nb, stride, off;
-  if (v == 0) { src = pd; nb = nbd; stride = 5; off = 0; }
-  else if (v <= 9) { src = pf; nb = nbf; stride = 13; off = v - 1; }
-  else if (v == 10) { src = pk; nb = nbk; stride = 1; off = 0; }
-  else if (v <= 14) { src = pd; nb = nbd; stride = 5; off = v - 10; }
-  else { src = pf; nb = nbf; stride = 13; off = 9 + (v - 15); }
-  if (src == nullptr) return;
-  long long t = 0;
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) t += src[(size_t)b * stride + off];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    t = red[threadIdx.x];                              // FIN_THREADS / 32 == 32 warp sums
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  }
-  if (threadIdx.x == 0) {
-    const long long tot = t;
-    sums[v] = v <= 10 ? (double)tot * FIX_INV : (double)tot;       // energies/virial are fixed point
-    if (counters != nullptr && v >= 11) counters[v - 11] += tot;
-    if (counters != nullptr && v == 0) counters[8] += 1;
-  }
+  add_kinetic(sums, acc);
 }
 
 // [n][3] float64 (original order) -> SoA float64, ids = 0..n-1.
@@ -362,55 +286,43 @@ __global__ void k_store_neighbors(int n, int cap_in, int cap_out, const int *__r
 // ---------------------------------------------------------------------------------------------------
 static int bl(long long m, int b) { return (int)((m + b - 1) / b); }
 
-constexpr int MD_BLOCK = 256;
-int md_blocks(int n) { return bl(n, MD_BLOCK); }
-
-cudaError_t launch_kick_drift(int n, double *x, double *y, double *z, double *vx, double *vy, double *vz, const long long *F,
+cudaError_t launch_kick_drift(int n, double *x, double *y, double *z, double *vx, double *vy, double *vz, long long *F,
                               float4 *pos, const float4 *pos_ref, double kick, double dt, const double l[3],
                               float half_skin2, Control *ctrl, cudaStream_t st) {
-  if (n > 0)
-    k_kick_drift<<<bl(n, MD_BLOCK), MD_BLOCK, 0, st>>>(n, x, y, z, vx, vy, vz, F, pos, pos_ref, kick, dt, l[0], l[1],
-                                                       l[2], half_skin2, ctrl);
+  if (n <= 0) return cudaSuccess;
+  // FP64-bound and short: small systems in small blocks, so that every SM's narrow pipe takes part
+  const int block = n <= 16384 ? 64 : MD_BLOCK;
+  k_kick_drift<<<bl(n, block), block, 0, st>>>(n, x, y, z, vx, vy, vz, F, pos, pos_ref, kick, dt, l[0], l[1], l[2],
+                                               half_skin2, ctrl);
   return cudaGetLastError();
 }
 
+// The rebuild decision of kind `decide` (nep_control.cuh) as a kernel of its own; cond: also sets the condition of
+// the graph node that holds the rebuild chain.
+cudaError_t launch_control(Control *ctrl, int decide, cudaStream_t st) {
+  k_control_as<<<1, 32, 0, st>>>(ctrl, decide);
+  return cudaGetLastError();
+}
 cudaError_t launch_control_cond(Control *ctrl, cudaGraphConditionalHandle cond, cudaStream_t st) {
   k_control_cond<<<1, 32, 0, st>>>(ctrl, cond);
   return cudaGetLastError();
 }
 
-cudaError_t launch_control(Control *ctrl, bool force, cudaStream_t st) {
-  if (force) k_control_force<<<1, 32, 0, st>>>(ctrl);
-  else k_control<<<1, 32, 0, st>>>(ctrl);
+cudaError_t launch_kick(int n, double *vx, double *vy, double *vz, const long long *F, double kick, double mass,
+                        const EvalSums &sums, Control *ctrl, cudaStream_t st) {
+  if (n > 0) k_kick<<<bl(n, MD_BLOCK), MD_BLOCK, 0, st>>>(n, vx, vy, vz, F, kick, mass, sums, ctrl);
   return cudaGetLastError();
 }
 
-cudaError_t launch_kick(int n, double *vx, double *vy, double *vz, const long long *F, double kick, double mass, long long *part,
-                        Control *ctrl, cudaStream_t st) {
-  if (n > 0) k_kick<<<bl(n, MD_BLOCK), MD_BLOCK, 0, st>>>(n, vx, vy, vz, F, kick, mass, part, ctrl);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_kinetic(int n, const double *vx, const double *vy, const double *vz, double mass, long long *part,
-                           cudaStream_t st) {
-  if (n > 0) k_kinetic<<<bl(n, MD_BLOCK), MD_BLOCK, 0, st>>>(n, vx, vy, vz, mass, part);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_finalize(const long long *pd, int nbd, const long long *pf, int nbf, const long long *pk, int nbk,
-                            double *sums, long long *counters, cudaStream_t st) {
-  k_finalize<<<N_SUMS, FIN_THREADS, 0, st>>>(pd, nbd, pf, nbf, pk, nbk, sums, counters);
+cudaError_t launch_kinetic(int n, const double *vx, const double *vy, const double *vz, double mass,
+                           const EvalSums &sums, cudaStream_t st) {
+  if (n > 0) k_kinetic<<<bl(n, MD_BLOCK), MD_BLOCK, 0, st>>>(n, vx, vy, vz, mass, sums);
   return cudaGetLastError();
 }
 
 cudaError_t launch_load_state(int n, const double *xin, const double *vin, double *x, double *y, double *z, double *vx,
                               double *vy, double *vz, int *id, int *status, cudaStream_t st) {
   if (n > 0) k_load_state<<<bl(n, 256), 256, 0, st>>>(n, xin, vin, x, y, z, vx, vy, vz, id, status);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_control_check(Control *ctrl, cudaStream_t st) {
-  k_control_check<<<1, 32, 0, st>>>(ctrl);
   return cudaGetLastError();
 }
 

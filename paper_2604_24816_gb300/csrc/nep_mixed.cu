@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(MIX_BLOCK, S::NLM > 8 ? NEP_MIX_MINB_TM : 6)
 k_descriptor_mixed(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
                    const int32_t *__restrict__ nbr, const RowExt X, __half *__restrict__ G,
                    float *__restrict__ usite, float *__restrict__ qout, long long *__restrict__ Ffix,
-                   long long *__restrict__ part, int *__restrict__ status, const __grid_constant__ Fallback fb) {
+                   const EvalSums sums, int *__restrict__ status, const __grid_constant__ Fallback fb) {
   static_assert(S::NDES <= MIX_K && S::NNEU <= MIX_N, "network larger than one tensor-core tile");
   constexpr bool TM = S::NLM > 8;
   constexpr int NT = 4;                                   // TM: channels whose sums live in TMEM
@@ -229,29 +229,25 @@ k_descriptor_mixed(const __grid_constant__ Model<S> P, const Geom geom, const in
   tc_fence_before();
   __syncthreads();
   if (t < 32) tmem_dealloc(tmem, TCOLS);
-  block_sum_store<5, MIX_BLOCK / 32>(acc, part);
+  eval_add_d<MIX_BLOCK / 32>(sums, acc);
 }
 
 template <class S, class MT>
 cudaError_t launch_descriptor_mixed(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
                                     const RowExt &X, __half *G, float *usite, float *qout, long long *Ffix,
-                                    long long *part, int *status, const Fallback &fb, cudaStream_t st) {
+                                    const EvalSums &sums, int *status, const Fallback &fb, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int grid = (n + MIX_BLOCK - 1) / MIX_BLOCK;
-  k_descriptor_mixed<S, MT><<<grid, MIX_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, G, usite, qout, Ffix, part, status,
+  k_descriptor_mixed<S, MT><<<grid, MIX_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, G, usite, qout, Ffix, sums, status,
                                                         fb);
   return cudaGetLastError();
 }
 
-int mixed_descriptor_blocks(int n) { return (n + MIX_BLOCK - 1) / MIX_BLOCK; }
-
 #define NEP_INSTANTIATE(SH, MT)                                                                                \
   template cudaError_t launch_descriptor_mixed<SH, MT>(const Model<SH> &, const Geom &, int, const float4 *,          \
                                                        const int32_t *, const RowExt &, __half *, float *, float *,   \
-                                                       long long *, long long *, int *, const Fallback &,             \
+                                                       long long *, const EvalSums &, int *, const Fallback &,        \
                                                        cudaStream_t);
-NEP_INSTANTIATE(CuShape, __nv_bfloat16)
-NEP_INSTANTIATE(CuShape, __half)
 NEP_INSTANTIATE(StudentShape, __nv_bfloat16)
 NEP_INSTANTIATE(StudentShape, __half)
 #undef NEP_INSTANTIATE

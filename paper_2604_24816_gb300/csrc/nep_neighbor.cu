@@ -10,7 +10,8 @@
 //                   the positions, independent of launch timing and of the previous order; gathers x, v,
 //                   id into it and forms the cell-relative float32 coordinates
 //   k_copy_back     copy the gathered arrays back (fixed device pointers for graph replay)
-//   k_rebuild_small all of the above in one block, for small systems
+//   k_rebuild_small, k_rebuild_cluster   all of the above in one block or one cluster, for small systems; these can
+//                   also take the rebuild decision themselves
 //   k_neighbors     for each atom, every j with |r_ij| < rc_R + skin among the 27 neighbouring cell
 //                   images, split into the pairs this atom owns (one owner per unordered pair) and the
 //                   rest, each part grouped by distance band so that the per-pair branches of the
@@ -18,6 +19,7 @@
 // Distances use cell-relative float32 coordinates plus the image offset of the neighbouring cell, so
 // their error does not grow with the box size (float64 appears only in the wrap and cell assignment).
 #include "nep_common.cuh"
+#include "nep_control.cuh"
 
 #include <algorithm>
 
@@ -229,8 +231,8 @@ __global__ void k_copy_back(int n, double *__restrict__ x, double *__restrict__ 
 // The whole cell sort of a small system (n <= SMALL_ATOMS, ncell <= SMALL_CELLS) in one block: histogram,
 // scan, slots and ranks in shared memory, the state in registers between reading the old order and writing
 // the new one (no second buffer).  The same order and coordinates as the kernels above.  At this size every
-// kernel of the chain is a launch and a few dependent loads: 6.2 us at 862 atoms, and 1.5 us on a step that
-// does not rebuild, against nine launches (26 us and 13 us).
+// kernel of the chain is a launch and a few dependent loads: 6.2 us at 862 atoms, and 1.7 us on a step that
+// does not rebuild, the decision included, against nine launches (26 us and 13 us) and a control kernel.
 constexpr int SMALL_ATOMS = 2048, SMALL_CELLS = 2048;
 constexpr int SMALL_ITEMS = SMALL_ATOMS / SCAN_THREADS;
 static_assert(SMALL_ATOMS % SCAN_THREADS == 0 && SMALL_CELLS == 2 * SCAN_THREADS, "two cells per thread");
@@ -238,8 +240,11 @@ __global__ void __launch_bounds__(SCAN_THREADS)
 k_rebuild_small(int n, int ncell, double *__restrict__ x, double *__restrict__ y, double *__restrict__ z,
                 double *__restrict__ vx, double *__restrict__ vy, double *__restrict__ vz, int *__restrict__ id,
                 int *__restrict__ start, float4 *__restrict__ pos, float4 *__restrict__ pos_ref, const CellGrid g,
-                Control *ctrl) {
-  if (!ctrl->do_rebuild) return;
+                Control *ctrl, int decide) {
+  __shared__ int go;
+  if (threadIdx.x == 0) go = decide_rebuild(ctrl, decide);
+  __syncthreads();
+  if (!go) return;
   __shared__ int cnt[SMALL_CELLS];                 // histogram, then the running slots
   __shared__ int first[SMALL_CELLS + 1];           // cell_start
   __shared__ int sid[SMALL_ATOMS];                 // original ids by slot
@@ -283,6 +288,92 @@ k_rebuild_small(int n, int ncell, double *__restrict__ x, double *__restrict__ y
     const int b = first[cell[k]], e = first[cell[k] + 1];
     int d = b;
     for (int q = b; q < e; ++q) d += sid[q] < oid[k] ? 1 : 0;
+    x[d] = a[k].x; y[d] = a[k].y; z[d] = a[k].z;
+    vx[d] = u[k][0]; vy[d] = u[k][1]; vz[d] = u[k][2];
+    id[d] = oid[k];
+    const float4 p = cell_relative(a[k].x, a[k].y, a[k].z, a[k].cx, a[k].cy, a[k].cz, g);
+    pos[d] = p;
+    pos_ref[d] = p;
+  }
+}
+
+// The same for up to CLUSTER_ATOMS atoms and CLUSTER_CELLS cells by a cluster of eight blocks: the phases meet at
+// cluster barriers (hardware barriers; the blocks of a cluster are always resident together), cell counts, scan
+// and slots go through global memory, each thread keeps its atoms' old state in registers until every block has
+// read its share.  The histogram's own atomic gives each atom its slot, so there is no scatter counter.  One launch
+// instead of five per rebuild (25 us at 16,384 atoms: eight SMs' narrow FP64 pipes and six barriers, against 17 us
+// and four gaps) and, on the other steps, 1.9 us instead of the 8 us of a conditional graph node or five early
+// exits: a 10-step block of 16,384 atoms 789 -> 771 us.
+constexpr int CLUSTER_BLOCKS = 8;
+constexpr int CLUSTER_THREADS = CLUSTER_BLOCKS * SCAN_THREADS;
+constexpr int CLUSTER_ITEMS = 2;
+constexpr int CLUSTER_ATOMS = CLUSTER_THREADS * CLUSTER_ITEMS, CLUSTER_CELLS = CLUSTER_THREADS * 2;
+
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+__global__ void __cluster_dims__(CLUSTER_BLOCKS, 1, 1) __launch_bounds__(SCAN_THREADS)
+k_rebuild_cluster(int n, int ncell, double *__restrict__ x, double *__restrict__ y, double *__restrict__ z,
+                  double *__restrict__ vx, double *__restrict__ vy, double *__restrict__ vz, int *__restrict__ id,
+                  int *__restrict__ count, int *__restrict__ start, int *__restrict__ tile_sums,
+                  int *__restrict__ slot_id, float4 *__restrict__ pos, float4 *__restrict__ pos_ref, const CellGrid g,
+                  Control *ctrl, int decide) {
+  __shared__ int warp_tot[SCAN_THREADS / 32];
+  const int t = threadIdx.x, b = blockIdx.x;
+  if (b == 0 && t == 0) decide_rebuild(ctrl, decide);
+  __threadfence();
+  cluster_barrier();
+  if (!__ldcg(&ctrl->do_rebuild)) return;
+  if (b == 0 && t == 0) ctrl->nb_next = 0;
+  CellOf a[CLUSTER_ITEMS];
+  double u[CLUSTER_ITEMS][3];
+  int oid[CLUSTER_ITEMS], cell[CLUSTER_ITEMS], ord[CLUSTER_ITEMS];
+#pragma unroll
+  for (int k = 0; k < CLUSTER_ITEMS; ++k) {
+    const int s = (k * CLUSTER_BLOCKS + b) * SCAN_THREADS + t;
+    cell[k] = -1;
+    if (s < n) {
+      a[k] = cell_of_atom(x[s], y[s], z[s], g, &ctrl->status);
+      u[k][0] = vx[s]; u[k][1] = vy[s]; u[k][2] = vz[s];
+      oid[k] = id[s];
+      cell[k] = (a[k].cz * g.ncy + a[k].cy) * g.ncx + a[k].cx;
+      ord[k] = atomicAdd(count + cell[k], 1);
+    }
+  }
+  __threadfence();
+  cluster_barrier();                               // every atom is counted
+  // two cells per thread; reads past L1, where another block wrote
+  const int c = (b * SCAN_THREADS + t) * 2;
+  const int c0 = c < ncell ? __ldcg(count + c) : 0, c1 = c + 1 < ncell ? __ldcg(count + c + 1) : 0;
+  if (c < ncell) count[c] = 0;
+  if (c + 1 < ncell) count[c + 1] = 0;
+  const int excl = block_scan_excl(c0 + c1, warp_tot);
+  if (t == SCAN_THREADS - 1) tile_sums[b] = excl + c0 + c1;
+  __threadfence();
+  cluster_barrier();
+  int first = 0;
+  for (int k = 0; k < b; ++k) first += __ldcg(tile_sums + k);
+  if (c < ncell) start[c] = first + excl;
+  if (c + 1 < ncell) start[c + 1] = first + excl + c0;
+  if (b == CLUSTER_BLOCKS - 1 && t == SCAN_THREADS - 1) start[ncell] = first + excl + c0 + c1;
+  __threadfence();
+  cluster_barrier();
+  int lo[CLUSTER_ITEMS], hi[CLUSTER_ITEMS];
+#pragma unroll
+  for (int k = 0; k < CLUSTER_ITEMS; ++k) {
+    if (cell[k] < 0) continue;
+    lo[k] = __ldcg(start + cell[k]);
+    hi[k] = __ldcg(start + cell[k] + 1);
+    slot_id[lo[k] + ord[k]] = oid[k];
+  }
+  __threadfence();
+  cluster_barrier();                               // every slot is filled, every old value has been read
+#pragma unroll
+  for (int k = 0; k < CLUSTER_ITEMS; ++k) {
+    if (cell[k] < 0) continue;
+    int d = lo[k];
+    for (int q = lo[k]; q < hi[k]; ++q) d += __ldcg(slot_id + q) < oid[k] ? 1 : 0;
     x[d] = a[k].x; y[d] = a[k].y; z[d] = a[k].z;
     vx[d] = u[k][0]; vy[d] = u[k][1]; vz[d] = u[k][2];
     id[d] = oid[k];
@@ -539,23 +630,35 @@ static int resident_grid(K kernel, long long m, int per_block, int threads) {
   return (int)std::min<long long>(blocks_for(m, per_block), (long long)sm_count() * per_sm);
 }
 
-// Kernels that launch_cell_sort enqueues for a system of n atoms in ncell cells.
+// The forms of the cell sort: one block, one cluster, or the chain of kernels.
 static bool small_system(int n, int ncell) { return n <= SMALL_ATOMS && ncell <= SMALL_CELLS; }
+static bool cluster_system(int n, int ncell) { return n <= CLUSTER_ATOMS && ncell <= CLUSTER_CELLS; }
+// Whether the sort is a single kernel, which can also take the rebuild decision.
+bool cell_sort_decides(int n, int ncell) { return cluster_system(n, ncell); }
+// Kernels that launch_cell_sort enqueues for a system of n atoms in ncell cells.
 int cell_sort_launches(int n, int ncell) {
   if (n <= 0) return 0;
-  return small_system(n, ncell) ? 1 : (ncell <= SCAN_TILE ? 5 : 7);
+  return cluster_system(n, ncell) ? 1 : (ncell <= SCAN_TILE ? 5 : 7);
 }
 
-// a.count is zero on entry and on exit.
-cudaError_t launch_cell_sort(const RebuildArgs &a, cudaStream_t st) {
+// a.count is zero on entry and on exit.  decide (nep_control.cuh): a decision that the sort's only kernel takes
+// first (cell_sort_decides); DECIDE_DONE otherwise.
+cudaError_t launch_cell_sort(const RebuildArgs &a, int decide, cudaStream_t st) {
   if (a.n <= 0) return cudaSuccess;
   const CellGrid g{a.L[0], a.L[1], a.L[2], a.l[0], a.l[1], a.l[2], 1.0 / a.l[0], 1.0 / a.l[1], 1.0 / a.l[2],
                    a.nc[0], a.nc[1], a.nc[2]};
   if (small_system(a.n, a.ncell)) {
     k_rebuild_small<<<1, SCAN_THREADS, 0, st>>>(a.n, a.ncell, a.x, a.y, a.z, a.vx, a.vy, a.vz, a.id, a.start, a.pos,
-                                                a.pos_ref, g, a.ctrl);
+                                                a.pos_ref, g, a.ctrl, decide);
     return cudaGetLastError();
   }
+  if (cluster_system(a.n, a.ncell)) {
+    k_rebuild_cluster<<<CLUSTER_BLOCKS, SCAN_THREADS, 0, st>>>(a.n, a.ncell, a.x, a.y, a.z, a.vx, a.vy, a.vz, a.id,
+                                                               a.count, a.start, a.tile_sums, a.cell_of, a.pos,
+                                                               a.pos_ref, g, a.ctrl, decide);
+    return cudaGetLastError();
+  }
+  if (decide != DECIDE_DONE) return cudaErrorInvalidValue;
   k_cell_assign<<<resident_grid(k_cell_assign, a.n, 256, 256), 256, 0, st>>>(a.n, a.x, a.y, a.z, g, a.cell_of, a.count,
                                                                             a.ctrl);
   const int ntiles = blocks_for(a.ncell, SCAN_TILE);
@@ -586,6 +689,6 @@ cudaError_t launch_neighbors(const RebuildArgs &a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-int scan_tiles(int ncell) { return blocks_for(ncell, SCAN_TILE); }
+int scan_tiles(int ncell) { return std::max(CLUSTER_BLOCKS, blocks_for(ncell, SCAN_TILE)); }
 
 }  // namespace nep

@@ -24,6 +24,7 @@
 #include <thread>
 
 #include "nep_common.cuh"
+#include "nep_control.cuh"
 #include "nep_descriptor.cuh"
 #include "nep_gb300.h"
 
@@ -31,14 +32,12 @@ namespace nep {
 int wide_lanes(int n);
 template <class S, class MT>
 cudaError_t launch_wide(int, const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
-                        float *, float *, long long *, long long *, long long *, int *, const Fallback &, int *,
-                        cudaStream_t);
-cudaError_t launch_cell_sort(const RebuildArgs &, cudaStream_t);
+                        float *, float *, long long *, const EvalSums &, int *, const Fallback &, cudaStream_t);
+cudaError_t launch_cell_sort(const RebuildArgs &, int, cudaStream_t);
+bool cell_sort_decides(int n, int ncell);
 cudaError_t launch_neighbors(const RebuildArgs &, cudaStream_t);
 int scan_tiles(int ncell);
-cudaError_t launch_control(Control *, bool, cudaStream_t);
-cudaError_t launch_finalize(const long long *, int, const long long *, int, const long long *, int, double *,
-                            long long *, cudaStream_t);
+cudaError_t launch_control(Control *, int, cudaStream_t);
 cudaError_t launch_load_state(int, const double *, const double *, double *, double *, double *, double *, double *,
                               double *, int *, int *, cudaStream_t);
 cudaError_t launch_store_force(int, const int *, const long long *, double *, cudaStream_t);
@@ -58,7 +57,7 @@ constexpr size_t up256(size_t b) { return (b + 255) / 256 * 256; }
 // Byte offsets of the pieces inside the scratch array.
 struct Layout {
   size_t x, y, z, vx, vy, vz, xb, yb, zb, vxb, vyb, vzb, id, idb, cell_of, perm, pos, pos_ref, F, usite, nbr,
-      nnum, nang, nown, nband0, nfar, count, cursor, start, tile_sums, part_d, part_f, sums, counters, ctrl, io, total;
+      nnum, nang, nown, nband0, nfar, count, cursor, start, tile_sums, sums, counters, acc, ctrl, io, total;
 };
 
 constexpr Layout make_layout() {
@@ -72,12 +71,14 @@ constexpr Layout make_layout() {
   L.vxb = take(N * 8); L.vyb = take(N * 8); L.vzb = take(N * 8);
   L.id = take(N * 4); L.idb = take(N * 4); L.cell_of = take(N * 4); L.perm = take(N * 8);
   L.pos = take(N * 16); L.pos_ref = take(N * 16);
-  L.F = take(N * 3 * 8); L.usite = take(N * 4); L.nbr = take(N * CAP * 4);
+  L.usite = take(N * 4); L.nbr = take(N * CAP * 4);
   L.nnum = take(N * 4); L.nang = take(N * 4); L.nown = take(N * 4); L.nband0 = take(N * 4); L.nfar = take(N * 4);
+  // cleared by every call, up to the part of count that it uses: control block, counters, running totals (and the
+  // closing count behind them), forces, cell counters
+  L.ctrl = take(sizeof(Control)); L.counters = take(16 * 8); L.acc = take((N_SUMS + 1) * 8); L.F = take(N * 3 * 8);
   L.count = take((size_t)NC_MAX * 4); L.cursor = take((size_t)NC_MAX * 4); L.start = take(((size_t)NC_MAX + 1) * 4);
-  L.tile_sums = take(((size_t)NC_MAX / 4096 + 2) * 4);
-  L.part_d = take((size_t)WIDE_MAX_BLOCKS * 5 * 8); L.part_f = take((size_t)WIDE_MAX_BLOCKS * 13 * 8);
-  L.sums = take(32 * 8); L.counters = take(16 * 8); L.ctrl = take(sizeof(Control)); L.io = take(N * 3 * 8);
+  L.tile_sums = take(((size_t)NC_MAX / 4096 + 10) * 4);
+  L.sums = take(32 * 8); L.io = take(N * 3 * 8);
   L.total = o;
   return L;
 }
@@ -256,34 +257,29 @@ extern "C" nep_status nep_compute_noalloc(const nep_params *p, int64_t n, const 
   Control *ctrl = (Control *)at(LAYOUT.ctrl);
   a.ctrl = ctrl;
   long long *Ffix = (long long *)at(LAYOUT.F);
-  long long *pd = (long long *)at(LAYOUT.part_d), *pf = (long long *)at(LAYOUT.part_f);
   double *sums = (double *)at(LAYOUT.sums);
-  long long *counters = (long long *)at(LAYOUT.counters);
+  long long *acc = (long long *)at(LAYOUT.acc);
+  const EvalSums es{acc, (unsigned *)(acc + N_SUMS), sums, (long long *)at(LAYOUT.counters), 1};
   double *io = (double *)at(LAYOUT.io);
   Geom g;
   g.lx = (float)l[0]; g.ly = (float)l[1]; g.lz = (float)l[2];
   g.ncx = nc[0]; g.ncy = nc[1]; g.ncz = nc[2];
 
-  // The array keeps the previous call's contents: clear the status word, control block, counters and cell counters
-  // (force accumulators and partial sums are cleared or overwritten by the kernels).
-  NA_CUDA(cudaMemsetAsync(ctrl, 0, sizeof(Control), st));
-  NA_CUDA(cudaMemsetAsync(counters, 0, 16 * sizeof(long long), st));
-  NA_CUDA(cudaMemsetAsync(a.count, 0, (size_t)a.ncell * sizeof(int), st));
+  // The array keeps the previous call's contents: clear what must start from zero (one range, see Layout).
+  NA_CUDA(cudaMemsetAsync(ctrl, 0, LAYOUT.count - LAYOUT.ctrl + (size_t)a.ncell * sizeof(int), st));
   const double *xin = x;
   if (!device_pointer(x)) {
     NA_CUDA(cudaMemcpyAsync(io, x, 3 * (size_t)N * sizeof(double), cudaMemcpyHostToDevice, st));
     xin = io;
   }
   NA_CUDA(launch_load_state(N, xin, nullptr, a.x, a.y, a.z, a.vx, a.vy, a.vz, a.id, &ctrl->status, st));
-  NA_CUDA(launch_control(ctrl, true, st));
-  NA_CUDA(launch_cell_sort(a, st));
+  const bool decides = cell_sort_decides(N, a.ncell);
+  if (!decides) NA_CUDA(launch_control(ctrl, DECIDE_FORCE, st));
+  NA_CUDA(launch_cell_sort(a, decides ? DECIDE_FORCE : DECIDE_DONE, st));
   NA_CUDA(launch_neighbors(a, st));
   const RowExt rows{a.nnum, a.nown, a.nband0, a.nfar, nullptr};   // one evaluation: the whole rows
-  int blocks = 0;
-  NA_CUDA(cudaMemsetAsync(Ffix, 0, 3 * (size_t)N * sizeof(long long), st));
   NA_CUDA((launch_wide<S, float>(std::max(8, wide_lanes(N)), M, g, N, a.pos, a.nbr, rows, (float *)at(LAYOUT.usite),
-                                 nullptr, Ffix, pd, pf, &ctrl->status, Fallback{}, &blocks, st)));
-  NA_CUDA(launch_finalize(pd, blocks, pf, blocks, nullptr, 0, sums, counters, st));
+                                 nullptr, Ffix, es, &ctrl->status, Fallback{}, st)));
   const bool f_dev = F && device_pointer(F);
   const bool e_dev = E && device_pointer(E);
   const bool w_dev = virial && device_pointer(virial);

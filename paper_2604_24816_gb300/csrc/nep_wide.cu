@@ -113,8 +113,7 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
                                           const int m, const int32_t *__restrict__ list, const float4 *__restrict__ pos,
                                           const int32_t *__restrict__ nbr, const RowExt &X, float *__restrict__ usite,
                                           float *__restrict__ qout, unsigned long long *__restrict__ Ffix,
-                                          long long *__restrict__ part_d, long long *__restrict__ part_f,
-                                          int *__restrict__ status, const Fallback &fb) {
+                                          const EvalSums &sums, int *__restrict__ status, const Fallback &fb) {
   constexpr bool MIX = !std::is_same<MT, float>::value;
   constexpr int NG = 32 / G;                           // atoms per warp
   constexpr int LD = WideNet<S>::LD;
@@ -126,8 +125,6 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int gl = lane % G, grp = lane / G;
   int base = ((int)blockIdx.x * WIDE_WARPS + warp) * NG;
-  // a block without flagged atoms has nothing to add (block-uniform; in LIST no block writes a row of its own)
-  if (LIST && (int)blockIdx.x * WIDE_WARPS * NG >= m) return;
   const bool skip = skip_far(X);
   // an atom's row extent, first two entries per lane and first neighbour: loaded before the tables are staged
   // and at the end of the previous atom, so that the chain extent -> entry -> position starts early
@@ -148,6 +145,11 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
     e1 = entry(gl + G);
     pj = pos[e & J_MASK];
   };
+  __shared__ long long wsum_d[WIDE_WARPS][5], wsum_f[WIDE_WARPS][13];
+  if ((int)blockIdx.x * WIDE_WARPS * NG >= m) {        // a block without atoms only takes part in the closing count
+    if (threadIdx.x < 32) eval_add<WIDE_WARPS>(sums, nullptr, nullptr);
+    return;
+  }
   load_atom();
   fill_shift_table(shift, geom);
   for (int t = threadIdx.x; t < S::NNEU * S::NDES; t += WIDE_BLOCK)
@@ -457,24 +459,16 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
   }
   acc_f[3] = acc_f[1]; acc_f[6] = acc_f[2]; acc_f[7] = acc_f[5];
   if constexpr (LIST) {
-    // added to the sums of the student's kernels (integers: any order gives the same result)
-    __shared__ long long red[WIDE_WARPS][10];
-    long long v[10] = {acc_d[0], acc_f[0], acc_f[1], acc_f[2], acc_f[3], acc_f[4], acc_f[5], acc_f[6], acc_f[7], acc_f[8]};
-    warp_sum_stage<10>(v, red[warp]);
-    __syncthreads();
-    if (threadIdx.x < 10) {
-      long long t = 0;
-      for (int w = 0; w < WIDE_WARPS; ++w) t += red[w][threadIdx.x];
-      if (t != 0)
-        atomicAdd(reinterpret_cast<unsigned long long *>(threadIdx.x == 0 ? part_d : part_f + threadIdx.x - 1),
-                  (unsigned long long)t);
-    }
+    // the counts are the student's; these atoms only add energy and virial
+    acc_d[1] = acc_d[2] = acc_d[3] = acc_d[4] = 0;
   } else {
     // the force pass visits the walk's active pairs
     acc_f[9] = acc_d[3]; acc_f[10] = acc_d[4]; acc_f[11] = acc_d[1]; acc_f[12] = acc_d[2];
-    block_sum_store<5, WIDE_WARPS>(acc_d, part_d);
-    block_sum_store<13, WIDE_WARPS>(acc_f, part_f);
   }
+  warp_sum_stage<5>(acc_d, wsum_d[warp]);
+  warp_sum_stage<13>(acc_f, wsum_f[warp]);
+  __syncthreads();
+  eval_add<WIDE_WARPS>(sums, wsum_d, wsum_f);
 }
 
 // One evaluation of all n atoms.
@@ -482,10 +476,10 @@ template <class S, class MT, int G>
 __global__ void __launch_bounds__(WIDE_BLOCK, 4)
 k_nep_wide(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
            const int32_t *__restrict__ nbr, const RowExt X, float *__restrict__ usite, float *__restrict__ qout,
-           unsigned long long *__restrict__ Ffix, long long *__restrict__ part_d, long long *__restrict__ part_f,
-           int *__restrict__ status, const __grid_constant__ Fallback fb) {
+           unsigned long long *__restrict__ Ffix, const EvalSums sums, int *__restrict__ status,
+           const __grid_constant__ Fallback fb) {
   __shared__ WideShared<S, G> M;
-  wide_body<S, MT, G, false>(M, P, geom, n, n, nullptr, pos, nbr, X, usite, qout, Ffix, part_d, part_f, status, fb);
+  wide_body<S, MT, G, false>(M, P, geom, n, n, nullptr, pos, nbr, X, usite, qout, Ffix, sums, status, fb);
 }
 
 // The fallback model on the first min(*count, cap) atoms of list: only its network's part is added to usite, to
@@ -500,24 +494,22 @@ __global__ void __launch_bounds__(WIDE_BLOCK, 4)
 k_nep_wide_list(const __grid_constant__ Model<S> P, const Geom geom, const int n, const int32_t *__restrict__ list,
                 const int *__restrict__ count, const int cap, const float4 *__restrict__ pos,
                 const int32_t *__restrict__ nbr, const RowExt X, float *__restrict__ usite,
-                unsigned long long *__restrict__ Ffix, long long *__restrict__ part_d, long long *__restrict__ part_f,
-                long long *__restrict__ counters, int *__restrict__ status) {
+                unsigned long long *__restrict__ Ffix, const EvalSums sums, int *__restrict__ status) {
   __shared__ __align__(16) unsigned char raw[sizeof(WideShared<S, 8>)];
   static_assert(sizeof(WideShared<S, 8>) >= sizeof(WideShared<S, 32>), "one buffer for both splits");
   const int m = min(*count, cap);
   if (blockIdx.x == 0 && threadIdx.x == 0)
-    atomicAdd(reinterpret_cast<unsigned long long *>(counters + 9), (unsigned long long)m);
-  if (m == 0) return;
+    atomicAdd(reinterpret_cast<unsigned long long *>(sums.counters + 9), (unsigned long long)m);
   const Fallback none{};
   if (m <= LIST_WARP_MAX)
     wide_body<S, float, 32, true>(reinterpret_cast<WideShared<S, 32> &>(raw), P, geom, n, m, list, pos, nbr, X, usite,
-                                  nullptr, Ffix, part_d, part_f, status, none);
+                                  nullptr, Ffix, sums, status, none);
   else
     wide_body<S, float, 8, true>(reinterpret_cast<WideShared<S, 8> &>(raw), P, geom, n, m, list, pos, nbr, X, usite,
-                                 nullptr, Ffix, part_d, part_f, status, none);
+                                 nullptr, Ffix, sums, status, none);
 }
 
-// Blocks that fit on the device at once (at most WIDE_MAX_BLOCKS), or fewer for few atoms; the kernels loop.
+// Blocks that fit on the device at once, or fewer for few atoms; the kernels loop.
 template <class K>
 int wide_grid(K kernel, int atoms, int lanes) {
   int d = 0, sms = 0, per = 0;
@@ -528,7 +520,7 @@ int wide_grid(K kernel, int atoms, int lanes) {
     per = 1;
   }
   const long long need = ((long long)atoms * lanes + WIDE_BLOCK - 1) / WIDE_BLOCK;
-  return (int)std::max(1ll, std::min(need, (long long)std::min(sms * per, WIDE_MAX_BLOCKS)));
+  return (int)std::max(1ll, std::min(need, (long long)sms * per));
 }
 
 }  // namespace
@@ -542,17 +534,15 @@ int wide_grid(K kernel, int atoms, int lanes) {
 // mixed forms cross at the same sizes.
 int wide_lanes(int n) { return n <= 1024 ? 32 : (n <= 4096 ? 16 : (n <= 16384 ? 8 : 0)); }
 
-// One force evaluation with G = wide_lanes(n) lanes per atom; Ffix must be zero.  *blocks = partial-sum rows
-// written (at most WIDE_MAX_BLOCKS).
+// One force evaluation with `lanes` (8, 16 or 32) lanes per atom; Ffix must be zero.
 template <class S, class MT>
 cudaError_t launch_wide(int lanes, const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
-                        const RowExt &X, float *usite, float *qout, long long *Ffix, long long *part_d,
-                        long long *part_f, int *status, const Fallback &fb, int *blocks, cudaStream_t st) {
+                        const RowExt &X, float *usite, float *qout, long long *Ffix, const EvalSums &sums,
+                        int *status, const Fallback &fb, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   auto run = [&](auto kernel, int g_lanes) {
-    *blocks = wide_grid(kernel, n, g_lanes);
-    kernel<<<*blocks, WIDE_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, usite, qout,
-                                           reinterpret_cast<unsigned long long *>(Ffix), part_d, part_f, status, fb);
+    kernel<<<wide_grid(kernel, n, g_lanes), WIDE_BLOCK, 0, st>>>(
+        P, g, n, pos, nbr, X, usite, qout, reinterpret_cast<unsigned long long *>(Ffix), sums, status, fb);
   };
   if (lanes == 32) run(k_nep_wide<S, MT, 32>, 32);
   else if (lanes == 16) run(k_nep_wide<S, MT, 16>, 16);
@@ -560,26 +550,25 @@ cudaError_t launch_wide(int lanes, const Model<S> &P, const Geom &g, int n, cons
   return cudaGetLastError();
 }
 
-// The fallback model on the flagged atoms (list, count on the device): its site energies are added to usite and
-// to part_d[0], its forces to Ffix, its virial to part_f[0..8], the atom count to counters[9].
+// The fallback model on the flagged atoms (list, count on the device): its site energies are added to usite and to
+// the running energy, its forces to Ffix, its virial to the running virial, the atom count to counters[9].
 template <class S>
 cudaError_t launch_wide_list(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
                              const RowExt &X, const int *list, const int *count, int cap, float *usite, long long *Ffix,
-                             long long *part_d, long long *part_f, long long *counters, int *status, cudaStream_t st) {
+                             const EvalSums &sums, int *status, cudaStream_t st) {
   if (n <= 0 || cap <= 0) return cudaSuccess;
   k_nep_wide_list<S><<<wide_grid(k_nep_wide_list<S>, cap, 32), WIDE_BLOCK, 0, st>>>(
-      P, g, n, list, count, cap, pos, nbr, X, usite, reinterpret_cast<unsigned long long *>(Ffix), part_d, part_f,
-      counters, status);
+      P, g, n, list, count, cap, pos, nbr, X, usite, reinterpret_cast<unsigned long long *>(Ffix), sums, status);
   return cudaGetLastError();
 }
 template cudaError_t launch_wide_list<CuShape>(const Model<CuShape> &, const Geom &, int, const float4 *, const int32_t *,
                                                const RowExt &, const int *, const int *, int, float *, long long *,
-                                               long long *, long long *, long long *, int *, cudaStream_t);
+                                               const EvalSums &, int *, cudaStream_t);
 
 #define NEP_INSTANTIATE(SH, MT)                                                                                     \
   template cudaError_t launch_wide<SH, MT>(int, const Model<SH> &, const Geom &, int, const float4 *, const int32_t *, \
-                                           const RowExt &, float *, float *, long long *, long long *, long long *,   \
-                                           int *, const Fallback &, int *, cudaStream_t);
+                                           const RowExt &, float *, float *, long long *, const EvalSums &, int *,    \
+                                           const Fallback &, cudaStream_t);
 NEP_INSTANTIATE(CuShape, float)
 NEP_INSTANTIATE(CuShape, __nv_bfloat16)
 NEP_INSTANTIATE(CuShape, __half)

@@ -1,5 +1,5 @@
-"""The cell sort's forms at the sizes where they change: one block (up to 2,048 atoms and cells), one scan
-tile (up to 4,096 cells), several tiles, and more tiles than one pass of the carry scan holds.  The lists
+"""The cell sort's forms at the sizes where they change: one block (up to 2,048 atoms and cells), one cluster (up to
+16,384), a chain of kernels with several scan tiles, and more tiles than one pass of the carry scan holds.  The lists
 must be those of a brute-force search, and the same rows again when the build starts from its own order."""
 import numpy as np
 import pytest
@@ -41,8 +41,12 @@ CASES = {
     "2047 atoms": lambda: _crystal(2047, (8, 8, 8)),
     "2048 atoms": lambda: _crystal(2048, (8, 8, 8)),
     "2049 atoms": lambda: _crystal(2049, (8, 8, 9)),
+    "16384 atoms": lambda: _crystal(16384, (16, 16, 16)),
+    "16385 atoms": lambda: _crystal(16385, (16, 16, 17)),
+    "3000 atoms, 15625 cells": lambda: _clusters(3000, 150.5, 6),
+    "3000 atoms, 17576 cells": lambda: _clusters(3000, 156.5, 7),
     "2016 atoms, 2197 cells": lambda: _clusters(2016, 80.0, 3),
-    "1000 atoms, 4913 cells (two tiles)": lambda: _clusters(1000, 104.0, 4),
+    "1000 atoms, 4913 cells": lambda: _clusters(1000, 104.0, 4),
     "2500 atoms, 4.6M cells (1117 tiles)": lambda: _clusters(2500, 1000.0, 5),
 }
 
