@@ -402,8 +402,9 @@ __device__ __forceinline__ void radial_channels(const Model<S> &P, float r, bool
   }
 }
 // g_n and g_n': with p = E + x O, dp/dx = 4 x (E' + x O') + O, g' = p dh + dp/dx dxh.
-template <class S>
-__device__ __forceinline__ void radial_channels_d(const Model<S> &P, float r, float (&g)[S::NA], float (&dg)[S::NA]) {
+// (M: a Model, or any holder of inv_rcA, gE, gO, gL.)
+template <class S, class M>
+__device__ __forceinline__ void radial_channels_d(const M &P, float r, float (&g)[S::NA], float (&dg)[S::NA]) {
   float h, dh, dxh, x, y;
   cheb_args_d(r, P.inv_rcA, h, dh, dxh, x, y);
   const float x4 = 4.f * x;

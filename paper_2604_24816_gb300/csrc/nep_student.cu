@@ -19,6 +19,8 @@
 // zdot_mu = sum_nu W0_mu,nu s_nu dq_nu, whose derivatives are written out in st_grad.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "nep_common.cuh"
 #include "nep_student.h"
 
@@ -36,8 +38,15 @@ static_assert(NPAR == ST_NPAR && ND == ST_NDES && SS::GS == ST_GS, "header const
 static_assert(SS::KR == SS::KA, "one basis size for both cutoffs");
 
 constexpr int BLOCK = 128;
-constexpr int GRAD_BLOCK = 64;               // atoms per block of st_grad
-constexpr int GREC = NPAR;                   // floats per atom record in st_grad's shared memory
+constexpr int GRAD_ATOMS = 64;               // atoms per row of partial gradients, at least (st_grad_scratch)
+
+// The per-step kernels give each atom a group of eight lanes.  One thread per atom left a mini-batch of 40 cells
+// (21,000 atoms, 165 blocks of 128 threads) at about one block per SM, each thread walking its row alone, and
+// entered the angular branch for nearly every entry of the unsorted rows (some lane always has one) although two
+// in five are angular.
+constexpr int G = 8;
+static_assert(G == KB && G == NLM, "a lane per basis function, or per harmonic component");
+constexpr unsigned FULL = 0xffffffffu;
 
 struct Cut {
   float rcR2, rcA2, inv_rcR, inv_rcA;
@@ -45,6 +54,77 @@ struct Cut {
 Cut cut_of(st_cutoffs rc) { return Cut{rc.rc_R * rc.rc_R, rc.rc_A * rc.rc_A, 1.f / rc.rc_R, 1.f / rc.rc_A}; }
 
 __device__ __forceinline__ int l_of(int lm) { return lm < 3 ? 1 : 2; }
+
+// A group's sum of v, in every lane.
+__device__ __forceinline__ float group_sum(float v) {
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+  return v;
+}
+// The group's sums of 8 (4) values: lane gl gets the sum of value gl (gl & 3).
+__device__ __forceinline__ float group_scatter8(const float (&v)[8], int gl) {
+  float a[4], b[2];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float keep = gl & 4 ? v[4 + k] : v[k], give = gl & 4 ? v[k] : v[4 + k];
+    a[k] = keep + __shfl_xor_sync(FULL, give, 4);
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float keep = gl & 2 ? a[2 + k] : a[k], give = gl & 2 ? a[k] : a[2 + k];
+    b[k] = keep + __shfl_xor_sync(FULL, give, 2);
+  }
+  const float keep = gl & 1 ? b[1] : b[0], give = gl & 1 ? b[0] : b[1];
+  return keep + __shfl_xor_sync(FULL, give, 1);
+}
+__device__ __forceinline__ float group_scatter4(const float (&v)[4], int gl) {
+  float b[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float keep = gl & 2 ? v[2 + k] : v[k], give = gl & 2 ? v[k] : v[2 + k];
+    b[k] = keep + __shfl_xor_sync(FULL, give, 2);
+  }
+  const float keep = gl & 1 ? b[1] : b[0], give = gl & 1 ? b[0] : b[1];
+  const float c = keep + __shfl_xor_sync(FULL, give, 1);
+  return c + __shfl_xor_sync(FULL, c, 4);
+}
+__device__ __forceinline__ float from_lane(float v, int src) { return __shfl_sync(FULL, v, src, G); }
+
+// Radial functions of a set of channels as cubics (cheb_to_cubics), in shared memory.
+struct Cubics {
+  float inv_rcA;
+  float2 gE[2][4], gO[2][4], gL[4];
+};
+static_assert(NR == 4 && NA == 4, "two channel pairs");
+// Threads 0..3 fill R from theta's c_R, threads 4..7 A from c_A (a block barrier must follow).
+__device__ __forceinline__ void stage_cubics(const float *th, Cut C, Cubics *R, Cubics *A) {
+  const int t = threadIdx.x;
+  if (t >= 8) return;
+  Cubics &Q = t < 4 ? *R : *A;
+  const int n = t & 3;
+  float c[8], e[4], o[4];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) c[k] = th[(t < 4 ? OFF_CR : OFF_CA) + n * KB + k];
+  cheb_to_cubics(c, e, o);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    (&Q.gE[n >> 1][i].x)[n & 1] = e[i];
+    (&Q.gO[n >> 1][i].x)[n & 1] = o[i];
+  }
+  if (n == 0) Q.inv_rcA = t < 4 ? C.inv_rcR : C.inv_rcA;
+}
+
+// Four consecutive floats; V4: p is 16-byte aligned.
+template <bool V4>
+__device__ __forceinline__ float4 load4(const float *__restrict__ p) {
+  if constexpr (V4) return *reinterpret_cast<const float4 *>(p);
+  else return make_float4(p[0], p[1], p[2], p[3]);
+}
+
+// A row is walked in segments of SEG entries; the angular ones of a segment are listed per atom in shared memory
+// and evaluated G at a time.
+constexpr int SEG = 64;
+static_assert(SEG <= 256, "the lists hold bytes");
 
 // theta (and q_scale) staged in shared memory once per block.
 __device__ __forceinline__ void stage_theta(float *sth, const float *theta, float *sqs, const float *qs) {
@@ -125,89 +205,124 @@ __global__ void k_st_basis(int a0, int a1, int n, const int *__restrict__ nnum, 
     for (int c = 0; c < NLM; ++c) S[(size_t)a * NSB + k * NLM + c] = s[k][c];
 }
 
-// Per-atom forward pieces shared by st_forward and st_grad: descriptors, hidden layer, dU/dq.
-struct AtomNet {
-  float s[NA][NLM];     // s_nlm
-  float q[ND];          // unscaled descriptors
-  float h[NN];          // tanh activations
-  float Fp[ND];         // dU/dq (unscaled q)
-  float U;
+// An atom's forward pass over its eight lanes (shared by st_forward and st_grad).  Lane gl holds harmonic
+// component gl of the sums, the angular descriptor (n, l) = (gl & 3, gl / 4 + 1) and the radial descriptor gl & 3,
+// neurons gl and gl + 8.
+struct LaneNet {
+  float Sk[KB];         // S_k,gl
+  float s[NA];          // s_n,gl
+  float qr, qa;         // own radial and angular descriptor (unscaled)
+  float qt[ND];         // all scaled descriptors
+  float h[2], d1h[2];   // own neurons: tanh and 1 - tanh^2
+  float U;              // site energy, without the -b1 of the sum: added (every lane)
 };
+__device__ __forceinline__ int own_v(int gl) { return NR + 2 * (gl & 3) + (gl >> 2); }   // index of the own angular descriptor
 
-__device__ __forceinline__ void atom_net(const float *th, const float *qs, const float *Qa, const float *Sa,
-                                         AtomNet &A) {
+// Contractions with the expansion coefficients: s_n = sum_k cA_nk S_k (own component) and the own radial
+// descriptor sum_k cR_nk Q_k (n = gl & 3).
+__device__ __forceinline__ void contract(const float *th, const float (&Sk)[KB], float (&s)[NA]) {
 #pragma unroll
-  for (int nn = 0; nn < NR; ++nn) {
+  for (int n = 0; n < NA; ++n) {
     float t = 0.f;
 #pragma unroll
-    for (int k = 0; k < KB; ++k) t = fmaf(th[OFF_CR + nn * KB + k], Qa[k], t);
-    A.q[nn] = t;
+    for (int k = 0; k < KB; ++k) t = fmaf(th[OFF_CA + n * KB + k], Sk[k], t);
+    s[n] = t;
   }
+}
+__device__ __forceinline__ float radial_descriptor(const float *th, float Qgl, int gl) {
+  float t = 0.f;
 #pragma unroll
-  for (int nn = 0; nn < NA; ++nn) {
+  for (int k = 0; k < KB; ++k) t = fmaf(th[OFF_CR + (gl & 3) * KB + k], from_lane(Qgl, k), t);
+  return t;
+}
+// All ND values from the lanes' own radial and angular ones.
+__device__ __forceinline__ void gather_des(float r, float a, float (&v)[ND]) {
 #pragma unroll
-    for (int c = 0; c < NLM; ++c) {
-      float t = 0.f;
+  for (int n = 0; n < NR; ++n) v[n] = from_lane(r, n);
 #pragma unroll
-      for (int k = 0; k < KB; ++k) t = fmaf(th[OFF_CA + nn * KB + k], Sa[k * NLM + c], t);
-      A.s[nn][c] = t;
-    }
-    float q1 = 0.f, q2 = 0.f;
+  for (int g = 0; g < 8; ++g) v[NR + 2 * (g & 3) + (g >> 2)] = from_lane(a, g);
+}
+// sum_c x_n(c) over the components of each degree: lane gl gets (n, l) = (gl & 3, gl / 4 + 1).
+__device__ __forceinline__ float degree_sums(const float (&x)[NA], int gl) {
+  float v[8];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) q1 = fmaf(A.s[nn][c], A.s[nn][c], q1);
+  for (int n = 0; n < NA; ++n) { v[n] = gl < 3 ? x[n] : 0.f; v[4 + n] = gl < 3 ? 0.f : x[n]; }
+  return group_scatter8(v, gl);
+}
+// sum_mu w_mu W0_mu,v over all neurons (w: the own two): the own radial and angular v, not yet scaled.
+__device__ __forceinline__ void back_product(const float *th, const float (&w)[2], int gl, float &r, float &a) {
+  float vr[4], va[8];
 #pragma unroll
-    for (int c = 3; c < NLM; ++c) q2 = fmaf(A.s[nn][c], A.s[nn][c], q2);
-    A.q[NR + 2 * nn] = q1;
-    A.q[NR + 2 * nn + 1] = q2;
+  for (int v = 0; v < ND; ++v) {
+    const float t = fmaf(w[1], th[OFF_W0 + (gl + 8) * ND + v], w[0] * th[OFF_W0 + gl * ND + v]);
+    if (v < NR) vr[v < NR ? v : 0] = t;
+    else va[v < NR ? 0 : ((v - NR) & 1) * 4 + (v - NR) / 2] = t;
   }
-  float dq[ND];
+  r = group_scatter4(vr, gl);
+  a = group_scatter8(va, gl);
+}
+// One neuron's product with ND values.
+__device__ __forceinline__ float neuron(const float *th, int mu, const float (&v)[ND], float z0) {
+  float z = z0;
 #pragma unroll
-  for (int v = 0; v < ND; ++v) dq[v] = 0.f;
-  float U = -th[OFF_B1];
-#pragma unroll
-  for (int mu = 0; mu < NN; ++mu) {
-    float z = -th[OFF_B0 + mu];
-#pragma unroll
-    for (int v = 0; v < ND; ++v) z = fmaf(th[OFF_W0 + mu * ND + v], qs[v] * A.q[v], z);
-    const float h = tanhf(z);
-    A.h[mu] = h;
-    const float w1 = th[OFF_W1 + mu];
-    U = fmaf(w1, h, U);
-    const float t = w1 * (1.f - h * h);
-#pragma unroll
-    for (int v = 0; v < ND; ++v) dq[v] = fmaf(t, th[OFF_W0 + mu * ND + v], dq[v]);
-  }
-#pragma unroll
-  for (int v = 0; v < ND; ++v) A.Fp[v] = dq[v] * qs[v];
-  A.U = U;
+  for (int i = 0; i < ND; ++i) z = fmaf(th[OFF_W0 + mu * ND + i], v[i], z);
+  return z;
 }
 
-__global__ void k_st_forward(int a0, int a1, const float *__restrict__ theta, const float *__restrict__ qscale,
-                             const float *__restrict__ Q, const float *__restrict__ S, float *__restrict__ Uo,
-                             float *__restrict__ G, float *__restrict__ qout) {
+__device__ __forceinline__ void lane_net(const float *th, const float *qs, const float *__restrict__ Q,
+                                         const float *__restrict__ S, int a, int gl, LaneNet &A) {
+  const float Qgl = Q[(size_t)a * KB + gl];
+#pragma unroll
+  for (int k = 0; k < KB; ++k) A.Sk[k] = S[(size_t)a * NSB + k * NLM + gl];
+  contract(th, A.Sk, A.s);
+  A.qr = radial_descriptor(th, Qgl, gl);
+  float sq[NA];
+#pragma unroll
+  for (int n = 0; n < NA; ++n) sq[n] = A.s[n] * A.s[n];
+  A.qa = degree_sums(sq, gl);
+  gather_des(qs[gl & 3] * A.qr, qs[own_v(gl)] * A.qa, A.qt);
+  float u = 0.f;
+#pragma unroll
+  for (int m = 0; m < 2; ++m) {
+    const int mu = gl + 8 * m;
+    const float h = tanhf(neuron(th, mu, A.qt, -th[OFF_B0 + mu]));
+    A.h[m] = h;
+    A.d1h[m] = 1.f - h * h;
+    u = fmaf(th[OFF_W1 + mu], h, u);
+  }
+  A.U = group_sum(u) - th[OFF_B1];
+}
+
+__global__ void __launch_bounds__(BLOCK)
+k_st_forward(int a0, int a1, const float *__restrict__ theta, const float *__restrict__ qscale,
+             const float *__restrict__ Q, const float *__restrict__ S, float *__restrict__ Uo,
+             float *__restrict__ Gr, float *__restrict__ qout) {
   __shared__ float th[NPAR], qs[ND];
   stage_theta(th, theta, qs, qscale);
   __syncthreads();
-  const int a = a0 + blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= a1) return;
-  float Qa[KB], Sa[NSB];
+  const int gl = threadIdx.x % G;
+  const int at = a0 + (int)((blockIdx.x * BLOCK + threadIdx.x) / G);
+  const bool live = at < a1;
+  const int a = live ? at : a1 - 1;                    // lanes past the last atom repeat it and store nothing
+  LaneNet A;
+  lane_net(th, qs, Q, S, a, gl, A);
+  const float t[2] = {th[OFF_W1 + gl] * A.d1h[0], th[OFF_W1 + gl + 8] * A.d1h[1]};
+  float fr, fa;
+  back_product(th, t, gl, fr, fa);
+  fr *= qs[gl & 3];
+  fa *= qs[own_v(gl)];
+  float Fp[NA];                                        // dU/dq of (n, l(gl))
 #pragma unroll
-  for (int k = 0; k < KB; ++k) Qa[k] = Q[(size_t)a * KB + k];
+  for (int n = 0; n < NA; ++n) Fp[n] = from_lane(fa, (l_of(gl) - 1) * 4 + n);
+  if (!live) return;
+  if (gl == 0) Uo[a] = A.U;
+  float *g = Gr + (size_t)a * SS::GS;
 #pragma unroll
-  for (int c = 0; c < NSB; ++c) Sa[c] = S[(size_t)a * NSB + c];
-  AtomNet A;
-  atom_net(th, qs, Qa, Sa, A);
-  Uo[a] = A.U;
-  float *g = G + (size_t)a * SS::GS;
-#pragma unroll
-  for (int nn = 0; nn < NA; ++nn)
-#pragma unroll
-    for (int c = 0; c < NLM; ++c) g[nn * NLM + c] = 2.f * A.Fp[NR + 2 * nn + l_of(c) - 1] * A.s[nn][c];
-#pragma unroll
-  for (int t = 0; t < 8; ++t) g[NA * NLM + t] = t < NR ? A.Fp[t] : 0.f;
+  for (int n = 0; n < NA; ++n) g[n * NLM + gl] = 2.f * Fp[n] * A.s[n];
+  g[NA * NLM + gl] = gl < NR ? fr : 0.f;
   if (qout != nullptr) {
-#pragma unroll
-    for (int v = 0; v < ND; ++v) qout[(size_t)a * ND + v] = A.q[v];
+    if (gl < NR) qout[(size_t)a * ND + gl] = A.qr;
+    qout[(size_t)a * ND + own_v(gl)] = A.qa;
   }
 }
 
@@ -227,134 +342,246 @@ __global__ void k_st_energy(int s0, int s1, const int *__restrict__ start, const
 // ---------------------------------------------------------------------------------------------------
 // F_i = sum_j D_ij, D_ij = dU_i/dd_ij - dU_j/dd_ji: radial part (Fp_i + Fp_j) . g'(r) u, angular part
 // with H_nlm = G^i_nlm + (-1)^l G^j_nlm contracted with grad_d [g^A_n(r) Y_lm(d/r)].
-__global__ void k_st_force(int a0, int a1, int n, const int *__restrict__ nbr, const float4 *__restrict__ dvec,
-                           const int *__restrict__ nnum, Cut C, const float *__restrict__ theta,
-                           const float *__restrict__ G, float *__restrict__ F) {
-  __shared__ float th[NPAR];
-  stage_theta(th, theta, nullptr, nullptr);
+// Angular pairs are prepared one per lane (channel functions and direction, staged in shared memory) and evaluated
+// by the whole group, lane gl taking component gl: it keeps its four values of the own row, reads the neighbour's as
+// one coalesced 32-byte sector per channel, and forms its share of the force, which is linear in the components.
+// Y_c = m.u (l = 1) or u.M u (l = 2), so with the lane's constants K u + k = grad Y_c, and u . grad Y_c = l Y_c.
+// The kernel waits on its gathers (long scoreboard 9 of 14 cycles per issue, issue slots 31 % busy before): entries
+// are loaded a step ahead, neighbours' rows four pairs at a time.  103,000 atoms: 104 us (157 with one thread per
+// atom, 144 with whole pairs per lane, which gathered 128-byte rows from 32 places at once, 134 before the loads were
+// moved ahead); 21,000 atoms: 24 us (55).  Six resident blocks; five to eight differ by 5 %, and a loop of resident
+// blocks over the atoms measured 3 % slower.
+constexpr int ATOMS = BLOCK / G;
+
+template <bool V4>
+__global__ void __launch_bounds__(BLOCK, 6)
+k_st_force(int a0, int a1, int n, const int *__restrict__ nbr, const float4 *__restrict__ dvec,
+           const int *__restrict__ nnum, Cut C, const float *__restrict__ theta,
+           const float *__restrict__ Gr, float *__restrict__ F) {
+  constexpr int ROW = 20, GRP = G * ROW + 8;           // {g[4] | g'[4] | u, 1/r | j}; groups eight banks apart
+  __shared__ Cubics R, A;
+  __shared__ uint8_t list[ATOMS][SEG];
+  __shared__ __align__(16) float stage[ATOMS * GRP];
+  stage_cubics(theta, C, &R, &A);
   __syncthreads();
-  const int a = a0 + blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= a1) return;
-  float gi[SS::GS];
+  const int lane = threadIdx.x & 31, gl = lane % G, grp = lane / G;
+  const int at = a0 + (int)((blockIdx.x * BLOCK + threadIdx.x) / G);
+  const bool live = at < a1;
+  const int a = live ? at : a1 - 1;
+  const int cnt = live ? nnum[a] : 0;
+  const float *Ga = Gr + (size_t)a * SS::GS;
+  uint8_t *L = list[threadIdx.x / G];
+  float *sg = stage + (threadIdx.x / G) * GRP;
+  const float4 fi = load4<V4>(Ga + NA * NLM);
+  float gi[NA];
 #pragma unroll
-  for (int t = 0; t < SS::GS; ++t) gi[t] = G[(size_t)a * SS::GS + t];
+  for (int nn = 0; nn < NA; ++nn) gi[nn] = Ga[nn * NLM + gl];
+  // grad Y of the own component: (kx + xx ux + xy uy + xz uz, ...), symmetric; sgn = (-1)^l, il = 1 / l
+  const float s3 = 1.7320508075688772f;
+  const float kx = gl == 2 ? 1.f : 0.f, ky = gl == 0 ? 1.f : 0.f, kz = gl == 1 ? 1.f : 0.f;
+  const float xx = gl == 5 ? -1.f : (gl == 7 ? s3 : 0.f), yy = gl == 5 ? -1.f : (gl == 7 ? -s3 : 0.f);
+  const float zz = gl == 5 ? 2.f : 0.f, xy = gl == 3 ? s3 : 0.f, yz = gl == 4 ? s3 : 0.f, xz = gl == 6 ? s3 : 0.f;
+  const float sgn = gl < 3 ? -1.f : 1.f, il = gl < 3 ? 1.f : 0.5f;
   float fx = 0.f, fy = 0.f, fz = 0.f;
-  const int cnt = nnum[a];
-  for (int e = 0; e < cnt; ++e) {
-    const int j = nbr[(size_t)e * n + a];
-    const float4 d = dvec[(size_t)e * n + a];
-    const float *gj = G + (size_t)j * SS::GS;
-    const float r2 = d.x * d.x + d.y * d.y + d.z * d.z;
-    const float ir = rsqrtf(r2), r = r2 * ir;
-    float coef = 0.f, vx = 0.f, vy = 0.f, vz = 0.f;
-    if (r2 < C.rcR2) {
-      float f[KB], df[KB];
-      cheb_basis_d<KB>(r, C.inv_rcR, f, df);
-      float c = 0.f;
-#pragma unroll
-      for (int nn = 0; nn < NR; ++nn) {
-        float dg = 0.f;
-#pragma unroll
-        for (int k = 0; k < KB; ++k) dg = fmaf(th[OFF_CR + nn * KB + k], df[k], dg);
-        c = fmaf(gi[NA * NLM + nn] + gj[NA * NLM + nn], dg, c);
+  const int most = __reduce_max_sync(FULL, cnt);
+  const float4 none = make_float4(1e15f, 0.f, 0.f, 0.f);         // past the row: outside every cutoff
+  for (int seg = 0; seg < most; seg += SEG) {
+    int na = 0;
+    // entries one step ahead, the neighbour's radial adjoint requested before its distance is known
+    float4 d = seg + gl < cnt ? dvec[(size_t)(seg + gl) * n + a] : none;
+    int j = seg + gl < cnt ? nbr[(size_t)(seg + gl) * n + a] : a;
+    for (int it = 0; it < SEG && seg + it < most; it += G) {
+      const int e1 = seg + it + G + gl;
+      const bool more = it + G < SEG && e1 < cnt;
+      const float4 fj = load4<V4>(Gr + (size_t)j * SS::GS + NA * NLM);
+      const float4 d1 = more ? dvec[(size_t)e1 * n + a] : none;
+      const int j1 = more ? nbr[(size_t)e1 * n + a] : a;
+      const float r2 = d.x * d.x + d.y * d.y + d.z * d.z;
+      if (r2 < C.rcR2) {
+        const float ir = rsqrtf(r2), r = r2 * ir;
+        float g[NR], dg[NR];
+        radial_channels_d<SS>(R, r, g, dg);
+        const float2 c2 = fma2(add2(pr(fi.x, fi.y), pr(fj.x, fj.y)), pr(dg[0], dg[1]),
+                               mul2(add2(pr(fi.z, fi.w), pr(fj.z, fj.w)), pr(dg[2], dg[3])));
+        const float coef = hsum(c2) * ir;
+        fx = fmaf(coef, d.x, fx); fy = fmaf(coef, d.y, fy); fz = fmaf(coef, d.z, fz);
       }
-      coef = c * ir;
+      const bool ang = r2 < C.rcA2;
+      const unsigned m = (__ballot_sync(FULL, ang) >> (grp * G)) & 0xffu;
+      if (ang) L[na + __popc(m & ((1u << gl) - 1u))] = (uint8_t)(it + gl);
+      na += __popc(m);
+      d = d1; j = j1;
     }
-    if (r2 < C.rcA2) {
-      float f[KB], df[KB];
-      cheb_basis_d<KB>(r, C.inv_rcA, f, df);
-      float g[NA], dg[NA];
-#pragma unroll
-      for (int nn = 0; nn < NA; ++nn) {
-        float t = 0.f, dt = 0.f;
-#pragma unroll
-        for (int k = 0; k < KB; ++k) {
-          t = fmaf(th[OFF_CA + nn * KB + k], f[k], t);
-          dt = fmaf(th[OFF_CA + nn * KB + k], df[k], dt);
-        }
-        g[nn] = t; dg[nn] = dt;
+    __syncwarp();
+    const int chunks = __reduce_max_sync(FULL, (na + G - 1) / G);
+    for (int ch = 0; ch < chunks; ++ch) {
+      const int p = ch * G + gl;
+      // one pair per lane; a row without a pair is zero and points at the atom itself
+      float4 *mine = reinterpret_cast<float4 *>(sg + gl * ROW);
+      int jp = a;
+      if (p < na) {
+        const int e = seg + L[p];
+        const float4 dp = dvec[(size_t)e * n + a];
+        jp = nbr[(size_t)e * n + a];
+        const float r2 = dp.x * dp.x + dp.y * dp.y + dp.z * dp.z;
+        const float ir = rsqrtf(r2), r = r2 * ir;
+        float g[NA], dg[NA];
+        radial_channels_d<SS>(A, r, g, dg);
+        mine[0] = make_float4(g[0], g[1], g[2], g[3]);
+        mine[1] = make_float4(dg[0], dg[1], dg[2], dg[3]);
+        mine[2] = make_float4(dp.x * ir, dp.y * ir, dp.z * ir, ir);
+      } else {
+        mine[0] = mine[1] = mine[2] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
-      const float ux = d.x * ir, uy = d.y * ir, uz = d.z * ir;
-      float Y[NLM];
-      harmonics<NLM>(ux, uy, uz, Y);
-      float along = 0.f, bx = 0.f, by = 0.f, bz = 0.f;
+      sg[gl * ROW + 12] = __int_as_float(jp);
+      __syncwarp();
+      const int m = __reduce_max_sync(FULL, min(G, na - ch * G));
+      // four pairs at a time: sixteen loads of neighbours' rows in flight per lane
+      for (int i0 = 0; i0 < m; i0 += 4) {
 #pragma unroll
-      for (int c = 0; c < NLM; ++c) {
-        const float sgn = (l_of(c) & 1) ? -1.f : 1.f;
-        float av = 0.f, bv = 0.f;
-#pragma unroll
-        for (int nn = 0; nn < NA; ++nn) {
-          const float H = fmaf(sgn, gj[nn * NLM + c], gi[nn * NLM + c]);
-          av = fmaf(H, dg[nn], av);
-          bv = fmaf(H, g[nn], bv);
+        for (int i = i0; i < i0 + 4; ++i) {
+          const float4 *row = reinterpret_cast<const float4 *>(sg + i * ROW);
+          const float *Gj = Gr + (size_t)__float_as_int(sg[i * ROW + 12]) * SS::GS + gl;
+          const float4 g = row[0], dg = row[1], u = row[2];
+          const float h0 = fmaf(sgn, Gj[0], gi[0]), h1 = fmaf(sgn, Gj[NLM], gi[1]);
+          const float h2 = fmaf(sgn, Gj[2 * NLM], gi[2]), h3 = fmaf(sgn, Gj[3 * NLM], gi[3]);
+          const float av = fmaf(h0, dg.x, fmaf(h1, dg.y, fmaf(h2, dg.z, h3 * dg.w)));
+          const float bv = u.w * fmaf(h0, g.x, fmaf(h1, g.y, fmaf(h2, g.z, h3 * g.w)));      // B / r
+          const float gx = fmaf(xx, u.x, fmaf(xy, u.y, fmaf(xz, u.z, kx)));
+          const float gy = fmaf(xy, u.x, fmaf(yy, u.y, fmaf(yz, u.z, ky)));
+          const float gz = fmaf(xz, u.x, fmaf(yz, u.y, fmaf(zz, u.z, kz)));
+          const float ug = fmaf(u.x, gx, fmaf(u.y, gy, u.z * gz));                           // l Y
+          const float w = ug * fmaf(av, il, -bv);
+          fx = fmaf(w, u.x, fmaf(bv, gx, fx));
+          fy = fmaf(w, u.y, fmaf(bv, gy, fy));
+          fz = fmaf(w, u.z, fmaf(bv, gz, fz));
         }
-        along = fmaf(av - (float)l_of(c) * ir * bv, Y[c], along);
-        harmonic_grad_acc(c, ux, uy, uz, bv, bx, by, bz);
       }
-      coef = fmaf(along, ir, coef);
-      vx = bx * ir; vy = by * ir; vz = bz * ir;
+      __syncwarp();                                    // read before the next pairs (and lists) replace them
     }
-    fx += fmaf(coef, d.x, vx);
-    fy += fmaf(coef, d.y, vy);
-    fz += fmaf(coef, d.z, vz);
   }
-  F[3 * (size_t)a] = fx;
-  F[3 * (size_t)a + 1] = fy;
-  F[3 * (size_t)a + 2] = fz;
+  fx = group_sum(fx); fy = group_sum(fy); fz = group_sum(fz);
+  if (live && gl < 3) F[3 * (size_t)a + gl] = gl == 0 ? fx : (gl == 1 ? fy : fz);
 }
 
 // ---------------------------------------------------------------------------------------------------
 // dQ_k = sum_j f^R_k'(r) (u . w),  dS_klm = sum_j [f^A_k'(r) Y_lm (u . w) + f^A_k(r) (grad P_lm(u) . w
 // - l Y_lm (u . w)) / r],  w = v_j - v_i: the change of the basis sums when every atom moves along v.
-__global__ void k_st_jvp(int a0, int a1, int n, const int *__restrict__ nbr, const float4 *__restrict__ dvec,
-                         const int *__restrict__ nnum, Cut C, const float *__restrict__ v, float *__restrict__ dQ,
-                         float *__restrict__ dS) {
-  const int a = a0 + blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= a1) return;
+// Angular pairs are evaluated one per lane and staged in shared memory (f_k, f_k', and the two factors per
+// component); lane gl then adds them for its component.
+__global__ void __launch_bounds__(BLOCK)
+k_st_jvp(int a0, int a1, int n, const int *__restrict__ nbr, const float4 *__restrict__ dvec,
+         const int *__restrict__ nnum, Cut C, const float *__restrict__ v, float *__restrict__ dQ,
+         float *__restrict__ dS) {
+  constexpr int ROW = 4 * KB + 4, GRP = G * ROW + 8;   // 16-byte rows; groups eight banks apart
+  __shared__ uint8_t list[ATOMS][SEG];
+  __shared__ __align__(16) float stage[ATOMS * GRP];
+  const int lane = threadIdx.x & 31, gl = lane % G, grp = lane / G;
+  const int at = a0 + (int)((blockIdx.x * BLOCK + threadIdx.x) / G);
+  const bool live = at < a1;
+  const int a = live ? at : a1 - 1;
+  const int cnt = live ? nnum[a] : 0;
+  uint8_t *L = list[threadIdx.x / G];
+  float *sg = stage + (threadIdx.x / G) * GRP;
   const float vax = v[3 * (size_t)a], vay = v[3 * (size_t)a + 1], vaz = v[3 * (size_t)a + 2];
-  float q[KB], s[KB][NLM];
+  float2 q[4], s[4];
+  float qa = 0.f;                                      // the T_k-independent part of every dQ_k
 #pragma unroll
-  for (int k = 0; k < KB; ++k) {
-    q[k] = 0.f;
-#pragma unroll
-    for (int c = 0; c < NLM; ++c) s[k][c] = 0.f;
-  }
-  const int cnt = nnum[a];
-  for (int e = 0; e < cnt; ++e) {
-    const int j = nbr[(size_t)e * n + a];
-    const float4 d = dvec[(size_t)e * n + a];
-    const float wx = v[3 * (size_t)j] - vax, wy = v[3 * (size_t)j + 1] - vay, wz = v[3 * (size_t)j + 2] - vaz;
-    const float r2 = d.x * d.x + d.y * d.y + d.z * d.z;
-    const float ir = rsqrtf(r2), r = r2 * ir;
-    const float ux = d.x * ir, uy = d.y * ir, uz = d.z * ir;
-    const float uw = ux * wx + uy * wy + uz * wz;
-    if (r2 < C.rcR2) {
-      float f[KB], df[KB];
-      cheb_basis_d<KB>(r, C.inv_rcR, f, df);
-#pragma unroll
-      for (int k = 0; k < KB; ++k) q[k] = fmaf(df[k], uw, q[k]);
-    }
-    if (r2 < C.rcA2) {
-      float f[KB], df[KB], Y[NLM];
-      cheb_basis_d<KB>(r, C.inv_rcA, f, df);
-      harmonics<NLM>(ux, uy, uz, Y);
-#pragma unroll
-      for (int c = 0; c < NLM; ++c) {
-        float gx = 0.f, gy = 0.f, gz = 0.f;
-        harmonic_grad_acc(c, ux, uy, uz, 1.f, gx, gy, gz);
-        const float t1 = Y[c] * uw;
-        const float t2 = (gx * wx + gy * wy + gz * wz - (float)l_of(c) * t1) * ir;
-#pragma unroll
-        for (int k = 0; k < KB; ++k) s[k][c] = fmaf(df[k], t1, fmaf(f[k], t2, s[k][c]));
+  for (int k = 0; k < 4; ++k) { q[k] = bc2(0.f); s[k] = bc2(0.f); }
+  const int most = __reduce_max_sync(FULL, cnt);
+  for (int seg = 0; seg < most; seg += SEG) {
+    int na = 0;
+    for (int it = 0; it < SEG && seg + it < most; it += G) {
+      const int e = seg + it + gl;
+      const bool ok = e < cnt;
+      float r2 = 1e30f;
+      if (ok) {
+        const float4 d = dvec[(size_t)e * n + a];
+        r2 = d.x * d.x + d.y * d.y + d.z * d.z;
+        if (r2 < C.rcR2) {
+          const size_t j = 3 * (size_t)nbr[(size_t)e * n + a];
+          const float wx = v[j] - vax, wy = v[j + 1] - vay, wz = v[j + 2] - vaz;
+          const float ir = rsqrtf(r2), r = r2 * ir;
+          const float uw = (d.x * wx + d.y * wy + d.z * wz) * ir;
+          // f_k' = dh + T_k dh + T_k' dxh; the pairs (T_2m, T_2m+1) and their derivatives by the step-two recurrence
+          float h, dh, dxh, x, y;
+          cheb_args_d(r, C.inv_rcR, h, dh, dxh, x, y);
+          const float2 y2 = bc2(y + y), x8 = bc2(8.f * x), ta = bc2(uw * dh), tb = bc2(uw * dxh);
+          const float2 t01 = pr(1.f, x), t23 = pr(y, fmaf(y2.x, x, -x));
+          const float2 t45 = fma2(y2, t23, pr(-t01.x, -t01.y)), t67 = fma2(y2, t45, pr(-t23.x, -t23.y));
+          const float2 d01 = pr(0.f, 1.f), d23 = pr(4.f * x, fmaf(6.f, y, 3.f));
+          const float2 d45 = fma2(y2, d23, fma2(x8, t23, pr(0.f, -1.f)));
+          const float2 d67 = fma2(y2, d45, fma2(x8, t45, pr(-d23.x, -d23.y)));
+          qa += ta.x;
+          q[0] = fma2(ta, t01, fma2(tb, d01, q[0]));
+          q[1] = fma2(ta, t23, fma2(tb, d23, q[1]));
+          q[2] = fma2(ta, t45, fma2(tb, d45, q[2]));
+          q[3] = fma2(ta, t67, fma2(tb, d67, q[3]));
+        }
       }
+      const bool ang = ok && r2 < C.rcA2;
+      const unsigned m = (__ballot_sync(FULL, ang) >> (grp * G)) & 0xffu;
+      if (ang) L[na + __popc(m & ((1u << gl) - 1u))] = (uint8_t)(it + gl);
+      na += __popc(m);
+    }
+    __syncwarp();
+    const int chunks = __reduce_max_sync(FULL, (na + G - 1) / G);
+    for (int ch = 0; ch < chunks; ++ch) {
+      const int p = ch * G + gl;
+      if (p < na) {
+        const int e = seg + L[p];
+        const float4 d = dvec[(size_t)e * n + a];
+        const size_t j = 3 * (size_t)nbr[(size_t)e * n + a];
+        const float wx = v[j] - vax, wy = v[j + 1] - vay, wz = v[j + 2] - vaz;
+        const float r2 = d.x * d.x + d.y * d.y + d.z * d.z;
+        const float ir = rsqrtf(r2), r = r2 * ir;
+        const float ux = d.x * ir, uy = d.y * ir, uz = d.z * ir;
+        const float uw = ux * wx + uy * wy + uz * wz;
+        float f[KB], df[KB], Y[NLM], t1[NLM], t2[NLM];
+        cheb_basis_d<KB>(r, C.inv_rcA, f, df);
+        harmonics<NLM>(ux, uy, uz, Y);
+#pragma unroll
+        for (int c = 0; c < NLM; ++c) {
+          float gx = 0.f, gy = 0.f, gz = 0.f;
+          harmonic_grad_acc(c, ux, uy, uz, 1.f, gx, gy, gz);
+          t1[c] = Y[c] * uw;
+          t2[c] = (gx * wx + gy * wy + gz * wz - (float)(c < 3 ? 1 : 2) * t1[c]) * ir;
+        }
+        float4 *row = reinterpret_cast<float4 *>(sg + gl * ROW);
+        row[0] = make_float4(f[0], f[1], f[2], f[3]);
+        row[1] = make_float4(f[4], f[5], f[6], f[7]);
+        row[2] = make_float4(df[0], df[1], df[2], df[3]);
+        row[3] = make_float4(df[4], df[5], df[6], df[7]);
+        row[4] = make_float4(t1[0], t1[1], t1[2], t1[3]);
+        row[5] = make_float4(t1[4], t1[5], t1[6], t1[7]);
+        row[6] = make_float4(t2[0], t2[1], t2[2], t2[3]);
+        row[7] = make_float4(t2[4], t2[5], t2[6], t2[7]);
+      }
+      __syncwarp();
+      const int m = min(G, na - ch * G);               // group-uniform
+      for (int i = 0; i < m; ++i) {
+        const float4 *row = reinterpret_cast<const float4 *>(sg + i * ROW);
+        const float4 f0 = row[0], f1 = row[1], e0 = row[2], e1 = row[3];
+        const float2 t1 = bc2(sg[i * ROW + 2 * KB + gl]), t2 = bc2(sg[i * ROW + 3 * KB + gl]);
+        s[0] = fma2(pr(e0.x, e0.y), t1, fma2(pr(f0.x, f0.y), t2, s[0]));
+        s[1] = fma2(pr(e0.z, e0.w), t1, fma2(pr(f0.z, f0.w), t2, s[1]));
+        s[2] = fma2(pr(e1.x, e1.y), t1, fma2(pr(f1.x, f1.y), t2, s[2]));
+        s[3] = fma2(pr(e1.z, e1.w), t1, fma2(pr(f1.z, f1.w), t2, s[3]));
+      }
+      __syncwarp();                                    // read before the next pairs replace them
     }
   }
+  float qv[8];
 #pragma unroll
-  for (int k = 0; k < KB; ++k) dQ[(size_t)a * KB + k] = q[k];
+  for (int k = 0; k < 4; ++k) { qv[2 * k] = q[k].x + qa; qv[2 * k + 1] = q[k].y + qa; }
+  const float mine = group_scatter8(qv, gl);
+  if (!live) return;
+  dQ[(size_t)a * KB + gl] = mine;
 #pragma unroll
-  for (int k = 0; k < KB; ++k)
-#pragma unroll
-    for (int c = 0; c < NLM; ++c) dS[(size_t)a * NSB + k * NLM + c] = s[k][c];
+  for (int k = 0; k < 4; ++k) {
+    dS[(size_t)a * NSB + (2 * k) * NLM + gl] = s[k].x;
+    dS[(size_t)a * NSB + (2 * k + 1) * NLM + gl] = s[k].y;
+  }
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -369,164 +596,141 @@ __global__ void k_st_jvp(int a0, int a1, int n, const int *__restrict__ nbr, con
 //   cR_nk    : rho_n Q_k + sigma_n dQ_k,        rho = gE Fp - R (radial), sigma = -Fp (radial)
 //   cA_nk    : sum_lm kappa_nlm S_klm + lambda_nlm dS_klm,
 //              kappa = 2 (gE Fp_nl - R_nl) s_nlm - 2 Fp_nl ds_nlm,  lambda = -2 Fp_nl s_nlm.
-// Each thread builds its atom's record of these factors in shared memory; then thread t sums outputs
-// t, t + 64, ... over the block's atoms.  Block partials are summed over blocks in float64 by
-// k_st_grad_reduce in a fixed order.
-namespace rec {
-constexpr int QT = 0, U = QT + ND, AL = U + ND, BE = AL + NN, GW1 = BE + NN, GB1 = GW1 + NN, RHO = GB1 + 1,
-              SIG = RHO + NR, KAP = SIG + NR, LAM = KAP + NA * NLM, Q = LAM + NA * NLM, DQ = Q + KB, S = DQ + KB,
-              DS = S + NSB, END = DS + NSB;
-}
-static_assert(rec::END == GREC, "record layout");
+// Eight lanes hold these factors of an atom: lane gl its harmonic component of S, dS, kappa and lambda, neurons gl
+// and gl + 8, and k = gl of Q and dQ.  So every lane adds its own 65 products (32 of cA's from its component, 24 of
+// W0, 4 of cR, 2 of b0 and of w1, b1) in registers over the atoms of its group, and only the block's totals go
+// through shared memory, in a fixed order.  (Records of 289 floats per atom in shared memory, read back for every
+// product, held 6 warps per SM and took 34 us for 21,000 atoms.)  Block rows are summed by k_st_grad_reduce in
+// float64 in a fixed order.
+constexpr int GRAD_BLOCK = 256;
+constexpr int GRAD_WARPS = GRAD_BLOCK / 32;
 
 __global__ void __launch_bounds__(GRAD_BLOCK)
 k_st_grad(int a0, int a1, const float *__restrict__ theta, const float *__restrict__ qscale,
           const float4 *__restrict__ pos, const float *__restrict__ Q, const float *__restrict__ S,
           const float *__restrict__ dQ, const float *__restrict__ dS, const double *__restrict__ gE,
           float *__restrict__ part) {
-  extern __shared__ float smem[];
-  float *th = smem;                       // NPAR
-  float *qs = th + NPAR;                  // ND (padded to 16)
-  float *R = qs + 16;                     // GRAD_BLOCK records of GREC floats
+  __shared__ float th[NPAR], qs[ND];
+  __shared__ float tot[GRAD_WARPS][NPAR];
   stage_theta(th, theta, qs, qscale);
   __syncthreads();
-  const int t = threadIdx.x;
-  const int a = a0 + blockIdx.x * GRAD_BLOCK + t;
-  float *rc = R + t * GREC;
-  if (a < a1) {
-    float Qa[KB], Sa[NSB];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gl = lane % G;
+  float2 cA[NA][KB / 2], w0[2][ND / 2];
+  float cR[NR] = {0.f, 0.f, 0.f, 0.f}, b0[2] = {0.f, 0.f}, w1[2] = {0.f, 0.f}, b1 = 0.f;
 #pragma unroll
-    for (int k = 0; k < KB; ++k) Qa[k] = Q[(size_t)a * KB + k];
+  for (int i = 0; i < NA; ++i)
 #pragma unroll
-    for (int c = 0; c < NSB; ++c) Sa[c] = S[(size_t)a * NSB + c];
-    AtomNet A;
-    atom_net(th, qs, Qa, Sa, A);
-    const float ge = (float)gE[__float_as_int(pos[a].w)];
+    for (int k = 0; k < KB / 2; ++k) cA[i][k] = bc2(0.f);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int k = 0; k < ND / 2; ++k) w0[i][k] = bc2(0.f);
+  const int first = (int)((blockIdx.x * GRAD_BLOCK + threadIdx.x) / G), per_pass = (int)(gridDim.x * GRAD_BLOCK / G);
+  const int m = a1 - a0, trips = (m + per_pass - 1) / per_pass;   // grid-uniform: every lane takes part in the shuffles
+  for (int it = 0; it < trips; ++it) {
+    const int i = first + it * per_pass;
+    const bool live = i < m;
+    const int a = live ? a0 + i : a1 - 1;
+    LaneNet A;
+    lane_net(th, qs, Q, S, a, gl, A);
+    const float ge = live ? (float)gE[__float_as_int(pos[a].w)] : 0.f;
+    const float on = live ? 1.f : 0.f;                 // lanes past the last atom add zeros
     // directional derivatives of the descriptors
-    float dq[ND], ds[NA][NLM];
-    float dQa[KB];
+    float dSk[KB], ds[NA], x[NA], u[ND];
+    const float Qk = Q[(size_t)a * KB + gl], dQk = dQ[(size_t)a * KB + gl];
 #pragma unroll
-    for (int k = 0; k < KB; ++k) dQa[k] = dQ[(size_t)a * KB + k];
+    for (int k = 0; k < KB; ++k) dSk[k] = dS[(size_t)a * NSB + k * NLM + gl];
+    contract(th, dSk, ds);
 #pragma unroll
-    for (int nn = 0; nn < NR; ++nn) {
-      float tq = 0.f;
+    for (int n = 0; n < NA; ++n) x[n] = 2.f * A.s[n] * ds[n];
+    gather_des(qs[gl & 3] * radial_descriptor(th, dQk, gl), qs[own_v(gl)] * degree_sums(x, gl), u);
+    // neurons: t = w1 (1 - h^2) gives Fp; c = gE t + 2 w1 zd h (1 - h^2) gives rho = gE Fp - R and alpha
+    float t[2], c[2];
 #pragma unroll
-      for (int k = 0; k < KB; ++k) tq = fmaf(th[OFF_CR + nn * KB + k], dQa[k], tq);
-      dq[nn] = tq;
+    for (int k = 0; k < 2; ++k) {
+      const int mu = gl + 8 * k;
+      const float zd = neuron(th, mu, u, 0.f);
+      t[k] = th[OFF_W1 + mu] * A.d1h[k] * on;
+      c[k] = t[k] * (ge + 2.f * A.h[k] * zd);
+      b0[k] -= c[k];
+      w1[k] += on * (ge * A.h[k] - A.d1h[k] * zd);
+#pragma unroll
+      for (int v = 0; v < ND / 2; ++v)
+        w0[k][v] = fma2(bc2(c[k]), pr(A.qt[2 * v], A.qt[2 * v + 1]),
+                        fma2(bc2(-t[k]), pr(u[2 * v], u[2 * v + 1]), w0[k][v]));
     }
+    b1 -= ge;
+    float fr, fa, rr, ra;
+    back_product(th, t, gl, fr, fa);
+    back_product(th, c, gl, rr, ra);
+    fr *= qs[gl & 3]; rr *= qs[gl & 3];
+    fa *= qs[own_v(gl)]; ra *= qs[own_v(gl)];
 #pragma unroll
-    for (int nn = 0; nn < NA; ++nn) {
-      float d1 = 0.f, d2 = 0.f;
+    for (int n = 0; n < NR; ++n) cR[n] = fmaf(from_lane(rr, n), Qk, fmaf(-from_lane(fr, n), dQk, cR[n]));
 #pragma unroll
-      for (int c = 0; c < NLM; ++c) {
-        float tq = 0.f;
+    for (int n = 0; n < NA; ++n) {
+      const int src = (l_of(gl) - 1) * 4 + n;
+      const float Fp = from_lane(fa, src), rho = from_lane(ra, src);
+      const float kap = 2.f * rho * A.s[n] - 2.f * Fp * ds[n], lam = -2.f * Fp * A.s[n];
 #pragma unroll
-        for (int k = 0; k < KB; ++k) tq = fmaf(th[OFF_CA + nn * KB + k], dS[(size_t)a * NSB + k * NLM + c], tq);
-        ds[nn][c] = tq;
-        if (c < 3) d1 = fmaf(2.f * A.s[nn][c], tq, d1);
-        else d2 = fmaf(2.f * A.s[nn][c], tq, d2);
-      }
-      dq[NR + 2 * nn] = d1;
-      dq[NR + 2 * nn + 1] = d2;
+      for (int k = 0; k < KB / 2; ++k)
+        cA[n][k] = fma2(bc2(kap), pr(A.Sk[2 * k], A.Sk[2 * k + 1]),
+                        fma2(bc2(lam), pr(dSk[2 * k], dSk[2 * k + 1]), cA[n][k]));
     }
-    float u[ND], zd[NN];
+  }
+  // the warp's totals: over its four groups, and for cA over the eight components too
+  auto groups = [](float v) {
+    v += __shfl_xor_sync(FULL, v, 8);
+    return v + __shfl_xor_sync(FULL, v, 16);
+  };
+  float *T = tot[warp];
 #pragma unroll
-    for (int v = 0; v < ND; ++v) u[v] = qs[v] * dq[v];
+  for (int n = 0; n < NA; ++n) {
+    float v[8];
 #pragma unroll
-    for (int mu = 0; mu < NN; ++mu) {
-      float z = 0.f;
-#pragma unroll
-      for (int v = 0; v < ND; ++v) z = fmaf(th[OFF_W0 + mu * ND + v], u[v], z);
-      zd[mu] = z;
+    for (int k = 0; k < KB / 2; ++k) { v[2 * k] = cA[n][k].x; v[2 * k + 1] = cA[n][k].y; }
+    const float r = groups(group_scatter8(v, gl));     // k = gl
+    const float q = groups(cR[n]);
+    if (lane < G) {
+      T[OFF_CA + n * KB + gl] = r;
+      T[OFF_CR + n * KB + gl] = q;
     }
-    float Rq[ND];
+  }
 #pragma unroll
-    for (int v = 0; v < ND; ++v) Rq[v] = 0.f;
-#pragma unroll
-    for (int mu = 0; mu < NN; ++mu) {
-      const float h = A.h[mu], w1 = th[OFF_W1 + mu], d1h = 1.f - h * h;
-      const float cr = -2.f * w1 * zd[mu] * h * d1h;
-#pragma unroll
-      for (int v = 0; v < ND; ++v) Rq[v] = fmaf(cr, th[OFF_W0 + mu * ND + v], Rq[v]);
-      const float al = w1 * d1h * (ge + 2.f * h * zd[mu]);
-      rc[rec::AL + mu] = al;
-      rc[rec::BE + mu] = -w1 * d1h;
-      rc[rec::GW1 + mu] = ge * h - d1h * zd[mu];
-    }
+  for (int k = 0; k < 2; ++k) {
+    const int mu = gl + 8 * k;
 #pragma unroll
     for (int v = 0; v < ND; ++v) {
-      Rq[v] *= qs[v];
-      rc[rec::QT + v] = qs[v] * A.q[v];
-      rc[rec::U + v] = u[v];
+      const float r = groups(v & 1 ? w0[k][v / 2].y : w0[k][v / 2].x);
+      if (lane < G) T[OFF_W0 + mu * ND + v] = r;
     }
-    rc[rec::GB1] = -ge;
-#pragma unroll
-    for (int nn = 0; nn < NR; ++nn) {
-      rc[rec::RHO + nn] = ge * A.Fp[nn] - Rq[nn];
-      rc[rec::SIG + nn] = -A.Fp[nn];
+    const float rb = groups(b0[k]), rw = groups(w1[k]);
+    if (lane < G) {
+      T[OFF_B0 + mu] = rb;
+      T[OFF_W1 + mu] = rw;
     }
-#pragma unroll
-    for (int nn = 0; nn < NA; ++nn)
-#pragma unroll
-      for (int c = 0; c < NLM; ++c) {
-        const int v = NR + 2 * nn + l_of(c) - 1;
-        rc[rec::KAP + nn * NLM + c] = 2.f * (ge * A.Fp[v] - Rq[v]) * A.s[nn][c] - 2.f * A.Fp[v] * ds[nn][c];
-        rc[rec::LAM + nn * NLM + c] = -2.f * A.Fp[v] * A.s[nn][c];
-      }
-#pragma unroll
-    for (int k = 0; k < KB; ++k) {
-      rc[rec::Q + k] = Qa[k];
-      rc[rec::DQ + k] = dQa[k];
-    }
-#pragma unroll
-    for (int c = 0; c < NSB; ++c) {
-      rc[rec::S + c] = Sa[c];
-      rc[rec::DS + c] = dS[(size_t)a * NSB + c];
-    }
-  } else {
-    for (int c = 0; c < GREC; ++c) rc[c] = 0.f;
   }
+  b1 = groups(b1);
+  if (lane == 0) T[OFF_B1] = b1;
   __syncthreads();
-  for (int p = t; p < NPAR; p += GRAD_BLOCK) {
-    float acc = 0.f;
-    if (p < OFF_CA) {
-      const int nn = (p - OFF_CR) / KB, k = (p - OFF_CR) % KB;
-      for (int b = 0; b < GRAD_BLOCK; ++b) {
-        const float *r = R + b * GREC;
-        acc = fmaf(r[rec::RHO + nn], r[rec::Q + k], fmaf(r[rec::SIG + nn], r[rec::DQ + k], acc));
-      }
-    } else if (p < OFF_W0) {
-      const int nn = (p - OFF_CA) / KB, k = (p - OFF_CA) % KB;
-      for (int b = 0; b < GRAD_BLOCK; ++b) {
-        const float *r = R + b * GREC;
+  for (int p = threadIdx.x; p < NPAR; p += GRAD_BLOCK) {
+    float s = 0.f;
 #pragma unroll
-        for (int c = 0; c < NLM; ++c)
-          acc = fmaf(r[rec::KAP + nn * NLM + c], r[rec::S + k * NLM + c],
-                     fmaf(r[rec::LAM + nn * NLM + c], r[rec::DS + k * NLM + c], acc));
-      }
-    } else if (p < OFF_B0) {
-      const int mu = (p - OFF_W0) / ND, v = (p - OFF_W0) % ND;
-      for (int b = 0; b < GRAD_BLOCK; ++b) {
-        const float *r = R + b * GREC;
-        acc = fmaf(r[rec::AL + mu], r[rec::QT + v], fmaf(r[rec::BE + mu], r[rec::U + v], acc));
-      }
-    } else if (p < OFF_W1) {
-      for (int b = 0; b < GRAD_BLOCK; ++b) acc -= R[b * GREC + rec::AL + (p - OFF_B0)];
-    } else if (p < OFF_B1) {
-      for (int b = 0; b < GRAD_BLOCK; ++b) acc += R[b * GREC + rec::GW1 + (p - OFF_W1)];
-    } else {
-      for (int b = 0; b < GRAD_BLOCK; ++b) acc += R[b * GREC + rec::GB1];
-    }
-    part[(size_t)blockIdx.x * NPAR + p] = acc;
+    for (int w = 0; w < GRAD_WARPS; ++w) s += tot[w][p];
+    part[(size_t)blockIdx.x * NPAR + p] = s;
   }
 }
 
+// One warp per parameter: the lanes stride over the block rows in float64, then a fixed shuffle tree.  (One thread
+// per parameter took 30 us for 330 rows.)
 __global__ void k_st_grad_reduce(int nblk, const float *__restrict__ part, float *__restrict__ grad) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  const int p = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (p >= NPAR) return;
   double t = 0.0;
-  for (int b = 0; b < nblk; ++b) t += (double)part[(size_t)b * NPAR + p];
-  grad[p] = (float)t;
+  for (int b = lane; b < nblk; b += 32) t += (double)part[(size_t)b * NPAR + p];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(FULL, t, o);
+  if (lane == 0) grad[p] = (float)t;
 }
 
 __global__ void k_st_adam(int npar, float *__restrict__ theta, const float *__restrict__ grad, float *__restrict__ m,
@@ -540,8 +744,6 @@ __global__ void k_st_adam(int npar, float *__restrict__ theta, const float *__re
   v[p] = vp;
   theta[p] -= lr * (mp / c1) / (sqrtf(vp / c2) + eps);
 }
-
-constexpr size_t GRAD_SMEM = (NPAR + 16 + (size_t)GRAD_BLOCK * GREC) * sizeof(float);
 
 int blocks_of(int n, int b) { return (n + b - 1) / b; }
 
@@ -573,7 +775,7 @@ int st_basis(int a0, int a1, int n, int cap, const int *nbr, const float *dvec, 
 int st_forward(int a0, int a1, const float *theta, const float *q_scale, const float *Q, const float *S, float *U,
                float *G, float *q_out, void *stream) {
   if (a1 <= a0) return 0;
-  k_st_forward<<<blocks_of(a1 - a0, BLOCK), BLOCK, 0, (cudaStream_t)stream>>>(a0, a1, theta, q_scale, Q, S, U, G,
+  k_st_forward<<<blocks_of(a1 - a0, ATOMS), BLOCK, 0, (cudaStream_t)stream>>>(a0, a1, theta, q_scale, Q, S, U, G,
                                                                               q_out);
   return (int)cudaGetLastError();
 }
@@ -589,7 +791,9 @@ int st_force(int a0, int a1, int n, int cap, const int *nbr, const float *dvec, 
              const float *theta, const float *G, float *F, void *stream) {
   (void)cap;
   if (a1 <= a0) return 0;
-  k_st_force<<<blocks_of(a1 - a0, BLOCK), BLOCK, 0, (cudaStream_t)stream>>>(
+  // rows of 160 bytes: 16-byte loads when the array starts on a 16-byte boundary
+  auto kernel = (reinterpret_cast<uintptr_t>(G) & 15) == 0 ? k_st_force<true> : k_st_force<false>;
+  kernel<<<blocks_of(a1 - a0, ATOMS), BLOCK, 0, (cudaStream_t)stream>>>(
       a0, a1, n, nbr, reinterpret_cast<const float4 *>(dvec), nnum, cut_of(rc), theta, G, F);
   return (int)cudaGetLastError();
 }
@@ -598,13 +802,13 @@ int st_jvp(int a0, int a1, int n, int cap, const int *nbr, const float *dvec, co
            const float *v, float *dQ, float *dS, void *stream) {
   (void)cap;
   if (a1 <= a0) return 0;
-  k_st_jvp<<<blocks_of(a1 - a0, BLOCK), BLOCK, 0, (cudaStream_t)stream>>>(
+  k_st_jvp<<<blocks_of(a1 - a0, ATOMS), BLOCK, 0, (cudaStream_t)stream>>>(
       a0, a1, n, nbr, reinterpret_cast<const float4 *>(dvec), nnum, cut_of(rc), v, dQ, dS);
   return (int)cudaGetLastError();
 }
 
 int64_t st_grad_scratch(int a0, int a1) {
-  return a1 > a0 ? (int64_t)blocks_of(a1 - a0, GRAD_BLOCK) * NPAR : 0;
+  return a1 > a0 ? (int64_t)blocks_of(a1 - a0, GRAD_ATOMS) * NPAR : 0;
 }
 
 int st_grad(int a0, int a1, const float *theta, const float *q_scale, const float *pos, const float *Q,
@@ -612,19 +816,13 @@ int st_grad(int a0, int a1, const float *theta, const float *q_scale, const floa
             void *stream) {
   cudaStream_t st = (cudaStream_t)stream;
   if (a1 <= a0) return (int)cudaMemsetAsync(grad, 0, NPAR * sizeof(float), st);
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_st_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GRAD_SMEM);
-    if (e != cudaSuccess) return (int)e;
-    attr = true;
-  }
-  const int nblk = blocks_of(a1 - a0, GRAD_BLOCK);
-  k_st_grad<<<nblk, GRAD_BLOCK, GRAD_SMEM, st>>>(a0, a1, theta, q_scale, reinterpret_cast<const float4 *>(pos), Q, S,
-                                                 dQ, dS, gE, scratch);
+  // as many rows of partial sums as the scratch holds (GRAD_ATOMS atoms each, two per group), up to four blocks per SM
+  const int nblk = std::min(blocks_of(a1 - a0, GRAD_ATOMS), 152 * 4);
+  k_st_grad<<<nblk, GRAD_BLOCK, 0, st>>>(a0, a1, theta, q_scale, reinterpret_cast<const float4 *>(pos), Q, S, dQ, dS,
+                                         gE, scratch);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return (int)e;
-  k_st_grad_reduce<<<blocks_of(NPAR, BLOCK), BLOCK, 0, st>>>(nblk, scratch, grad);
+  k_st_grad_reduce<<<blocks_of(NPAR * 32, BLOCK), BLOCK, 0, st>>>(nblk, scratch, grad);
   return (int)cudaGetLastError();
 }
 

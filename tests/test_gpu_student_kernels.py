@@ -1,0 +1,72 @@
+"""The training kernels' groups of eight lanes at the edges of their ranges: cells of odd sizes (atoms past the last
+one in a warp), batches that start inside the set, rows that do not start on a 16-byte boundary, and the parameter
+gradient of a batch as the sum of its cells' gradients; and the fused loss against its plain form."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+import nep_inputs as ni
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env(trained_student_params):
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2604_24816_gb300 import build
+    build.build()
+    from paper_2604_24816_gb300 import student as st
+    rng = np.random.default_rng(3)
+    cells = [ni.student_cell(40 + k, c, 0.07, (0.02, -0.01, 0.0), k + 1) for k, c in enumerate([(4, 4, 4), (4, 4, 5), (4, 5, 4)])]
+    n = sum(p.shape[0] for p, _ in cells)
+    cs = st.CellSet(cells, E=rng.normal(0.0, 1.0, 3), F=rng.normal(0.0, 0.1, (n, 3)))
+    assert n % 4 != 0 and all(p.shape[0] % 2 for p, _ in cells[::2])
+    qs = torch.tensor(np.asarray(trained_student_params["q_scale"], np.float32), device="cuda")
+    return torch, st, cs, qs, st.pack(trained_student_params)
+
+
+def _run(env, s0, s1, wE=1.0, wF=10.0):
+    torch, st, cs, qs, th = env
+    theta = torch.tensor(th, device="cuda", requires_grad=True)
+    E, F = st.student_ef(theta, qs, cs, s0, s1)
+    loss = st.loss_fn(E, F, cs, s0, s1, wE, wF)
+    loss.backward()
+    return E.detach(), F.detach(), loss.detach(), theta.grad
+
+
+def test_batches_are_parts_of_the_set(env):
+    torch, st, cs, qs, th = env
+    E, F, _, _ = _run(env, 0, 3)
+    for s0, s1 in ((0, 1), (1, 2), (1, 3), (2, 3)):
+        e, f, _, _ = _run(env, s0, s1)
+        a0, a1 = cs.atoms(s0, s1)
+        assert torch.equal(e, E[s0:s1]) and torch.equal(f, F[a0:a1])
+
+
+def test_gradient_is_the_sum_over_cells(env):
+    """With a loss that is a sum over cells (each cell's mean weighted by its share)."""
+    torch, st, cs, qs, th = env
+    n = cs.n
+    total = _run(env, 0, 3)[3].double()
+    parts = torch.zeros_like(total)
+    for s in range(3):
+        a0, a1 = cs.atoms(s, s + 1)
+        parts += _run(env, s, s + 1, 1.0 / 3.0, 10.0 * (a1 - a0) / n)[3].double()
+    # float32 sums over some 1,000 atoms: errors add like their root at least, n at most, of 2^-24 of the terms
+    assert (total - parts).abs().max() <= 1e-4 * total.abs().max()
+
+
+def test_rows_off_a_16_byte_boundary(env):
+    torch, st, cs, qs, th = env
+    theta = torch.tensor(th, device="cuda")
+    st.student_ef(theta, qs, cs)                       # fills cs.G
+    rows = torch.zeros(cs.n * st.GS + 1, device="cuda")
+    rows[1:] = cs.G.reshape(-1)
+    F = [torch.zeros((cs.n, 3), device="cuda") for _ in range(2)]
+    for out, ptr in zip(F, (cs.G.data_ptr(), rows.data_ptr() + 4)):
+        rc = st.lib().st_force(0, cs.n, cs.n, cs.cap, st._p(cs.nbr), st._p(cs.dvec), st._p(cs.nnum), cs.rc, st._p(theta),
+                               C.c_void_p(ptr), st._p(out), st._stream())
+        assert rc == 0
+    assert torch.equal(F[0], F[1]) and F[0].abs().max() > 0
