@@ -16,6 +16,7 @@
  *                   dQ_k = sum_i v_i . dQ_k/dr_i, dS_klm likewise
  *   st_grad         dL/dtheta = sum_i [ gE_s(i) dU_i/dtheta - d(Fp_i . dq_i)/dtheta ]  (dq_i = the
  *                   directional derivative of q_i along v), reduced over atoms in a fixed order
+ *   st_loss, st_loss_grad   the training loss and its derivatives with respect to E and F
  *   st_adam         one Adam update of the parameter vector
  *
  * Parameter vector theta (float32, ST_NPAR = 289 values, in this order):
@@ -92,6 +93,19 @@ int64_t st_grad_scratch(int a0, int a1);
 int st_grad(int a0, int a1, const float *theta, const float *q_scale, const float *pos, const float *Q,
             const float *S, const float *dQ, const float *dS, const double *gE, float *scratch, float *grad,
             void *stream);
+
+/* Training loss of n_cells cells with n_comp force components (three per atom):
+ *   *loss = w_E mean_s ((E_s - E_ref_s) / natoms_s)^2 + w_F mean_k (F_k - F_ref_k)^2
+ * E, E_ref, natoms [n_cells], F, F_ref [n_comp], scratch: st_loss_scratch() doubles, loss: one double, all device
+ * memory.  Differences of forces in float32, everything else in float64; the sums run in a fixed order.
+ * n_cells and n_comp must be positive. */
+int64_t st_loss_scratch(void);
+int st_loss(int n_cells, int n_comp, const double *E, const double *E_ref, const double *natoms, const float *F,
+            const float *F_ref, double w_E, double w_F, double *scratch, double *loss, void *stream);
+
+/* *g times the derivatives of that loss: gE [n_cells] and gF [n_comp] (g: one double, device memory). */
+int st_loss_grad(int n_cells, int n_comp, const double *E, const double *E_ref, const double *natoms, const float *F,
+                 const float *F_ref, double w_E, double w_F, const double *g, double *gE, float *gF, void *stream);
 
 /* One Adam step on theta [npar] with moment buffers m, v (float32), step count t >= 1. */
 int st_adam(int npar, float *theta, const float *grad, float *m, float *v, float lr, float beta1, float beta2,

@@ -733,6 +733,53 @@ __global__ void k_st_grad_reduce(int nblk, const float *__restrict__ part, float
   if (lane == 0) grad[p] = (float)t;
 }
 
+// Loss w_E mean_s ((E_s - E*_s) / n_s)^2 + w_F mean (F - F*)^2 over force components: block sums in float64 (weights
+// and means applied), then one block adds them.  Differences of forces in float32, squares and sums in float64.
+constexpr int LOSS_BLOCK = 256, LOSS_BLOCKS = 128;
+template <int NT>
+__device__ __forceinline__ double block_sum(double v) {
+  __shared__ double w[NT / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
+  if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int k = 0; k < NT / 32; ++k) t += w[k];
+  return t;
+}
+__global__ void __launch_bounds__(LOSS_BLOCK)
+k_st_loss(int nc, int nf, const double *__restrict__ E, const double *__restrict__ Er, const double *__restrict__ na,
+          const float *__restrict__ F, const float *__restrict__ Fr, double wE, double wF, double *__restrict__ part) {
+  const int t = blockIdx.x * LOSS_BLOCK + threadIdx.x, stride = gridDim.x * LOSS_BLOCK;
+  double e = 0.0, f = 0.0;
+  for (int s = t; s < nc; s += stride) {
+    const double d = (E[s] - Er[s]) / na[s];
+    e = fma(d, d, e);
+  }
+  for (int k = t; k < nf; k += stride) {
+    const double d = (double)(F[k] - Fr[k]);
+    f = fma(d, d, f);
+  }
+  const double v = block_sum<LOSS_BLOCK>(e * (wE / nc) + f * (wF / nf));
+  if (threadIdx.x == 0) part[blockIdx.x] = v;
+}
+__global__ void __launch_bounds__(LOSS_BLOCKS)
+k_st_loss_sum(int nb, const double *__restrict__ part, double *__restrict__ loss) {
+  const double v = block_sum<LOSS_BLOCKS>((int)threadIdx.x < nb ? part[threadIdx.x] : 0.0);
+  if (threadIdx.x == 0) *loss = v;
+}
+// Its gradients times the upstream derivative *g.
+__global__ void __launch_bounds__(LOSS_BLOCK)
+k_st_loss_grad(int nc, int nf, const double *__restrict__ E, const double *__restrict__ Er,
+               const double *__restrict__ na, const float *__restrict__ F, const float *__restrict__ Fr, double wE,
+               double wF, const double *__restrict__ g, double *__restrict__ gE, float *__restrict__ gF) {
+  const int t = blockIdx.x * LOSS_BLOCK + threadIdx.x, stride = gridDim.x * LOSS_BLOCK;
+  const double up = *g, ce = 2.0 * up * wE / nc, cf = 2.0 * up * wF / nf;
+  for (int s = t; s < nc; s += stride) gE[s] = ce * ((E[s] - Er[s]) / na[s]) / na[s];
+  for (int k = t; k < nf; k += stride) gF[k] = (float)(cf * (double)(F[k] - Fr[k]));
+}
+
 __global__ void k_st_adam(int npar, float *__restrict__ theta, const float *__restrict__ grad, float *__restrict__ m,
                           float *__restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -823,6 +870,26 @@ int st_grad(int a0, int a1, const float *theta, const float *q_scale, const floa
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return (int)e;
   k_st_grad_reduce<<<blocks_of(NPAR * 32, BLOCK), BLOCK, 0, st>>>(nblk, scratch, grad);
+  return (int)cudaGetLastError();
+}
+
+int64_t st_loss_scratch(void) { return LOSS_BLOCKS; }
+
+int st_loss(int n_cells, int n_comp, const double *E, const double *E_ref, const double *natoms, const float *F,
+            const float *F_ref, double w_E, double w_F, double *scratch, double *loss, void *stream) {
+  if (n_cells <= 0 || n_comp <= 0) return (int)cudaErrorInvalidValue;
+  cudaStream_t st = (cudaStream_t)stream;
+  const int nb = std::min(LOSS_BLOCKS, blocks_of(std::max(n_cells, n_comp), LOSS_BLOCK));
+  k_st_loss<<<nb, LOSS_BLOCK, 0, st>>>(n_cells, n_comp, E, E_ref, natoms, F, F_ref, w_E, w_F, scratch);
+  k_st_loss_sum<<<1, LOSS_BLOCKS, 0, st>>>(nb, scratch, loss);
+  return (int)cudaGetLastError();
+}
+
+int st_loss_grad(int n_cells, int n_comp, const double *E, const double *E_ref, const double *natoms, const float *F,
+                 const float *F_ref, double w_E, double w_F, const double *g, double *gE, float *gF, void *stream) {
+  if (n_cells <= 0 || n_comp <= 0) return (int)cudaErrorInvalidValue;
+  k_st_loss_grad<<<std::min(152 * 8, blocks_of(std::max(n_cells, n_comp), LOSS_BLOCK)), LOSS_BLOCK, 0,
+                   (cudaStream_t)stream>>>(n_cells, n_comp, E, E_ref, natoms, F, F_ref, w_E, w_F, g, gE, gF);
   return (int)cudaGetLastError();
 }
 

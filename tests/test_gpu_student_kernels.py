@@ -27,11 +27,11 @@ def env(trained_student_params):
     return torch, st, cs, qs, st.pack(trained_student_params)
 
 
-def _run(env, s0, s1, wE=1.0, wF=10.0):
+def _run(env, s0, s1, wE=1.0, wF=10.0, plain=False):
     torch, st, cs, qs, th = env
     theta = torch.tensor(th, device="cuda", requires_grad=True)
     E, F = st.student_ef(theta, qs, cs, s0, s1)
-    loss = st.loss_fn(E, F, cs, s0, s1, wE, wF)
+    loss = (st._loss_plain if plain else st.loss_fn)(E, F, cs, s0, s1, wE, wF)
     loss.backward()
     return E.detach(), F.detach(), loss.detach(), theta.grad
 
@@ -70,3 +70,34 @@ def test_rows_off_a_16_byte_boundary(env):
                                C.c_void_p(ptr), st._p(out), st._stream())
         assert rc == 0
     assert torch.equal(F[0], F[1]) and F[0].abs().max() > 0
+
+
+@pytest.mark.parametrize("s0,s1", [(0, 3), (1, 2), (1, 3)])
+def test_loss_matches_its_plain_form(env, s0, s1):
+    torch, st, cs, qs, th = env
+    fused, plain = _run(env, s0, s1), _run(env, s0, s1, plain=True)
+    assert abs(float(fused[2] - plain[2])) <= 1e-13 * abs(float(plain[2]))    # float64 sums in another order
+    assert (fused[3] - plain[3]).abs().max() <= 1e-6 * plain[3].abs().max()   # one float32 rounding of each dL/dF
+
+
+def test_loss_keeps_what_autograd_could_do(env):
+    """A second derivative, other strides, and a call under forward mode give what the plain form gives."""
+    torch, st, cs, qs, th = env
+    a0, a1 = cs.atoms(1, 3)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    E = torch.randn(2, generator=g, device="cuda", dtype=torch.float64, requires_grad=True)
+    F = torch.randn((a1 - a0, 3), generator=g, device="cuda", requires_grad=True)
+
+    def second(loss):
+        gE, gF = torch.autograd.grad(loss(E, F, cs, 1, 3), (E, F), create_graph=True)
+        return torch.autograd.grad((gE * gE).sum() + (gF * gF).sum().double(), (E, F))
+
+    for a, b in zip(second(st.loss_fn), second(st._loss_plain)):
+        assert torch.allclose(a, b, rtol=1e-5)
+    strided = F.detach().t().contiguous().t()
+    assert torch.allclose(st.loss_fn(E, strided, cs, 1, 3), st._loss_plain(E, strided, cs, 1, 3), rtol=1e-12)
+    import torch.autograd.forward_ad as fwad
+    with fwad.dual_level():
+        dual = fwad.make_dual(F.detach(), torch.ones_like(F))
+        t = [fwad.unpack_dual(f(E.detach(), dual, cs, 1, 3)).tangent for f in (st.loss_fn, st._loss_plain)]
+    assert torch.allclose(t[0], t[1], rtol=1e-6)
