@@ -83,6 +83,7 @@ cudaError_t launch_cell_sort(const RebuildArgs &, int, cudaStream_t);
 bool cell_sort_decides(int n, int ncell);
 cudaError_t launch_neighbors(const RebuildArgs &, cudaStream_t);
 int scan_tiles(int ncell);
+int slice_shift(int n, int64_t ncell);
 int cell_sort_launches(int n, int ncell);
 // nep_md.cu
 cudaError_t launch_kick_drift(int, double *, double *, double *, double *, double *, double *, long long *, float4 *,
@@ -168,7 +169,7 @@ struct nep_handle {
   int n = 0;
   double L[3] = {0, 0, 0}, l[3] = {0, 0, 0};
   int nc[3] = {0, 0, 0};
-  int ncell = 0;
+  int ncell = 0, ssh = 0;   // slices of cells along x (2^ssh per cell)
   bool have_state = false, have_nlist = false, have_forces = false;
   bool recheck = false;   // an upload kept the list: check the displacements before the next evaluation
 
@@ -374,7 +375,7 @@ cudaError_t reset_report(nep_handle *h) {
 
 RebuildArgs rebuild_args(nep_handle *h) {
   RebuildArgs a;
-  a.n = h->n; a.ncell = h->ncell;
+  a.n = h->n; a.ncell = h->ncell; a.ssh = h->ssh;
   for (int d = 0; d < 3; ++d) { a.L[d] = h->L[d]; a.l[d] = h->l[d]; a.nc[d] = h->nc[d]; }
   a.x = h->x; a.y = h->y; a.z = h->z; a.vx = h->vx; a.vy = h->vy; a.vz = h->vz;
   a.xb = h->xb; a.yb = h->yb; a.zb = h->zb; a.vxb = h->vxb; a.vyb = h->vyb; a.vzb = h->vzb;
@@ -920,7 +921,8 @@ nep_status nep_set_state(nep_handle *h, int64_t n, const double *x, const double
     ncell *= nc;
   }
   if (ncell > (int64_t)1 << 30) return fail(h, NEP_ERR_ARG, "too many cells");
-  h->ncell = (int)ncell;
+  h->ssh = slice_shift(h->n, ncell);
+  h->ncell = (int)(ncell << h->ssh);
   h->wide = wide_lanes(h->n);
   const size_t N = (size_t)std::max(h->n, 1);
   cudaError_t e = cudaSuccess;

@@ -61,7 +61,8 @@ struct Control {
 
 // Arguments of the rebuild chain (cell sort + neighbour list).
 struct RebuildArgs {
-  int n, ncell;
+  int n, ncell;               // ncell: slices of cells (see slice_shift in nep_neighbor.cu)
+  int ssh;
   double L[3], l[3];
   int nc[3];
   double *x, *y, *z, *vx, *vy, *vz, *xb, *yb, *zb, *vxb, *vyb, *vzb;

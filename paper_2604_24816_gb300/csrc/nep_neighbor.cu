@@ -25,10 +25,12 @@
 
 namespace nep {
 
-// Box edges, cell edges and their reciprocals, cells per dimension (float64 side of the cell sort).
+// Box edges, cell edges, cells per dimension (float64 side of the cell sort), and the reciprocal edges that index
+// them.  The sort divides each cell into 2^ssh slices along x: a slice row (fixed y and z) is contiguous, so that
+// the neighbour scan reads only the slices that its atom can reach.  ilx: slices per Angstrom.
 struct CellGrid {
   double Lx, Ly, Lz, lx, ly, lz, ilx, ily, ilz;
-  int ncx, ncy, ncz;
+  int ncx, ncy, ncz, ssh;
 };
 
 constexpr int SCAN_THREADS = 1024;
@@ -52,6 +54,7 @@ __device__ __forceinline__ double wrap_coord(double x, double L) {
 struct CellOf {
   double x, y, z;
   int cx, cy, cz;
+  int slice;             // index of its slice of cell in the sorted order
 };
 __device__ __forceinline__ CellOf cell_of_atom(double px, double py, double pz, const CellGrid &g, int *status) {
   if (!(isfinite(px) && isfinite(py) && isfinite(pz))) {
@@ -60,9 +63,11 @@ __device__ __forceinline__ CellOf cell_of_atom(double px, double py, double pz, 
   }
   CellOf c;
   c.x = wrap_coord(px, g.Lx); c.y = wrap_coord(py, g.Ly); c.z = wrap_coord(pz, g.Lz);
-  c.cx = min((int)(c.x * g.ilx), g.ncx - 1);
+  const int sx = min((int)(c.x * g.ilx), (g.ncx << g.ssh) - 1);
+  c.cx = sx >> g.ssh;
   c.cy = min((int)(c.y * g.ily), g.ncy - 1);
   c.cz = min((int)(c.z * g.ilz), g.ncz - 1);
+  c.slice = (c.cz * g.ncy + c.cy) * (g.ncx << g.ssh) + sx;
   return c;
 }
 // Cell-relative float32 coordinates: the same expression as the drift and upload kernels (nep_md.cu), so
@@ -82,9 +87,8 @@ __global__ void k_cell_assign(int n, double *__restrict__ x, double *__restrict_
     if (a.x != px || a.y != py || a.z != pz) {          // also true for NaN: the wrapped position replaces it
       x[s] = a.x; y[s] = a.y; z[s] = a.z;
     }
-    const int c = (a.cz * g.ncy + a.cy) * g.ncx + a.cx;
-    cell_of[s] = c;
-    atomicAdd(count + c, 1);
+    cell_of[s] = a.slice;
+    atomicAdd(count + a.slice, 1);
   }
 }
 
@@ -207,7 +211,8 @@ __global__ void k_permute(int n, const int2 *__restrict__ perm, const int *__res
     xb[t] = px; yb[t] = py; zb[t] = pz;
     vxb[t] = vx[s]; vyb[t] = vy[s]; vzb[t] = vz[s];
     idb[t] = sp.y;
-    const int cx = c % g.ncx, cy = (c / g.ncx) % g.ncy, cz = c / (g.ncx * g.ncy);
+    const int nsx = g.ncx << g.ssh;
+    const int cx = (c % nsx) >> g.ssh, cy = (c / nsx) % g.ncy, cz = c / (nsx * g.ncy);
     const float4 p = cell_relative(px, py, pz, cx, cy, cz, g);
     pos[t] = p;
     pos_ref[t] = p;
@@ -265,7 +270,7 @@ k_rebuild_small(int n, int ncell, double *__restrict__ x, double *__restrict__ y
       a[k] = cell_of_atom(x[s], y[s], z[s], g, &ctrl->status);
       u[k][0] = vx[s]; u[k][1] = vy[s]; u[k][2] = vz[s];
       oid[k] = id[s];
-      cell[k] = (a[k].cz * g.ncy + a[k].cy) * g.ncx + a[k].cx;
+      cell[k] = a[k].slice;
       atomicAdd(&cnt[cell[k]], 1);
     }
   }
@@ -337,7 +342,7 @@ k_rebuild_cluster(int n, int ncell, double *__restrict__ x, double *__restrict__
       a[k] = cell_of_atom(x[s], y[s], z[s], g, &ctrl->status);
       u[k][0] = vx[s]; u[k][1] = vy[s]; u[k][2] = vz[s];
       oid[k] = id[s];
-      cell[k] = (a[k].cz * g.ncy + a[k].cy) * g.ncx + a[k].cx;
+      cell[k] = a[k].slice;
       ord[k] = atomicAdd(count + cell[k], 1);
     }
   }
@@ -398,6 +403,8 @@ k_rebuild_cluster(int n, int ncell, double *__restrict__ x, double *__restrict__
 // The placement's 4-byte stores into the neighbour-major list are scattered across rows; L2 merges
 // them into full sectors before they reach DRAM.
 constexpr int NB_WARPS = 8;            // atoms (one warp each) per block
+constexpr int NB_TAKE_MIN = 262144;    // atoms from which a block takes four groups of NB_WARPS atoms at a time: fewer
+                                       // barriers (1,339 -> 1,299 us at 1,048,576), but too coarse for small systems (16,384: 30 -> 47)
 constexpr int NB_STAGE = 128;          // staged entries per atom (lists longer than this are an overflow)
 constexpr float OWN_EPS = 0.5f;        // Angstrom; lattice-vector components are either ~0 or >= a/2
 
@@ -439,9 +446,9 @@ __device__ __forceinline__ int segment_counts(int key, int lane, unsigned fsh) {
 
 // The candidate scan and segment placement of atom i by one warp (see k_neighbors).
 __device__ __forceinline__ void neighbors_of_atom(int i, int n, const float4 *__restrict__ pos,
-                                                  const int *__restrict__ cell_start, const Geom &geom,
-                                                  const Bands &B, int limit, float4 *stage,
-                                                  uint8_t *skey, int lane, int32_t *__restrict__ nbr,
+                                                  const int *__restrict__ cell_start, const Geom &geom, int ssh,
+                                                  float slices, const Bands &B, int limit, float4 *stage, float4 *tab,
+                                                  int lane, int32_t *__restrict__ nbr,
                                                   int32_t *__restrict__ nnum, int32_t *__restrict__ nang,
                                                   int32_t *__restrict__ nown, int32_t *__restrict__ nband0,
                                                   int32_t *__restrict__ nfar, Control *ctrl) {
@@ -451,11 +458,10 @@ __device__ __forceinline__ void neighbors_of_atom(int i, int n, const float4 *__
   const bool xwrap = cx == 0 || cx == geom.ncx - 1;
   int acc = 0;                                         // accepted so far (warp-uniform)
   // The candidate ranges in stencil order (dz, dy, then the x part), set up one per lane L = 9 (dz + 1)
-  // + 3 (dy + 1) + part: a row of three cells that does not wrap around x is one range (part 0; its
-  // left or right cell left out when atom i lies farther from its own cell's face than the reach left
-  // after the row's (y, z) gap: every candidate there is at least that far away in x), a row that
-  // wraps is three; rows whose (y, z) slab lies beyond the list radius are empty.  The 1e-4 margin
-  // keeps every candidate a float32 distance test could accept, so the lists are unchanged.
+  // + 3 (dy + 1) + part: a row of three cells that does not wrap around x is one range (part 0), a row that wraps is
+  // three; rows whose (y, z) slab lies beyond the list radius are empty.  A range holds the x slices within the reach
+  // left after the row's (y, z) gap: every candidate outside is at least that far away in x.  The 1e-4 margin
+  // (0.0036 Angstrom^2) keeps every candidate a float32 distance test could accept, so the lists are unchanged.
   int rb = 0, rlen = 0;
   float roy = 0.f, roz = 0.f;
   int rcode = 0;                                       // shift-table base (dy, dz) | x part << 8
@@ -468,86 +474,102 @@ __device__ __forceinline__ void neighbors_of_atom(int i, int n, const float4 *__
     zz += zz < 0 ? geom.ncz : (zz >= geom.ncz ? -geom.ncz : 0);
     int yy = cy + dy;
     yy += yy < 0 ? geom.ncy : (yy >= geom.ncy ? -geom.ncy : 0);
-    const int row = (zz * geom.ncy + yy) * geom.ncx;
+    const int sub = 1 << ssh, row = (zz * geom.ncy + yy) * (geom.ncx << ssh);
     const float gy = dy < 0 ? pi.y : (dy > 0 ? geom.ly - pi.y : 0.f);
     const float gz = dz < 0 ? pi.z : (dz > 0 ? geom.lz - pi.z : 0.f);
     const float reach2 = B.b4 * 1.0001f - (gy * gy + gz * gz);
     if (reach2 >= 0.f) {
-      const bool need_l = pi.x * pi.x <= reach2, need_r = (geom.lx - pi.x) * (geom.lx - pi.x) <= reach2;
-      if (!xwrap) {
-        if (part == 0) {
-          rb = cell_start[row + cx - (need_l ? 1 : 0)];
-          rlen = cell_start[row + cx + (need_r ? 2 : 1)] - rb;
-        }
-      } else if (!((part == 0 && !need_l) || (part == 2 && !need_r))) {
-        int xx = cx + part - 1;
-        xx += xx < 0 ? geom.ncx : (xx >= geom.ncx ? -geom.ncx : 0);
-        rb = cell_start[row + xx];
-        rlen = cell_start[row + xx + 1] - rb;
+      // slices from this cell's first: s0..s1 within the three cells
+      const float reach = sqrtf(reach2);
+      int s0 = max(__float2int_rd((pi.x - reach) * slices), -sub), s1 = min(__float2int_rd((pi.x + reach) * slices), 2 * sub - 1);
+      int at = cx;                                     // the cell that s0 is counted from
+      if (xwrap) {
+        const int o = (part - 1) * sub;
+        s0 = max(s0, o) - o;
+        s1 = min(s1, o + sub - 1) - o;
+        at = cx + part - 1;
+        at += at < 0 ? geom.ncx : (at >= geom.ncx ? -geom.ncx : 0);
+      }
+      if ((xwrap || part == 0) && s1 >= s0) {
+        rb = cell_start[row + at * sub + s0];
+        rlen = cell_start[row + at * sub + s1 + 1] - rb;
       }
     }
   }
-  // the non-empty ranges, walked in order (every lane takes part in each shuffle); each candidate is
-  // tested on every lane without a branch (the load index clamped into the range), and an accepted
-  // pair's displacement and entry go to the stage as one 16-byte record in candidate order
-  unsigned ne = __ballot_sync(0xffffffffu, rlen > 0);
-  while (ne != 0u) {
-    const int L = __ffs(ne) - 1;                       // warp-uniform
-    ne &= ne - 1u;
-    const int b = __shfl_sync(0xffffffffu, rb, L), e = b + __shfl_sync(0xffffffffu, rlen, L);
-    const float oz = __shfl_sync(0xffffffffu, roz, L), oy = __shfl_sync(0xffffffffu, roy, L);
-    const int code = __shfl_sync(0xffffffffu, rcode, L);
-    const int shb = code & 255, part = code >> 8;
-    for (int j0 = b; j0 < e; j0 += 32) {
-      const int j = j0 + lane;
-      const bool inr = j < e;
-      const float4 pj = pos[inr ? j : e - 1];          // j0 < e: always inside the range
-      const int dx = xwrap ? part - 1 : cell_x(pj.w) - cx;
-      const float ox = (float)dx * geom.lx;            // exact: dx is -1, 0 or 1
-      const float ddx = pj.x - pi.x + ox, ddy = pj.y - pi.y + oy, ddz = pj.z - pi.z + oz;
-      const bool ok = inr && j != i && nb_r2(ddx, ddy, ddz) < B.b4;
-      const uint32_t ent = (uint32_t)j | ((uint32_t)((dx + 1) + shb) << J_BITS);
-      const unsigned m = __ballot_sync(0xffffffffu, ok);
-      const int slot = acc + __popc(m & lower);
-      if (ok && slot < NB_STAGE) stage[slot] = make_float4(ddx, ddy, ddz, __uint_as_float(ent));
-      acc += __popc(m);
-    }
+  // The non-empty ranges form one sequence, walked 32 candidates at a time (8.4 turns per atom of an fcc crystal; range
+  // by range it takes 13.2, half of the ranges needing a second, mostly empty one).  A lane finds its range as the
+  // number of range starts up to its place: one bit per start inside the turn, combined over the warp.  Each candidate
+  // is tested without a branch (the load index clamped), and an accepted pair's displacement and entry go to the
+  // stage as one 16-byte record in candidate order.
+  int incl = rlen;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += t;
+  }
+  const int total = __shfl_sync(0xffffffffu, incl, 31), first = incl - rlen;
+  const unsigned ne = __ballot_sync(0xffffffffu, rlen > 0);
+  if (rlen > 0) tab[__popc(ne & lower)] = make_float4(__int_as_float(rb - first), roy, roz, __int_as_float(rcode));
+  __syncwarp();
+  const unsigned upto = lower | (1u << lane);
+  int started = 0;                                     // ranges that began before this turn (warp-uniform)
+  for (int c0 = 0; c0 < total; c0 += 32) {
+    const unsigned rel = (unsigned)(first - c0);
+    const unsigned starts = __reduce_or_sync(0xffffffffu, rlen > 0 && rel < 32u ? 1u << rel : 0u);
+    const float4 t = tab[started + __popc(starts & upto) - 1];
+    started += __popc(starts);
+    const bool inr = c0 + lane < total;
+    const int j = __float_as_int(t.x) + c0 + lane;     // past the end of the last range when !inr
+    const int code = __float_as_int(t.w);
+    const float4 pj = pos[inr ? j : i];
+    const int dx = xwrap ? (code >> 8) - 1 : cell_x(pj.w) - cx;
+    const float ox = (float)dx * geom.lx;              // exact: dx is -1, 0 or 1
+    const float ddx = pj.x - pi.x + ox, ddy = pj.y - pi.y + t.y, ddz = pj.z - pi.z + t.z;
+    const bool ok = inr && j != i && nb_r2(ddx, ddy, ddz) < B.b4;
+    const uint32_t ent = (uint32_t)j | ((uint32_t)((dx + 1) + (code & 255)) << J_BITS);
+    const unsigned m = __ballot_sync(0xffffffffu, ok);
+    const int slot = acc + __popc(m & lower);
+    if (ok && slot < NB_STAGE) stage[slot] = make_float4(ddx, ddy, ddz, __uint_as_float(ent));
+    acc += __popc(m);
   }
   __syncwarp();
   // Segments of the staged entries (classified here, 32 accepted pairs at a time, rather than in the
-  // sparse candidate loop; the same float32 arithmetic as the acceptance test), their sizes and offsets,
-  // then placement in candidate order within each segment.  Lane g < NB_SEG keeps segment g's count
-  // and running offset; a chunk of 32 staged entries is counted with two warp reductions of one-hot
-  // 6-bit fields (segments 0..4 and 5..9: at most 32 per field, no carries).
+  // sparse candidate loop; the same float32 arithmetic as the acceptance test): each entry's rank among the
+  // turn's entries of its segment, and per lane g < NB_SEG the segment's count (two warp reductions of one-hot
+  // 6-bit fields, segments 0..4 and 5..9: at most 32 per field, no carries) before and after the turn.  Then the
+  // segments' offsets, and placement in candidate order within each segment.
+  constexpr int TURNS = NB_STAGE / 32;
   const int ms = min(acc, NB_STAGE);
   const unsigned fsh = 6u * (unsigned)(lane % 5);
   int mycnt = 0;
-  for (int s0 = 0; s0 < ms; s0 += 32) {
+  int keyrank[TURNS], before[TURNS];
+#pragma unroll
+  for (int t = 0; t < TURNS; ++t) {
+    keyrank[t] = NB_SEG;
+    before[t] = 0;
+    if (32 * t >= ms) continue;                        // warp-uniform
     int key = NB_SEG;
-    if (s0 + lane < ms) {
-      const float4 sd = stage[s0 + lane];
+    if (32 * t + lane < ms) {
+      const float4 sd = stage[32 * t + lane];
       key = segment_of(sd.x, sd.y, sd.z, nb_r2(sd.x, sd.y, sd.z), B);
-      skey[s0 + lane] = (uint8_t)key;
     }
+    keyrank[t] = key | (__popc(__match_any_sync(0xffffffffu, key) & lower) << 8);
+    before[t] = mycnt;
     mycnt += segment_counts(key, lane, fsh);
   }
-  __syncwarp();
   if (lane >= NB_SEG) mycnt = 0;
-  int incl = mycnt;                                    // inclusive prefix over lanes 0..NB_SEG-1
+  incl = mycnt;                                        // inclusive prefix over lanes 0..NB_SEG-1
 #pragma unroll
   for (int d = 1; d < 16; d <<= 1) {
     const int t = __shfl_up_sync(0xffffffffu, incl, d);
     if (lane >= d) incl += t;
   }
-  int myrun = incl - mycnt;                            // next slot of segment `lane`
-  for (int s0 = 0; s0 < ms; s0 += 32) {
-    const bool valid = s0 + lane < ms;
-    const int key = valid ? (int)skey[s0 + lane] : NB_SEG;
-    const uint32_t ent = valid ? __float_as_uint(stage[s0 + lane].w) : 0u;
-    const unsigned grp = __match_any_sync(0xffffffffu, key);
-    const int k = __shfl_sync(0xffffffffu, myrun, key) + __popc(grp & lower);
-    if (valid && k < limit) nbr[(size_t)k * n + i] = (int32_t)ent;
-    myrun += segment_counts(key, lane, fsh);
+#pragma unroll
+  for (int t = 0; t < TURNS; ++t) {
+    if (32 * t >= ms) continue;
+    const int k = __shfl_sync(0xffffffffu, incl - mycnt + before[t], keyrank[t] & 255) + (keyrank[t] >> 8);
+    if (32 * t + lane < ms && k < limit)
+      nbr[(size_t)k * n + i] = (int32_t)__float_as_uint(stage[32 * t + lane].w);
   }
   const int c0 = __shfl_sync(0xffffffffu, mycnt, 0), c1 = __shfl_sync(0xffffffffu, mycnt, 1);
   const int c4 = __shfl_sync(0xffffffffu, mycnt, 4), c5 = __shfl_sync(0xffffffffu, mycnt, 5);
@@ -567,24 +589,28 @@ __device__ __forceinline__ void neighbors_of_atom(int i, int n, const float4 *__
 }
 
 // One warp per atom i.  The lanes test 32 candidates at a time (coalesced position loads, the atom's
-// own position broadcast): for each of the 9 (dy, dz) rows of the 27-cell stencil the three cells
-// x-1, x, x+1 are consecutive in the cell-sorted arrays, so the row is one contiguous range and a
+// own position broadcast): for each of the 9 (dy, dz) rows of the 27-cell stencil the x slices within reach
+// are consecutive in the sorted arrays, so the row is one contiguous range and a
 // candidate's x offset comes from its packed cell coordinate (rows that wrap around the periodic x
-// boundary are walked cell by cell; the bounds of all ranges are read up front, one lane each).
-// Accepted entries go to a per-warp shared-memory stage in
+// boundary are walked cell by cell; the bounds of all ranges are read up front, one lane each), and the ranges are
+// walked as one sequence.  Accepted entries go to a per-warp shared-memory stage in
 // candidate order (ballot + popc), then are placed by segment: [owned | not owned] x band, candidate
 // order inside a segment -- the same row as the thread-per-atom formulation, with 32-wide work
-// instead of divergent per-thread cell loops.
+// instead of divergent per-thread cell loops.  The kernel is bound by issue slots (85 % busy), so what counts is the
+// number of turns and what each costs.  1,048,576 atoms: 1,608 us per build over whole cells, range by range; 1,500
+// with four x slices per cell (269 candidates per atom instead of 385; eight slices 2 % less again, for twice the
+// cells); 1,353 with the ranges as one sequence; 1,331 with segment ranks kept in registers between counting and
+// placement; 1,299 with four groups per take.  Two candidates per lane and turn in float2 pairs: no gain.
 __global__ void __launch_bounds__(NB_WARPS * 32, 6)   // 40 registers at most: 6 resident blocks
-k_neighbors(int n, const float4 *__restrict__ pos, const int *__restrict__ cell_start, const Geom geom, int cap,
-            Bands B, int32_t *__restrict__ nbr, int32_t *__restrict__ nnum, int32_t *__restrict__ nang,
+k_neighbors(int n, const float4 *__restrict__ pos, const int *__restrict__ cell_start, const Geom geom, int ssh,
+            float slices, int take, int cap, Bands B, int32_t *__restrict__ nbr, int32_t *__restrict__ nnum, int32_t *__restrict__ nang,
             int32_t *__restrict__ nown, int32_t *__restrict__ nband0, int32_t *__restrict__ nfar, Control *ctrl) {
   if (!ctrl->do_rebuild) return;
   __shared__ float4 stage[NB_WARPS][NB_STAGE];         // staged (displacement, entry)
-  __shared__ uint8_t skey[NB_WARPS][NB_STAGE];
+  __shared__ float4 tab[NB_WARPS][28];                 // candidate ranges
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   // The grid is capped at the resident blocks (a launch on a step without a rebuild then costs a few
-  // microseconds whatever the atom count); each block takes the next group of NB_WARPS consecutive
+  // microseconds whatever the atom count); each block takes the next `take` groups of NB_WARPS consecutive
   // atoms from a counter, which keeps the order of the hardware's own block scheduling (a static
   // stride over the atoms measured 25 % slower).
   __shared__ int group;
@@ -593,12 +619,14 @@ k_neighbors(int n, const float4 *__restrict__ pos, const int *__restrict__ cell_
     __syncthreads();
     const int g = group;
     __syncthreads();                                   // read by every warp before the next take
-    if ((long long)g * NB_WARPS >= n) break;           // block-uniform
-    const int i = g * NB_WARPS + w;                    // warp-uniform
-    if (i < n)
-      neighbors_of_atom(i, n, pos, cell_start, geom, B, min(cap, NB_STAGE), stage[w], skey[w], lane, nbr, nnum,
+    if ((long long)g * (NB_WARPS * take) >= n) break;   // block-uniform
+    for (int k = 0; k < take; ++k) {
+      const int i = (g * take + k) * NB_WARPS + w;  // warp-uniform
+      if (i >= n) break;
+      neighbors_of_atom(i, n, pos, cell_start, geom, ssh, slices, B, min(cap, NB_STAGE), stage[w], tab[w], lane, nbr, nnum,
                         nang, nown, nband0, nfar, ctrl);
-    __syncwarp();                                      // the stage is reused by the warp's next atom
+      __syncwarp();                                    // the stage is reused by the warp's next atom
+    }
   }
 }
 
@@ -630,6 +658,10 @@ static int resident_grid(K kernel, long long m, int per_block, int threads) {
   return (int)std::min<long long>(blocks_for(m, per_block), (long long)sm_count() * per_sm);
 }
 
+// Slices per cell along x as a shift, for n atoms in ncell cells: four, unless the box is sparse (no gain, and four
+// times the cells to clear and scan).
+int slice_shift(int n, int64_t ncell) { return ncell <= n ? 2 : 0; }
+
 // The forms of the cell sort: one block, one cluster, or the chain of kernels.
 static bool small_system(int n, int ncell) { return n <= SMALL_ATOMS && ncell <= SMALL_CELLS; }
 static bool cluster_system(int n, int ncell) { return n <= CLUSTER_ATOMS && ncell <= CLUSTER_CELLS; }
@@ -645,8 +677,8 @@ int cell_sort_launches(int n, int ncell) {
 // first (cell_sort_decides); DECIDE_DONE otherwise.
 cudaError_t launch_cell_sort(const RebuildArgs &a, int decide, cudaStream_t st) {
   if (a.n <= 0) return cudaSuccess;
-  const CellGrid g{a.L[0], a.L[1], a.L[2], a.l[0], a.l[1], a.l[2], 1.0 / a.l[0], 1.0 / a.l[1], 1.0 / a.l[2],
-                   a.nc[0], a.nc[1], a.nc[2]};
+  const CellGrid g{a.L[0], a.L[1], a.L[2], a.l[0], a.l[1], a.l[2], (1 << a.ssh) / a.l[0], 1.0 / a.l[1], 1.0 / a.l[2],
+                   a.nc[0], a.nc[1], a.nc[2], a.ssh};
   if (small_system(a.n, a.ncell)) {
     k_rebuild_small<<<1, SCAN_THREADS, 0, st>>>(a.n, a.ncell, a.x, a.y, a.z, a.vx, a.vy, a.vz, a.id, a.start, a.pos,
                                                 a.pos_ref, g, a.ctrl, decide);
@@ -685,7 +717,7 @@ cudaError_t launch_neighbors(const RebuildArgs &a, cudaStream_t st) {
   Bands B;
   B.b0 = a.ba2; B.b1 = a.ra2; B.b2 = a.br2; B.b3 = std::min(a.fs2, a.rl2); B.b4 = a.rl2;
   k_neighbors<<<resident_grid(k_neighbors, a.n, NB_WARPS, NB_WARPS * 32), NB_WARPS * 32, 0, st>>>(
-      a.n, a.pos, a.start, g, a.cap, B, a.nbr, a.nnum, a.nang, a.nown, a.nband0, a.nfar, a.ctrl);
+      a.n, a.pos, a.start, g, a.ssh, (float)((1 << a.ssh) / a.l[0]), a.n >= NB_TAKE_MIN ? 4 : 1, a.cap, B, a.nbr, a.nnum, a.nang, a.nown, a.nband0, a.nfar, a.ctrl);
   return cudaGetLastError();
 }
 

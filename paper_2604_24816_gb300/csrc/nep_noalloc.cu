@@ -36,7 +36,7 @@ cudaError_t launch_wide(int, const Model<S> &, const Geom &, int, const float4 *
 cudaError_t launch_cell_sort(const RebuildArgs &, int, cudaStream_t);
 bool cell_sort_decides(int n, int ncell);
 cudaError_t launch_neighbors(const RebuildArgs &, cudaStream_t);
-int scan_tiles(int ncell);
+int slice_shift(int n, int64_t ncell);
 cudaError_t launch_control(Control *, int, cudaStream_t);
 cudaError_t launch_load_state(int, const double *, const double *, double *, double *, double *, double *, double *,
                               double *, int *, int *, cudaStream_t);
@@ -239,7 +239,10 @@ extern "C" nep_status nep_compute_noalloc(const nep_params *p, int64_t n, const 
 
   RebuildArgs a{};
   a.n = N;
-  a.ncell = (int)ncell;
+  // at most NC_MAX slices: cells are divided only when there are no more of them than atoms
+  static_assert((NA_MAX << 2) <= NC_MAX, "slices of a dense system fit the cell arrays");
+  a.ssh = slice_shift(N, ncell);
+  a.ncell = (int)(ncell << a.ssh);
   for (int d = 0; d < 3; ++d) { a.L[d] = box[d]; a.l[d] = l[d]; a.nc[d] = nc[d]; }
   a.x = (double *)at(LAYOUT.x); a.y = (double *)at(LAYOUT.y); a.z = (double *)at(LAYOUT.z);
   a.vx = (double *)at(LAYOUT.vx); a.vy = (double *)at(LAYOUT.vy); a.vz = (double *)at(LAYOUT.vz);
