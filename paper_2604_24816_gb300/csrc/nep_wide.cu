@@ -3,7 +3,7 @@
 // The fused kernels of nep_force.cu give each atom one thread, which walks its row alone: 45 us from one block
 // to one block per SM, whatever the atom count, since a warp then issues one instruction every three cycles.
 // Systems that leave the chip empty that way (and the few atoms that a student's fallback hands to the
-// teacher) take k_nep_wide: a group of G = 8, 16 or 32 lanes shares an atom.
+// teacher) take k_nep_wide: a group of G = 4, 8, 16 or 32 lanes shares an atom.
 //   walk      the lanes stride over the neighbour row; entries inside the cutoff are compacted by ballot into
 //             the group's shared memory (angular pairs from the front, the others from the back), radial
 //             basis sums and LJ energy in registers, combined by shuffles;
@@ -38,10 +38,13 @@ __device__ __forceinline__ float round_to(float x) {
 }
 
 // The model tables the lanes index (read from shared memory; the constant bank serves one address at a time).
+// W0 by rows and by columns, zero-padded to whole 16-byte vectors: a product reads a lane's row and the atom's
+// values four at a time, eight lanes' rows without bank conflicts.
 template <class S>
-struct WideNet {
-  static constexpr int LD = S::NDES | 1;
-  float W0[S::NNEU * LD];
+struct __align__(16) WideNet {
+  static constexpr int NV = (S::NDES + 3) / 4, NM = (S::NNEU + 3) / 4;      // vectors per row, per column
+  static constexpr int LD = S::NDES > 16 ? 4 * NV + 4 : 4 * NV, LDT = 4 * NM + 4;
+  float W0[S::NNEU * LD], W0t[S::NDES * LDT];
   float cR[S::NR * S::KR];
   float qs[S::NDES], b0[S::NNEU], w1[S::NNEU], norm[S::NLM];
 };
@@ -50,11 +53,23 @@ struct WideNet {
 template <class S>
 struct __align__(16) WideAtom {
   uint32_t ent[WIDE_CAP];              // active list entries: angular from the front, others from the back
-  float row[S::NA][S::NLM];            // s', then the adjoint row (16-byte rows: NLM is a multiple of 4)
+  float q[32], t[32];                  // scaled descriptors then dU/dq; backward factors (zero past the last)
   float Q[8];                          // radial sums, then the radial adjoint
-  float q[32], t[32];                  // scaled descriptors then dU/dq; backward factors
   float g4[S::FOURBODY ? S::NA : 1][5];
 };
+
+// sum of w[k] v[k] over 4 N values, both on 16-byte boundaries.
+template <int N>
+__device__ __forceinline__ float dot4(const float *w, const float *v, float z0) {
+  float2 a = pr(z0, 0.f), b = bc2(0.f);
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    const float4 x = reinterpret_cast<const float4 *>(w)[k], y = reinterpret_cast<const float4 *>(v)[k];
+    a = fma2(pr(x.x, x.y), pr(y.x, y.y), a);
+    b = fma2(pr(x.z, x.w), pr(y.z, y.w), b);
+  }
+  return hsum(add2(a, b));
+}
 
 template <class S>
 struct RowShared {
@@ -75,11 +90,11 @@ __device__ __forceinline__ float group_sum(float v) {
   return v;
 }
 
-// Sums of the 8 values over the group: lane gl ends with value gl / (G / 8).
+// Sums of the 8 values over the group, to dst[0..7] (lane gl holds value gl / (G / 8), or values 2 gl and 2 gl + 1).
 template <int G>
-__device__ __forceinline__ float group_sum8(const float (&v)[8], int gl) {
+__device__ __forceinline__ void group_sum8(const float (&v)[8], int gl, float *dst) {
   float a[4], b[2];
-  const bool h0 = (gl & (G / 2)) != 0, h1 = (gl & (G / 4)) != 0, h2 = (gl & (G / 8)) != 0;
+  const bool h0 = (gl & (G / 2)) != 0, h1 = (gl & (G / 4)) != 0;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const float keep = h0 ? v[4 + k] : v[k], give = h0 ? v[k] : v[4 + k];
@@ -90,11 +105,17 @@ __device__ __forceinline__ float group_sum8(const float (&v)[8], int gl) {
     const float keep = h1 ? a[2 + k] : a[k], give = h1 ? a[k] : a[2 + k];
     b[k] = keep + __shfl_xor_sync(0xffffffffu, give, G / 4);
   }
-  const float keep = h2 ? b[1] : b[0], give = h2 ? b[0] : b[1];
-  float c = keep + __shfl_xor_sync(0xffffffffu, give, G / 8);
+  if constexpr (G >= 8) {
+    const bool h2 = (gl & (G / 8)) != 0;
+    const float keep = h2 ? b[1] : b[0], give = h2 ? b[0] : b[1];
+    float c = keep + __shfl_xor_sync(0xffffffffu, give, G / 8);
 #pragma unroll
-  for (int o = G / 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  return c;
+    for (int o = G / 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if ((gl & (G / 8 - 1)) == 0) dst[gl / (G / 8)] = c;
+  } else {
+    dst[2 * gl] = b[0];
+    dst[2 * gl + 1] = b[1];
+  }
 }
 
 template <class S, int G>
@@ -104,8 +125,11 @@ struct __align__(16) WideShared {
   WideNet<S> net;
   // one staged pair per lane; with rows of an odd length the lanes write their own rows, and the lanes of a
   // group read consecutive values of one row, G rows apart from the next group's, without bank conflicts
-  static constexpr int STP = (S::NA + S::NLM) | 1;
-  float stage[WIDE_WARPS][32 * STP];
+  // (when all pairs are summed, the groups' rows take the same memory: s', then the adjoint row, 16-byte vectors)
+  static constexpr int STP = (S::NA + S::NLM) | 1, ROW = S::NA * S::NLM;
+  static constexpr int STAGE = 32 * STP > 32 / G * ROW ? 32 * STP : 32 / G * ROW;
+  static_assert(STAGE % 4 == 0 && ROW % 4 == 0, "16-byte rows");
+  __align__(16) float stage[WIDE_WARPS][STAGE];
 };
 
 template <class S, class MT, int G, bool LIST>
@@ -116,7 +140,7 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
                                           const EvalSums &sums, int *__restrict__ status, const Fallback &fb) {
   constexpr bool MIX = !std::is_same<MT, float>::value;
   constexpr int NG = 32 / G;                           // atoms per warp
-  constexpr int LD = WideNet<S>::LD;
+  constexpr int LD = WideNet<S>::LD, LDT = WideNet<S>::LDT, NV = WideNet<S>::NV, NM = WideNet<S>::NM;
   constexpr int STP = WideShared<S, G>::STP;
   constexpr int CPL = (S::NLM + G - 1) / G;            // components per lane
   constexpr int NP2 = 2 * solid_pairs(S::NLM);
@@ -152,8 +176,12 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
   }
   load_atom();
   fill_shift_table(shift, geom);
-  for (int t = threadIdx.x; t < S::NNEU * S::NDES; t += WIDE_BLOCK)
-    net.W0[(t / S::NDES) * LD + t % S::NDES] = round_to<MT>(P.W0[t / S::NDES][t % S::NDES]);
+  for (int t = threadIdx.x; t < 4 * NM * 4 * NV; t += WIDE_BLOCK) {
+    const int mu = t / (4 * NV), v = t % (4 * NV);
+    const float w = mu < S::NNEU && v < S::NDES ? round_to<MT>(P.W0[mu < S::NNEU ? mu : 0][v < S::NDES ? v : 0]) : 0.f;
+    if (mu < S::NNEU) net.W0[mu * LD + v] = w;
+    if (v < S::NDES) net.W0t[v * LDT + mu] = w;
+  }
   for (int t = threadIdx.x; t < S::NR * S::KR; t += WIDE_BLOCK) net.cR[t] = P.cR[t / S::KR][t % S::KR];
   for (int t = threadIdx.x; t < S::NDES; t += WIDE_BLOCK) net.qs[t] = P.qs[t];
   for (int t = threadIdx.x; t < S::NNEU; t += WIDE_BLOCK) { net.b0[t] = P.b0[t]; net.w1[t] = P.w1[t]; }
@@ -168,6 +196,11 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
   const unsigned gmask = (G == 32 ? 0xffffffffu : ((1u << G) - 1u)), below = (1u << gl) - 1u;
   WideAtom<S> &A = M.ws[warp * NG + grp];
   float *st = M.stage[warp] + lane * STP;              // this lane's staged pair
+  float *row = M.stage[warp] + grp * WideShared<S, G>::ROW;   // the atom's row
+  for (int k = gl; k < 32; k += G) {
+    if (k >= S::NDES) A.q[k] = 0.f;
+    if (k >= S::NNEU) A.t[k] = 0.f;
+  }
   const float *sg = M.stage[warp] + grp * G * STP;     // the group's
   long long acc_d[5] = {0, 0, 0, 0, 0}, acc_f[13] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   const int per_pass = (int)gridDim.x * WIDE_WARPS * NG;
@@ -212,8 +245,7 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
     {
       float v[8];
       cheb_sums(Q, v);                                 // linear: the lanes' sums add up to the atom's
-      const float t = group_sum8<G>(v, gl);
-      if ((gl & (G / 8 - 1)) == 0) A.Q[gl / (G / 8)] = t;
+      group_sum8<G>(v, gl, A.Q);
     }
     elj = group_sum<G>(elj);
     __syncwarp();
@@ -269,7 +301,7 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
     for (int c = 0; c < CPL; ++c)
       if (gl + c * G < S::NLM) {
 #pragma unroll
-        for (int a = 0; a < S::NA; ++a) A.row[a][gl + c * G] = s[a][c];
+        for (int a = 0; a < S::NA; ++a) row[a * S::NLM + gl + c * G] = s[a][c];
       }
     __syncwarp();
 
@@ -283,10 +315,10 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
         for (int k = 0; k < S::KR; ++k) q = fmaf(net.cR[d * S::KR + k], A.Q[k], q);
       } else if (d < S::NR + S::NA * S::LMAX) {
         const int a = (d - S::NR) / S::LMAX, l = (d - S::NR) % S::LMAX + 1;
-        const float z = net.norm[NP2 + l - 1] * A.row[a][NP2 + l - 1];
+        const float z = net.norm[NP2 + l - 1] * row[a * S::NLM + NP2 + l - 1];
         q = z * z;
         for (int c = l * (l - 1); c < l * (l + 1); ++c) {
-          const float v = net.norm[c] * A.row[a][c];
+          const float v = net.norm[c] * row[a * S::NLM + c];
           q = fmaf(v, v, q);
         }
       } else {
@@ -299,7 +331,7 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
 #pragma unroll
           for (int p = 0; p < S::NLM; ++p) {
             const int m2 = solid_quadrupole(S::NLM, p);
-            if (m2 >= 0) s2[0][m2 < 0 ? 0 : m2] = solid_norm(S::NLM, p) * A.row[a][p];
+            if (m2 >= 0) s2[0][m2 < 0 ? 0 : m2] = solid_norm(S::NLM, p) * row[a * S::NLM + p];
           }
           FourBody<One> T;
           fourbody_tensors<One>(s2, T, q1);
@@ -327,15 +359,7 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
     // network: neurons, then their backward products
     float U = 0.f;
     for (int mu = gl; mu < S::NNEU; mu += G) {
-      const float *w = net.W0 + mu * LD;
-      float z0 = -net.b0[mu], z1 = 0.f;
-#pragma unroll
-      for (int v = 0; v + 1 < S::NDES; v += 2) {
-        z0 = fmaf(w[v], A.q[v], z0);
-        z1 = fmaf(w[v + 1], A.q[v + 1], z1);
-      }
-      if (S::NDES & 1) z0 = fmaf(w[S::NDES - 1], A.q[S::NDES - 1], z0);
-      const float z = z0 + z1;
+      const float z = dot4<NV>(net.W0 + mu * LD, A.q, -net.b0[mu]);
       const float h = MIX ? tanh_sfu(z) : tanhf(z);
       U = fmaf(net.w1[mu], h, U);
       A.t[mu] = round_to<MT>(net.w1[mu] * (1.f - h * h));
@@ -343,15 +367,8 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
     U = group_sum<G>(U) - P.b1;
     __syncwarp();                                      // t is complete, q has been read
     for (int v = gl; v < S::NDES; v += G) {
-      const float *w = net.W0 + v;
-      float d0 = 0.f, d1 = 0.f;
-#pragma unroll
-      for (int mu = 0; mu + 1 < S::NNEU; mu += 2) {
-        d0 = fmaf(A.t[mu], w[mu * LD], d0);
-        d1 = fmaf(A.t[mu + 1], w[(mu + 1) * LD], d1);
-      }
-      if (S::NNEU & 1) d0 = fmaf(A.t[S::NNEU - 1], w[(S::NNEU - 1) * LD], d0);
-      A.q[v] = flagged ? 0.f : (d0 + d1) * net.qs[v];  // dU/dq
+      const float d = dot4<NM>(net.W0t + v * LDT, A.t, 0.f);
+      A.q[v] = flagged ? 0.f : d * net.qs[v];          // dU/dq
     }
     __syncwarp();
 
@@ -372,7 +389,7 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
           if constexpr (S::FOURBODY) {
             if (m2 >= 0) gl_ = fmaf(h * A.q[S::NR + S::NA * S::LMAX + a], A.g4[a][m2], gl_);
           }
-          A.row[a][p] = gl_;
+          row[a * S::NLM + p] = gl_;
         }
       }
     }
@@ -403,7 +420,7 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
     acc_d[1] += nrad;
 
     // forces: the compacted entries, angular ones first
-    const RowShared<S> row{&A.row[0][0]};
+    const RowShared<S> adjoint{row};
     float fx = 0.f, fy = 0.f, fz = 0.f;
     float wxx = 0.f, wxy = 0.f, wxz = 0.f, wyy = 0.f, wyz = 0.f, wzz = 0.f;
     const int nact = na + no;
@@ -425,7 +442,7 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
       float vx = 0.f, vy = 0.f, vz = 0.f;
       if (ang) {
         float ca;
-        angular_pair_solid<S>(P, row, false, r, ir, dx, dy, dz, ca, vx, vy, vz);
+        angular_pair_solid<S>(P, adjoint, false, r, ir, dx, dy, dz, ca, vx, vy, vz);
         coef += ca;
       }
       if (valid) {
@@ -478,8 +495,8 @@ k_nep_wide(const __grid_constant__ Model<S> P, const Geom geom, const int n, con
            const int32_t *__restrict__ nbr, const RowExt X, float *__restrict__ usite, float *__restrict__ qout,
            unsigned long long *__restrict__ Ffix, const EvalSums sums, int *__restrict__ status,
            const __grid_constant__ Fallback fb) {
-  __shared__ WideShared<S, G> M;
-  wide_body<S, MT, G, false>(M, P, geom, n, n, nullptr, pos, nbr, X, usite, qout, Ffix, sums, status, fb);
+  extern __shared__ __align__(16) unsigned char raw[];
+  wide_body<S, MT, G, false>(*reinterpret_cast<WideShared<S, G> *>(raw), P, geom, n, n, nullptr, pos, nbr, X, usite, qout, Ffix, sums, status, fb);
 }
 
 // The fallback model on the first min(*count, cap) atoms of list: only its network's part is added to usite, to
@@ -511,10 +528,11 @@ k_nep_wide_list(const __grid_constant__ Model<S> P, const Geom geom, const int n
 
 // Blocks that fit on the device at once, or fewer for few atoms; the kernels loop.
 template <class K>
-int wide_grid(K kernel, int atoms, int lanes) {
+int wide_grid(K kernel, int atoms, int lanes, size_t smem) {
   int d = 0, sms = 0, per = 0;
-  if (cudaGetDevice(&d) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, WIDE_BLOCK, 0) != cudaSuccess || sms * per <= 0) {
+  if ((smem > 48 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) ||
+      cudaGetDevice(&d) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, WIDE_BLOCK, smem) != cudaSuccess || sms * per <= 0) {
     cudaGetLastError();
     sms = 152;
     per = 1;
@@ -525,28 +543,30 @@ int wide_grid(K kernel, int atoms, int lanes) {
 
 }  // namespace
 
-// Lanes per atom for a system of n atoms, 0: one thread per atom (the fused kernels of nep_force.cu).  Measured
-// per evaluation (eager, with the launch's own 7 us) for the teacher: at 256 atoms 50 us with one thread per atom,
-// 25 / 19 / 17 us with 8 / 16 / 32 lanes; at 2,048 51, 26 / 22 / 23; at 4,000 50, 28 / 28 / 30; at 10,976 53,
-// 45 / 46 / 50; at 16,384 53 (MD step 72.5), 54 (70.9) / 57 / 67; at 32,000 66, 83 / 93 / 112, where the wide
-// form's extra work (1.6 x the instructions per atom) is no longer hidden.  The student (40 us with one thread
-// per atom up to 16,384 atoms; 15 at 256 with 32 lanes, 20 at 4,000 with 16, 36 at 16,384 with 8) and the
-// mixed forms cross at the same sizes.
-int wide_lanes(int n) { return n <= 1024 ? 32 : (n <= 4096 ? 16 : (n <= 16384 ? 8 : 0)); }
+// Lanes per atom for a system of n atoms, 0: one thread per atom (the fused kernels of nep_force.cu).  The last
+// two lines are where all atoms still fit the resident warps at once (608 blocks of 16 and of 32 atoms).  Measured per
+// evaluation of the teacher (eager, with the launch's own 7 us), one thread per atom, then 4 / 8 / 16 / 32 lanes:
+// 256 atoms 49, 30 / 23 / 19 / 17 us; 2,048 49, 32 / 24 / 21 / 23; 4,000 50, 32 / 26 / 27 / 29; 6,912 50,
+// 36 / 30 / 36 / 38; 10,976 51, 42 / 43 / 46 / 50; 16,384 51 (MD step 60.3), 49 (58.0) / 52 (61.3) / 57 / 67; 23,328 64,
+// 69 / 62 / 73 / 88; 32,000 66, 81 / 80 / 92 / 113, where the wide forms' extra work is no longer
+// hidden.  The student (39 us with one thread per atom up to 16,384 atoms; 19 at 4,000 with 16, 22 at 6,912 with 8,
+// 34 at 16,384 with 4) and the mixed forms cross at the same sizes.
+int wide_lanes(int n) { return n <= 1024 ? 32 : (n <= 4096 ? 16 : (n <= 9728 ? 8 : (n <= 19456 ? 4 : 0))); }
 
-// One force evaluation with `lanes` (8, 16 or 32) lanes per atom; Ffix must be zero.
+// One force evaluation with `lanes` (4, 8, 16 or 32) lanes per atom; Ffix must be zero.
 template <class S, class MT>
 cudaError_t launch_wide(int lanes, const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
                         const RowExt &X, float *usite, float *qout, long long *Ffix, const EvalSums &sums,
                         int *status, const Fallback &fb, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  auto run = [&](auto kernel, int g_lanes) {
-    kernel<<<wide_grid(kernel, n, g_lanes), WIDE_BLOCK, 0, st>>>(
+  auto run = [&](auto kernel, int g_lanes, size_t smem) {
+    kernel<<<wide_grid(kernel, n, g_lanes, smem), WIDE_BLOCK, smem, st>>>(
         P, g, n, pos, nbr, X, usite, qout, reinterpret_cast<unsigned long long *>(Ffix), sums, status, fb);
   };
-  if (lanes == 32) run(k_nep_wide<S, MT, 32>, 32);
-  else if (lanes == 16) run(k_nep_wide<S, MT, 16>, 16);
-  else run(k_nep_wide<S, MT, 8>, 8);
+  if (lanes == 32) run(k_nep_wide<S, MT, 32>, 32, sizeof(WideShared<S, 32>));
+  else if (lanes == 16) run(k_nep_wide<S, MT, 16>, 16, sizeof(WideShared<S, 16>));
+  else if (lanes == 8) run(k_nep_wide<S, MT, 8>, 8, sizeof(WideShared<S, 8>));
+  else run(k_nep_wide<S, MT, 4>, 4, sizeof(WideShared<S, 4>));
   return cudaGetLastError();
 }
 
@@ -557,7 +577,7 @@ cudaError_t launch_wide_list(const Model<S> &P, const Geom &g, int n, const floa
                              const RowExt &X, const int *list, const int *count, int cap, float *usite, long long *Ffix,
                              const EvalSums &sums, int *status, cudaStream_t st) {
   if (n <= 0 || cap <= 0) return cudaSuccess;
-  k_nep_wide_list<S><<<wide_grid(k_nep_wide_list<S>, cap, 32), WIDE_BLOCK, 0, st>>>(
+  k_nep_wide_list<S><<<wide_grid(k_nep_wide_list<S>, cap, 32, 0), WIDE_BLOCK, 0, st>>>(
       P, g, n, list, count, cap, pos, nbr, X, usite, reinterpret_cast<unsigned long long *>(Ffix), sums, status);
   return cudaGetLastError();
 }

@@ -10,8 +10,8 @@ import oracle
 
 pytestmark = pytest.mark.gpu
 
-# lanes per atom: 32 up to 1,024 atoms, 16 up to 4,096, 8 up to 16,384, then one thread per atom
-SIZES = [1, 5, 129, 1024, 1025, 4096, 4097, 16384, 16385]
+# lanes per atom: 32 up to 1,024 atoms, 16 up to 4,096, 8 up to 9,728, 4 up to 19,456, then one thread per atom
+SIZES = [1, 5, 129, 1024, 1025, 4096, 4097, 9728, 9729, 19456, 19457]
 
 
 @pytest.fixture(scope="module")
@@ -51,7 +51,7 @@ def test_teacher(api, model_params, model, n):
 
 
 @pytest.mark.parametrize("precision", ["mix_bf16", "mix_fp16"])
-@pytest.mark.parametrize("n", [5, 1024, 1025, 4097])
+@pytest.mark.parametrize("n", [5, 1024, 1025, 4097, 9729])
 def test_mixed(api, model_params, model, trained_student_params, n, precision):
     # the bounds of the tensor-core forms' tests: RMSE 5 meV/A, largest 20 (bf16) or 3 meV/A (f16)
     pos, box = _cell(n)
@@ -64,7 +64,7 @@ def test_mixed(api, model_params, model, trained_student_params, n, precision):
         assert np.abs(dF).max() <= (2e-2 if precision == "mix_bf16" else 3e-3)
 
 
-@pytest.mark.parametrize("n", [1, 1024, 1025, 4097, 16385])
+@pytest.mark.parametrize("n", [1, 1024, 1025, 4097, 9729, 19457])
 def test_student(api, trained_student_params, n):
     pos, box = _cell(n)
     Eo, Uo, Fo, Wo = oracle.energy_forces(oracle.Model(trained_student_params), pos, box)
@@ -79,7 +79,7 @@ def test_student(api, trained_student_params, n):
 @pytest.mark.parametrize("n,share", [(257, 0.5), (1024, 1.0), (4096, 1.0), (4097, 1.0), (20000, 0.03), (20000, 0.4)])
 def test_fallback_list(api, model_params, model, trained_student_params, n, share):
     """1 to 4,096 flagged atoms take a warp each, more a quarter of one; the student's own kernel is a wide one
-    up to 16,384 atoms."""
+    up to 19,456 atoms."""
     pos, box = _cell(n)
     sm = oracle.Model(trained_student_params)
     qt = oracle.descriptors(sm, pos, box) * np.asarray(trained_student_params["q_scale"], np.float32)
