@@ -90,17 +90,18 @@ cudaError_t launch_kick_drift(int, double *, double *, double *, double *, doubl
                               const float4 *, double, double, const double *, float, Control *, cudaStream_t);
 cudaError_t launch_control(Control *, int, cudaStream_t);
 cudaError_t launch_control_cond(Control *, cudaGraphConditionalHandle, cudaStream_t);
-cudaError_t launch_inverse_order(int, const int *, int *, cudaStream_t);
+cudaError_t launch_inverse_order(int, const int *, int *, Control *, cudaStream_t);
 cudaError_t launch_load_state_sorted(int, const double *, const double *, const int *, double *, double *, double *,
                                      double *, double *, double *, float4 *, const float4 *, const double *,
                                      const double *, float, Control *, cudaStream_t);
 cudaError_t launch_kick(int, double *, double *, double *, const long long *, double, double, const EvalSums &, Control *,
                         cudaStream_t);
-cudaError_t launch_kinetic(int, const double *, const double *, const double *, double, const EvalSums &, cudaStream_t);
+cudaError_t launch_kinetic(int, const double *, const double *, const double *, double, const EvalSums &, const int *,
+                           const long long *, double *, cudaStream_t);
 cudaError_t launch_load_state(int, const double *, const double *, double *, double *, double *, double *, double *,
                               double *, int *, int *, cudaStream_t);
 cudaError_t launch_store_vec(int, const int *, const double *, const double *, const double *, const double *, int,
-                             double *, cudaStream_t);
+                             double *, const double *, const double *, const double *, double *, cudaStream_t);
 cudaError_t launch_store_force(int, const int *, const long long *, double *, cudaStream_t);
 cudaError_t launch_store_scalar(int, const int *, const float *, double *, cudaStream_t);
 cudaError_t launch_store_rows(int, int, const int *, const float *, float *, cudaStream_t);
@@ -195,6 +196,7 @@ struct nep_handle {
 
   // host mirror (pinned)
   DeviceReport *h_rep = nullptr;
+  double *h_io = nullptr;          // page-locked staging 2 x [HOST_ATOMS][3] of small systems' pageable arrays
   cudaEvent_t done = nullptr;
 
   // graphs of MD steps: one step, and several
@@ -215,7 +217,7 @@ struct nep_handle {
   float fb_lo[16] = {0}, fb_hi[16] = {0};
   double fb_frac = 1.0 / 16.0;
   int fb_cap = 0;
-  int *fb_list = nullptr, *fb_count = nullptr;
+  int *fb_list = nullptr, *fb_count = nullptr;   // fb_count: in the control block
 
   // buffers of the ablation variants (allocated on first use)
   float *abl_f = nullptr, *abl_s = nullptr;
@@ -288,7 +290,7 @@ void free_system(nep_handle *h) {
   dfree(h->nbr); dfree(h->nnum); dfree(h->nang); dfree(h->nown); dfree(h->nband0); dfree(h->nfar);
   dfree(h->count); dfree(h->cursor); dfree(h->start); dfree(h->tile_sums);
   dfree(h->io); dfree(h->io_i);
-  dfree(h->fb_list); dfree(h->fb_count);
+  dfree(h->fb_list);
   dfree(h->abl_f); dfree(h->abl_s); dfree(h->abl_cnt);
   dfree(h->pc_rec); dfree(h->pc_mask); dfree(h->inv);
   h->pc_nsm = 0;
@@ -297,6 +299,15 @@ void free_system(nep_handle *h) {
   h->n = 0;
   h->have_state = h->have_nlist = h->have_forces = false;
 }
+
+// Pageable arrays of up to HOST_ATOMS atoms pass through page-locked memory that the load and store kernels read and
+// write themselves: a pageable copy costs the host 5 us (to the device) or a wait of its own (from it).  Through copies
+// and through staging: nep_set_state + nep_compute 90 and 86 us at 256 atoms, 114 and 108 at 4,000, 137 and 150 at
+// 10,976 (scattered 24-byte accesses over the host link); nep_get_state 41 and 19, 51 and 32, 59 and 53.
+constexpr int HOST_ATOMS = 4096;
+
+// A host array's stand-in that kernels can reach, nullptr for arrays of larger systems (which are copied).
+double *host_stage(nep_handle *h, int which) { return h->n <= HOST_ATOMS ? h->h_io + which * 3 * (size_t)HOST_ATOMS : nullptr; }
 
 template <class T>
 cudaError_t dalloc(T *&p, size_t elems) {
@@ -446,7 +457,8 @@ cudaError_t forces_of(nep_handle *h, const Model<S> &M, float *qout, bool zeroed
     for (int v = 0; v < 16; ++v) { fb.lo[v] = h->fb_lo[v]; fb.hi[v] = h->fb_hi[v]; }
   }
   cudaError_t e;
-  if (fb.on && (e = cudaMemsetAsync(h->fb_count, 0, sizeof(int), h->stream)) != cudaSuccess) return e;
+  // (an MD step's rebuild decision has cleared the count)
+  if (fb.on && !zeroed && (e = cudaMemsetAsync(h->fb_count, 0, sizeof(int), h->stream)) != cudaSuccess) return e;
   if (h->wide > 0 || teacher || h->precision == NEP_FP32) {
     // descriptors, network and full-row forces in one kernel, then the teacher on the flagged atoms; the network
     // in float32, or with bf16 / f16 operands in the mixed-precision forms
@@ -517,9 +529,10 @@ cudaError_t enqueue_forces(nep_handle *h, float *qout, bool zeroed = false) {
                        : forces_of<StudentShape>(h, h->model_s, qout, zeroed);
 }
 
-cudaError_t enqueue_kinetic(nep_handle *h) {
+// The kinetic energy; with the evaluation's forces in the caller's order (Fout, or nullptr).
+cudaError_t enqueue_kinetic(nep_handle *h, double *Fout = nullptr) {
   Scope sc(h, KC_OTHER, 1);
-  return launch_kinetic(h->n, h->vx, h->vy, h->vz, h->mass, eval_sums(h, true), h->stream);
+  return launch_kinetic(h->n, h->vx, h->vy, h->vz, h->mass, eval_sums(h, true), h->id, h->F, Fout, h->stream);
 }
 
 // One MD step.  Launched eagerly (capture = false) the rebuild chain's kernels run every step and
@@ -627,11 +640,11 @@ nep_status ensure_nlist(nep_handle *h) {
   return NEP_OK;
 }
 
-nep_status compute_internal(nep_handle *h, float *qout) {
+nep_status compute_internal(nep_handle *h, float *qout, double *Fout = nullptr) {
   nep_status s = ensure_nlist(h);
   if (s != NEP_OK) return s;
   NEP_CUDA(h, enqueue_forces(h, qout));
-  NEP_CUDA(h, enqueue_kinetic(h));
+  NEP_CUDA(h, enqueue_kinetic(h, Fout));
   h->have_forces = true;
   return NEP_OK;
 }
@@ -662,21 +675,29 @@ nep_status build_graph(nep_handle *h, StepGraph &sg, double dt, int steps) {
   return NEP_OK;
 }
 
+// Where the load kernels read a host array a of the caller (which: 0 positions, 1 velocities): small ones from
+// page-locked staging (the previous call has waited for the kernels that used it), others from a device copy.
+nep_status stage_input(nep_handle *h, const double *a, int which, const double *&src) {
+  const size_t N3 = 3 * (size_t)h->n;
+  if (double *t = host_stage(h, which)) {
+    std::memcpy(t, a, N3 * sizeof(double));
+    src = t;
+    return NEP_OK;
+  }
+  NEP_CUDA(h, cudaMemcpyAsync(h->io + which * N3, a, N3 * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+  src = h->io + which * N3;
+  return NEP_OK;
+}
+
 // Copy [n][3] positions/velocities (host or device) into the SoA state, ids = 0..n-1, and reset the
 // device status word.
 nep_status upload_state(nep_handle *h, const double *x, const double *v) {
   if (h->n > 0) {
-    const size_t N = (size_t)h->n;
     NEP_CUDA(h, cudaMemsetAsync(&h->ctrl->status, 0, sizeof(int), h->stream));
     const double *xs = x, *vs = v;
-    if (!is_device_ptr(x)) {
-      NEP_CUDA(h, cudaMemcpyAsync(h->io, x, 3 * N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-      xs = h->io;
-    }
-    if (v && !is_device_ptr(v)) {
-      NEP_CUDA(h, cudaMemcpyAsync(h->io + 3 * N, v, 3 * N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-      vs = h->io + 3 * N;
-    }
+    nep_status t = is_device_ptr(x) ? NEP_OK : stage_input(h, x, 0, xs);
+    if (t == NEP_OK && v && !is_device_ptr(v)) t = stage_input(h, v, 1, vs);
+    if (t != NEP_OK) return t;
     {
       Scope sc(h, KC_OTHER, 1);
       NEP_CUDA(h, launch_load_state(h->n, xs, vs, h->x, h->y, h->z, h->vx, h->vy, h->vz, h->id, &h->ctrl->status,
@@ -694,26 +715,18 @@ nep_status upload_state(nep_handle *h, const double *x, const double *v) {
 // nep_get_state is uploaded again, velocities possibly altered) the forces, energy and virial of the
 // last evaluation still hold: they are kept, and only the kinetic energy is summed again.
 nep_status upload_state_sorted(nep_handle *h, const double *x, const double *v) {
-  const size_t N = (size_t)h->n;
   const bool had_forces = h->have_forces, had_recheck = h->recheck;
   h->have_forces = false;
-  NEP_CUDA(h, cudaMemsetAsync(&h->ctrl->status, 0, sizeof(int), h->stream));
-  NEP_CUDA(h, cudaMemsetAsync(&h->ctrl->changed, 0, sizeof(int), h->stream));
   // device arrays and page-locked host arrays are read by the kernel itself (in the caller's order,
-  // contiguously); other host arrays are copied to the device first
+  // contiguously); other host arrays through stage_input
   const double *xs = x, *vs = v;
-  if (!is_device_ptr(x) && !(xs = pinned_alias(x))) {
-    NEP_CUDA(h, cudaMemcpyAsync(h->io, x, 3 * N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-    xs = h->io;
-  }
-  if (v && !is_device_ptr(v) && !(vs = pinned_alias(v))) {
-    NEP_CUDA(h, cudaMemcpyAsync(h->io + 3 * N, v, 3 * N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-    vs = h->io + 3 * N;
-  }
+  nep_status t = is_device_ptr(x) || (xs = pinned_alias(x)) ? NEP_OK : stage_input(h, x, 0, xs);
+  if (t == NEP_OK && v && !is_device_ptr(v) && !(vs = pinned_alias(v))) t = stage_input(h, v, 1, vs);
+  if (t != NEP_OK) return t;
   const float hs = 0.5f * h->skin;
   {
     Scope sc(h, KC_OTHER, 2);
-    NEP_CUDA(h, launch_inverse_order(h->n, h->id, h->inv, h->stream));
+    NEP_CUDA(h, launch_inverse_order(h->n, h->id, h->inv, h->ctrl, h->stream));
     NEP_CUDA(h, launch_load_state_sorted(h->n, xs, vs, h->inv, h->x, h->y, h->z, h->vx, h->vy, h->vz, h->pos,
                                          h->pos_ref, h->l, h->L, hs * hs, h->ctrl, h->stream));
   }
@@ -730,11 +743,10 @@ nep_status upload_state_sorted(nep_handle *h, const double *x, const double *v) 
 
 // Fallback buffers for the current system: flagged-atom list and its length.
 cudaError_t alloc_fallback(nep_handle *h) {
-  dfree(h->fb_list); dfree(h->fb_count);
+  dfree(h->fb_list);
   const size_t N = (size_t)std::max(h->n, 1);
   h->fb_cap = (int)std::min<double>((double)N, std::max(1.0, std::ceil((double)N * h->fb_frac)));
   cudaError_t e = dalloc(h->fb_list, (size_t)h->fb_cap);
-  if (e == cudaSuccess) e = dalloc(h->fb_count, 1);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->fb_count, 0, sizeof(int), h->stream);
   return e;
 }
@@ -856,11 +868,13 @@ nep_status nep_create(const nep_params *p, void *cuda_stream, nep_handle **out) 
   }
   if ((e = cudaEventCreateWithFlags(&h->done, cudaEventDisableTiming)) != cudaSuccess ||
       (e = dalloc(h->rep, 1)) != cudaSuccess ||
-      (e = cudaMallocHost((void **)&h->h_rep, sizeof(DeviceReport))) != cudaSuccess) {
+      (e = cudaMallocHost((void **)&h->h_rep, sizeof(DeviceReport))) != cudaSuccess ||
+      (e = cudaMallocHost((void **)&h->h_io, 6 * (size_t)HOST_ATOMS * sizeof(double))) != cudaSuccess) {
     nep_destroy(h);
     return NEP_ERR_CUDA;
   }
   h->ctrl = &h->rep->ctrl;
+  h->fb_count = &h->ctrl->fb_count;
   h->sums = h->rep->sums;
   h->counters = h->rep->counters;
   if ((e = reset_report(h)) != cudaSuccess || (e = cudaStreamSynchronize(h->stream)) != cudaSuccess) {
@@ -877,6 +891,7 @@ nep_status nep_destroy(nep_handle *h) {
   free_system(h);
   dfree(h->rep);
   if (h->h_rep) cudaFreeHost(h->h_rep);
+  if (h->h_io) cudaFreeHost(h->h_io);
   for (auto &t : h->timers) { cudaEventDestroy(t.a); cudaEventDestroy(t.b); }
   if (h->done) cudaEventDestroy(h->done);
   for (cudaEvent_t ev : h->aux_ev)
@@ -981,16 +996,15 @@ nep_status nep_compute(nep_handle *h, double *E, double *F, double *virial) {
     if (virial) for (int k = 0; k < 9; ++k) virial[k] = 0.0;
     return NEP_OK;
   }
-  nep_status s = compute_internal(h, nullptr);
-  if (s != NEP_OK) return s;
+  // the forces: to a device array, or to page-locked staging (small systems), or through a device copy
+  const size_t F_bytes = 3 * (size_t)h->n * sizeof(double);
   const bool fdev = F && is_device_ptr(F);
-  if (F) {
-    Scope sc(h, KC_OTHER, 1);
-    NEP_CUDA(h, launch_store_force(h->n, h->id, h->F, fdev ? F : h->io, h->stream));
-    if (!fdev)
-      NEP_CUDA(h, cudaMemcpyAsync(F, h->io, 3 * (size_t)h->n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  }
+  double *stage = F && !fdev ? host_stage(h, 0) : nullptr;
+  nep_status s = compute_internal(h, nullptr, F ? (fdev ? F : (stage ? stage : h->io)) : nullptr);
+  if (s != NEP_OK) return s;
+  if (F && !fdev && !stage) NEP_CUDA(h, cudaMemcpyAsync(F, h->io, F_bytes, cudaMemcpyDeviceToHost, h->stream));
   s = check_device_status(h);
+  if (stage && s != NEP_ERR_CUDA) std::memcpy(F, stage, F_bytes);
   if (s != NEP_OK) return s;
   if (E) *E = h->h_rep->sums[0];
   if (virial) for (int k = 0; k < 9; ++k) virial[k] = h->h_rep->sums[1 + k];
@@ -1054,40 +1068,52 @@ nep_status nep_get_state(nep_handle *h, double *x, double *v) {
   const size_t N3 = 3 * (size_t)h->n;
   {
     Scope sc(h, KC_OTHER, 1);
-    NEP_CUDA(h, launch_inverse_order(h->n, h->id, h->inv, h->stream));
+    NEP_CUDA(h, launch_inverse_order(h->n, h->id, h->inv, nullptr, h->stream));
   }
   // device arrays and page-locked host arrays are written by the store kernel itself (16-byte stores of
-  // whole rows: over the host link this outruns a staging buffer and a copy); pageable host arrays
-  // through the staging buffer and a copy, the positions' copy on a second stream beside the
-  // velocities' store and copy.
-  if (!h->aux) NEP_CUDA(h, cudaStreamCreateWithFlags(&h->aux, cudaStreamNonBlocking));
-  for (cudaEvent_t &ev : h->aux_ev)
-    if (!ev) NEP_CUDA(h, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+  // whole rows: over the host link this outruns a staging buffer and a copy), and so is the page-locked staging of
+  // small pageable arrays; larger ones go through a device buffer and a copy, the positions' copy on a second stream
+  // beside the velocities' store and copy.
+  double *out[2] = {x, v}, *to[2] = {nullptr, nullptr};
+  bool staged[2] = {false, false};
+  for (int k = 0; k < 2; ++k) {
+    if (!out[k]) continue;
+    to[k] = is_device_ptr(out[k]) ? out[k] : pinned_alias(out[k]);
+    if (!to[k] && (to[k] = host_stage(h, k)) != nullptr) staged[k] = true;
+  }
   bool aux_used = false;
-  for (int which = 0; which < 2; ++which) {
-    double *out = which == 0 ? x : v;
-    if (!out) continue;
-    double *direct = is_device_ptr(out) ? out : pinned_alias(out);
-    const bool dev = direct != nullptr;
-    double *stage = dev ? direct : h->io + which * N3;
-    {
-      Scope sc(h, KC_OTHER, 1);
-      if (which == 0) NEP_CUDA(h, launch_store_vec(h->n, h->inv, h->x, h->y, h->z, h->L, 1, stage, h->stream));
-      else NEP_CUDA(h, launch_store_vec(h->n, h->inv, h->vx, h->vy, h->vz, h->L, 0, stage, h->stream));
-    }
-    if (dev) continue;
-    if (which == 0) {
-      NEP_CUDA(h, cudaEventRecord(h->aux_ev[0], h->stream));
-      NEP_CUDA(h, cudaStreamWaitEvent(h->aux, h->aux_ev[0], 0));
-      NEP_CUDA(h, cudaMemcpyAsync(out, stage, N3 * sizeof(double), cudaMemcpyDeviceToHost, h->aux));
-      NEP_CUDA(h, cudaEventRecord(h->aux_ev[1], h->aux));
-      aux_used = true;
-    } else {
-      NEP_CUDA(h, cudaMemcpyAsync(out, stage, N3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  if (to[0] && to[1] && (((uintptr_t)to[0] ^ (uintptr_t)to[1]) & 15) == 0) {
+    Scope sc(h, KC_OTHER, 1);
+    NEP_CUDA(h, launch_store_vec(h->n, h->inv, h->x, h->y, h->z, h->L, 1, to[0], h->vx, h->vy, h->vz, to[1], h->stream));
+  } else {
+    for (int k = 0; k < 2; ++k) {
+      if (!out[k]) continue;
+      double *stage = to[k] ? to[k] : h->io + k * N3;
+      {
+        Scope sc(h, KC_OTHER, 1);
+        NEP_CUDA(h, launch_store_vec(h->n, h->inv, k ? h->vx : h->x, k ? h->vy : h->y, k ? h->vz : h->z, h->L, k ? 0 : 1, stage,
+                                     nullptr, nullptr, nullptr, nullptr, h->stream));
+      }
+      if (to[k]) continue;
+      if (k == 0 && v) {
+        if (!h->aux) NEP_CUDA(h, cudaStreamCreateWithFlags(&h->aux, cudaStreamNonBlocking));
+        for (cudaEvent_t &ev : h->aux_ev)
+          if (!ev) NEP_CUDA(h, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        NEP_CUDA(h, cudaEventRecord(h->aux_ev[0], h->stream));
+        NEP_CUDA(h, cudaStreamWaitEvent(h->aux, h->aux_ev[0], 0));
+        NEP_CUDA(h, cudaMemcpyAsync(x, stage, N3 * sizeof(double), cudaMemcpyDeviceToHost, h->aux));
+        NEP_CUDA(h, cudaEventRecord(h->aux_ev[1], h->aux));
+        aux_used = true;
+      } else {
+        NEP_CUDA(h, cudaMemcpyAsync(out[k], stage, N3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+      }
     }
   }
   if (aux_used) NEP_CUDA(h, cudaStreamWaitEvent(h->stream, h->aux_ev[1], 0));
-  return wait_stream(h);
+  const nep_status s = wait_stream(h);
+  for (int k = 0; k < 2 && s == NEP_OK; ++k)
+    if (staged[k]) std::memcpy(out[k], to[k], N3 * sizeof(double));
+  return s;
 }
 
 nep_status nep_get_thermo(nep_handle *h, double out[8]) {

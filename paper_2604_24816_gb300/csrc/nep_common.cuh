@@ -57,6 +57,7 @@ struct Control {
   int changed;          // an upload into the kept cell order changed some atom's float32 position
   int pending;          // the last MD step's closing half kick is still owed (applied by the next step's
                         // opening kick, or by the kick that ends md_verlet_step)
+  int fb_count;         // atoms the last evaluation handed to the fallback model
 };
 
 // Arguments of the rebuild chain (cell sort + neighbour list).

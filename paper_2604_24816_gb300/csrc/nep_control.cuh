@@ -20,6 +20,7 @@ __device__ __forceinline__ int decide_rebuild(Control *ctrl, int decide) {
     ctrl->steps += 1;
     ctrl->steps_since += 1;
     if (ctrl->rebuild_every > 0 && ctrl->steps_since >= ctrl->rebuild_every) rb = 1;
+    ctrl->fb_count = 0; // of the evaluation to come
     ctrl->pending = 1;  // this step's closing half kick: done by the next step's opening kick or the final one
   }
   if (decide == DECIDE_FORCE) rb = 1;

@@ -115,11 +115,23 @@ __global__ void k_kick(int n, double *__restrict__ vx, double *__restrict__ vy, 
   add_kinetic(sums, acc);
 }
 
-// Kinetic energy only (no kick): for thermo outside MD steps.
+// Forces of slot s to original-order float64 rows.
+__device__ __forceinline__ void store_force(int s, int n, const int *__restrict__ id, const long long *__restrict__ F,
+                                            double *__restrict__ out) {
+  const size_t o = 3 * (size_t)id[s];
+  out[o] = fix_to_double(F[s]);
+  out[o + 1] = fix_to_double(F[(size_t)n + s]);
+  out[o + 2] = fix_to_double(F[2 * (size_t)n + s]);
+}
+
+// Kinetic energy only (no kick): for thermo outside MD steps; with the forces of the evaluation (out, or nullptr) in
+// the caller's order.
 __global__ void k_kinetic(int n, const double *__restrict__ vx, const double *__restrict__ vy,
-                          const double *__restrict__ vz, double mass, const EvalSums sums) {
+                          const double *__restrict__ vz, double mass, const EvalSums sums, const int *__restrict__ id,
+                          const long long *__restrict__ F, double *__restrict__ out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   long long acc[1] = {0};
+  if (i < n && out != nullptr) store_force(i, n, id, F, out);
   if (i < n) acc[0] = __double2ll_rn(0.5 * mass * KE_CONV * (vx[i] * vx[i] + vy[i] * vy[i] + vz[i] * vz[i]) * 4294967296.0);
   add_kinetic(sums, acc);
 }
@@ -147,9 +159,11 @@ __global__ void k_load_state(int n, const double *__restrict__ xin, const double
 // position (so the cell-relative coordinate stays continuous, as between rebuilds), the cell-relative
 // float32 coordinate is refreshed in the slot's cell, and an atom that moved more than skin/2 from
 // the positions the list was built for sets ctrl->moved (the next evaluation then rebuilds).
-// inv[id[s]] = s: the cell-order slot of every atom (original order).
-__global__ void k_inverse_order(int n, const int *__restrict__ id, int *__restrict__ inv) {
+// inv[id[s]] = s: the cell-order slot of every atom (original order).  upload (or nullptr): the control block of an
+// upload that follows, whose status word and change mark are cleared.
+__global__ void k_inverse_order(int n, const int *__restrict__ id, int *__restrict__ inv, Control *upload) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s == 0 && upload != nullptr) upload->status = upload->changed = 0;
   if (s < n) inv[id[s]] = s;
 }
 
@@ -213,11 +227,18 @@ constexpr int MD_STAGE = 256;   // threads per block of the row-staging form
 // WIDE: out is 16-byte aligned; the block's rows go through shared memory and leave with 16-byte stores
 // of consecutive addresses (blockDim.x == MD_STAGE), so page-locked host memory is written by the
 // kernel itself in full lines.
+// A second set (out2 != nullptr: gridDim.y = 2) is written as it is, without the wrap.
 template <bool WIDE>
 __global__ void k_store_vec(int n, const int *__restrict__ inv, const double *__restrict__ a, const double *__restrict__ b,
                             const double *__restrict__ c, double Lx, double Ly, double Lz, int wrap,
-                            double *__restrict__ out) {
+                            double *__restrict__ out, const double *__restrict__ a2, const double *__restrict__ b2,
+                            const double *__restrict__ c2, double *__restrict__ out2) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (blockIdx.y == 1) {
+    a = a2; b = b2; c = c2;
+    out = out2;
+    wrap = 0;
+  }
   __shared__ double so[WIDE ? 3 * MD_STAGE : 1];
   if (i < n) {
     const int s = inv[i];
@@ -247,11 +268,7 @@ __global__ void k_store_vec(int n, const int *__restrict__ inv, const double *__
 __global__ void k_store_force(int n, const int *__restrict__ id, const long long *__restrict__ F,
                               double *__restrict__ out) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const size_t o = 3 * (size_t)id[s];
-  out[o] = fix_to_double(F[s]);
-  out[o + 1] = fix_to_double(F[(size_t)n + s]);
-  out[o + 2] = fix_to_double(F[2 * (size_t)n + s]);
+  if (s < n) store_force(s, n, id, F, out);
 }
 
 __global__ void k_store_scalar(int n, const int *__restrict__ id, const float *__restrict__ u, double *__restrict__ out) {
@@ -315,8 +332,8 @@ cudaError_t launch_kick(int n, double *vx, double *vy, double *vz, const long lo
 }
 
 cudaError_t launch_kinetic(int n, const double *vx, const double *vy, const double *vz, double mass,
-                           const EvalSums &sums, cudaStream_t st) {
-  if (n > 0) k_kinetic<<<bl(n, MD_BLOCK), MD_BLOCK, 0, st>>>(n, vx, vy, vz, mass, sums);
+                           const EvalSums &sums, const int *id, const long long *F, double *out, cudaStream_t st) {
+  if (n > 0) k_kinetic<<<bl(n, MD_BLOCK), MD_BLOCK, 0, st>>>(n, vx, vy, vz, mass, sums, id, F, out);
   return cudaGetLastError();
 }
 
@@ -326,8 +343,8 @@ cudaError_t launch_load_state(int n, const double *xin, const double *vin, doubl
   return cudaGetLastError();
 }
 
-cudaError_t launch_inverse_order(int n, const int *id, int *inv, cudaStream_t st) {
-  if (n > 0) k_inverse_order<<<bl(n, 256), 256, 0, st>>>(n, id, inv);
+cudaError_t launch_inverse_order(int n, const int *id, int *inv, Control *upload, cudaStream_t st) {
+  if (n > 0) k_inverse_order<<<bl(n, 256), 256, 0, st>>>(n, id, inv, upload);
   return cudaGetLastError();
 }
 
@@ -342,12 +359,14 @@ cudaError_t launch_load_state_sorted(int n, const double *xin, const double *vin
 }
 
 cudaError_t launch_store_vec(int n, const int *inv, const double *a, const double *b, const double *c, const double L[3],
-                             int wrap, double *out, cudaStream_t st) {
+                             int wrap, double *out, const double *a2, const double *b2, const double *c2, double *out2,
+                             cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  if (((uintptr_t)out & 15) == 0)
-    k_store_vec<true><<<bl(n, MD_STAGE), MD_STAGE, 0, st>>>(n, inv, a, b, c, L[0], L[1], L[2], wrap, out);
+  const dim3 grid(bl(n, MD_STAGE), out2 != nullptr ? 2 : 1);
+  if ((((uintptr_t)out | (uintptr_t)out2) & 15) == 0)
+    k_store_vec<true><<<grid, MD_STAGE, 0, st>>>(n, inv, a, b, c, L[0], L[1], L[2], wrap, out, a2, b2, c2, out2);
   else
-    k_store_vec<false><<<bl(n, 256), 256, 0, st>>>(n, inv, a, b, c, L[0], L[1], L[2], wrap, out);
+    k_store_vec<false><<<grid, MD_STAGE, 0, st>>>(n, inv, a, b, c, L[0], L[1], L[2], wrap, out, a2, b2, c2, out2);
   return cudaGetLastError();
 }
 
