@@ -730,13 +730,14 @@ __device__ __forceinline__ void lj_pair(const Model<S> &P, float r2, float r, fl
   de = fmaf(ir6 * fmaf(P.lj_m12, ir6, P.lj_p6), ir, -P.lj_de_rc);
 }
 
-// lj_pair's derivative dE/dr for two pairs at once.
+// lj_pair for two pairs at once.
 template <class S>
-__device__ __forceinline__ float2 lj_deriv_x2(const Model<S> &P, float2 r2, float2 ir) {
+__device__ __forceinline__ void lj_pair_x2(const Model<S> &P, float2 r2, float2 r, float2 ir, float2 &e, float2 &de) {
   float2 ir2 = mul2(ir, ir);
   ir2 = fma2(ir2, fma2(make_float2(-r2.x, -r2.y), ir2, bc2(1.f)), ir2);
   const float2 ir6 = mul2(mul2(ir2, ir2), ir2);
-  return fma2(mul2(ir6, fma2(bc2(P.lj_m12), ir6, bc2(P.lj_p6))), ir, bc2(-P.lj_de_rc));
+  e = fma2(ir6, fma2(bc2(P.lj_c12), ir6, bc2(-P.lj_c6)), fma2(bc2(-P.lj_de_rc), r, bc2(P.lj_e0)));
+  de = fma2(mul2(ir6, fma2(bc2(P.lj_m12), ir6, bc2(P.lj_p6))), ir, bc2(-P.lj_de_rc));
 }
 
 // Exact conversion of a float to 64-bit fixed point with 32 fractional bits, without a 64-bit

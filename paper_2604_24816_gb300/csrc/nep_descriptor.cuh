@@ -132,7 +132,7 @@ __device__ __forceinline__ void accumulate_atom(const Model<S> &P, const float4 
       cheb_accumulate(r, P.inv_rcR, Q);
       ++A.nrad;
     }
-    if (P.lj_on != 0.f && r2 < P.lj_rc2) {
+    if (!REC && P.lj_on != 0.f && r2 < P.lj_rc2) {
       float el, dl;
       lj_pair<S>(P, r2, r, ir, el, dl);
       A.elj = fmaf(0.5f, el, A.elj);
@@ -423,7 +423,7 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
         cheb_accumulate(r, P.inv_rcR, Q);
         ++nrad;
       }
-      if (P.lj_on != 0.f && r2 < P.lj_rc2) {
+      if (!REC && P.lj_on != 0.f && r2 < P.lj_rc2) {
         float el, dl;
         lj_pair<S>(P, r2, r, ir, el, dl);
         elj = fmaf(0.5f, el, elj);

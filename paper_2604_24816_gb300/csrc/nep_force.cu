@@ -452,14 +452,16 @@ __device__ __forceinline__ void force_pairs(const Model<S> &P, const float4 *shi
 // nr other active pairs (slots pmax-1 down to pmax-nr; no TMEM).  Each pair gets the arithmetic of
 // force_pairs<S, float, false, true> on the displacement the descriptor walk computed: d_ij added to F_i,
 // subtracted from F_j (fixed point), W -= r_ij (x) d_ij (upper triangle, mirrored).  The row is over the
-// solid harmonics (angular_pair_solid), the radial tail at fps in radial_tail_cubics' form.
+// solid harmonics (angular_pair_solid), the radial tail at fps in radial_tail_cubics' form.  elj: the atom's half of
+// its pairs' LJ energy, which here costs three instructions beside the derivative and in the descriptor walk twelve.
 template <class S, int DQ, class Row>
 __device__ __forceinline__ void force_pairs_rec(const Model<S> &P, const Row &row, const float4 *fps, int i, bool live,
                                                 int n, const float4 *rec, unsigned off, int pmax, int na, int nr,
                                                 float4 *ring,
                                                 unsigned long long *__restrict__ Ffix, int *__restrict__ status,
-                                                long long (&acc)[13]) {
+                                                long long (&acc)[13], float &elj) {
   constexpr bool TM = ForceCfg<S>::TM;
+  float2 e2 = bc2(0.f);
   float fx = 0.f, fy = 0.f, fz = 0.f;
   float wxx = 0.f, wxy = 0.f, wxz = 0.f, wyy = 0.f, wyz = 0.f, wzz = 0.f;
   auto apply = [&](float dx, float dy, float dz, int j, float coef, float vx, float vy, float vz) {
@@ -485,7 +487,7 @@ __device__ __forceinline__ void force_pairs_rec(const Model<S> &P, const Row &ro
       const float r2 = q.x * q.x + q.y * q.y + q.z * q.z;
       const float ir = rsqrtf(r2);
       const float r = r2 * ir;
-      float coef = valid ? radial_lj_coef<S, true>(P, fps[0], fps[FORCE_BLOCK], r2, r, ir) : 0.f;
+      float coef = valid ? radial_lj_coef<S, true>(P, fps[0], fps[FORCE_BLOCK], r2, r, ir, &e2.x) : 0.f;
       if constexpr (TM) __syncwarp();
       float ca, vx, vy, vz;
       angular_pair_solid<S>(P, row, !valid, r, ir, q.x, q.y, q.z, ca, vx, vy, vz);
@@ -517,7 +519,9 @@ __device__ __forceinline__ void force_pairs_rec(const Model<S> &P, const Row &ro
         if (P.lj_on != 0.f) {
           const bool la = r2.x < P.lj_rc2, lb = r2.y < P.lj_rc2;
           if (la || lb) {
-            const float2 dl = lj_deriv_x2<S>(P, r2, ir);
+            float2 el, dl;
+            lj_pair_x2<S>(P, r2, r, ir, el, dl);
+            e2 = add2(e2, pr(la ? el.x : 0.f, lb ? el.y : 0.f));
             const float2 t = mul2(mul2(bc2(0.5f), dl), ir);
             coef = add2(coef, pr(la ? t.x : 0.f, lb ? t.y : 0.f));
           }
@@ -531,10 +535,11 @@ __device__ __forceinline__ void force_pairs_rec(const Model<S> &P, const Row &ro
       const float r2 = q.x * q.x + q.y * q.y + q.z * q.z;
       const float ir = rsqrtf(r2);
       const float r = r2 * ir;
-      apply(q.x, q.y, q.z, __float_as_int(q.w), radial_lj_coef<S>(P, fps[0], fps[FORCE_BLOCK], r2, r, ir), 0.f, 0.f, 0.f);
+      apply(q.x, q.y, q.z, __float_as_int(q.w), radial_lj_coef<S>(P, fps[0], fps[FORCE_BLOCK], r2, r, ir, &e2.x), 0.f, 0.f, 0.f);
     }
     pb.finish();
   }
+  elj = 0.5f * (e2.x + e2.y);
   if (live) {
     red_add(Ffix + i, to_fix32(fx));
     red_add(Ffix + (size_t)n + i, to_fix32(fy));
@@ -544,6 +549,20 @@ __device__ __forceinline__ void force_pairs_rec(const Model<S> &P, const Row &ro
     acc[3] = acc[1]; acc[4] = -to_fix32(wyy); acc[5] = -to_fix32(wyz);
     acc[6] = acc[2]; acc[7] = acc[5]; acc[8] = -to_fix32(wzz);
   }
+}
+
+// The site energy u + elj after the force pass: stored, and its warp's sum (lane 0) into the block's first partial.
+__device__ __forceinline__ void site_energy(float u, float elj, bool live, int i, float *usite, int *status,
+                                            long long &part) {
+  const float ui = u + elj;
+  long long e[1] = {0};
+  if (live) {
+    usite[i] = ui;
+    if (!isfinite(ui)) atomicOr(status, ST_NAN);
+    e[0] = to_fix32(ui);
+  }
+  __syncwarp();                                        // the counters' lane 0 has cleared this partial
+  warp_sum_stage<1>(e, &part);
 }
 
 // FULL = true walks the whole row with atom i's own adjoint only; FULL = false walks the owned half
@@ -669,6 +688,7 @@ k_nep_fused(const __grid_constant__ Model<S> P, const Geom geom, const int n, co
   __shared__ uint32_t tmem_base;
   __shared__ __align__(16) NetSmem<S> net;
   __shared__ float4 fp_s[2 * DESC_BLOCK];
+  __shared__ float u_s[DESC_BLOCK];                 // the network's energies, until the pair energies are known
   __shared__ int s_slot;
   if (threadIdx.x < 32) tmem_alloc(&tmem_base, TCOLS);
   if (threadIdx.x == 0) {
@@ -730,11 +750,8 @@ k_nep_fused(const __grid_constant__ Model<S> P, const Geom geom, const int n, co
   }
   long long acc_d[5] = {0, 0, 0, 0, 0};
   long long acc_f[13] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  u_s[threadIdx.x] = U;
   if (live) {
-    const float ui = U + elj;
-    usite[i] = ui;
-    if (!isfinite(ui)) atomicOr(status, ST_NAN);
-    acc_d[0] = to_fix32(ui);
     acc_d[1] = nrad;
     acc_d[2] = nang;
     acc_d[3] = cnt;
@@ -742,15 +759,16 @@ k_nep_fused(const __grid_constant__ Model<S> P, const Geom geom, const int n, co
     // the force pass visits the descriptor walk's active pairs
     acc_f[9] = cnt; acc_f[10] = nact; acc_f[11] = nrad; acc_f[12] = nang;
   }
-  // the energy and counters: summed over the warp now (fewer live registers in the force pass), over
-  // the block after the closing barrier
+  // the counters: summed over the warp now (fewer live registers in the force pass), over the block after the
+  // closing barrier
   __shared__ long long wsum_d[DESC_BLOCK / 32][5], wsum_f[DESC_BLOCK / 32][13];
   warp_sum_stage<5>(acc_d, wsum_d[threadIdx.x >> 5]);
 
   // forces: every active pair of the row with the own adjoint row, from the pair records
   force_pairs_rec<S, PIPE_DP>(P, RowTmem<S>{trow}, fp_s + threadIdx.x, i, live, n, pc.rec, rec_off, pc.pmax, nang,
-                                    nact - nang, ring_p, Ffix, status, acc_f);
+                                    nact - nang, ring_p, Ffix, status, acc_f, elj);
   warp_sum_stage<13>(acc_f, wsum_f[threadIdx.x >> 5]);
+  site_energy(u_s[threadIdx.x], elj, live, i, usite, status, wsum_d[threadIdx.x >> 5][0]);
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x < 32) {
@@ -788,6 +806,7 @@ k_nep_fused_reg(const __grid_constant__ Model<S> P, const Geom geom, const int n
   __shared__ uint32_t ring_e[PIPE_DE * DESC_BLOCK];
   __shared__ float4 ring_p[PIPE_DP * DESC_BLOCK];
   __shared__ float4 fp_s[2 * DESC_BLOCK];
+  __shared__ float u_s[DESC_BLOCK];                 // the network's energies, until the pair energies are known
   __shared__ int s_slot;
   if (threadIdx.x == 0) {
     const int slot = acquire_record_slot(pc);
@@ -802,6 +821,7 @@ k_nep_fused_reg(const __grid_constant__ Model<S> P, const Geom geom, const int n
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   long long acc_d[5] = {0, 0, 0, 0, 0};
   long long acc_f[13] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  float elj = 0.f;
   if (i < n) {
     AtomSums<S> A;
     accumulate_atom<S, PIPE_DE, PIPE_DP, DESC_BLOCK, true, true>(P, shift, i, n, pos, nbr, full_row(X, i, skip_far(X)),
@@ -825,21 +845,19 @@ k_nep_fused_reg(const __grid_constant__ Model<S> P, const Geom geom, const int n
       radial_tail<S>(P, Fp, tail);
       radial_tail_cubics(tail, fp_s[threadIdx.x], fp_s[DESC_BLOCK + threadIdx.x]);   // the force pass's form (force_pairs_rec)
     }
-    const float ui = flagged ? A.elj : U + A.elj;
-    usite[i] = ui;
-    if (!isfinite(ui)) atomicOr(status, ST_NAN);
-    acc_d[0] = to_fix32(ui);
+    u_s[threadIdx.x] = flagged ? 0.f : U;
     acc_d[1] = A.nrad;
     acc_d[2] = A.nang;
     acc_d[3] = A.cnt;
     acc_d[4] = A.nact;
     acc_f[9] = A.cnt; acc_f[10] = A.nact; acc_f[11] = A.nrad; acc_f[12] = A.nang;
     force_pairs_rec<S, PIPE_DP>(P, RowReg<S>{gi}, fp_s + threadIdx.x, i, true, n, pc.rec, rec_off, pc.pmax, A.nang,
-                                A.nact - A.nang, ring_p, Ffix, status, acc_f);
+                                A.nact - A.nang, ring_p, Ffix, status, acc_f, elj);
   }
   __shared__ long long wsum_d[DESC_BLOCK / 32][5], wsum_f[DESC_BLOCK / 32][13];
   warp_sum_stage<5>(acc_d, wsum_d[threadIdx.x >> 5]);
   warp_sum_stage<13>(acc_f, wsum_f[threadIdx.x >> 5]);
+  site_energy(u_s[threadIdx.x], elj, i < n, i, usite, status, wsum_d[threadIdx.x >> 5][0]);
   __syncthreads();
   if (threadIdx.x == 0 && slot >= 0) {
     __threadfence();          // this block's record reads are complete (cp.async waited, barrier above)
@@ -887,6 +905,7 @@ k_nep_fused_mixed(const __grid_constant__ Model<S> P, const Geom geom, const int
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tmem_base;
   __shared__ float4 fp_s[2 * DESC_BLOCK];
+  __shared__ float u_s[DESC_BLOCK];                 // the network's energies, until the pair energies are known
   __shared__ int s_slot;
   const int t = threadIdx.x;
   if (t < 32) {
@@ -1025,11 +1044,8 @@ k_nep_fused_mixed(const __grid_constant__ Model<S> P, const Geom geom, const int
   }
   long long acc_d[5] = {0, 0, 0, 0, 0};
   long long acc_f[13] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  u_s[threadIdx.x] = U;
   if (live) {
-    const float ui = U + elj;
-    usite[i] = ui;
-    if (!isfinite(ui)) atomicOr(status, ST_NAN);
-    acc_d[0] = to_fix32(ui);
     acc_d[1] = nrad;
     acc_d[2] = nang;
     acc_d[3] = cnt;
@@ -1039,8 +1055,9 @@ k_nep_fused_mixed(const __grid_constant__ Model<S> P, const Geom geom, const int
   __shared__ long long wsum_d[DESC_BLOCK / 32][5], wsum_f[DESC_BLOCK / 32][13];
   warp_sum_stage<5>(acc_d, wsum_d[t >> 5]);
   force_pairs_rec<S, PIPE_DP>(P, RowTmem<S>{trow}, fp_s + t, i, live, n, pc.rec, rec_off, pc.pmax, nang, nact - nang, ring_p,
-                              Ffix, status, acc_f);
+                              Ffix, status, acc_f, elj);
   warp_sum_stage<13>(acc_f, wsum_f[threadIdx.x >> 5]);
+  site_energy(u_s[threadIdx.x], elj, live, i, usite, status, wsum_d[threadIdx.x >> 5][0]);
   tc_fence_before();
   __syncthreads();
   if (t < 32) {

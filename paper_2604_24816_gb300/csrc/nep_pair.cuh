@@ -86,15 +86,17 @@ __device__ __forceinline__ void angular_pair_solid(const Model<S> &P, const Row 
 // Radial and LJ part of one active pair's force coefficient (d = coef * r_ij + angular part): the
 // radial adjoint (the two cubics c0, c1 of radial_tail_cubics) against the basis derivatives, plus half of the shifted-force LJ pair force.  INSIDE_RC: the caller knows that
 // r < rc_R (an angular pair: rc_A <= rc_R is checked by nep_create).  LJ = false: without
-// the pair term.
+// the pair term.  e2: gets the pair's LJ energy added.
 template <class S, bool INSIDE_RC = false, bool LJ = true>
-__device__ __forceinline__ float radial_lj_coef(const Model<S> &P, float4 c0, float4 c1, float r2, float r, float ir) {
+__device__ __forceinline__ float radial_lj_coef(const Model<S> &P, float4 c0, float4 c1, float r2, float r, float ir,
+                                                float *e2 = nullptr) {
   float coef = 0.f;
   if (INSIDE_RC || r2 < P.rcR2) coef = cubics_deriv(c0, c1, r, P.inv_rcR) * ir;
   if (LJ && P.lj_on != 0.f && r2 < P.lj_rc2) {
     float el, dl;
     lj_pair<S>(P, r2, r, ir, el, dl);
     coef = fmaf(0.5f * dl, ir, coef);
+    if (e2 != nullptr) *e2 += el;
   }
   return coef;
 }
