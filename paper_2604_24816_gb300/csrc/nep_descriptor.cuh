@@ -113,6 +113,8 @@ __device__ __forceinline__ void accumulate_atom(const Model<S> &P, const float4 
   A.nrad = 0; A.nang = 0; A.nact = 0; A.cnt = cnt;
   NbrPipe<DE, DP, BLOCK> pipe;
   pipe.start(ring_e, ring_p, nbr + i, (size_t)n, pos, sp);
+  const unsigned last = off + (unsigned)(pmax - 1) * BLOCK;
+  unsigned oa = off, oo = last;                        // REC: where the next angular and the next other record go
   for (int k = 0; k < cnt; ++k) {
     uint32_t e;
     float4 pj;
@@ -122,15 +124,18 @@ __device__ __forceinline__ void accumulate_atom(const Model<S> &P, const float4 
     const float r2 = dx * dx + dy * dy + dz * dz;
     if (r2 >= P.rmax2) continue;
     if constexpr (REC) {
-      const int slot = r2 < P.rcA2 ? A.nang : pmax - 1 - (A.nact - A.nang);
-      rec[off + (unsigned)slot * BLOCK] = make_float4(dx, dy, dz, __int_as_float((int)(e & J_MASK)));
+      const bool in_a = r2 < P.rcA2;
+      rec[in_a ? oa : oo] = make_float4(dx, dy, dz, __int_as_float((int)(e & J_MASK)));
+      if (in_a) oa += BLOCK;
+      else oo -= BLOCK;
+    } else {
+      ++A.nact;
     }
-    ++A.nact;
     const float ir = rsqrtf(r2);
     const float r = r2 * ir;
-    if (r2 < P.rcR2) {
+    if (REC || r2 < P.rcR2) {                          // (the pair term's cutoff is at most rc_R: nep_create)
       cheb_accumulate(r, P.inv_rcR, Q);
-      ++A.nrad;
+      if (!REC) ++A.nrad;
     }
     if (!REC && P.lj_on != 0.f && r2 < P.lj_rc2) {
       float el, dl;
@@ -156,8 +161,12 @@ __device__ __forceinline__ void accumulate_atom(const Model<S> &P, const float4 
       for (int a = 0; a < S::NA; ++a)
 #pragma unroll
         for (int c = 0; c < S::NLM; ++c) A.s[a][c] = fmaf(g[a], Y[c], A.s[a][c]);
-      ++A.nang;
+      if (!REC) ++A.nang;
     }
+  }
+  if constexpr (REC) {
+    A.nang = (int)((oa - off) / BLOCK);
+    A.nact = A.nrad = A.nang + (int)((last - oo) / BLOCK);
   }
   pipe.finish();
   cheb_sums(Q, A.QR);
@@ -399,6 +408,8 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
   NbrPipe<DE, DP, BLOCK> pipe;
   pipe.start(ring_e, ring_p, nbr + ii, (size_t)n, pos, sp);
   const int trip = __reduce_max_sync(0xffffffffu, cnt);
+  const unsigned last = off + (unsigned)(pmax - 1) * BLOCK;
+  unsigned oa = off, oo = last;                        // REC: where the next angular and the next other record go
   for (int k = 0; k < trip; ++k) {
     const bool valid = k < cnt;
     uint32_t e;
@@ -415,13 +426,16 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
     const float r = r2 * ir;
     if (act) {
       if constexpr (REC) {
-        const int slot = r2 < P.rcA2 ? nang : pmax - 1 - (nact - nang);
-        rec[off + (unsigned)slot * BLOCK] = make_float4(dx, dy, dz, __int_as_float((int)(e & J_MASK)));
+        const bool in_a = r2 < P.rcA2;
+        rec[in_a ? oa : oo] = make_float4(dx, dy, dz, __int_as_float((int)(e & J_MASK)));
+        if (in_a) oa += BLOCK;
+        else oo -= BLOCK;
+      } else {
+        ++nact;
       }
-      ++nact;
-      if (r2 < P.rcR2) {
+      if (REC || r2 < P.rcR2) {                        // (the pair term's cutoff is at most rc_R: nep_create)
         cheb_accumulate(r, P.inv_rcR, Q);
-        ++nrad;
+        if (!REC) ++nrad;
       }
       if (!REC && P.lj_on != 0.f && r2 < P.lj_rc2) {
         float el, dl;
@@ -467,8 +481,12 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
 #pragma unroll
         for (int c = 0; c < S::NLM; ++c) R.s[a - NT][c] = fmaf(g[a], Y[c], R.s[a - NT][c]);
       tmem_wait_st();
-      if (ang) ++nang;
+      if (!REC && ang) ++nang;
     }
+  }
+  if constexpr (REC) {
+    nang = (int)((oa - off) / BLOCK);
+    nact = nrad = nang + (int)((last - oo) / BLOCK);
   }
   pipe.finish();
   cheb_sums(Q, QR);

@@ -510,12 +510,7 @@ __device__ __forceinline__ void force_pairs_rec(const Model<S> &P, const Row &ro
         const float2 r2 = fma2(dzv, dzv, fma2(dyv, dyv, mul2(dxv, dxv)));
         const float2 ir = pr(rsqrtf(r2.x), rsqrtf(r2.y));
         const float2 r = mul2(r2, ir);
-        float2 coef = bc2(0.f);
-        const bool ra = r2.x < P.rcR2, rb = r2.y < P.rcR2;
-        if (ra || rb) {
-          const float2 dot = mul2(cubics_deriv_x2(ta, tb, r, P.inv_rcR), ir);
-          coef = pr(ra ? dot.x : 0.f, rb ? dot.y : 0.f);
-        }
+        float2 coef = mul2(cubics_deriv_x2(ta, tb, r, P.inv_rcR), ir);   // every record is inside rc_R
         if (P.lj_on != 0.f) {
           const bool la = r2.x < P.lj_rc2, lb = r2.y < P.lj_rc2;
           if (la || lb) {
@@ -535,7 +530,8 @@ __device__ __forceinline__ void force_pairs_rec(const Model<S> &P, const Row &ro
       const float r2 = q.x * q.x + q.y * q.y + q.z * q.z;
       const float ir = rsqrtf(r2);
       const float r = r2 * ir;
-      apply(q.x, q.y, q.z, __float_as_int(q.w), radial_lj_coef<S>(P, fps[0], fps[FORCE_BLOCK], r2, r, ir, &e2.x), 0.f, 0.f, 0.f);
+      apply(q.x, q.y, q.z, __float_as_int(q.w), radial_lj_coef<S, true>(P, fps[0], fps[FORCE_BLOCK], r2, r, ir, &e2.x), 0.f, 0.f,
+            0.f);
     }
     pb.finish();
   }
