@@ -360,7 +360,7 @@ __device__ __forceinline__ void wide_body(WideShared<S, G> &M, const Model<S> &P
     float U = 0.f;
     for (int mu = gl; mu < S::NNEU; mu += G) {
       const float z = dot4<NV>(net.W0 + mu * LD, A.q, -net.b0[mu]);
-      const float h = MIX ? tanh_sfu(z) : tanhf(z);
+      const float h = MIX && S::NLM > 8 ? tanh_sfu(z) : tanhf(z);   // as the forms of one thread per atom
       U = fmaf(net.w1[mu], h, U);
       A.t[mu] = round_to<MT>(net.w1[mu] * (1.f - h * h));
     }
