@@ -40,10 +40,11 @@ cudaError_t launch_fused(const Model<S> &, const Geom &, int, const float4 *, co
 template <class S, class MT>
 cudaError_t launch_fused_mixed(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
                                float *, float *, long long *, const EvalSums &, int *, const PairCache &, cudaStream_t);
-template <class S>
+template <class S, class MT>
 cudaError_t launch_fused_reg(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
                              float *, float *, long long *, const EvalSums &, int *, const Fallback &,
                              const PairCache &, cudaStream_t);
+cudaError_t fused_reg_resident(int *atoms);
 cudaError_t pair_cache_sm_bound(int *nsm);
 size_t pair_cache_region_elems(int pmax);
 // nep_mixed.cu
@@ -192,6 +193,7 @@ struct nep_handle {
   double *io = nullptr;            // staging 2 x [n][3] float64 for host transfers
   int32_t *io_i = nullptr;         // staging for neighbour output
   size_t io_i_elems = 0;
+  bool split = false;              // the mixed student in two kernels (student_split)
   int wide = 0;                    // lanes per atom of the wide kernels, 0: one thread per atom
 
   // host mirror (pinned)
@@ -444,6 +446,22 @@ cudaError_t enqueue_fallback(nep_handle *h, const Geom &g) {
                                    h->usite, h->F, eval_sums(h, true), &h->ctrl->status, h->stream);
 }
 
+// Whether the mixed student of the current size runs as two kernels (tensor-core descriptor kernel, half-list force
+// kernel over float16 rows) instead of the fused one.  The fused kernel needs no rows in memory and no gathers, but keeps
+// 97,280 atoms resident (R: 152 SMs x 5 blocks) and leaves the chip half empty in a second round that is less than half
+// full; the two kernels' rounds differ (6 and 4 blocks).  MD steps, fused and split: 55,296 atoms 73 and 81 us, 94,192
+// (0.97 R) 113 and 124, 108,000 (1.11 R) 138 and 134, 123,008 151 and 149, 139,392 (1.43 R) 159 and 157, 166,600 (1.71 R)
+// 177 and 191, 256,000 255 and 275, 1,048,576 850 and 952.
+bool student_split(nep_handle *h) {
+  if (h->shape != 1 || h->precision == NEP_FP32) return false;
+  int R = 0;
+  if (fused_reg_resident(&R) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return h->n > R && h->n <= R + R / 2;
+}
+
 // Descriptors + network + forces, energy, virial and counters.  zeroed: the forces are already clear (the drift
 // kernel of an MD step clears them).
 template <class S>
@@ -459,7 +477,7 @@ cudaError_t forces_of(nep_handle *h, const Model<S> &M, float *qout, bool zeroed
   cudaError_t e;
   // (an MD step's rebuild decision has cleared the count)
   if (fb.on && !zeroed && (e = cudaMemsetAsync(h->fb_count, 0, sizeof(int), h->stream)) != cudaSuccess) return e;
-  if (h->wide > 0 || teacher || h->precision == NEP_FP32) {
+  if (!h->split) {
     // descriptors, network and full-row forces in one kernel, then the teacher on the flagged atoms; the network
     // in float32, or with bf16 / f16 operands in the mixed-precision forms
     {
@@ -492,8 +510,15 @@ cudaError_t forces_of(nep_handle *h, const Model<S> &M, float *qout, bool zeroed
             e = launch_fused_mixed<CuShape, __half>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status,
                                                     pc, h->stream);
         } else {
-          e = launch_fused_reg<StudentShape>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status, fb, pc,
-                                             h->stream);
+          if (h->precision == NEP_FP32)
+            e = launch_fused_reg<S, float>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status, fb, pc,
+                                           h->stream);
+          else if (h->precision == NEP_MIX_BF16)
+            e = launch_fused_reg<S, __nv_bfloat16>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status, fb,
+                                                   pc, h->stream);
+          else
+            e = launch_fused_reg<S, __half>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status, fb, pc,
+                                            h->stream);
         }
       }
     }
@@ -850,6 +875,10 @@ nep_status nep_create(const nep_params *p, void *cuda_stream, nep_handle **out) 
   h->shape = shape;
   if (shape == 0) fill_model(h->model_t, p);
   else fill_model(h->model_s, p);
+  if (p->precision != NEP_FP32)                        // the mixed student's kernels read W0 as their products use it
+    for (auto &row : h->model_s.W0)
+      for (float &w : row)
+        w = p->precision == NEP_MIX_BF16 ? __bfloat162float(__float2bfloat16_rn(w)) : __half2float(__float2half_rn(w));
   h->mass = p->mass_amu;
   h->skin = p->skin;
   h->rcR = p->rc_R;
@@ -939,6 +968,7 @@ nep_status nep_set_state(nep_handle *h, int64_t n, const double *x, const double
   h->ssh = slice_shift(h->n, ncell);
   h->ncell = (int)(ncell << h->ssh);
   h->wide = wide_lanes(h->n);
+  h->split = h->wide == 0 && student_split(h);
   const size_t N = (size_t)std::max(h->n, 1);
   cudaError_t e = cudaSuccess;
   auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
@@ -947,14 +977,15 @@ nep_status nep_set_state(nep_handle *h, int64_t n, const double *x, const double
   A(dalloc(h->id, N)); A(dalloc(h->idb, N)); A(dalloc(h->cell_of, N)); A(dalloc(h->perm, N)); A(dalloc(h->inv, N));
   A(dalloc(h->pos, N)); A(dalloc(h->pos_ref, N));
   A(dalloc(h->F, 3 * N)); A(dalloc(h->usite, N));
-  A(dalloc(reinterpret_cast<char *&>(h->G), N * (size_t)h->gs() * (h->precision == NEP_FP32 ? 4 : 2)));
+  if (h->split || (h->shape == 0 && h->precision == NEP_FP32))   // else no kernel keeps adjoint rows
+    A(dalloc(reinterpret_cast<char *&>(h->G), N * (size_t)h->gs() * (h->precision == NEP_FP32 ? 4 : 2)));
   A(dalloc(h->nbr, N * (size_t)h->cap)); A(dalloc(h->nnum, N)); A(dalloc(h->nang, N)); A(dalloc(h->nown, N));
   A(dalloc(h->nband0, N)); A(dalloc(h->nfar, N));
   A(dalloc(h->count, (size_t)h->ncell)); A(dalloc(h->cursor, (size_t)h->ncell)); A(dalloc(h->start, (size_t)h->ncell + 1));
   A(dalloc(h->tile_sums, (size_t)scan_tiles(h->ncell) + 1));
   A(dalloc(h->io, 6 * N));
   if (h->fb_on) A(alloc_fallback(h));
-  if (e == cudaSuccess && h->wide == 0 && (h->shape == 0 || h->precision == NEP_FP32)) {
+  if (e == cudaSuccess && h->wide == 0 && !h->split) {
     // pair records of the fused kernels: pc_slots regions per SM index, list capacity records per atom
     h->pc_slots = h->shape == 0 ? PC_SLOTS : PC_SLOTS_REG;
     A(pair_cache_sm_bound(&h->pc_nsm));

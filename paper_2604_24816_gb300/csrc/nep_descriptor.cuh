@@ -234,12 +234,13 @@ __device__ __forceinline__ void descriptors_of(const Model<S> &P, const AtomSums
 // The one-hidden-layer network (Section III.B equation): U = sum_mu w1_mu tanh(sum_nu W0_mu,nu q~_nu -
 // b0_mu) - b1 with q~ = q_scale q; returns U and Fp_nu = dU/dq_nu (zero for an atom flagged for the
 // fallback model, whose site energy comes from the other model).
-template <class S>
+// MT: the operands of its two products are rounded to that type (W0 by the host already), sums in float32.
+template <class S, class MT = float>
 __device__ __forceinline__ float network(const Model<S> &P, const float (&q)[S::NDES], bool flagged,
                                          float (&Fp)[S::NDES]) {
   float qt[S::NDES], dq[S::NDES];
 #pragma unroll
-  for (int v = 0; v < S::NDES; ++v) { qt[v] = q[v] * P.qs[v]; dq[v] = 0.f; }
+  for (int v = 0; v < S::NDES; ++v) { qt[v] = round_to<MT>(q[v] * P.qs[v]); dq[v] = 0.f; }
   float U = -P.b1;
   // The teacher's 30 x 30 network, fully unrolled, is ~2k instructions of straight-line code that the
   // row-walk loops share the instruction cache with; one neuron per iteration (weights read from the
@@ -252,7 +253,7 @@ __device__ __forceinline__ float network(const Model<S> &P, const float (&q)[S::
     for (int v = 0; v < S::NDES; ++v) z = fmaf(P.W0[mu][v], qt[v], z);
     const float h = tanhf(z);
     U = fmaf(P.w1[mu], h, U);
-    const float t = P.w1[mu] * (1.f - h * h);
+    const float t = round_to<MT>(P.w1[mu] * (1.f - h * h));
 #pragma unroll
     for (int v = 0; v < S::NDES; ++v) dq[v] = fmaf(t, P.W0[mu][v], dq[v]);
   }

@@ -18,8 +18,8 @@
 //                full row (the float32 teacher): every ordered pair (i, j) of i's row gives
 //                d_ij = dU_i/dr_ij from atom i's own row only -- radial sum_k dU/dQ_k f_k'(r) r^, angular
 //                sum_nlm G_nlm d[g_n(r) Yh_lm(u)]/dr_ij, half of the LJ pair force -- which is added to F_i
-//                and subtracted from F_j; no neighbour row is read.  Half list (float16 rows, the
-//                student): D_ij = dU_i/dr_ij - dU_j/dr_ji for each unordered pair once, by its owner (the
+//                and subtracted from F_j; no neighbour row is read.  Half list (float16 rows of
+//                the mixed student's two-kernel form): D_ij = dU_i/dr_ij - dU_j/dr_ji for each unordered pair once, by its owner (the
 //                owned part of the list), with H_nlm = G^i_nlm + (-1)^l G^j_nlm because the pair geometry
 //                g_n(r) Yh_lm(u) is shared by both directions (Yh_lm(-u) = (-1)^l Yh_lm(u)) and D_ji = -D_ij
 //                exactly; the owner adds D_ij to F_i and -D_ij to F_j.  The scatter uses 64-bit fixed-point
@@ -786,11 +786,12 @@ k_nep_fused(const __grid_constant__ Model<S> P, const Geom geom, const int n, co
 // the fallback on, an atom whose descriptors leave the training range is flagged as in k_descriptor
 // (zero adjoint row, LJ energy only), and the teacher kernels then add its own model's part.  Ffix is
 // zeroed by the caller before the launch.  Five resident blocks (at most 102 registers) measured 4 %
-// faster than four.
+// faster than four.  MT = __nv_bfloat16 / __half (the mixed student): the network's operands rounded to that type, W0 by
+// the host; 16 neurons of 12 inputs cost less here than the two block barriers of a tensor-core form.
 #ifndef NEP_FUSED_REG_MINB
 #define NEP_FUSED_REG_MINB 5
 #endif
-template <class S>
+template <class S, class MT>
 __global__ void __launch_bounds__(DESC_BLOCK, NEP_FUSED_REG_MINB)
 k_nep_fused_reg(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
                 const int32_t *__restrict__ nbr, const RowExt X, float *__restrict__ usite,
@@ -832,7 +833,7 @@ k_nep_fused_reg(const __grid_constant__ Model<S> P, const Geom geom, const int n
     const bool flagged = fb.on && out_of_range<S>(fb, P, q);
     if (flagged) flag_atom(fb, i, status);
     float Fp[S::NDES];
-    const float U = network<S>(P, q, flagged, Fp);   // flagged: no U_i from this model, Fp = 0
+    const float U = network<S, MT>(P, q, flagged, Fp);   // flagged: no U_i from this model, Fp = 0
     float gi[S::NA][S::NLM];
 #pragma unroll
     for (int a = 0; a < S::NA; ++a) adjoint_channel<S, true>(a, A, T, Fp, gi[a]);
@@ -1158,26 +1159,45 @@ template cudaError_t launch_fused<CuShape>(const Model<CuShape> &, const Geom &,
 
 // Fused evaluation of a register-resident shape (k_nep_fused_reg); Ffix must be zero.  Fails with
 // cudaErrorInvalidConfiguration if more blocks than PC_SLOTS_REG could be resident on an SM.
-template <class S>
+template <class S, class MT>
 cudaError_t launch_fused_reg(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
                              const RowExt &X, float *usite, float *qout, long long *Ffix, const EvalSums &sums,
                          int *status, const Fallback &fb, const PairCache &pc,
                              cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_nep_fused_reg<S>, DESC_BLOCK, 0);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_nep_fused_reg<S, MT>, DESC_BLOCK, 0);
   if (e != cudaSuccess) return e;
   if (per_sm > pc.slots) return cudaErrorInvalidConfiguration;
   const int grid = (n + DESC_BLOCK - 1) / DESC_BLOCK;
-  k_nep_fused_reg<S><<<grid, DESC_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, usite, qout,
+  k_nep_fused_reg<S, MT><<<grid, DESC_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, usite, qout,
                                                   reinterpret_cast<unsigned long long *>(Ffix), sums,
                                                   status, fb, pc);
   return cudaGetLastError();
 }
-template cudaError_t launch_fused_reg<StudentShape>(const Model<StudentShape> &, const Geom &, int, const float4 *,
+template cudaError_t launch_fused_reg<StudentShape, float>(const Model<StudentShape> &, const Geom &, int, const float4 *,
                                                     const int32_t *, const RowExt &, float *, float *, long long *,
                                                     const EvalSums &, int *, const Fallback &,
                                                     const PairCache &, cudaStream_t);
+template cudaError_t launch_fused_reg<StudentShape, __nv_bfloat16>(const Model<StudentShape> &, const Geom &, int, const float4 *,
+                                                    const int32_t *, const RowExt &, float *, float *, long long *,
+                                                    const EvalSums &, int *, const Fallback &,
+                                                    const PairCache &, cudaStream_t);
+template cudaError_t launch_fused_reg<StudentShape, __half>(const Model<StudentShape> &, const Geom &, int, const float4 *,
+                                                    const int32_t *, const RowExt &, float *, float *, long long *,
+                                                    const EvalSums &, int *, const Fallback &,
+                                                    const PairCache &, cudaStream_t);
+
+// Atoms that k_nep_fused_reg keeps resident on the current device.
+cudaError_t fused_reg_resident(int *atoms) {
+  int d = 0, sms = 0, per = 0;
+  cudaError_t e = cudaGetDevice(&d);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_nep_fused_reg<StudentShape, __nv_bfloat16>, DESC_BLOCK, 0);
+  *atoms = sms * per * DESC_BLOCK;
+  return e;
+}
 
 // Mixed-precision fused evaluation of the teacher (k_nep_fused_mixed); Ffix must be zero.
 template <class S, class MT>

@@ -59,6 +59,14 @@ struct MmaKind<__half> {
   static constexpr int bf16 = 0;
 };
 
+template <class MT>
+__device__ __forceinline__ float round_to(float x) {
+  if constexpr (std::is_same<MT, float>::value) return x;
+  else if constexpr (std::is_same<MT, __half>::value) return __half2float(__float2half_rn(x));
+  else return __bfloat162float(__float2bfloat16_rn(x));
+}
+
+
 // tanh of the hardware's special-function unit (PTX tanh.approx.f32: relative error about 2^-11, the unit
 // roundoff of the 16-bit operands it feeds in the mixed-precision network).
 __device__ __forceinline__ float tanh_sfu(float x) {

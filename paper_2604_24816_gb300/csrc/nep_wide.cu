@@ -30,13 +30,6 @@ constexpr int WIDE_BLOCK = 128;
 constexpr int WIDE_WARPS = WIDE_BLOCK / 32;
 constexpr int WIDE_CAP = 128;          // entries per atom: the largest list capacity
 
-template <class MT>
-__device__ __forceinline__ float round_to(float x) {
-  if constexpr (std::is_same<MT, float>::value) return x;
-  else if constexpr (std::is_same<MT, __half>::value) return __half2float(__float2half_rn(x));
-  else return __bfloat162float(__float2bfloat16_rn(x));
-}
-
 // The model tables the lanes index (read from shared memory; the constant bank serves one address at a time).
 // W0 by rows and by columns, zero-padded to whole 16-byte vectors: a product reads a lane's row and the atom's
 // values four at a time, eight lanes' rows without bank conflicts.
