@@ -50,8 +50,8 @@ import nep_inputs as ni  # noqa: E402
 METRIC = "NEP MD atom-steps/s on 1 GB300: plain FP32 vs mixed/student at stated force RMSE"
 UNIT = "atom-steps/s"
 
-# Algorithmic FP32 FLOPs of the method per unit: a static count of the arithmetic each unit needs in the
-# kernels (FMA = 2, add/mul = 1, each transcendental = 1, a packed float2 operation counts both halves),
+# FP32 FLOPs of the method per unit in its basis formulation (Chebyshev basis values, harmonic polynomials and their
+# gradients, as the separate list-walking kernels compute them): a static count of the arithmetic each unit needs (FMA = 2, add/mul = 1, each transcendental = 1, a packed float2 operation counts both halves),
 # for the compiled teacher shape (5 radial + 5 angular channels, 8 basis functions, l = 1..4, 4-body,
 # 30 neurons).  Fixed-point conversions of the force scatter and of the sums, the stand-in pairs of
 # lanes that only take part in warp-collective loads and the zero padding of the network row are not
@@ -88,12 +88,11 @@ UNIT = "atom-steps/s"
 #     FMAs 116 + 9; the list-walking force kernels over Yh_lm: 1177 (harmonics 81, gradients 129);
 #   the half-list force (float16 rows): H = G^i + (-1)^l G^j adds 240 per angular pair and 8 per radial
 #     pair; its LJ term is the whole pair force (14).
-# The FP32 op counters of one fused launch (ffma, fadd, fmul, paired ops, MUFU) agree with this count to
-# within the conversions and padding named above (profiles/k_nep_fused_cu64x64x64.md).
-# The mixed-precision forms run the same fused kernel with the network as two tensor-core GEMMs
-# (32 x 32 tiles, bf16/f16 operands): per atom 1514 FP32 FLOPs remain (5114 - 3870 for the float32
-# network + scaling 30, per neuron z - b0, tanh, energy FMA and gradient factor 7, Fp 30); the GEMMs'
-# 4096 tensor FLOPs per atom are not part of the FP32 count.
+# The fused kernels need fewer operations than this for the same results: FUSED_FLOPS below is their own count, and
+# the one the roofline uses for them.
+# "descriptor_mixed": with the network as two tensor-core GEMMs (32 x 32 tiles, bf16/f16 operands) 1514 FP32 FLOPs per
+# atom remain (5114 - 3870 for the float32 network + scaling 30, per neuron z - b0, tanh, energy FMA and gradient
+# factor 7, Fp 30).
 FLOPS = {
     "descriptor": dict(list_entry=11, active_pair=2, radial_pair=38, lj_pair=15, angular_pair=410, atom=5114),
     "descriptor_mixed": dict(list_entry=11, active_pair=2, radial_pair=38, lj_pair=15, angular_pair=410, atom=1514),
@@ -117,6 +116,35 @@ FLOPS_STUDENT = {
     "force": dict(list_entry=11, active_pair=23, radial_pair=125, lj_pair=14, angular_pair=510, atom=0),
     "force_rec": dict(list_entry=0, active_pair=28, radial_pair=84, lj_pair=15, angular_pair=442, atom=0),
 }
+# The fused kernels' static count: the radial functions as cubics in T_2 (no basis values), the angular sums and
+# the adjoint row over the solid harmonics (gradients from the lower degree's values), the LJ energy summed by the
+# force pass.  Teacher:
+#   radial pair, descriptor 39: r/rc, the hardware cosine, the cutoff half h = (1 + cos) / 4, x = 2 (r/rc - 1)^2 - 1 and
+#     y = 2 x^2 - 1 12, T_2..T_7 in pairs by the step-two recurrence 11, the sums h T_k in 4 paired FMAs 16;
+#   angular pair, descriptor 382: unit vector 3 + cutoff, x and y 12 + 5 channels h (E(y) + x O(y)) 75 + the 24 solid
+#     harmonics 52 + 120 paired FMAs into s_nlm 240;
+#   atom 5159: the radial sums' 8 adds, q_n 80, q_nl 355 (240 + 115 scalings of the sums), 4-body tensors and q4 130,
+#     network 3870, 4-body adjoint 355 (330 + 25 scalings), adjoint row 255 (14 distinct scaled factors per channel 70,
+#     120 products, 15 scaled 4-body factors, 25 FMAs), radial adjoint in basis space 80 and as two cubics 23, site
+#     energy 3;
+#   radial pair, force 47: cutoff and its derivative, x, y and x'(r) h 16, the two cubics and their derivatives 20, their
+#     combination 11;
+#   LJ pair, force 22: 1/r^2 with one Newton step 5, r^-6 2, the energy in three FMAs and its sum 7, dE/dr 5, half of
+#     it / r added to the pair coefficient 3;
+#   angular pair, force 850: unit vector 3 + cutoff, x, y and derivatives 17 + 5 channels with derivatives 150 + solid
+#     harmonics 52 + A_lm, B_lm over the channels 432 + the sum of A R 48 + the gradient 135 + its projection 13.
+# Student: 8 solid harmonics 12, 4 channels 60 (with derivatives 120), sums 64, A_lm and B_lm 112, A R 16, gradient 31;
+# per atom 28 scalings of the sums, 12 more adjoint factors and the two cubics beside the separate kernel's 1153.
+# The FP32 op counters of one fused launch (ffma, fadd, fmul, paired ops, MUFU) agree with this count to
+# within the conversions and padding named above (profiles/k_nep_fused_cu64x64x64.md).
+FUSED_FLOPS = {
+    "descriptor": dict(list_entry=11, active_pair=2, radial_pair=39, lj_pair=0, angular_pair=382, atom=5159),
+    "force_rec": dict(list_entry=0, active_pair=28, radial_pair=47, lj_pair=22, angular_pair=850, atom=0),
+}
+FUSED_FLOPS_STUDENT = {
+    "descriptor_rec": dict(list_entry=11, active_pair=2, radial_pair=39, lj_pair=0, angular_pair=151, atom=1218),
+    "force_rec": dict(list_entry=0, active_pair=28, radial_pair=47, lj_pair=22, angular_pair=324, atom=0),
+}
 # Algorithmic HBM bytes per atom-step: the integrator reads and writes x, v (96) in the kick + drift and
 # v (48) in the second kick, and reads the forces in both kicks (48); the force kernel reads the atom's
 # position (16) and its walked neighbour-list entries (4 each), writes the site energy (4) and the
@@ -134,7 +162,7 @@ def force_kind(form: str) -> str:
 
 def descriptor_kind(form: str) -> str:
     """FLOP table of the descriptor part: the mixed-precision teacher forms' network is on the tensor
-    cores; the float32 student runs its fused kernel (descriptor_rec of FLOPS_STUDENT)."""
+    cores; the float32 student runs its fused kernel (descriptor_rec of FUSED_FLOPS_STUDENT)."""
     f = FORMS[form]
     if f["model"] == "student":
         return "descriptor_rec" if f["precision"] == "fp32" else "descriptor"
@@ -154,17 +182,17 @@ def kernel_flops(kind: str, c: dict, n_atoms_evals: int, table: dict = FLOPS) ->
 
 # The sources each profiled kernel is built from: a committed traffic figure is used only while they
 # are unchanged (kernel names as in profiles/traffic_per_launch.txt; ":form" for the non-plain forms).
-_CORE = ("nep_common.cuh", "nep_descriptor.cuh", "nep_tc.cuh")
+_CORE = ("nep_common.cuh", "nep_descriptor.cuh", "nep_pair.cuh", "nep_solid.cuh", "nep_tc.cuh")
 KERNEL_SOURCES = {
-    "neighbors": ("nep_neighbor.cu", "nep_common.cuh"),
+    "neighbors": ("nep_neighbor.cu", "nep_common.cuh", "nep_control.cuh"),
     "descriptor": ("nep_force.cu",) + _CORE,
     "force": ("nep_force.cu",) + _CORE,
     "fused": ("nep_force.cu",) + _CORE,
     "fused:mix_bf16": ("nep_force.cu",) + _CORE,
     "fused:mix_fp16": ("nep_force.cu",) + _CORE,
     "fused:student": ("nep_force.cu",) + _CORE,
-    "descriptor:student_bf16_fallback": ("nep_mixed.cu", "nep_fallback.cu") + _CORE,
-    "force:student_bf16_fallback": ("nep_force.cu", "nep_fallback.cu") + _CORE,
+    "descriptor:student_bf16_fallback": ("nep_mixed.cu",) + _CORE,
+    "force:student_bf16_fallback": ("nep_force.cu",) + _CORE,
 }
 SOURCE_FILES = tuple(sorted({f for v in KERNEL_SOURCES.values() for f in v}))
 
@@ -403,11 +431,8 @@ def measure_fp32_peak(stream, local: int) -> dict:
 
 # form name -> library precision, model (teacher or distilled student), per-atom fallback to the
 # teacher, arithmetic types, description
-_MIX = ("network GEMMs on tcgen05 tensor cores with {} operands and f32 accumulation inside the fused "
-        "kernel, FP32 descriptors and forces, float64 integration and sums")
-_MIX_STUDENT = ("network GEMMs on tcgen05 tensor cores with {} operands and f32 accumulation, float16 adjoint "
-                "rows between its descriptor and half-list force kernels, FP32 descriptors and forces, float64 "
-                "integration and sums")
+_MIX = ("network products with {} operands and f32 accumulation inside the fused kernel, FP32 descriptors and "
+        "forces, float64 integration and sums")
 FORMS = {
     "plain": dict(precision="fp32", model="teacher", fallback=False, dtype="f32",
                   desc="plain FP32 NEP, seeded teacher weights (float64 integration and sums)"),
@@ -418,7 +443,7 @@ FORMS = {
     "student": dict(precision="fp32", model="student", fallback=False, dtype="f32",
                     desc="distilled student NEP (n_max 3/3, l_max 2, no 4-body, 16 neurons), FP32"),
     "student_bf16_fallback": dict(precision="mix_bf16", model="student", fallback=True, dtype="bf16/f32",
-                                  desc="distilled student NEP, " + _MIX_STUDENT.format("bf16") + "; per-atom fallback to the "
+                                  desc="distilled student NEP, " + _MIX.format("bf16") + "; per-atom fallback to the "
                                        "FP32 teacher for atoms outside the student's training range (5 % margin)"),
     "student_fallback": dict(precision="fp32", model="student", fallback=True, dtype="f32",
                              desc="distilled student NEP, FP32 (one fused kernel); per-atom fallback to the FP32 teacher "
@@ -629,13 +654,17 @@ def run_ours(args, rank: int, ws: int, local: int):
     c2 = nep.counters()
     dc = {k: c2[k] - c1[k] for k in c2}          # the eager pass with per-kernel events
     evals = dc["evaluations"]
-    table = FLOPS_STUDENT if FORMS[args.form]["model"] == "student" else FLOPS
-    f_desc = kernel_flops(descriptor_kind(args.form), dc, evals * wl.n, table)
-    f_force = kernel_flops(force_kind(args.form), dc, evals * wl.n, table)
+    is_student = FORMS[args.form]["model"] == "student"
+    fused = tim["descriptor"][1] == 0 and tim["force"][1] > 0      # one kernel does descriptors and forces
+    table = ((FUSED_FLOPS_STUDENT if is_student else FUSED_FLOPS) if fused else
+             (FLOPS_STUDENT if is_student else FLOPS))
+    # the fused kernels' parts are the same in every precision
+    f_desc = kernel_flops(("descriptor_rec" if is_student else "descriptor") if fused else descriptor_kind(args.form), dc,
+                          evals * wl.n, table)
+    f_force = kernel_flops("force_rec" if fused else force_kind(args.form), dc, evals * wl.n, table)
     clk = clocks.summary(t_host0, t_host1)
     clk_kernels = clocks.summary(t_host2, t_host3)
     kern = {k: {"ms": round(v[0], 4), "launches": v[1]} for k, v in tim.items()}
-    fused = tim["descriptor"][1] == 0 and tim["force"][1] > 0      # one kernel does descriptors and forces
     dominant = "force" if fused else max(("descriptor", "force"), key=lambda k: tim[k][0])
     dom_flops = f_desc + f_force if fused else (f_force if dominant == "force" else f_desc)
     dom_ms = tim[dominant][0]
@@ -644,7 +673,7 @@ def run_ours(args, rank: int, ws: int, local: int):
     kind = "fused" if fused else dominant
     traffic = profiled_traffic(kind if args.form == "plain" else f"{kind}:{args.form}")
     dom_name = (("k_nep_fused_reg" if FORMS[args.form]["model"] == "student" else
-                 "k_nep_fused" if args.form == "plain" else "k_nep_fused_mixed") if fused else
+                 "k_nep_fused") if fused else
                 "k_descriptor_mixed" if dominant == "descriptor" and args.form != "plain" else f"k_{dominant}")
     pk_mhz, kn_mhz = peak["clocks"].get("sm_mhz"), clk_kernels.get("sm_mhz")
     roofline = {

@@ -56,8 +56,8 @@ typedef enum {
 
 /* Arithmetic of the force evaluation.  NEP_FP32: everything in float32 (float64 integration and sums).
  * NEP_MIX_BF16 / NEP_MIX_FP16: descriptors in float32; the network's products (forward and gradient) with
- * bf16 / f16 operands and float32 accumulation, on the tensor cores where that is faster (the paper's mixed
- * precision, Section V.B Optimization 4 and Section VII.A).  The teacher keeps its per-atom adjoint rows in float32
+ * bf16 / f16 operands and float32 accumulation (the paper's mixed precision, Section V.B Optimization 4 and Section
+ * VII.A).  The teacher keeps its per-atom adjoint rows in float32
  * and takes the network's tanh from the special-function unit (relative error about 2^-11, below that of the 16-bit
  * inputs); the student's adjoint rows are float32 too, except in a range of sizes (about 97,000 to 146,000 atoms)
  * where its evaluation runs as two kernels with float16 rows between them. */

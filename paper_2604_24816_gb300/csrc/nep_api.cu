@@ -34,12 +34,9 @@ cudaError_t launch_descriptor(const Model<S> &, const Geom &, int, const float4 
 template <class S, class GT>
 cudaError_t launch_force(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
                          const GT *, long long *, const EvalSums &, int *, cudaStream_t);
-template <class S>
+template <class S, class MT>
 cudaError_t launch_fused(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &, float *,
                          float *, long long *, const EvalSums &, int *, const PairCache &, cudaStream_t);
-template <class S, class MT>
-cudaError_t launch_fused_mixed(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
-                               float *, float *, long long *, const EvalSums &, int *, const PairCache &, cudaStream_t);
 template <class S, class MT>
 cudaError_t launch_fused_reg(const Model<S> &, const Geom &, int, const float4 *, const int32_t *, const RowExt &,
                              float *, float *, long long *, const EvalSums &, int *, const Fallback &,
@@ -502,12 +499,12 @@ cudaError_t forces_of(nep_handle *h, const Model<S> &M, float *qout, bool zeroed
         const PairCache pc{h->pc_rec, h->pc_mask, h->pc_nsm, h->cap, h->pc_slots};
         if constexpr (teacher) {
           if (h->precision == NEP_FP32)
-            e = launch_fused<CuShape>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status, pc, h->stream);
+            e = launch_fused<CuShape, float>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status, pc, h->stream);
           else if (h->precision == NEP_MIX_BF16)
-            e = launch_fused_mixed<CuShape, __nv_bfloat16>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es,
+            e = launch_fused<CuShape, __nv_bfloat16>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es,
                                                            status, pc, h->stream);
           else
-            e = launch_fused_mixed<CuShape, __half>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status,
+            e = launch_fused<CuShape, __half>(M, g, h->n, h->pos, h->nbr, rows, h->usite, qout, h->F, es, status,
                                                     pc, h->stream);
         } else {
           if (h->precision == NEP_FP32)

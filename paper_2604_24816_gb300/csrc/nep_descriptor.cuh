@@ -596,14 +596,14 @@ struct NetSmem {
   static constexpr int NDP = (S::NDES + 3) / 4 * 4;
   float W0[S::NNEU][NDP];
 };
-template <class S>
+template <class MT, class S>
 __device__ __forceinline__ void stage_network(const Model<S> &P, NetSmem<S> &N) {
   for (int t = threadIdx.x; t < S::NNEU * NetSmem<S>::NDP; t += blockDim.x) {
     const int mu = t / NetSmem<S>::NDP, v = t % NetSmem<S>::NDP;
-    N.W0[mu][v] = v < S::NDES ? P.W0[mu][v] : 0.f;
+    N.W0[mu][v] = v < S::NDES ? round_to<MT>(P.W0[mu][v]) : 0.f;
   }
 }
-template <class S>
+template <class MT, class S>
 __device__ __forceinline__ float network_smem(const Model<S> &P, const NetSmem<S> &N, const float (&q)[S::NDES],
                                               bool flagged, float (&Fp)[S::NDES]) {
   constexpr int NDP = NetSmem<S>::NDP, NP = NDP / 2;
@@ -611,8 +611,8 @@ __device__ __forceinline__ float network_smem(const Model<S> &P, const NetSmem<S
 #pragma unroll
   for (int p = 0; p < NP; ++p) {
     const int v0 = 2 * p, v1 = 2 * p + 1;
-    qt[p] = pr(v0 < S::NDES ? q[v0 < S::NDES ? v0 : 0] * P.qs[v0 < S::NDES ? v0 : 0] : 0.f,
-               v1 < S::NDES ? q[v1 < S::NDES ? v1 : 0] * P.qs[v1 < S::NDES ? v1 : 0] : 0.f);
+    qt[p] = pr(v0 < S::NDES ? round_to<MT>(q[v0 < S::NDES ? v0 : 0] * P.qs[v0 < S::NDES ? v0 : 0]) : 0.f,
+               v1 < S::NDES ? round_to<MT>(q[v1 < S::NDES ? v1 : 0] * P.qs[v1 < S::NDES ? v1 : 0]) : 0.f);
     dq[p] = bc2(0.f);
   }
   float U = -P.b1;
@@ -627,9 +627,10 @@ __device__ __forceinline__ float network_smem(const Model<S> &P, const NetSmem<S
       z2 = fma2(pr(t.x, t.y), qt[2 * p], z2);
       z2 = fma2(pr(t.z, t.w), qt[2 * p + 1], z2);
     }
-    const float h = tanhf(hsum(z2));
+    // mixed: error 2^-11, below that of z (16-bit inputs)
+    const float h = std::is_same<MT, float>::value ? tanhf(hsum(z2)) : tanh_sfu(hsum(z2));
     U = fmaf(P.w1[mu], h, U);
-    const float2 t2 = bc2(P.w1[mu] * (1.f - h * h));
+    const float2 t2 = bc2(round_to<MT>(P.w1[mu] * (1.f - h * h)));
 #pragma unroll
     for (int p = 0; p < NDP / 4; ++p) {
       const float4 t = row[p];

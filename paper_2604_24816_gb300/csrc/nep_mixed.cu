@@ -32,27 +32,15 @@ __device__ __forceinline__ uint4 pack8_half(const float *v) {
   return w;
 }
 
-// Teacher shape: the angular sums of 4 of the 5 channels are accumulated in TMEM (96 columns,
-// accumulate_atom_tm), the fifth channel's 24 in registers, and the two network GEMMs take turns in the
-// remaining 32 columns (the forward result is read out before the backward GEMM overwrites it): 128
-// columns per block and 4 resident blocks (124 registers) instead of 245 registers and 2.  The student shape keeps its
-// sums in registers and asks for 6 resident blocks (measured best).
-#ifndef NEP_MIX_MINB_TM
-#define NEP_MIX_MINB_TM 4
-#endif
+// Six resident blocks (at most 80 registers) measured best.
 template <class S, class MT>
-__global__ void __launch_bounds__(MIX_BLOCK, S::NLM > 8 ? NEP_MIX_MINB_TM : 6)
+__global__ void __launch_bounds__(MIX_BLOCK, 6)
 k_descriptor_mixed(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
                    const int32_t *__restrict__ nbr, const RowExt X, __half *__restrict__ G,
                    float *__restrict__ usite, float *__restrict__ qout, long long *__restrict__ Ffix,
                    const EvalSums sums, int *__restrict__ status, const __grid_constant__ Fallback fb) {
   static_assert(S::NDES <= MIX_K && S::NNEU <= MIX_N, "network larger than one tensor-core tile");
-  constexpr bool TM = S::NLM > 8;
-  constexpr int NT = 4;                                   // TM: channels whose sums live in TMEM
-  constexpr uint32_t TCOLS = TM ? 128 : 64;
-  constexpr uint32_t ZCOL = TM ? NT * S::NLM : 0;         // forward GEMM result
-  constexpr uint32_t DCOL = TM ? NT * S::NLM : 32;        // backward GEMM result (TM: the same columns)
-  static_assert(!TM || (NT * S::NLM + MIX_N <= (int)TCOLS && MIX_BLOCK == 128), "TMEM budget");
+  constexpr uint32_t TCOLS = 64, ZCOL = 0, DCOL = 32;     // forward and backward GEMM results
   __shared__ float4 shift[27];
   // The neighbour-pipeline ring is dead once every thread has walked its row, so the GEMMs' A tile
   // (q~ rows, then T rows) overlays it: less shared memory per block leaves more of the unified
@@ -87,26 +75,7 @@ k_descriptor_mixed(const __grid_constant__ Model<S> P, const Geom geom, const in
   float q[S::NDES];
   long long acc[5] = {0, 0, 0, 0, 0};
   bool flagged = false;
-  RegSums<S, NT> R;
-  uint32_t trow = 0;
-  if constexpr (TM) {
-    tc_fence_after();
-    trow = tmem_base + ((uint32_t)(t & ~31) << 16);
-    const RowSpan sp = live ? full_row(X, i, skip_far(X)) : RowSpan{0, 0, 0};
-    A.cnt = sp.c;
-    if (live) { Ffix[i] = 0; Ffix[(size_t)n + i] = 0; Ffix[2 * (size_t)n + i] = 0; }
-    accumulate_atom_tm<S, NT, MIX_DE, MIX_DP, MIX_BLOCK>(P, shift, trow, live ? i : 0, n, pos, nbr, sp, ring_e,
-                                                         ring_p, A.QR, R, A.elj, A.nrad, A.nang, A.nact);
-    descriptors_tm<S, NT>(P, trow, A.QR, R, q, T);        // zero for threads past the last atom (empty row)
-    if (live) {
-      if (qout != nullptr) {
-#pragma unroll
-        for (int v = 0; v < S::NDES; ++v) qout[(size_t)i * S::NDES + v] = q[v];
-      }
-      flagged = fb.on && out_of_range<S>(fb, P, q);
-      if (flagged) flag_atom(fb, i, status);
-    }
-  } else if (live) {
+  if (live) {
     Ffix[i] = 0; Ffix[(size_t)n + i] = 0; Ffix[2 * (size_t)n + i] = 0;
     accumulate_atom<S, MIX_DE, MIX_DP, MIX_BLOCK>(P, shift, i, n, pos, nbr, full_row(X, i, skip_far(X)), ring_e,
                                                   ring_p, A);
@@ -181,36 +150,13 @@ k_descriptor_mixed(const __grid_constant__ Model<S> P, const Geom geom, const in
 #pragma unroll
   for (int v = 0; v < S::NDES; ++v) Fp[v] = flagged ? 0.f : dq[v] * P.qs[v];   // flagged: no U_i here
   __half *Gi = G + (size_t)(live ? i : 0) * S::GS;
-  if constexpr (TM) {
-    // adjoint from the sums (TMEM chunks read by whole warps; rows stored for live atoms only)
-    float g4[S::NA][5];
-#pragma unroll
-    for (int a = 0; a < S::NA; ++a) fourbody_adjoint<S>(a, T, g4[a]);
-#pragma unroll
-    for (int k = 0; k < S::NLM / TMEM_W; ++k) {
-      const int c = TMEM_W * k;
-      float sv[S::NA][TMEM_W];
-      sums_chunk<S, NT>(trow, k, R, sv);
-#pragma unroll
-      for (int a = 0; a < S::NA; ++a) {
-        float gl[TMEM_W];
-        adjoint_chunk<S>(a, c, sv[a], g4[a], Fp, gl);
-        const __half2 h0 = __floats2half2_rn(gl[0], gl[1]), h1 = __floats2half2_rn(gl[2], gl[3]);
-        if (live)
-          *reinterpret_cast<uint2 *>(Gi + a * S::NLM + c) =
-              make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
-      }
-    }
-  }
   if (live) {
-    if constexpr (!TM) {
 #pragma unroll
-      for (int a = 0; a < S::NA; ++a) {
-        float gl[S::NLM];
-        adjoint_channel<S>(a, A, T, Fp, gl);
+    for (int a = 0; a < S::NA; ++a) {
+      float gl[S::NLM];
+      adjoint_channel<S>(a, A, T, Fp, gl);
 #pragma unroll
-        for (int c = 0; c < S::NLM; c += 8) *reinterpret_cast<uint4 *>(Gi + a * S::NLM + c) = pack8_half(gl + c);
-      }
+      for (int c = 0; c < S::NLM; c += 8) *reinterpret_cast<uint4 *>(Gi + a * S::NLM + c) = pack8_half(gl + c);
     }
     {
       float tail[8];
