@@ -180,7 +180,7 @@ struct nep_handle {
   float4 *pos = nullptr, *pos_ref = nullptr;
   long long *F = nullptr;          // fixed-point forces [3][n]
   float *usite = nullptr, *qbuf = nullptr;
-  void *G = nullptr;               // adjoint rows: float32 (plain) or float16 (mixed) [n][GS]
+  void *G = nullptr;               // adjoint rows of the separate kernels: float32 or float16 (split) [n][GS]
   int32_t *nbr = nullptr, *nnum = nullptr, *nang = nullptr, *nown = nullptr, *nband0 = nullptr, *nfar = nullptr;
   int *count = nullptr, *cursor = nullptr, *start = nullptr, *tile_sums = nullptr;
   DeviceReport *rep = nullptr;     // control block, sums and counters, read back together

@@ -13,7 +13,7 @@
 
 namespace nep {
 
-// Adjoint rows are stored as float32 (plain form) or float16 (mixed-precision form); the force
+// Adjoint rows in memory are float32 (the teacher's separate kernels) or float16 (the mixed student's); the force
 // kernel reads them W values per 16-byte load.
 template <class GT>
 struct GTraits;
@@ -326,8 +326,7 @@ __device__ __forceinline__ void adjoint_channel(int a, const AtomSums<S> &A, con
 }
 
 // ---------------------------------------------------------------------------------------------------
-// Teacher shape with the angular sums s_nlm of the first NT channels in tensor memory (TMEM) instead
-// of registers (NT = 5: all 120; NT = 4: 96, the fifth channel's 24 in registers), in the chunked layout
+// Teacher shape with the 120 angular sums s_nlm in tensor memory (TMEM) instead of registers, in the chunked layout
 // of tm_col (chunk k = components 4k..4k+3 of every channel: one x16 access for channels 0..3 and one x4
 // access for channel 4), which the force pass's adjoint row shares.  All TMEM accesses are
 // warp-collective, so the neighbour walk runs to the warp's longest row (threads past their own row, or
@@ -335,55 +334,31 @@ __device__ __forceinline__ void adjoint_channel(int a, const AtomSums<S> &A, con
 // without an angular pair adding g = 0.
 constexpr int TMEM_W = 4;
 
-// The sums of the channels kept in registers (NA - NT of them; one unused row when NT = NA).
-template <class S, int NT>
-struct RegSums {
-  float s[S::NA > NT ? S::NA - NT : 1][S::NLM];
-};
-
-// Chunk k of the NT TMEM channels into v[0..NT-1] (one statement, waited for).
-template <class S, int NT>
+// Chunk k of every channel into v (one statement, waited for), and v into it.
+template <class S>
 __device__ __forceinline__ void tm_load(uint32_t trow, int k, float (&v)[S::NA][TMEM_W]) {
-  if constexpr (NT == 5) {
-    tmem_ld_chunk<S::NLM>(trow, k, v);
-  } else {
-    float t[4][TMEM_W];
-    tmem_ld_chunk<S::NLM>(trow, k, t);
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int c = 0; c < TMEM_W; ++c) v[a][c] = t[a][c];
-  }
+  tmem_ld_chunk<S::NLM>(trow, k, v);
 }
-template <class S, int NT>
+template <class S>
 __device__ __forceinline__ void tm_store(uint32_t trow, int k, const float (&v)[S::NA][TMEM_W]) {
-  if constexpr (NT == 5) {
-    tmem_st_chunk<S::NLM, 5>(trow, k, v);
-  } else {
-    float t[4][TMEM_W];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int c = 0; c < TMEM_W; ++c) t[a][c] = v[a][c];
-    tmem_st_chunk<S::NLM, 4>(trow, k, t);
-  }
+  tmem_st_chunk<S::NLM>(trow, k, v);
 }
 
 // Zero the sums, then walk atom ii's row (cnt entries; cnt = 0 for threads past the last atom):
-// radial basis sums QR and the LJ energy in registers, s_nlm in TMEM (channels < NT) and R.
+// radial basis sums QR and the LJ energy in registers, s_nlm in TMEM.
 // The accumulations run in float2 pairs (two basis functions, or two (l, m) components, per instruction).
 // REC: every active pair is also recorded as (dx, dy, dz, j) at rec[off + slot * BLOCK] (off: this
 // thread's column of a [pmax][BLOCK] array): angular pairs (r < rc_A) from
 // slot 0 up in walk order, the other active pairs from slot pmax - 1 down (pmax >= the row length, so
 // the two never meet).
-template <class S, int NT, int DE, int DP, int BLOCK, bool REC = false, bool SOLID = false>
+template <class S, int DE, int DP, int BLOCK, bool REC = false, bool SOLID = false>
 __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const float4 *shift, uint32_t trow, int ii,
                                                    int n, const float4 *__restrict__ pos,
                                                    const int32_t *__restrict__ nbr, RowSpan sp, uint32_t *ring_e,
-                                                   float4 *ring_p, float (&QR)[S::KR], RegSums<S, NT> &R,
+                                                   float4 *ring_p, float (&QR)[S::KR],
                                                    float &elj, int &nrad, int &nang, int &nact,
                                                    float4 *__restrict__ rec = nullptr, unsigned off = 0, int pmax = 0) {
-  static_assert(S::NA == 5 && S::NLM == 24 && (NT == 4 || NT == 5), "teacher shape");
+  static_assert(S::NA == 5 && S::NLM == 24, "teacher shape");
   static_assert(S::KR == 8, "eight basis functions");
   constexpr int W = TMEM_W;
   constexpr int NC = S::NLM / W;
@@ -394,13 +369,9 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
 #pragma unroll
       for (int c = 0; c < W; ++c) z[a][c] = 0.f;
 #pragma unroll
-    for (int k = 0; k < NC; ++k) tm_store<S, NT>(trow, k, z);
+    for (int k = 0; k < NC; ++k) tm_store<S>(trow, k, z);
     tmem_wait_st();
   }
-#pragma unroll
-  for (int a = NT; a < S::NA; ++a)
-#pragma unroll
-    for (int c = 0; c < S::NLM; ++c) R.s[a - NT][c] = 0.f;
   float2 Q[4] = {bc2(0.f), bc2(0.f), bc2(0.f), bc2(0.f)};
   elj = 0.f;
   nrad = 0; nang = 0; nact = 0;
@@ -451,15 +422,14 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
       const float ux = ang ? dx * ir : 1.f, uy = ang ? dy * ir : 0.f, uz = ang ? dz * ir : 0.f;
       float g[S::NA];
       radial_channels<S>(P, ar, ang, g);
-      // SOLID: the components chunk by chunk (fewer live registers than 24 values); all channels in TMEM
-      static_assert(!SOLID || NT == S::NA, "register-resident channels take the normalised harmonics");
+      // SOLID: the components chunk by chunk (fewer live registers than 24 values)
       const Solid<S::NLM> H(ux, uy, uz);
       float Y[S::NLM];
       if constexpr (!SOLID) harmonics<S::NLM>(ux, uy, uz, Y);
 #pragma unroll
       for (int k = 0; k < NC; ++k) {
         float sv[S::NA][W];
-        tm_load<S, NT>(trow, k, sv);
+        tm_load<S>(trow, k, sv);
         float2 y01, y23;
         if constexpr (SOLID) {
           H.chunk(k, y01, y23);
@@ -468,19 +438,14 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
           y23 = pr(Y[W * k + 2], Y[W * k + 3]);
         }
 #pragma unroll
-        for (int a = 0; a < NT; ++a) {
+        for (int a = 0; a < S::NA; ++a) {
           const float2 g2 = bc2(g[a]);
           const float2 lo = fma2(g2, y01, pr(sv[a][0], sv[a][1]));
           const float2 hi = fma2(g2, y23, pr(sv[a][2], sv[a][3]));
           sv[a][0] = lo.x; sv[a][1] = lo.y; sv[a][2] = hi.x; sv[a][3] = hi.y;
         }
-        tm_store<S, NT>(trow, k, sv);
+        tm_store<S>(trow, k, sv);
       }
-      // register-resident channels: scalar (paired updates would pin the sums to aligned register pairs)
-#pragma unroll
-      for (int a = NT; a < S::NA; ++a)
-#pragma unroll
-        for (int c = 0; c < S::NLM; ++c) R.s[a - NT][c] = fmaf(g[a], Y[c], R.s[a - NT][c]);
       tmem_wait_st();
       if (!REC && ang) ++nang;
     }
@@ -493,22 +458,12 @@ __device__ __forceinline__ void accumulate_atom_tm(const Model<S> &P, const floa
   cheb_sums(Q, QR);
 }
 
-// The sums of chunk k (components 4k..4k+3) of every channel: TMEM for a < NT, registers after.
-template <class S, int NT>
-__device__ __forceinline__ void sums_chunk(uint32_t trow, int k, const RegSums<S, NT> &R, float (&sv)[S::NA][TMEM_W]) {
-  tm_load<S, NT>(trow, k, sv);
-#pragma unroll
-  for (int a = NT; a < S::NA; ++a)
-#pragma unroll
-    for (int cc = 0; cc < TMEM_W; ++cc) sv[a][cc] = R.s[a < NT ? 0 : a - NT][TMEM_W * k + cc];
-}
-
 // Descriptors from the radial basis sums and the sums s_nlm (q_nl = sum_m s_nlm^2, 4-body from the
 // l = 2 sums), as descriptors_of.
 // SOLID: sums over the solid harmonics (accumulate_atom_tm), scaled by solid_norm here.
-template <class S, int NT, bool SOLID = false>
+template <class S, bool SOLID = false>
 __device__ __forceinline__ void descriptors_tm(const Model<S> &P, uint32_t trow, const float (&QR)[S::KR],
-                                               const RegSums<S, NT> &R, float (&q)[S::NDES], FourBody<S> &T) {
+                                               float (&q)[S::NDES], FourBody<S> &T) {
   constexpr int W = TMEM_W;
 #pragma unroll
   for (int a = 0; a < S::NR; ++a) {
@@ -523,7 +478,7 @@ __device__ __forceinline__ void descriptors_tm(const Model<S> &P, uint32_t trow,
 #pragma unroll
   for (int k = 0; k < S::NLM / W; ++k) {
     float sv[S::NA][W];
-    sums_chunk<S, NT>(trow, k, R, sv);
+    tm_load<S>(trow, k, sv);
 #pragma unroll
     for (int a = 0; a < S::NA; ++a)
 #pragma unroll
@@ -542,15 +497,15 @@ __device__ __forceinline__ void descriptors_tm(const Model<S> &P, uint32_t trow,
 // 4-body adjoint factors g4[a] = 3 (T_a^2) : dT_a/ds_m of every channel, with the tensors T_a rebuilt
 // from the l = 2 sums (chunks 0 and 1, and the zonal component of chunk 5 with SOLID), so that T need not
 // stay live across the network.
-template <class S, int NT, bool SOLID = false>
-__device__ __forceinline__ void fourbody_adjoint_tm(uint32_t trow, const RegSums<S, NT> &R, float (&g4)[S::NA][5]) {
+template <class S, bool SOLID = false>
+__device__ __forceinline__ void fourbody_adjoint_tm(uint32_t trow, float (&g4)[S::NA][5]) {
   static_assert(S::FOURBODY && S::NLM == 24, "teacher shape");
   float s2[S::NA][5];
 #pragma unroll
   for (int k = 0; k < S::NLM / TMEM_W; ++k) {
     if (!(k < 2 || (SOLID && k == 5))) continue;
     float sv[S::NA][TMEM_W];
-    sums_chunk<S, NT>(trow, k, R, sv);
+    tm_load<S>(trow, k, sv);
 #pragma unroll
     for (int cc = 0; cc < TMEM_W; ++cc) {
       const int lm = TMEM_W * k + cc;

@@ -1,11 +1,12 @@
 // nep_force.cu -- NEP descriptors, network and chain-rule forces on sm_103a.
 //
-// Two kernels per force evaluation, one thread per atom (cell-sorted order), both reading the
-// distance-sorted neighbour list of nep_neighbor.cu.  For the teacher shape both keep their 120-value
-// per-atom arrays (the sums s_nlm, the adjoint row G_i) in tensor memory (TMEM) rather than registers,
-// which doubles (descriptor) or 1.5x (force) the resident warps:
+// One evaluation is one kernel, one thread per atom (cell-sorted order) over the distance-sorted neighbour list of
+// nep_neighbor.cu: k_nep_fused (teacher; its 120-value per-atom arrays in tensor memory) or k_nep_fused_reg (student; in
+// registers), in float32 or with 16-bit operands in the network.  Systems that leave the chip empty that way run the
+// kernels of nep_wide.cu.  The same work in two kernels is kept for the ablations and one range of the mixed student
+// (which has its descriptor kernel in nep_mixed.cu):
 //
-//  k_descriptor  radial descriptors q_n (Section III.B), shifted-force LJ energy, angular sums
+//  k_descriptor_tm  radial descriptors q_n (Section III.B), shifted-force LJ energy, angular sums
 //                s_nlm = sum_j g_n(r_ij) Yh_lm(u_ij) for l = 1..4 (24 (l,m) components per channel,
 //                all NA channels updated in one neighbour pass: the geometry -- cutoff, Chebyshev
 //                basis, harmonics -- is computed once per neighbour and reused, the channel tiling of
@@ -46,9 +47,6 @@ constexpr int DESC_BLOCK = 128;
 constexpr int FORCE_BLOCK = NEP_FORCE_BLOCK;
 // Minimum resident blocks per SM requested from the compiler (register budget per thread =
 // 65536 / (block * min_blocks)); the defaults are the measured best on GB300.
-#ifndef NEP_DESC_MINB
-#define NEP_DESC_MINB 2
-#endif
 #ifndef NEP_FORCE_MINB
 #define NEP_FORCE_MINB 2
 #endif
@@ -59,65 +57,6 @@ constexpr int PIPE_DE = 8;    // list entries in flight per thread (descriptor k
 constexpr int PIPE_DP = 2;    // neighbour positions (and the fused force pass's records) in flight per thread
 constexpr int FPIPE_DE = 6;   // the same for the force kernel, whose pairs take longer
 constexpr int FPIPE_DP = 3;
-
-template <class S>
-__global__ void __launch_bounds__(DESC_BLOCK, NEP_DESC_MINB)
-k_descriptor(const __grid_constant__ Model<S> P, const Geom geom, const int n, const float4 *__restrict__ pos,
-             const int32_t *__restrict__ nbr, const RowExt X, float *__restrict__ G,
-             float *__restrict__ usite, float *__restrict__ qout, long long *__restrict__ Ffix,
-             const EvalSums sums, int *__restrict__ status, const __grid_constant__ Fallback fb) {
-  __shared__ float4 shift[27];
-  __shared__ uint32_t ring_e[PIPE_DE * DESC_BLOCK];
-  __shared__ float4 ring_p[PIPE_DP * DESC_BLOCK];
-  fill_shift_table(shift, geom);
-  __syncthreads();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  long long acc[5] = {0, 0, 0, 0, 0};
-  const bool skip = skip_far(X);
-  if (i < n) {
-    Ffix[i] = 0; Ffix[(size_t)n + i] = 0; Ffix[2 * (size_t)n + i] = 0;
-    AtomSums<S> A;
-    accumulate_atom<S, PIPE_DE, PIPE_DP, DESC_BLOCK>(P, shift, i, n, pos, nbr, full_row(X, i, skip), ring_e, ring_p,
-                                                     A);
-    float q[S::NDES];
-    FourBody<S> T;
-    descriptors_of<S>(P, A, q, T);
-    if (qout != nullptr) {
-#pragma unroll
-      for (int v = 0; v < S::NDES; ++v) qout[(size_t)i * S::NDES + v] = q[v];
-    }
-    const bool flagged = fb.on && out_of_range<S>(fb, P, q);
-    if (flagged) flag_atom(fb, i, status);
-
-    float Fp[S::NDES];
-    const float U = network<S>(P, q, flagged, Fp);   // flagged: no U_i from this model
-
-    float *Gi = G + (size_t)i * S::GS;
-#pragma unroll
-    for (int a = 0; a < S::NA; ++a) {
-      float gl[S::NLM];
-      adjoint_channel<S>(a, A, T, Fp, gl);
-#pragma unroll
-      for (int c = 0; c < S::NLM; c += 4)
-        *reinterpret_cast<float4 *>(Gi + a * S::NLM + c) = make_float4(gl[c], gl[c + 1], gl[c + 2], gl[c + 3]);
-    }
-    {
-      float tail[8];
-      radial_tail<S>(P, Fp, tail);
-      *reinterpret_cast<float4 *>(Gi + S::NA * S::NLM) = make_float4(tail[0], tail[1], tail[2], tail[3]);
-      *reinterpret_cast<float4 *>(Gi + S::NA * S::NLM + 4) = make_float4(tail[4], tail[5], tail[6], tail[7]);
-    }
-    const float ui = flagged ? A.elj : U + A.elj;
-    usite[i] = ui;
-    if (!isfinite(ui)) atomicOr(status, ST_NAN);
-    acc[0] = to_fix32(ui);
-    acc[1] = A.nrad;
-    acc[2] = A.nang;
-    acc[3] = A.cnt;
-    acc[4] = A.nact;
-  }
-  eval_add_d<DESC_BLOCK / 32>(sums, acc);
-}
 
 // Teacher-shape descriptor kernel with the 120 angular sums s_nlm accumulated in tensor memory (TMEM)
 // instead of registers (accumulate_atom_tm), so that 4 blocks fit per SM instead of 2 (128 registers,
@@ -155,12 +94,11 @@ k_descriptor_tm(const __grid_constant__ Model<S> P, const Geom geom, const int n
   const int cnt = sp.c;
   float QR[S::KR], elj;
   int nrad, nang, nact;
-  RegSums<S, S::NA> R;                      // empty: every channel in TMEM
-  accumulate_atom_tm<S, S::NA, PIPE_DE, PIPE_DP, DESC_BLOCK>(P, shift, trow, ii, n, pos, nbr, sp, ring_e, ring_p,
-                                                             QR, R, elj, nrad, nang, nact);
+  accumulate_atom_tm<S, PIPE_DE, PIPE_DP, DESC_BLOCK>(P, shift, trow, ii, n, pos, nbr, sp, ring_e, ring_p,
+                                                             QR, elj, nrad, nang, nact);
   float q[S::NDES];
   FourBody<S> T;
-  descriptors_tm<S, S::NA>(P, trow, QR, R, q, T);
+  descriptors_tm<S>(P, trow, QR, q, T);
   if (live && qout != nullptr) {
 #pragma unroll
     for (int v = 0; v < S::NDES; ++v) qout[(size_t)i * S::NDES + v] = q[v];
@@ -173,12 +111,12 @@ k_descriptor_tm(const __grid_constant__ Model<S> P, const Geom geom, const int n
   // adjoint row from the TMEM sums, then the radial tail
   float *Gi = G + (size_t)ii * S::GS;
   float g4[S::NA][5];
-  fourbody_adjoint_tm<S, S::NA>(trow, R, g4);
+  fourbody_adjoint_tm<S>(trow, g4);
 #pragma unroll
   for (int k = 0; k < S::NLM / W; ++k) {
     const int c = W * k;
     float sv[S::NA][W];
-    sums_chunk<S, S::NA>(trow, k, R, sv);
+    tm_load<S>(trow, k, sv);
 #pragma unroll
     for (int a = 0; a < S::NA; ++a) {
       float gl[W];
@@ -269,7 +207,7 @@ __device__ __forceinline__ void angular_pair(const Model<S> &P, uint32_t trow,
     const int lm0 = 4 * k;
     float hi[S::NA][4];
     if constexpr (TM) {
-      tm_load<S, S::NA>(trow, k, hi);
+      tm_load<S>(trow, k, hi);
     } else {
 #pragma unroll
       for (int a = 0; a < S::NA; ++a)
@@ -622,7 +560,7 @@ k_force(const __grid_constant__ Model<S> P, const Geom geom, const int n, const 
           for (int cc = 0; cc < 4; ++cc) v[a][cc] = t[(4 * k) % W + cc];
         }
       }
-      tm_store<S, S::NA>(trow, k, v);
+      tm_store<S>(trow, k, v);
     }
     tmem_wait_st();
   } else {
@@ -718,13 +656,12 @@ k_nep_fused(const __grid_constant__ Model<S> P, const Geom geom, const int n, co
   // descriptors and network (as k_descriptor_tm), recording the active pairs
   float QR[S::KR], elj;
   int nrad, nang, nact;
-  RegSums<S, S::NA> R;
-  accumulate_atom_tm<S, S::NA, PIPE_DE, PIPE_DP, DESC_BLOCK, true, true>(P, shift, trow, ii, n, pos, nbr, sp, ring_e,
-                                                                         ring_p, QR, R, elj, nrad, nang, nact, pc.rec,
+  accumulate_atom_tm<S, PIPE_DE, PIPE_DP, DESC_BLOCK, true, true>(P, shift, trow, ii, n, pos, nbr, sp, ring_e,
+                                                                         ring_p, QR, elj, nrad, nang, nact, pc.rec,
                                                                          rec_off, pc.pmax);
   float q[S::NDES];
   FourBody<S> T;
-  descriptors_tm<S, S::NA, true>(P, trow, QR, R, q, T);
+  descriptors_tm<S, true>(P, trow, QR, q, T);
   if (live && qout != nullptr) {
 #pragma unroll
     for (int v = 0; v < S::NDES; ++v) qout[(size_t)i * S::NDES + v] = q[v];
@@ -734,14 +671,14 @@ k_nep_fused(const __grid_constant__ Model<S> P, const Geom geom, const int n, co
 
   // the adjoint row replaces the sums in TMEM (same columns, chunk by chunk); radial tail in registers
   float g4[S::NA][5];
-  fourbody_adjoint_tm<S, S::NA, true>(trow, R, g4);
+  fourbody_adjoint_tm<S, true>(trow, g4);
 #pragma unroll
   for (int k = 0; k < S::NLM / W; ++k) {
     float sv[S::NA][W], gl[S::NA][W];
-    sums_chunk<S, S::NA>(trow, k, R, sv);
+    tm_load<S>(trow, k, sv);
 #pragma unroll
     for (int a = 0; a < S::NA; ++a) adjoint_chunk<S, true>(a, W * k, sv[a], g4[a], Fp, gl[a]);
-    tm_store<S, S::NA>(trow, k, gl);
+    tm_store<S>(trow, k, gl);
   }
   tmem_wait_st();
   {
@@ -788,7 +725,7 @@ k_nep_fused(const __grid_constant__ Model<S> P, const Geom geom, const int n, co
 // with no tensor memory, so every thread walks its own row (no warp-collective steps).  The descriptor
 // walk records the active pairs (PairCache, PC_SLOTS_REG regions per SM: the launch checks that no more
 // blocks are resident), the adjoint row stays in registers and the force pass reads the records.  With
-// the fallback on, an atom whose descriptors leave the training range is flagged as in k_descriptor
+// the fallback on, an atom whose descriptors leave the training range is flagged (flag_atom)
 // (zero adjoint row, LJ energy only), and the teacher kernels then add its own model's part.  Ffix is
 // zeroed by the caller before the launch.  Five resident blocks (at most 102 registers) measured 4 %
 // faster than four.  MT = __nv_bfloat16 / __half (the mixed student): the network's operands rounded to that type, W0 by
@@ -871,19 +808,13 @@ k_nep_fused_reg(const __grid_constant__ Model<S> P, const Geom geom, const int n
 // ---------------------------------------------------------------------------------------------------
 // Host launchers (called from nep_api.cu).
 
-#ifndef NEP_DESC_TM
-#define NEP_DESC_TM 1
-#endif
 template <class S>
 cudaError_t launch_descriptor(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
                               const RowExt &X, float *G, float *usite, float *qout, long long *Ffix, const EvalSums &sums,
                          int *status, const Fallback &fb, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int grid = (n + DESC_BLOCK - 1) / DESC_BLOCK;
-  if constexpr (ForceCfg<S>::TM && NEP_DESC_TM)
-    k_descriptor_tm<S><<<grid, DESC_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, G, usite, qout, Ffix, sums, status, fb);
-  else
-    k_descriptor<S><<<grid, DESC_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, G, usite, qout, Ffix, sums, status, fb);
+  k_descriptor_tm<S><<<grid, DESC_BLOCK, 0, st>>>(P, g, n, pos, nbr, X, G, usite, qout, Ffix, sums, status, fb);
   return cudaGetLastError();
 }
 
@@ -1020,18 +951,14 @@ cudaError_t pair_cache_sm_bound(int *nsm) {
 // Pair records per region: one float4 per record, DESC_BLOCK threads.
 size_t pair_cache_region_elems(int pmax) { return (size_t)pmax * DESC_BLOCK; }
 
-#define NEP_INSTANTIATE(SH)                                                                                    \
-  template cudaError_t launch_descriptor<SH>(const Model<SH> &, const Geom &, int, const float4 *, const int32_t *,   \
-                                             const RowExt &, float *, float *, float *, long long *, const EvalSums &, \
-                                             int *, const Fallback &, cudaStream_t);                                  \
-  template cudaError_t launch_force<SH, float>(const Model<SH> &, const Geom &, int, const float4 *, const int32_t *, \
-                                               const RowExt &, const float *, long long *, const EvalSums &, int *,    \
-                                               cudaStream_t);                                                         \
-  template cudaError_t launch_force<SH, __half>(const Model<SH> &, const Geom &, int, const float4 *,                 \
-                                                const int32_t *, const RowExt &, const __half *, long long *,         \
-                                                const EvalSums &, int *, cudaStream_t);
-NEP_INSTANTIATE(CuShape)
-NEP_INSTANTIATE(StudentShape)
-#undef NEP_INSTANTIATE
+template cudaError_t launch_descriptor<CuShape>(const Model<CuShape> &, const Geom &, int, const float4 *, const int32_t *,
+                                                const RowExt &, float *, float *, float *, long long *, const EvalSums &,
+                                                int *, const Fallback &, cudaStream_t);
+template cudaError_t launch_force<CuShape, float>(const Model<CuShape> &, const Geom &, int, const float4 *,
+                                                  const int32_t *, const RowExt &, const float *, long long *,
+                                                  const EvalSums &, int *, cudaStream_t);
+template cudaError_t launch_force<StudentShape, __half>(const Model<StudentShape> &, const Geom &, int, const float4 *,
+                                                        const int32_t *, const RowExt &, const __half *, long long *,
+                                                        const EvalSums &, int *, cudaStream_t);
 
 }  // namespace nep

@@ -71,7 +71,7 @@ __global__ void k_kick_drift(int n, double *__restrict__ x, double *__restrict__
   note_displacement(moved, dd, ctrl);
 }
 
-// The step's rebuild decision (step_control) in a kernel of its own: with a condition, in a captured MD step whose
+// The step's rebuild decision in a kernel of its own: with a condition, in a captured MD step whose
 // rebuild chain is the body of a conditional graph node, so that a step without a rebuild launches none of the
 // chain's kernels.
 __global__ void k_control_cond(Control *ctrl, cudaGraphConditionalHandle cond) {

@@ -1,7 +1,7 @@
-// nep_mixed.cu -- mixed-precision descriptor + network kernel (sm_103a, tcgen05 tensor cores).
+// nep_mixed.cu -- mixed-precision descriptor + network kernel of the student's two-kernel form (sm_103a, tcgen05 tensor
+// cores; see student_split in nep_api.cu for when it runs).
 //
-// Same descriptors as k_descriptor (float32 neighbour walk, Section III.B), but the one-hidden-layer
-// network runs as two GEMMs on the 5th-generation tensor cores, one CTA = one 128-atom tile:
+// Descriptors by the float32 neighbour walk (Section III.B); the one-hidden-layer network runs as two GEMMs on the 5th-generation tensor cores, one CTA = one 128-atom tile:
 //   forward   Z[128 x 32]  = Q~[128 x 32] . W0^T      (bf16 or f16 operands, f32 accumulation in TMEM)
 //   backward  dQ[128 x 32] = T[128 x 32] . W0          T_mu = w1_mu (1 - tanh(z_mu - b0_mu)^2)
 // (the batched network GEMM of Section V.B, Optimization 1 and Fig. 2c, with the half-precision network

@@ -10,7 +10,7 @@ namespace nep {
 template <class S>
 struct RowTmem {
   uint32_t trow;
-  __device__ __forceinline__ void load(int k, float (&h)[S::NA][4]) const { tm_load<S, S::NA>(trow, k, h); }
+  __device__ __forceinline__ void load(int k, float (&h)[S::NA][4]) const { tm_load<S>(trow, k, h); }
 };
 template <class S>
 struct RowReg {

@@ -138,18 +138,11 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 // of warp w owns lane 32 (w mod 4) + t, and a thread's values occupy consecutive columns of its lane.
 // All of these are warp-collective (.sync.aligned): the whole warp executes them together.
 
-// Columns [taddr, taddr + W) of this thread's lane <- v (W = 4 or 8).
+// Columns [taddr, taddr + 4), and [taddr, taddr + 16), of this thread's lane <- v.
 __device__ __forceinline__ void tmem_st(uint32_t taddr, const float (&v)[4]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(__float_as_uint(v[0])),
                "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])));
 }
-__device__ __forceinline__ void tmem_st(uint32_t taddr, const float (&v)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
-               "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-               "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
-               "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])));
-}
-// Columns [taddr, taddr + 16) of this thread's lane <- v.
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
@@ -162,73 +155,15 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) 
 // Wait until this thread's TMEM stores have completed.
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Five (or four) groups of W columns (W = 4 or 8) at c[0..] of this thread's lane, loaded and waited
-// for in one statement, so that no use of the values can be scheduled before the wait.
-__device__ __forceinline__ void tmem_ld5(const uint32_t (&c)[5], float (&v)[5][4]) {
-  uint32_t r[20];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%20];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4, %5, %6, %7}, [%21];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8, %9, %10, %11}, [%22];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%12, %13, %14, %15}, [%23];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%16, %17, %18, %19}, [%24];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19])
-      : "r"(c[0]), "r"(c[1]), "r"(c[2]), "r"(c[3]), "r"(c[4]));
-#pragma unroll
-  for (int a = 0; a < 5; ++a)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[a][k] = __uint_as_float(r[4 * a + k]);
-}
-__device__ __forceinline__ void tmem_ld5(const uint32_t (&c)[4], float (&v)[4][4]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%16];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4, %5, %6, %7}, [%17];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8, %9, %10, %11}, [%18];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%12, %13, %14, %15}, [%19];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(c[0]), "r"(c[1]), "r"(c[2]), "r"(c[3]));
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[a][k] = __uint_as_float(r[4 * a + k]);
-}
-__device__ __forceinline__ void tmem_ld5(const uint32_t (&c)[5], float (&v)[5][8]) {
-  uint32_t r[40];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%40];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%41];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16, %17, %18, %19, %20, %21, %22, %23}, [%42];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24, %25, %26, %27, %28, %29, %30, %31}, [%43];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%32, %33, %34, %35, %36, %37, %38, %39}, [%44];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]),
-        "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39])
-      : "r"(c[0]), "r"(c[1]), "r"(c[2]), "r"(c[3]), "r"(c[4]));
-#pragma unroll
-  for (int a = 0; a < 5; ++a)
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[a][k] = __uint_as_float(r[8 * a + k]);
-}
-
 // Per-thread rows of 5 channels x NLM components in TMEM ("chunked" layout): chunk k holds the
 // components lm = 4k..4k+3; channels 0..3 of chunk k sit in the 16 columns 16k + 4a + (lm mod 4)
 // (one x16 access at a 16-aligned column) and channel 4 in the 4 columns 16 NC + lm (one x4 access at a
-// 4-aligned column), NC = NLM / 4 chunks.  With NLM = 24: 96 + 24 = 120 columns; with only channels 0..3
-// (the mixed-precision kernel) the first 96.  Every access is aligned to its own width.
+// 4-aligned column), NC = NLM / 4 chunks.  With NLM = 24: 96 + 24 = 120 columns.  Every access is aligned to its own width.
 __host__ __device__ constexpr uint32_t tm_col(int a, int lm, int nlm) {
   return a < 4 ? (uint32_t)((lm >> 2) * 16 + a * 4 + (lm & 3)) : (uint32_t)((nlm >> 2) * 16 + lm);
 }
 
-// Chunk k of channels 0..NT-1 (NT = 4 or 5), loaded and waited for in one statement.
+// Chunk k of the five channels, loaded and waited for in one statement.
 template <int NLM>
 __device__ __forceinline__ void tmem_ld_chunk(uint32_t trow, int k, float (&v)[5][4]) {
   uint32_t r[20];
@@ -246,32 +181,16 @@ __device__ __forceinline__ void tmem_ld_chunk(uint32_t trow, int k, float (&v)[5
 #pragma unroll
     for (int c = 0; c < 4; ++c) v[a][c] = __uint_as_float(r[4 * a + c]);
 }
+// Chunk k of the five channels <- v (not waited for: tmem_wait_st before the columns are read again).
 template <int NLM>
-__device__ __forceinline__ void tmem_ld_chunk(uint32_t trow, int k, float (&v)[4][4]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
-      "[%16];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(trow + tm_col(0, 4 * k, NLM)));
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) v[a][c] = __uint_as_float(r[4 * a + c]);
-}
-// Chunk k of channels 0..NT-1 <- v (not waited for: tmem_wait_st before the columns are read again).
-template <int NLM, int NT>
-__device__ __forceinline__ void tmem_st_chunk(uint32_t trow, int k, const float (&v)[NT][4]) {
-  static_assert(NT == 4 || NT == 5, "4 or 5 channels");
+__device__ __forceinline__ void tmem_st_chunk(uint32_t trow, int k, const float (&v)[5][4]) {
   float w[16];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int c = 0; c < 4; ++c) w[4 * a + c] = v[a][c];
   tmem_st16(trow + tm_col(0, 4 * k, NLM), w);
-  if constexpr (NT == 5) tmem_st(trow + tm_col(4, 4 * k, NLM), v[NT - 1]);
+  tmem_st(trow + tm_col(4, 4 * k, NLM), v[4]);
 }
 
 }  // namespace nep
