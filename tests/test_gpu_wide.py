@@ -51,7 +51,7 @@ def test_teacher(api, model_params, model, n):
 
 
 @pytest.mark.parametrize("precision", ["mix_bf16", "mix_fp16"])
-@pytest.mark.parametrize("n", [5, 1024, 1025, 4097, 9729])
+@pytest.mark.parametrize("n", [5, 1024, 1025, 4097, 9729, 19457])
 def test_mixed(api, model_params, model, trained_student_params, n, precision):
     # the bounds of the tensor-core forms' tests: RMSE 5 meV/A, largest 20 (bf16) or 3 meV/A (f16)
     pos, box = _cell(n)
