@@ -269,17 +269,22 @@ _LOSS = None
 
 
 def _takes_fused_loss(E, F, cells, s0, s1, w_E, w_F) -> bool:
-    """Plain CUDA tensors as student_ef returns them, labels that are not differentiated, and none of the modes that
-    a custom autograd function without their rules would refuse (forward mode, functorch transforms, tracing)."""
+    """Plain CUDA tensors as student_ef returns them, labels as CellSet makes them for one label per cell and atom (the
+    kernels read them by address) that are not differentiated, and none of the modes that a custom autograd function
+    without their rules would refuse (forward mode, functorch transforms, tracing)."""
     import torch
+
+    def label(t, dtype, *shape):
+        return (type(t) is torch.Tensor and t.device == E.device and t.dtype == dtype and t.shape == shape
+                and t.is_contiguous() and not t.requires_grad)
+
     a0, a1 = cells.atoms(s0, s1)
     return (type(E) is torch.Tensor and type(F) is torch.Tensor and E.is_cuda and F.device == E.device
-            and cells.F_ref.device == E.device and E.dtype == torch.float64 and F.dtype == torch.float32
-            and E.shape == (s1 - s0,) and F.shape == (a1 - a0, 3) and s1 > s0 and a1 > a0
+            and E.dtype == torch.float64 and F.dtype == torch.float32
+            and E.shape == (s1 - s0,) and F.shape == (a1 - a0, 3) and 0 <= s0 < s1 and a1 > a0
             and E.is_contiguous() and F.is_contiguous()
-            and cells.E_ref.dtype == torch.float64 and cells.F_ref.dtype == torch.float32
-            and cells.E_ref.is_contiguous() and cells.F_ref.is_contiguous()
-            and not (cells.E_ref.requires_grad or cells.F_ref.requires_grad)
+            and label(cells.E_ref, torch.float64, cells.n_cells) and label(cells.F_ref, torch.float32, cells.n, 3)
+            and label(cells.natoms, torch.float64, cells.n_cells)
             and isinstance(w_E, (int, float)) and isinstance(w_F, (int, float))
             and torch.autograd.forward_ad._current_level < 0 and not torch._C._are_functorch_transforms_active()
             and not torch.jit.is_tracing() and not torch.compiler.is_compiling())
