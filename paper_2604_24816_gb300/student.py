@@ -18,7 +18,7 @@ import numpy as np
 from . import nep as _nep
 
 EXPORTED = ("st_pairs", "st_basis", "st_forward", "st_energy", "st_force", "st_jvp", "st_grad_scratch", "st_grad",
-            "st_loss_scratch", "st_loss", "st_loss_grad", "st_adam")
+            "st_loss_scratch", "st_loss", "st_loss_diff", "st_loss_grad", "st_adam")
 DIMS = dict(n_max_R=3, n_max_A=3, basis_R=8, basis_A=8, l_max_3b=2, l_max_4b=0, n_neu=16)
 NR, NA, KB, NLM, NDES, NNEU, GS = 4, 4, 8, 8, 12, 16, 40
 NSB = KB * NLM
@@ -52,6 +52,7 @@ def lib():
         L.st_loss_scratch.argtypes = []
         L.st_loss_scratch.restype = C.c_int64
         L.st_loss.argtypes = [i, i, vp, vp, vp, vp, vp, d, d, vp, vp, vp]
+        L.st_loss_diff.argtypes = [i, i, vp, vp, vp, vp, vp, d, d, vp, vp, vp, vp, vp]
         L.st_loss_grad.argtypes = [i, i, vp, vp, vp, vp, vp, d, d, vp, vp, vp, vp]
         L.st_adam.argtypes = [i, vp, vp, vp, vp, C.c_float, C.c_float, C.c_float, C.c_float, i, vp]
         for f in EXPORTED:
@@ -230,37 +231,42 @@ def _loss_ef():
     import torch
 
     class LossEF(torch.autograd.Function):
-        """(E, F, cells, s0, s1, w_E, w_F) -> loss, by st_loss and st_loss_grad."""
+        """(E, F, cells, s0, s1, w_E, w_F) -> (loss, E - E*, F - F*), by st_loss_diff and st_loss_grad.  The differences
+        are what the gradient needs: they are outputs so that it stays the gradient of the value returned whatever is
+        done to E, F and the labels afterwards, and a second derivative finds its way through them."""
 
         @staticmethod
         def forward(ctx, E, F, cells, s0, s1, w_E, w_F):
             L = lib()
+            a0 = cells.atoms(s0, s1)[0]
             ws = torch.empty(int(L.st_loss_scratch()), dtype=torch.float64, device=E.device)
             loss = torch.empty((), dtype=torch.float64, device=E.device)
-            ctx.args = (cells, s0, s1, w_E, w_F)
-            _chk(L.st_loss(*LossEF.arrays(E, F, cells, s0, s1), w_E, w_F, _p(ws), _p(loss), _stream()), "st_loss")
-            ctx.save_for_backward(E, F)
-            return loss
+            dE, dF = torch.empty_like(E), torch.empty_like(F)
+            _chk(L.st_loss_diff(E.numel(), F.numel(), _p(E), _at(cells.E_ref, -8 * s0), _at(cells.natoms, -8 * s0), _p(F),
+                                _at(cells.F_ref, -12 * a0), w_E, w_F, _p(dE), _p(dF), _p(ws), _p(loss), _stream()),
+                 "st_loss_diff")
+            ctx.set_materialize_grads(False)
+            ctx.save_for_backward(dE, dF, cells.natoms)
+            ctx.args = (s0, s1, w_E, w_F)
+            return loss, dE, dF
 
         @staticmethod
-        def arrays(E, F, cells, s0, s1):
-            return (E.numel(), F.numel(), _p(E), _at(cells.E_ref, -8 * s0), _at(cells.natoms, -8 * s0), _p(F),
-                    _at(cells.F_ref, -12 * cells.atoms(s0, s1)[0]))
-
-        @staticmethod
-        def backward(ctx, g):
-            E, F = ctx.saved_tensors
-            cells, s0, s1, w_E, w_F = ctx.args
-            if torch.is_grad_enabled():      # a derivative of this derivative is asked for: differentiable operations
-                a0, a1 = cells.atoms(s0, s1)
-                n = cells.natoms[s0:s1]
-                gE = g * (2.0 * w_E / E.numel()) * ((E - cells.E_ref[s0:s1]) / n) / n
-                gF = (g * (2.0 * w_F / F.numel()) * (F - cells.F_ref[a0:a1]).double()).to(F.dtype)
-            else:
-                gE, gF = torch.empty_like(E), torch.empty_like(F)
-                _chk(lib().st_loss_grad(*LossEF.arrays(E, F, cells, s0, s1), w_E, w_F, _p(g.contiguous()), _p(gE), _p(gF),
-                                        _stream()), "st_loss_grad")
-            return gE, gF, None, None, None, None, None
+        def backward(ctx, g, gdE, gdF):
+            dE, dF, natoms = ctx.saved_tensors
+            s0, s1, w_E, w_F = ctx.args
+            if g is not None and gdE is None and gdF is None and not torch.is_grad_enabled():
+                gE, gF = torch.empty_like(dE), torch.empty_like(dF)
+                _chk(lib().st_loss_grad(dE.numel(), dF.numel(), _p(dE), None, _at(natoms, -8 * s0), _p(dF), None, w_E, w_F,
+                                        _p(g.contiguous()), _p(gE), _p(gF), _stream()), "st_loss_grad")
+                return gE, gF, None, None, None, None, None
+            # a derivative of this derivative is asked for, or this is one: differentiable operations
+            if g is not None:
+                n = natoms[s0:s1]
+                gE = g * (2.0 * w_E / dE.numel()) * (dE / n) / n
+                gF = (g * (2.0 * w_F / dF.numel()) * dF.double()).to(dF.dtype)
+                gdE = gE if gdE is None else gdE + gE
+                gdF = gF if gdF is None else gdF + gF
+            return gdE, gdF, None, None, None, None, None
 
     return LossEF
 
@@ -301,7 +307,7 @@ def loss_fn(E, F, cells: CellSet, s0: int, s1: int, w_E: float = 1.0, w_F: float
         return _loss_plain(E, F, cells, s0, s1, w_E, w_F)
     if _LOSS is None:
         _LOSS = _loss_ef()
-    return _LOSS.apply(E, F, cells, s0, s1, float(w_E), float(w_F))
+    return _LOSS.apply(E, F, cells, s0, s1, float(w_E), float(w_F))[0]
 
 
 def adam_step(theta, grad, m, v, lr: float, t: int, beta1: float = 0.9, beta2: float = 0.999, eps: float = 1e-8):

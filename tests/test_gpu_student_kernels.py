@@ -101,3 +101,47 @@ def test_loss_keeps_what_autograd_could_do(env):
         dual = fwad.make_dual(F.detach(), torch.ones_like(F))
         t = [fwad.unpack_dual(f(E.detach(), dual, cs, 1, 3)).tangent for f in (st.loss_fn, st._loss_plain)]
     assert torch.allclose(t[0], t[1], rtol=1e-6)
+
+
+def test_loss_gradient_is_of_the_value_returned(env):
+    """Labels, energies and forces replaced or rewritten between the loss and its backward pass: the gradient stays that
+    of the loss returned, once and as a second derivative."""
+    torch, st, cs, qs, th = env
+    a0, a1 = cs.atoms(1, 3)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    E0 = torch.randn(2, generator=g, device="cuda", dtype=torch.float64)
+    F0 = torch.randn((a1 - a0, 3), generator=g, device="cuda")
+    keep = cs.E_ref, cs.F_ref
+
+    def swap(E, F):
+        cs.E_ref, cs.F_ref = keep[0] + 1.0, keep[1] - 2.0
+
+    def rewrite(E, F):
+        cs.E_ref.mul_(3.0)
+        cs.F_ref.zero_()
+
+    def outputs(E, F):
+        with torch.no_grad():
+            E.zero_()
+            F.mul_(-1.0)
+
+    def derivatives(loss, change):
+        cs.E_ref, cs.F_ref = keep[0].clone(), keep[1].clone()
+        x, y = E0.clone().requires_grad_(), F0.clone().requires_grad_()
+        E, F = x * 1.0, y * 1.0
+        value = loss(E, F, cs, 1, 3)
+        change(E, F)
+        first = torch.autograd.grad(value, (x, y), retain_graph=True)
+        gE, gF = torch.autograd.grad(value, (x, y), create_graph=True)
+        return (*first, *torch.autograd.grad((gE * gE).sum() + (gF * gF).sum().double(), (x, y)))
+
+    try:
+        for change in (swap, rewrite, outputs):
+            for a, b in zip(derivatives(st.loss_fn, change), derivatives(st._loss_plain, change)):
+                assert b.abs().max() > 0 and torch.allclose(a, b, rtol=1e-5), change.__name__
+    finally:
+        cs.E_ref, cs.F_ref = keep
+    # and through hooks on what is saved
+    with torch.autograd.graph.save_on_cpu():
+        a, b = _run(env, 0, 3)[3], _run(env, 0, 3, plain=True)[3]
+    assert (a - b).abs().max() <= 1e-6 * b.abs().max()
