@@ -1,5 +1,5 @@
-"""Which calls of the training loss reach the fused kernels, which read the labels by address: decided on the CPU, with
-host tensors that report themselves as CUDA ones.  Every other call takes the loss in PyTorch operations."""
+"""Ranges of cells that student_ef accepts, and which calls of the training loss reach the fused kernels, which read the labels by address: on the CPU,
+with host tensors that report themselves as CUDA ones.  Every other call takes the loss in PyTorch operations."""
 from types import SimpleNamespace
 
 import numpy as np
@@ -92,3 +92,40 @@ def test_ranges_from_the_end_take_the_plain_loss():
     out = torch.randn(1, dtype=torch.float64), torch.randn(5, 3)
     assert not _fused(c, -3, -2, outputs=out)
     assert torch.equal(st.loss_fn(*out, c, -3, -2), st._loss_plain(*out, c, -3, -2))
+
+
+class _Calls:
+    """Records the kernel library's calls (every one succeeds)."""
+
+    def __init__(self):
+        self.args = {}
+
+    def __getattr__(self, name):
+        return lambda *a: self.args.setdefault(name, a) and 0
+
+
+@pytest.fixture
+def calls(monkeypatch):
+    L = _Calls()
+    monkeypatch.setattr(st, "lib", lambda: L)
+    monkeypatch.setattr(st, "_stream", lambda: None)
+    return L
+
+
+def _resident(c):
+    for k, shape in dict(pos=(12, 4), Q=(12, 8), S=(12, 64), U=(12,), G=(12, 40), nbr=(96, 12), dvec=(96, 12, 4), nnum=(12,),
+                         dQ=(12, 8), dS=(12, 64), scratch=(289,), start=(4,)).items():
+        setattr(c, k, torch.zeros(shape))
+    c.cap, c.rc = 96, st.st_cutoffs(5.0, 4.0)
+    return c
+
+
+@pytest.mark.parametrize("as_int", [int, np.int64, np.int32, torch.tensor])
+def test_ranges_of_any_integer_type(calls, as_int):
+    c = _resident(_cells())
+    theta, qs = torch.zeros(st.NPAR, requires_grad=True), torch.ones(12)
+    E, F = st.student_ef(theta, qs, c, as_int(1), as_int(3))
+    assert E.shape == (2,) and F.shape == (9, 3)
+    assert calls.args["st_energy"][-2].value == E.data_ptr() - 8 and calls.args["st_force"][-2].value == F.data_ptr() - 36
+    (E.sum() + F.sum().double()).backward()
+    assert theta.grad.shape == (st.NPAR,)
