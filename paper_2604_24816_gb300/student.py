@@ -174,8 +174,8 @@ def _student_ef():
             s0, s1 = int(s0), int(s1)
             a0, a1 = cells.atoms(s0, s1)
             dev = cells.pos.device
-            E = torch.empty(s1 - s0, dtype=torch.float64, device=dev)
-            F = torch.empty((a1 - a0, 3), dtype=torch.float32, device=dev)
+            E = torch.empty(max(s1 - s0, 0), dtype=torch.float64, device=dev)      # s1 < s0: an empty range
+            F = torch.empty((max(a1 - a0, 0), 3), dtype=torch.float32, device=dev)
             st = _stream()
             _chk(L.st_forward(a0, a1, _p(theta), _p(q_scale), _p(cells.Q), _p(cells.S), _p(cells.U), _p(cells.G),
                               None, st), "st_forward")
@@ -194,9 +194,9 @@ def _student_ef():
             L = lib()
             dev = cells.pos.device
             # neighbours and cell energies lie inside the batch, so its own derivatives are all the kernels read
-            gE = torch.zeros(s1 - s0, dtype=torch.float64, device=dev) if gE is None else \
+            gE = torch.zeros(max(s1 - s0, 0), dtype=torch.float64, device=dev) if gE is None else \
                 gE.to(torch.float64).contiguous()
-            v = torch.zeros((a1 - a0, 3), dtype=torch.float32, device=dev) if gF is None else \
+            v = torch.zeros((max(a1 - a0, 0), 3), dtype=torch.float32, device=dev) if gF is None else \
                 gF.to(torch.float32).contiguous()
             st = _stream()
             _chk(L.st_jvp(a0, a1, cells.n, cells.cap, _p(cells.nbr), _p(cells.dvec), _p(cells.nnum), cells.rc,

@@ -129,3 +129,12 @@ def test_ranges_of_any_integer_type(calls, as_int):
     assert calls.args["st_energy"][-2].value == E.data_ptr() - 8 and calls.args["st_force"][-2].value == F.data_ptr() - 36
     (E.sum() + F.sum().double()).backward()
     assert theta.grad.shape == (st.NPAR,)
+
+
+def test_an_empty_range(calls):
+    c = _resident(_cells())
+    theta = torch.zeros(st.NPAR, requires_grad=True)
+    for s0, s1 in ((1, 1), (2, 1)):
+        E, F = st.student_ef(theta, torch.ones(12), c, s0, s1)
+        assert E.shape == (0,) and F.shape == (0, 3)
+        (E.sum() + F.sum().double()).backward()
