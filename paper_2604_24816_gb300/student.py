@@ -12,6 +12,7 @@ kernels; this module only allocates device buffers (PyTorch) and marshals pointe
 from __future__ import annotations
 
 import ctypes as C
+import operator
 
 import numpy as np
 
@@ -171,7 +172,7 @@ def _student_ef():
         @staticmethod
         def forward(ctx, theta, q_scale, cells, s0, s1):
             L = lib()
-            s0, s1 = int(s0), int(s1)
+            s0, s1 = operator.index(s0), operator.index(s1)
             a0, a1 = cells.atoms(s0, s1)
             dev = cells.pos.device
             E = torch.empty(max(s1 - s0, 0), dtype=torch.float64, device=dev)      # s1 < s0: an empty range
@@ -308,7 +309,7 @@ def loss_fn(E, F, cells: CellSet, s0: int, s1: int, w_E: float = 1.0, w_F: float
         return _loss_plain(E, F, cells, s0, s1, w_E, w_F)
     if _LOSS is None:
         _LOSS = _loss_ef()
-    return _LOSS.apply(E, F, cells, int(s0), int(s1), float(w_E), float(w_F))[0]
+    return _LOSS.apply(E, F, cells, operator.index(s0), operator.index(s1), float(w_E), float(w_F))[0]
 
 
 def adam_step(theta, grad, m, v, lr: float, t: int, beta1: float = 0.9, beta2: float = 0.999, eps: float = 1e-8):

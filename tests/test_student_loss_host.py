@@ -138,3 +138,9 @@ def test_an_empty_range(calls):
         E, F = st.student_ef(theta, torch.ones(12), c, s0, s1)
         assert E.shape == (0,) and F.shape == (0, 3)
         (E.sum() + F.sum().double()).backward()
+
+
+def test_a_fraction_is_no_cell(calls):
+    c = _resident(_cells())
+    with pytest.raises((TypeError, IndexError)):
+        st.student_ef(torch.zeros(st.NPAR), torch.ones(12), c, 0.5, 3)
