@@ -671,8 +671,12 @@ nep_status compute_internal(nep_handle *h, float *qout, double *Fout = nullptr) 
   return NEP_OK;
 }
 
-// Steps that a replayed graph holds at most.
-constexpr int GRAPH_STEPS = 16;
+// Steps that a replayed graph holds at most: of plain kernels, and with a conditional rebuild chain per step.  A
+// chain costs its capture and instantiation 30 us, and more than two per replay gain nothing: ten steps of 55,296
+// student atoms from graphs of 1 / 2 / 4 / 8 / 16 steps 830 / 821 / 820 / 825 / 816 us, the call that builds the graph
+// 917 (one step) / 906 / 969 / 1,096 / 1,143; 23,328 teacher atoms 775 / 764 / 769 / 772 / 764, built in 850 / 848 /
+// 907 / 1,019 / 1,073.
+constexpr int GRAPH_STEPS = 16, GRAPH_COND_STEPS = 2;
 
 // Captures `steps` MD steps: with the rebuild chain behind a conditional node, or (small systems, whose chain is
 // two kernels that take the decision themselves) as plain kernels.
@@ -1052,15 +1056,16 @@ nep_status md_verlet_step(nep_handle *h, double dt_fs, int n_steps) {
   const long long rebuilds_before = h->h_rep->ctrl.rebuilds;
   int left = n_steps;
   if (!h->timing) {
-    // A graph of several steps (as many as the first such call has, at most GRAPH_STEPS) saves the 5 us between
-    // replays and, for small systems, the 2 us between launches: ten steps of 256 atoms take 254 us, against 347
-    // launch by launch and 361 from a one-step graph with a conditional node (8 us per step).  Larger systems'
-    // graphs hold a conditional chain per step, whose capture costs a call of 10 steps 80 us; they are built when
-    // a second call comes (56,000 student atoms: 1,043 -> 998 us per call).
+    // A graph of several steps saves the 5 us between replays and, for small systems, the 2 us between launches: ten
+    // steps of 256 atoms take 212 us from a graph, 230 launch by launch.  Small systems' graphs hold as many steps as
+    // the first call that builds one has (up to GRAPH_STEPS); one from a short call is replaced when a call comes that
+    // is long enough to repay it (a graph of 4 steps costs 64 steps of 256 atoms 37 us of 1,254 against one of 16, which
+    // is built in 130).  Larger systems, whose graphs hold a conditional chain per step, get theirs in a second call.
     const bool conditional = !cell_sort_decides(h->n, h->ncell);
-    if (left >= 4 && (!h->graphk.exec || h->graphk.dt != dt_fs) &&
-        (!conditional || (h->graph1.exec && h->graph1.dt == dt_fs))) {
-      nep_status s = build_graph(h, h->graphk, dt_fs, std::min(left, GRAPH_STEPS));
+    const bool fresh = h->graphk.exec && h->graphk.dt == dt_fs;
+    const bool replace = fresh && !conditional && h->graphk.steps < GRAPH_STEPS && left >= 16 * GRAPH_STEPS;
+    if (left >= 4 && (!fresh || replace) && (!conditional || (h->graph1.exec && h->graph1.dt == dt_fs))) {
+      nep_status s = build_graph(h, h->graphk, dt_fs, std::min(left, conditional ? GRAPH_COND_STEPS : GRAPH_STEPS));
       if (s != NEP_OK) return s;
     }
     const bool several = h->graphk.exec && h->graphk.dt == dt_fs;

@@ -310,8 +310,8 @@ def test_checkpoint_resume_is_bit_identical(api, model_params):
 def test_step_grouping_is_bit_identical(api, model_params):
     """md_verlet_step(20) and twenty md_verlet_step(1) give the same bits: each step's closing half kick
     is applied by the next step's opening kick kernel or, after the last step of a call, by the kick
-    that ends the call, with the same two FMAs either way; the rebuild chain runs inside the captured
-    step only when the control kernel asks for it."""
+    that ends the call, with the same two FMAs either way.  (At this size the twenty steps are a graph of plain
+    kernels, single steps are launched one by one; test_gpu_step_graphs.py has the sizes with a conditional chain.)"""
     wl = ni.fcc_cu_workload(6, 300.0, 0.05, seed=99)
     with api.NEP(model_params, rebuild_every=10) as nep:
         nep.set_state(wl.pos, wl.vel, wl.box)
