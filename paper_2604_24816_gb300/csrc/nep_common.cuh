@@ -20,6 +20,17 @@
 
 namespace nep {
 
+// SMs of the current device (152 if that cannot be read).
+inline int sm_count() {
+  int d = 0, sms = 0;
+  if (cudaGetDevice(&d) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d) != cudaSuccess ||
+      sms <= 0) {
+    cudaGetLastError();
+    sms = 152;
+  }
+  return sms;
+}
+
 constexpr int J_BITS = 27;
 constexpr uint32_t J_MASK = (1u << J_BITS) - 1u;
 constexpr float FIX_SCALE = 4294967296.0f;        // 2^32 fixed-point units per eV/Angstrom

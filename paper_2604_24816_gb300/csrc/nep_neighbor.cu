@@ -640,16 +640,6 @@ static int blocks_for(long long m, int b) { return (int)((m + b - 1) / b); }
 // occupancy calculator's blocks per SM x the SM count); the kernels loop over the rest.  Every step
 // launches the chain and the kernels return at once when it does not rebuild, so the grid size is
 // what such a step pays for.
-static int sm_count() {
-  static int sms = 0;
-  if (sms <= 0) {
-    int d = 0;
-    if (cudaGetDevice(&d) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d) != cudaSuccess ||
-        sms <= 0)
-      sms = 152;
-  }
-  return sms;
-}
 template <class K>
 static int resident_grid(K kernel, long long m, int per_block, int threads) {
   int per_sm = 0;

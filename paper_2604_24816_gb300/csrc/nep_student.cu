@@ -39,6 +39,7 @@ static_assert(SS::KR == SS::KA, "one basis size for both cutoffs");
 
 constexpr int BLOCK = 128;
 constexpr int GRAD_ATOMS = 64;               // atoms per row of partial gradients, at least (st_grad_scratch)
+constexpr int GRAD_SERIAL = 32;              // atoms that one lane's float32 sums run over, at most
 
 // The per-step kernels give each atom a group of eight lanes.  One thread per atom left a mini-batch of 40 cells
 // (21,000 atoms, 165 blocks of 128 threads) at about one block per SM, each thread walking its row alone, and
@@ -601,7 +602,7 @@ k_st_jvp(int a0, int a1, int n, const int *__restrict__ nbr, const float4 *__res
 // W0, 4 of cR, 2 of b0 and of w1, b1) in registers over the atoms of its group, and only the block's totals go
 // through shared memory, in a fixed order.  (Records of 289 floats per atom in shared memory, read back for every
 // product, held 6 warps per SM and took 34 us for 21,000 atoms.)  Block rows are summed by k_st_grad_reduce in
-// float64 in a fixed order.
+// float64 in a fixed order, and there are enough of them that no float32 sum runs over more than GRAD_SERIAL atoms.
 constexpr int GRAD_BLOCK = 256;
 constexpr int GRAD_WARPS = GRAD_BLOCK / 32;
 
@@ -868,8 +869,10 @@ int st_grad(int a0, int a1, const float *theta, const float *q_scale, const floa
             void *stream) {
   cudaStream_t st = (cudaStream_t)stream;
   if (a1 <= a0) return (int)cudaMemsetAsync(grad, 0, NPAR * sizeof(float), st);
-  // as many rows of partial sums as the scratch holds (GRAD_ATOMS atoms each, two per group), up to four blocks per SM
-  const int nblk = std::min(blocks_of(a1 - a0, GRAD_ATOMS), 152 * 4);
+  // as many rows of partial sums as the scratch holds (GRAD_ATOMS atoms each, two per group), up to four blocks per SM;
+  // above 1,024 atoms for each of those, as many as keep the float32 sums at GRAD_SERIAL atoms
+  const int m = a1 - a0;
+  const int nblk = std::max(std::min(blocks_of(m, GRAD_ATOMS), 4 * sm_count()), blocks_of(m, GRAD_BLOCK / G * GRAD_SERIAL));
   k_st_grad<<<nblk, GRAD_BLOCK, 0, st>>>(a0, a1, theta, q_scale, reinterpret_cast<const float4 *>(pos), Q, S, dQ, dS,
                                          gE, scratch);
   cudaError_t e = cudaGetLastError();
@@ -899,7 +902,7 @@ int st_loss(int n_cells, int n_comp, const double *E, const double *E_ref, const
 int st_loss_grad(int n_cells, int n_comp, const double *E, const double *E_ref, const double *natoms, const float *F,
                  const float *F_ref, double w_E, double w_F, const double *g, double *gE, float *gF, void *stream) {
   if (n_cells <= 0 || n_comp <= 0) return (int)cudaErrorInvalidValue;
-  k_st_loss_grad<<<std::min(152 * 8, blocks_of(std::max(n_cells, n_comp), LOSS_BLOCK)), LOSS_BLOCK, 0,
+  k_st_loss_grad<<<std::min(8 * sm_count(), blocks_of(std::max(n_cells, n_comp), LOSS_BLOCK)), LOSS_BLOCK, 0,
                    (cudaStream_t)stream>>>(n_cells, n_comp, E, E_ref, natoms, F, F_ref, w_E, w_F, g, gE, gF);
   return (int)cudaGetLastError();
 }

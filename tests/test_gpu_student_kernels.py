@@ -145,3 +145,29 @@ def test_loss_gradient_is_of_the_value_returned(env):
     with torch.autograd.graph.save_on_cpu():
         a, b = _run(env, 0, 3)[3], _run(env, 0, 3, plain=True)[3]
     assert (a - b).abs().max() <= 1e-6 * b.abs().max()
+
+
+def test_gradient_of_many_atoms_is_summed_in_float64(env):
+    """Equal atoms without directional derivatives, so that every term of a parameter has one sign (c_A's, which come from
+    eight components of two degrees, left out): a lane adds at most 32 atoms' two products in float32 and the block 2 + 8
+    partial sums, each with a relative error of 2^-24 or less; the product itself and the result are rounded once more."""
+    torch, st, cs, qs, th = env
+    n = 12_000_000
+    theta = torch.tensor(th, device="cuda")
+    full = lambda *shape: torch.ones(shape, device="cuda")
+    Q, S, zero = full(n, st.KB) * cs.Q[:1], full(n, st.NSB) * cs.S[:1], torch.zeros(n * st.NSB, device="cuda")
+    pos = torch.zeros((n, 4), device="cuda")                       # cell 0
+    gE = torch.tensor([0.7], dtype=torch.float64, device="cuda")
+
+    def grad(m):
+        out = torch.empty(st.NPAR, device="cuda")
+        ws = torch.empty(int(st.lib().st_grad_scratch(0, m)), device="cuda")
+        rc = st.lib().st_grad(0, m, st._p(theta), st._p(qs), st._p(pos), st._p(Q), st._p(S), st._p(zero), st._p(zero),
+                              st._p(gE), st._p(ws), st._p(out), st._stream())
+        assert rc == 0
+        return out.double()
+
+    one, many = grad(1) * n, grad(n)
+    for o, m in ((0, 32), (64, st.NPAR - 64)):                     # c_R; W0, b0, w1, b1
+        a, b = one[o:o + m], many[o:o + m]
+        assert a.abs().min() > 0 and ((a - b).abs() / a.abs()).max() <= 76 * 2.0 ** -24
