@@ -8,6 +8,8 @@
                 same loss evaluated by the FP64 oracle, for parameters of every group
   Adam          the st_adam kernel vs the textbook update written in numpy
   determinism   two gradient evaluations are bitwise equal
+  long rows     forward, JVP and gradient again on compressed cells, whose rows end before, at and past the first
+                segment of the row walks (64 entries), up to the list capacity
 """
 import numpy as np
 import pytest
@@ -158,6 +160,38 @@ def test_parameter_gradient_matches_oracle_finite_differences(api, cells, labels
         fd = (_oracle_loss(api, tp, student_params, cells, E_ref, F_ref) -
               _oracle_loss(api, tm, student_params, cells, E_ref, F_ref)) / (2 * h)
         assert abs(g[p] - fd) <= 2e-3 * abs(fd) + 1e-4 * gmax, (p, g[p], fd)
+
+
+def test_rows_of_more_than_one_segment(api, model, student_params):
+    # on a grid of 2^-20 Angstrom, so that float32 holds every displacement (these cells are stiff: rounded positions
+    # alone would change the forces by 1e-4 eV/Angstrom)
+    grid = lambda a: np.round(np.asarray(a) * 2.0 ** 20) / 2.0 ** 20
+    cells = [(grid(np.mod(p, b)), grid(b)) for p, b in (ni.student_cell(91, (4, 4, 4), 0.05, (-0.126,) * 3, 1),
+                                                        ni.student_cell(96, (4, 4, 4), 0.04, (-0.245,) * 3, 1))]
+    cs = api.CellSet(cells)
+    rows = cs.nnum.cpu().numpy()
+    assert all((rows == k).any() for k in (63, 64, 65)) and 90 <= rows.max() <= cs.cap
+    r2 = (cs.dvec[64:, :, :3].double() ** 2).sum(-1).cpu().numpy()
+    past = np.arange(64, cs.cap)[:, None] < rows[None, :]
+    assert (r2[past] < 16.0).any() and (r2[past] >= 16.0).any()    # angular and other pairs in the second segment
+    import torch
+    th = _theta32(api, student_params)
+    m = _oracle_student(api, th, student_params)
+    E, F = api.student_ef(torch.tensor(th, device="cuda"),
+                          torch.tensor(np.asarray(student_params["q_scale"], np.float32), device="cuda"), cs)
+    for s, (p, b) in enumerate(cells):
+        a0, a1 = cs.atoms(s, s + 1)
+        eo, uo, fo, wo = oracle.energy_forces(m, p, b)
+        moved = p + np.eye(1, p.size).reshape(p.shape) * 1e-4
+        stiff = np.abs(oracle.energy_forces(m, moved, b)[2] - fo).max() / 1e-4     # 1.5 and 22.6 eV/Angstrom^2, bulk 0.7
+        # the bulk cells' bound, and distances of up to 5 Angstrom rounded to two units of 2^-21 Angstrom
+        assert np.abs(F[a0:a1].cpu().numpy() - fo).max() <= 2e-5 + stiff * 2.0 ** -20
+        assert abs(float(E[s]) - eo) <= 1e-6 * abs(eo) + 1e-6
+    test_jvp_matches_oracle_directional_derivative(api, cells, student_params)
+    m0 = model.with_changes(lj_eps=0.0)
+    ref = [oracle.energy_forces(m0, p, b) for p, b in cells]
+    test_parameter_gradient_matches_oracle_finite_differences(
+        api, cells, (np.array([r[0] for r in ref]), np.concatenate([r[2] for r in ref])), student_params)
 
 
 def test_gradient_is_deterministic(api, cells, labels, student_params):
