@@ -145,6 +145,18 @@ FUSED_FLOPS_STUDENT = {
     "descriptor_rec": dict(list_entry=11, active_pair=2, radial_pair=39, lj_pair=0, angular_pair=151, atom=1218),
     "force_rec": dict(list_entry=0, active_pair=28, radial_pair=47, lj_pair=22, angular_pair=324, atom=0),
 }
+# k_nep_wide (several lanes per atom): the fused kernels' arithmetic without pair records.  The angular sums and the force
+# pass form each pair's displacement again (11, and rsqrt and r 2), the walk sums the LJ energy (15 per LJ pair, the
+# force pass 15); adds of the lanes' partial sums and work on padding are not counted.
+WIDE_FLOPS = {
+    "descriptor": dict(list_entry=11, active_pair=2, radial_pair=39, lj_pair=15, angular_pair=382 + 13, atom=5159),
+    "force": dict(list_entry=0, active_pair=28 + 6, radial_pair=47, lj_pair=15, angular_pair=850, atom=0),
+}
+WIDE_FLOPS_STUDENT = {
+    "descriptor": dict(list_entry=11, active_pair=2, radial_pair=39, lj_pair=15, angular_pair=151 + 13, atom=1218),
+    "force": dict(list_entry=0, active_pair=28 + 6, radial_pair=47, lj_pair=15, angular_pair=324, atom=0),
+}
+WIDE_MAX_ATOMS = 19456             # the largest system that takes k_nep_wide (wide_lanes in nep_wide.cu)
 # Algorithmic HBM bytes per atom-step: the integrator reads and writes x, v (96) in the kick + drift and
 # v (48) in the second kick, and reads the forces in both kicks (48); the force kernel reads the atom's
 # position (16) and its walked neighbour-list entries (4 each), writes the site energy (4) and the
@@ -153,20 +165,37 @@ BYTES = dict(per_atom=96 + 48 + 48 + 16 + 4 + 24, per_list_entry=4)
 
 
 def force_kind(form: str) -> str:
-    """FLOP table of the force pass a form runs: the fused kernels' pass over their pair records for the
-    teacher (float32 or mixed-precision network) and the float32 student, the half list for the
-    student's mixed-precision form."""
+    """Entry of FLOPS / FLOPS_STUDENT for a form's force pass: over the pair records for the teacher and the float32
+    student, the half list for the student's mixed-precision form (its two-kernel form, student_split in nep_api.cu)."""
     f = FORMS[form]
     return "force_rec" if f["model"] == "teacher" or f["precision"] == "fp32" else "force"
 
 
 def descriptor_kind(form: str) -> str:
-    """FLOP table of the descriptor part: the mixed-precision teacher forms' network is on the tensor
-    cores; the float32 student runs its fused kernel (descriptor_rec of FUSED_FLOPS_STUDENT)."""
+    """Entry of FLOPS / FLOPS_STUDENT for a form's descriptor part: the mixed-precision teacher's without the network's
+    products, the float32 student's over the polynomials without their constants."""
     f = FORMS[form]
     if f["model"] == "student":
         return "descriptor_rec" if f["precision"] == "fp32" else "descriptor"
     return "descriptor_mixed" if form in ("mix_bf16", "mix_fp16") else "descriptor"
+
+
+def evaluation_kernels(form: str, n: int, separate: bool) -> dict:
+    """What one evaluation of n atoms runs and how its arithmetic is counted: kind (the name that profiles know it by:
+    wide or fused for one kernel, separate for descriptors and forces apart), the kernel's name, the two FLOP tables.
+    separate: the evaluation launched a descriptor kernel of its own."""
+    student = FORMS[form]["model"] == "student"
+    if separate:
+        t = FLOPS_STUDENT if student else FLOPS
+        return dict(kind="separate", name=None, descriptor=t[descriptor_kind(form)], force=t[force_kind(form)])
+    if n <= WIDE_MAX_ATOMS:
+        t = WIDE_FLOPS_STUDENT if student else WIDE_FLOPS
+        return dict(kind="wide", name="k_nep_wide", descriptor=t["descriptor"], force=t["force"])
+    # the fused kernels' parts are the same in every precision
+    if student:
+        return dict(kind="fused", name="k_nep_fused_reg", descriptor=FUSED_FLOPS_STUDENT["descriptor_rec"],
+                    force=FUSED_FLOPS_STUDENT["force_rec"])
+    return dict(kind="fused", name="k_nep_fused", descriptor=FUSED_FLOPS["descriptor"], force=FUSED_FLOPS["force_rec"])
 
 
 def kernel_flops(kind: str, c: dict, n_atoms_evals: int, table: dict = FLOPS) -> float:
@@ -188,6 +217,7 @@ KERNEL_SOURCES = {
     "descriptor": ("nep_force.cu",) + _CORE,
     "force": ("nep_force.cu",) + _CORE,
     "fused": ("nep_force.cu",) + _CORE,
+    "wide": ("nep_wide.cu",) + _CORE,
     "fused:mix_bf16": ("nep_force.cu",) + _CORE,
     "fused:mix_fp16": ("nep_force.cu",) + _CORE,
     "fused:student": ("nep_force.cu",) + _CORE,
@@ -654,27 +684,22 @@ def run_ours(args, rank: int, ws: int, local: int):
     c2 = nep.counters()
     dc = {k: c2[k] - c1[k] for k in c2}          # the eager pass with per-kernel events
     evals = dc["evaluations"]
-    is_student = FORMS[args.form]["model"] == "student"
-    fused = tim["descriptor"][1] == 0 and tim["force"][1] > 0      # one kernel does descriptors and forces
-    table = ((FUSED_FLOPS_STUDENT if is_student else FUSED_FLOPS) if fused else
-             (FLOPS_STUDENT if is_student else FLOPS))
-    # the fused kernels' parts are the same in every precision
-    f_desc = kernel_flops(("descriptor_rec" if is_student else "descriptor") if fused else descriptor_kind(args.form), dc,
-                          evals * wl.n, table)
-    f_force = kernel_flops("force_rec" if fused else force_kind(args.form), dc, evals * wl.n, table)
+    ev = evaluation_kernels(args.form, wl.n, separate=tim["descriptor"][1] > 0)
+    one = ev["kind"] != "separate"               # one kernel does descriptors and forces
+    f_desc = kernel_flops("descriptor", dc, evals * wl.n, ev)
+    f_force = kernel_flops("force", dc, evals * wl.n, ev)
     clk = clocks.summary(t_host0, t_host1)
     clk_kernels = clocks.summary(t_host2, t_host3)
     kern = {k: {"ms": round(v[0], 4), "launches": v[1]} for k, v in tim.items()}
-    dominant = "force" if fused else max(("descriptor", "force"), key=lambda k: tim[k][0])
-    dom_flops = f_desc + f_force if fused else (f_force if dominant == "force" else f_desc)
+    dominant = "force" if one else max(("descriptor", "force"), key=lambda k: tim[k][0])
+    dom_flops = f_desc + f_force if one else (f_force if dominant == "force" else f_desc)
     dom_ms = tim[dominant][0]
     dom_launches = max(1, tim[dominant][1])
     achieved = dom_flops / (dom_ms * 1e-3) / 1e12
-    kind = "fused" if fused else dominant
+    kind = ev["kind"] if one else dominant
     traffic = profiled_traffic(kind if args.form == "plain" else f"{kind}:{args.form}")
-    dom_name = (("k_nep_fused_reg" if FORMS[args.form]["model"] == "student" else
-                 "k_nep_fused") if fused else
-                "k_descriptor_mixed" if dominant == "descriptor" and args.form != "plain" else f"k_{dominant}")
+    dom_name = ev["name"] if one else ("k_descriptor_mixed" if dominant == "descriptor" and args.form != "plain"
+                                       else f"k_{dominant}")
     pk_mhz, kn_mhz = peak["clocks"].get("sm_mhz"), clk_kernels.get("sm_mhz")
     roofline = {
         "bound": "alu",

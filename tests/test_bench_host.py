@@ -107,6 +107,26 @@ def test_flop_model_counts_units():
     assert g["active_pair"] == 2 + 6 + 3 + 12 and h["active_pair"] == g["active_pair"]
 
 
+def test_evaluation_kernels_follow_the_librarys_size_rule():
+    """Up to the last line of wide_lanes an evaluation is k_nep_wide, above it the fused kernel of the model's shape; the
+    roofline counts the one that ran, and DRAM traffic captured for another kernel is not used."""
+    import re
+    src = open(os.path.join(bench.ROOT, "paper_2604_24816_gb300", "csrc", "nep_wide.cu")).read()
+    rule = re.search(r"int wide_lanes\(int n\) \{(.*)\}", src).group(1)
+    assert bench.WIDE_MAX_ATOMS == max(int(v) for v in re.findall(r"n <= (\d+)", rule))
+    for form, m in bench.FORMS.items():
+        at, above = (bench.evaluation_kernels(form, bench.WIDE_MAX_ATOMS + k, False) for k in (0, 1))
+        assert (at["kind"], at["name"]) == ("wide", "k_nep_wide")
+        assert above["kind"] == "fused"
+        assert above["name"] == ("k_nep_fused_reg" if m["model"] == "student" else "k_nep_fused")
+        # the wide kernel forms displacements again instead of keeping records, and sums the pair energy in its walk
+        for part, more in (("descriptor", dict(angular_pair=13, lj_pair=15)), ("force", dict(active_pair=6, lj_pair=-7))):
+            assert all(at[part][k] - above[part][k] == more.get(k, 0) for k in above[part])
+    two = bench.evaluation_kernels("student_bf16_fallback", 123008, True)
+    assert two["kind"] == "separate" and two["force"] is bench.FLOPS_STUDENT["force"]
+    assert "nep_wide.cu" in bench.KERNEL_SOURCES["wide"] and bench.profiled_traffic("wide:mix_bf16") is None
+
+
 def test_traffic_lookup_requires_matching_source(tmp_path, monkeypatch):
     monkeypatch.setattr(bench, "ROOT", str(tmp_path))
     (tmp_path / "profiles").mkdir()
