@@ -6,8 +6,8 @@
 
 namespace nep {
 
-// What decides: an earlier kernel already did; an MD step (displacement past skin/2, a request, or every
-// rebuild_every steps); a check after an upload that kept the list (displacement or request, the step counters are
+// What decides: an earlier kernel already did; an MD step (displacement past skin/2, or every
+// rebuild_every steps); a check after an upload that kept the list (displacement only, the step counters are
 // not touched); or a rebuild in any case.
 enum : int { DECIDE_DONE = 0, DECIDE_STEP = 1, DECIDE_CHECK = 2, DECIDE_FORCE = 3 };
 
@@ -15,7 +15,7 @@ enum : int { DECIDE_DONE = 0, DECIDE_STEP = 1, DECIDE_CHECK = 2, DECIDE_FORCE = 
 // atom moved far enough since the build to bring a far-band pair inside rc_R.  Returns do_rebuild.
 __device__ __forceinline__ int decide_rebuild(Control *ctrl, int decide) {
   if (decide == DECIDE_DONE) return ctrl->do_rebuild;
-  int rb = ctrl->moved | ctrl->force_rebuild;
+  int rb = ctrl->moved;
   if (decide == DECIDE_STEP) {
     ctrl->steps += 1;
     ctrl->steps_since += 1;
@@ -27,7 +27,6 @@ __device__ __forceinline__ int decide_rebuild(Control *ctrl, int decide) {
   ctrl->do_rebuild = rb;
   if (rb) {
     ctrl->moved = 0;
-    ctrl->force_rebuild = 0;
     ctrl->steps_since = 0;
     ctrl->rebuilds += 1;
     ctrl->dmax2 = 0.f;

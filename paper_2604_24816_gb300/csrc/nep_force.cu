@@ -29,7 +29,7 @@
 //                paper's consolidated backward kernel (Section V.B, Optimization 1) made deterministic.
 //                Virial W = -sum over the evaluated pairs of r_ij (x) (d_ij or D_ij).
 //
-// Everything is float32 except the per-block energy/virial partial sums (float64).
+// Everything is float32 except the fixed-point sums (int64: forces, energy, virial).
 #include "nep_descriptor.cuh"
 #include "nep_pair.cuh"
 #include "nep_tc.cuh"
@@ -873,7 +873,7 @@ template cudaError_t launch_force_float_scatter<CuShape>(const Model<CuShape> &,
                                                          const int32_t *, const RowExt &, const float *, float *,
                                                          const EvalSums &, int *, cudaStream_t);
 
-// Fused descriptor + force evaluation of the float32 teacher (k_nep_fused); Ffix must be zero.
+// Fused descriptor + force evaluation of the teacher (k_nep_fused; MT: type of the network's operands); Ffix must be zero.
 template <class S, class MT>
 cudaError_t launch_fused(const Model<S> &P, const Geom &g, int n, const float4 *pos, const int32_t *nbr,
                          const RowExt &X, float *usite, float *qout, long long *Ffix, const EvalSums &sums,

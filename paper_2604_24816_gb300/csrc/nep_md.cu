@@ -307,8 +307,10 @@ cudaError_t launch_kick_drift(int n, double *x, double *y, double *z, double *vx
                               float4 *pos, const float4 *pos_ref, double kick, double dt, const double l[3],
                               float half_skin2, Control *ctrl, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  // FP64-bound and short: small systems in small blocks, so that every SM's narrow pipe takes part
-  const int block = n <= 16384 ? 64 : MD_BLOCK;
+  // FP64-bound and short: blocks of 64 threads while blocks of 256 would leave an SM's narrow pipe without one.  Of 64 and
+  // 256 threads, eager, with 6 us of launch: 256 atoms 6.9 and 7.6 us, 4,000 7.9 and 8.3, 8,064 8.0 and 8.5, 23,328 8.4
+  // and 8.6, 38,808 8.6 and 8.6; 70,304 10.1 and 10.1, 131,072 12.7 and 12.8, 500,000 30.6 and 27.8.
+  const int block = n <= sm_count() * MD_BLOCK ? 64 : MD_BLOCK;
   k_kick_drift<<<bl(n, block), block, 0, st>>>(n, x, y, z, vx, vy, vz, F, pos, pos_ref, kick, dt, l[0], l[1], l[2],
                                                half_skin2, ctrl);
   return cudaGetLastError();

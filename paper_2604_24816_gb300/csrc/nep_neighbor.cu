@@ -403,8 +403,10 @@ k_rebuild_cluster(int n, int ncell, double *__restrict__ x, double *__restrict__
 // The placement's 4-byte stores into the neighbour-major list are scattered across rows; L2 merges
 // them into full sectors before they reach DRAM.
 constexpr int NB_WARPS = 8;            // atoms (one warp each) per block
-constexpr int NB_TAKE_MIN = 262144;    // atoms from which a block takes four groups of NB_WARPS atoms at a time: fewer
-                                       // barriers (1,339 -> 1,299 us at 1,048,576), but too coarse for small systems (16,384: 30 -> 47)
+// Atoms from which a block takes four groups of NB_WARPS atoms at a time: fewer barriers, but too coarse for small
+// systems.  One and four groups per take: 16,384 atoms 32 and 47 us, 55,296 80 and 86, 131,072 170 and 172, 157,216 205
+// and 205, 262,400 336 and 330, 500,000 627 and 602, 1,048,576 1,360 and 1,311 (eight: 1,309).
+constexpr int NB_TAKE_MIN = 160000;
 constexpr int NB_STAGE = 128;          // staged entries per atom (lists longer than this are an overflow)
 constexpr float OWN_EPS = 0.5f;        // Angstrom; lattice-vector components are either ~0 or >= a/2
 
