@@ -16,7 +16,8 @@
  *                   dQ_k = sum_i v_i . dQ_k/dr_i, dS_klm likewise
  *   st_grad         dL/dtheta = sum_i [ gE_s(i) dU_i/dtheta - d(Fp_i . dq_i)/dtheta ]  (dq_i = the
  *                   directional derivative of q_i along v), reduced over atoms in a fixed order
- *   st_loss, st_loss_diff, st_loss_grad   the training loss and its derivatives with respect to E and F
+ *   st_loss, st_loss_grad   the training loss and its derivatives with respect to E and F; st_loss_keep and
+ *                   st_loss_kept_grad the same with what the derivatives need kept by the former
  *   st_adam         one Adam update of the parameter vector
  *
  * Parameter vector theta (float32, ST_NPAR = 289 values, in this order):
@@ -103,15 +104,18 @@ int64_t st_loss_scratch(void);
 int st_loss(int n_cells, int n_comp, const double *E, const double *E_ref, const double *natoms, const float *F,
             const float *F_ref, double w_E, double w_F, double *scratch, double *loss, void *stream);
 
-/* st_loss that also stores the differences dE = E - E_ref [n_cells] and dF = F - F_ref [n_comp] (either may be NULL). */
-int st_loss_diff(int n_cells, int n_comp, const double *E, const double *E_ref, const double *natoms, const float *F,
-                 const float *F_ref, double w_E, double w_F, double *dE, float *dF, double *scratch, double *loss,
-                 void *stream);
-
-/* *g times the derivatives of that loss: gE [n_cells] and gF [n_comp] (g: one double, device memory).  E_ref (F_ref)
- * NULL: E (F) holds the differences. */
+/* *g times the derivatives of that loss: gE [n_cells] and gF [n_comp] (g: one double, device memory). */
 int st_loss_grad(int n_cells, int n_comp, const double *E, const double *E_ref, const double *natoms, const float *F,
                  const float *F_ref, double w_E, double w_F, const double *g, double *gE, float *gF, void *stream);
+
+/* st_loss that also stores in kept [st_loss_kept()] what its derivatives need, whatever is written to the inputs later:
+ * (E - E_ref) / natoms^2 [n_cells], 1 / natoms^2 [n_cells], F - F_ref [n_comp].  st_loss_kept_grad: the derivatives
+ * from it, times *g. */
+int64_t st_loss_kept(int n_cells, int n_comp);
+int st_loss_keep(int n_cells, int n_comp, const double *E, const double *E_ref, const double *natoms, const float *F,
+                 const float *F_ref, double w_E, double w_F, double *kept, double *scratch, double *loss, void *stream);
+int st_loss_kept_grad(int n_cells, int n_comp, const double *kept, double w_E, double w_F, const double *g, double *gE,
+                      float *gF, void *stream);
 
 /* One Adam step on theta [npar] with moment buffers m, v (float32), step count t >= 1. */
 int st_adam(int npar, float *theta, const float *grad, float *m, float *v, float lr, float beta1, float beta2,

@@ -736,7 +736,8 @@ __global__ void k_st_grad_reduce(int nblk, const float *__restrict__ part, float
 
 // Loss w_E mean_s ((E_s - E*_s) / n_s)^2 + w_F mean (F - F*)^2 over force components: block sums in float64 (weights
 // and means applied), then one block adds them.  Differences of forces in float32, squares and sums in float64.
-// dE, dF (or nullptr): the differences, which the gradient is formed from later whatever becomes of the labels.
+// keep (or nullptr): what the gradient is formed from later, whatever becomes of the labels, {(E - E*) / n^2 [nc] |
+// 1 / n^2 [nc] | F - F* [nf]} (st_loss_keep).
 constexpr int LOSS_BLOCK = 256, LOSS_BLOCKS = 128;
 template <int NT>
 __device__ __forceinline__ double block_sum(double v) {
@@ -752,19 +753,21 @@ __device__ __forceinline__ double block_sum(double v) {
 }
 __global__ void __launch_bounds__(LOSS_BLOCK)
 k_st_loss(int nc, int nf, const double *__restrict__ E, const double *__restrict__ Er, const double *__restrict__ na,
-          const float *__restrict__ F, const float *__restrict__ Fr, double wE, double wF, double *__restrict__ dE,
-          float *__restrict__ dF, double *__restrict__ part) {
+          const float *__restrict__ F, const float *__restrict__ Fr, double wE, double wF, double *__restrict__ keep,
+          double *__restrict__ part) {
   const int t = blockIdx.x * LOSS_BLOCK + threadIdx.x, stride = gridDim.x * LOSS_BLOCK;
   double e = 0.0, f = 0.0;
   for (int s = t; s < nc; s += stride) {
-    const double x = E[s] - Er[s], d = x / na[s];
-    if (dE != nullptr) dE[s] = x;
+    const double d = (E[s] - Er[s]) / na[s];
+    if (keep != nullptr) {
+      keep[s] = d / na[s];
+      keep[nc + s] = 1.0 / (na[s] * na[s]);
+    }
     e = fma(d, d, e);
   }
   for (int k = t; k < nf; k += stride) {
-    const float x = F[k] - Fr[k];
-    if (dF != nullptr) dF[k] = x;
-    const double d = (double)x;
+    const double d = (double)(F[k] - Fr[k]);
+    if (keep != nullptr) keep[2 * (size_t)nc + k] = d;
     f = fma(d, d, f);
   }
   const double v = block_sum<LOSS_BLOCK>(e * (wE / nc) + f * (wF / nf));
@@ -775,15 +778,16 @@ k_st_loss_sum(int nb, const double *__restrict__ part, double *__restrict__ loss
   const double v = block_sum<LOSS_BLOCKS>((int)threadIdx.x < nb ? part[threadIdx.x] : 0.0);
   if (threadIdx.x == 0) *loss = v;
 }
-// Its gradients times the upstream derivative *g.  Er, Fr nullptr: E and F are the differences.
+// Its gradients times the upstream derivative *g, from what k_st_loss kept or (keep nullptr) from E, F and the labels.
 __global__ void __launch_bounds__(LOSS_BLOCK)
-k_st_loss_grad(int nc, int nf, const double *__restrict__ E, const double *__restrict__ Er,
+k_st_loss_grad(int nc, int nf, const double *__restrict__ keep, const double *__restrict__ E, const double *__restrict__ Er,
                const double *__restrict__ na, const float *__restrict__ F, const float *__restrict__ Fr, double wE,
                double wF, const double *__restrict__ g, double *__restrict__ gE, float *__restrict__ gF) {
   const int t = blockIdx.x * LOSS_BLOCK + threadIdx.x, stride = gridDim.x * LOSS_BLOCK;
   const double up = *g, ce = 2.0 * up * wE / nc, cf = 2.0 * up * wF / nf;
-  for (int s = t; s < nc; s += stride) gE[s] = ce * ((Er != nullptr ? E[s] - Er[s] : E[s]) / na[s]) / na[s];
-  for (int k = t; k < nf; k += stride) gF[k] = (float)(cf * (double)(Fr != nullptr ? F[k] - Fr[k] : F[k]));
+  for (int s = t; s < nc; s += stride) gE[s] = ce * (keep != nullptr ? keep[s] : (E[s] - Er[s]) / na[s] / na[s]);
+  for (int k = t; k < nf; k += stride)
+    gF[k] = (float)(cf * (keep != nullptr ? keep[2 * (size_t)nc + k] : (double)(F[k] - Fr[k])));
 }
 
 __global__ void k_st_adam(int npar, float *__restrict__ theta, const float *__restrict__ grad, float *__restrict__ m,
@@ -883,28 +887,40 @@ int st_grad(int a0, int a1, const float *theta, const float *q_scale, const floa
 
 int64_t st_loss_scratch(void) { return LOSS_BLOCKS; }
 
-int st_loss_diff(int n_cells, int n_comp, const double *E, const double *E_ref, const double *natoms, const float *F,
-                 const float *F_ref, double w_E, double w_F, double *dE, float *dF, double *scratch, double *loss,
-                 void *stream) {
+int64_t st_loss_kept(int n_cells, int n_comp) { return 2 * (int64_t)n_cells + n_comp; }
+
+int st_loss_keep(int n_cells, int n_comp, const double *E, const double *E_ref, const double *natoms, const float *F,
+                 const float *F_ref, double w_E, double w_F, double *kept, double *scratch, double *loss, void *stream) {
   if (n_cells <= 0 || n_comp <= 0) return (int)cudaErrorInvalidValue;
   cudaStream_t st = (cudaStream_t)stream;
   const int nb = std::min(LOSS_BLOCKS, blocks_of(std::max(n_cells, n_comp), LOSS_BLOCK));
-  k_st_loss<<<nb, LOSS_BLOCK, 0, st>>>(n_cells, n_comp, E, E_ref, natoms, F, F_ref, w_E, w_F, dE, dF, scratch);
+  k_st_loss<<<nb, LOSS_BLOCK, 0, st>>>(n_cells, n_comp, E, E_ref, natoms, F, F_ref, w_E, w_F, kept, scratch);
   k_st_loss_sum<<<1, LOSS_BLOCKS, 0, st>>>(nb, scratch, loss);
   return (int)cudaGetLastError();
 }
 
 int st_loss(int n_cells, int n_comp, const double *E, const double *E_ref, const double *natoms, const float *F,
             const float *F_ref, double w_E, double w_F, double *scratch, double *loss, void *stream) {
-  return st_loss_diff(n_cells, n_comp, E, E_ref, natoms, F, F_ref, w_E, w_F, nullptr, nullptr, scratch, loss, stream);
+  return st_loss_keep(n_cells, n_comp, E, E_ref, natoms, F, F_ref, w_E, w_F, nullptr, scratch, loss, stream);
+}
+
+static int loss_grad(int n_cells, int n_comp, const double *kept, const double *E, const double *E_ref,
+                     const double *natoms, const float *F, const float *F_ref, double w_E, double w_F, const double *g,
+                     double *gE, float *gF, void *stream) {
+  if (n_cells <= 0 || n_comp <= 0) return (int)cudaErrorInvalidValue;
+  k_st_loss_grad<<<std::min(8 * sm_count(), blocks_of(std::max(n_cells, n_comp), LOSS_BLOCK)), LOSS_BLOCK, 0,
+                   (cudaStream_t)stream>>>(n_cells, n_comp, kept, E, E_ref, natoms, F, F_ref, w_E, w_F, g, gE, gF);
+  return (int)cudaGetLastError();
 }
 
 int st_loss_grad(int n_cells, int n_comp, const double *E, const double *E_ref, const double *natoms, const float *F,
                  const float *F_ref, double w_E, double w_F, const double *g, double *gE, float *gF, void *stream) {
-  if (n_cells <= 0 || n_comp <= 0) return (int)cudaErrorInvalidValue;
-  k_st_loss_grad<<<std::min(8 * sm_count(), blocks_of(std::max(n_cells, n_comp), LOSS_BLOCK)), LOSS_BLOCK, 0,
-                   (cudaStream_t)stream>>>(n_cells, n_comp, E, E_ref, natoms, F, F_ref, w_E, w_F, g, gE, gF);
-  return (int)cudaGetLastError();
+  return loss_grad(n_cells, n_comp, nullptr, E, E_ref, natoms, F, F_ref, w_E, w_F, g, gE, gF, stream);
+}
+
+int st_loss_kept_grad(int n_cells, int n_comp, const double *kept, double w_E, double w_F, const double *g, double *gE,
+                      float *gF, void *stream) {
+  return loss_grad(n_cells, n_comp, kept, nullptr, nullptr, nullptr, nullptr, nullptr, w_E, w_F, g, gE, gF, stream);
 }
 
 int st_adam(int npar, float *theta, const float *grad, float *m, float *v, float lr, float beta1, float beta2,

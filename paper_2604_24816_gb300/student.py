@@ -19,7 +19,7 @@ import numpy as np
 from . import nep as _nep
 
 EXPORTED = ("st_pairs", "st_basis", "st_forward", "st_energy", "st_force", "st_jvp", "st_grad_scratch", "st_grad",
-            "st_loss_scratch", "st_loss", "st_loss_diff", "st_loss_grad", "st_adam")
+            "st_loss_scratch", "st_loss", "st_loss_grad", "st_loss_kept", "st_loss_keep", "st_loss_kept_grad", "st_adam")
 DIMS = dict(n_max_R=3, n_max_A=3, basis_R=8, basis_A=8, l_max_3b=2, l_max_4b=0, n_neu=16)
 NR, NA, KB, NLM, NDES, NNEU, GS = 4, 4, 8, 8, 12, 16, 40
 NSB = KB * NLM
@@ -53,11 +53,14 @@ def lib():
         L.st_loss_scratch.argtypes = []
         L.st_loss_scratch.restype = C.c_int64
         L.st_loss.argtypes = [i, i, vp, vp, vp, vp, vp, d, d, vp, vp, vp]
-        L.st_loss_diff.argtypes = [i, i, vp, vp, vp, vp, vp, d, d, vp, vp, vp, vp, vp]
         L.st_loss_grad.argtypes = [i, i, vp, vp, vp, vp, vp, d, d, vp, vp, vp, vp]
+        L.st_loss_kept.argtypes = [i, i]
+        L.st_loss_kept.restype = C.c_int64
+        L.st_loss_keep.argtypes = [i, i, vp, vp, vp, vp, vp, d, d, vp, vp, vp, vp]
+        L.st_loss_kept_grad.argtypes = [i, i, vp, d, d, vp, vp, vp, vp]
         L.st_adam.argtypes = [i, vp, vp, vp, vp, C.c_float, C.c_float, C.c_float, C.c_float, i, vp]
         for f in EXPORTED:
-            if f not in ("st_grad_scratch", "st_loss_scratch"):
+            if f not in ("st_grad_scratch", "st_loss_scratch", "st_loss_kept"):
                 getattr(L, f).restype = C.c_int
         _ready = True
     return L
@@ -233,42 +236,46 @@ def _loss_ef():
     import torch
 
     class LossEF(torch.autograd.Function):
-        """(E, F, cells, s0, s1, w_E, w_F) -> (loss, E - E*, F - F*), by st_loss_diff and st_loss_grad.  The differences
-        are what the gradient needs: they are outputs so that it stays the gradient of the value returned whatever is
-        done to E, F and the labels afterwards, and a second derivative finds its way through them."""
+        """(E, F, cells, s0, s1, w_E, w_F) -> (loss, what st_loss_keep kept and its scratch).  The gradient is formed from
+        that (st_loss_kept_grad), so it stays the one of the value returned whatever is done to E, F and the labels
+        afterwards; as an output it is part of the graph, where second derivatives find it."""
 
         @staticmethod
         def forward(ctx, E, F, cells, s0, s1, w_E, w_F):
             L = lib()
-            a0 = cells.atoms(s0, s1)[0]
-            ws = torch.empty(int(L.st_loss_scratch()), dtype=torch.float64, device=E.device)
+            nc, nf = s1 - s0, F.numel()
+            kept = torch.empty(2 * nc + nf + L.st_loss_scratch(), dtype=torch.float64, device=E.device)
             loss = torch.empty((), dtype=torch.float64, device=E.device)
-            dE, dF = torch.empty_like(E), torch.empty_like(F)
-            _chk(L.st_loss_diff(E.numel(), F.numel(), _p(E), _at(cells.E_ref, -8 * s0), _at(cells.natoms, -8 * s0), _p(F),
-                                _at(cells.F_ref, -12 * a0), w_E, w_F, _p(dE), _p(dF), _p(ws), _p(loss), _stream()),
-                 "st_loss_diff")
+            _chk(L.st_loss_keep(nc, nf, _p(E), _at(cells.E_ref, -8 * s0), _at(cells.natoms, -8 * s0), _p(F),
+                                _at(cells.F_ref, -12 * cells.atoms(s0, s1)[0]), w_E, w_F, _p(kept),
+                                _at(kept, -8 * (2 * nc + nf)), _p(loss), _stream()), "st_loss_keep")
             ctx.set_materialize_grads(False)
-            ctx.save_for_backward(dE, dF, cells.natoms)
-            ctx.args = (s0, s1, w_E, w_F)
-            return loss, dE, dF
+            ctx.save_for_backward(kept)
+            ctx.args = (nc, F.shape, w_E, w_F)
+            return loss, kept
 
         @staticmethod
-        def backward(ctx, g, gdE, gdF):
-            dE, dF, natoms = ctx.saved_tensors
-            s0, s1, w_E, w_F = ctx.args
-            if g is not None and gdE is None and gdF is None and not torch.is_grad_enabled():
-                gE, gF = torch.empty_like(dE), torch.empty_like(dF)
-                _chk(lib().st_loss_grad(dE.numel(), dF.numel(), _p(dE), None, _at(natoms, -8 * s0), _p(dF), None, w_E, w_F,
-                                        _p(g.contiguous()), _p(gE), _p(gF), _stream()), "st_loss_grad")
+        def backward(ctx, g, g_kept):
+            kept, = ctx.saved_tensors
+            nc, shape, w_E, w_F = ctx.args
+            nf = shape.numel()
+            if g is not None and g_kept is None and not torch.is_grad_enabled():
+                gE = torch.empty(nc, dtype=torch.float64, device=kept.device)
+                gF = torch.empty(shape, dtype=torch.float32, device=kept.device)
+                _chk(lib().st_loss_kept_grad(nc, nf, _p(kept), w_E, w_F, _p(g.contiguous()), _p(gE), _p(gF), _stream()),
+                     "st_loss_kept_grad")
                 return gE, gF, None, None, None, None, None
             # a derivative of this derivative is asked for, or this is one: differentiable operations
+            gE = gF = 0.0
             if g is not None:
-                n = natoms[s0:s1]
-                gE = g * (2.0 * w_E / dE.numel()) * (dE / n) / n
-                gF = (g * (2.0 * w_F / dF.numel()) * dF.double()).to(dF.dtype)
-                gdE = gE if gdE is None else gdE + gE
-                gdF = gF if gdF is None else gdF + gF
-            return gdE, gdF, None, None, None, None, None
+                gE = g * (2.0 * w_E / nc) * kept[:nc]
+                gF = g * (2.0 * w_F / nf) * kept[2 * nc:2 * nc + nf]
+            if g_kept is not None:
+                gE = gE + g_kept[:nc] * kept[nc:2 * nc]
+                gF = gF + g_kept[2 * nc:2 * nc + nf]
+            if g is None and g_kept is None:
+                return (None,) * 7
+            return gE, gF.view(shape).to(torch.float32), None, None, None, None, None
 
     return LossEF
 
@@ -282,17 +289,18 @@ def _takes_fused_loss(E, F, cells, s0, s1, w_E, w_F) -> bool:
     without their rules would refuse (forward mode, functorch transforms, tracing)."""
     import torch
 
-    def label(t, dtype, *shape):
-        return (type(t) is torch.Tensor and t.device == E.device and t.dtype == dtype and t.shape == shape
-                and t.is_contiguous() and not t.requires_grad)
-
-    a0, a1 = cells.atoms(s0, s1)
-    return (type(E) is torch.Tensor and type(F) is torch.Tensor and E.is_cuda and F.device == E.device
-            and E.dtype == torch.float64 and F.dtype == torch.float32
-            and E.shape == (s1 - s0,) and F.shape == (a1 - a0, 3) and 0 <= s0 < s1 and a1 > a0
+    T, f64, f32 = torch.Tensor, torch.float64, torch.float32
+    Er, Fr, na = cells.E_ref, cells.F_ref, cells.natoms
+    if not (type(E) is T and type(F) is T and type(Er) is T and type(Fr) is T and type(na) is T and E.is_cuda):
+        return False
+    (a0, a1), dev, per_cell = cells.atoms(s0, s1), E.device, (cells.n_cells,)
+    return (0 <= s0 < s1 and a1 > a0 and E.shape == (s1 - s0,) and F.shape == (a1 - a0, 3)
+            and Er.shape == per_cell and na.shape == per_cell and Fr.shape == (cells.n, 3)
+            and E.dtype is f64 and F.dtype is f32 and Er.dtype is f64 and na.dtype is f64 and Fr.dtype is f32
+            and F.device == dev and Er.device == dev and na.device == dev and Fr.device == dev
             and E.is_contiguous() and F.is_contiguous()
-            and label(cells.E_ref, torch.float64, cells.n_cells) and label(cells.F_ref, torch.float32, cells.n, 3)
-            and label(cells.natoms, torch.float64, cells.n_cells)
+            and Er.is_contiguous() and na.is_contiguous() and Fr.is_contiguous()
+            and not (Er.requires_grad or na.requires_grad or Fr.requires_grad)
             and isinstance(w_E, (int, float)) and isinstance(w_F, (int, float))
             and torch.autograd.forward_ad._current_level < 0 and not torch._C._are_functorch_transforms_active()
             and not torch.jit.is_tracing() and not torch.compiler.is_compiling())
