@@ -494,10 +494,13 @@ k_nep_wide(const __grid_constant__ Model<S> P, const Geom geom, const int n, con
 
 // The fallback model on the first min(*count, cap) atoms of list: only its network's part is added to usite, to
 // the forces and to the partial sums (the pair term is the student's).  Few flagged atoms take a warp each, many
-// a quarter of one: at 131,072 atoms 20 us against 28 for 1,311 flagged ones, 39 against 33 for 8,192 (of
-// 16,384), 426 against 264 for all (eager times, with 6 us of launch).  The two kernels of one thread per flagged
-// atom that this replaces took 66 us from one to 16,384 flagged atoms (their serial row walk), 321 for 131,072 and
-// 2.02 ms for 1,048,576, where this takes 2.1.
+// a quarter of one: at 131,072 atoms 20 us against 27 for 1,311 flagged ones, 39 against 35 for 6,554, 440 against 272
+// for all (eager times, with 6 us of launch).  The two kernels of one thread per flagged
+// atom that this replaces took 70 us from one to 16,384 flagged atoms (their serial row walk), 322 for 131,072, 549 for
+// 262,400 (this: 544), and less than this only above 450,000: 992 against 1,007 for 500,000, 2,011 against 2,097 for
+// 1,048,576.  Not kept for those: eight lanes alone (2,029 there, but 28 us instead of 18 for a few flagged atoms, which
+// is what a range is set for), and four lanes above 81,920 flagged ones (1,859, but 56 KB of shared memory per block
+// instead of 40, taken from L1: 55 us instead of 46 for 7,805 of 780,448 atoms).
 constexpr int LIST_WARP_MAX = 4096;
 template <class S>
 __global__ void __launch_bounds__(WIDE_BLOCK, 4)
