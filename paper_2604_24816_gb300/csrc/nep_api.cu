@@ -200,6 +200,7 @@ struct nep_handle {
 
   // graphs of MD steps: one step, and several
   StepGraph graph1, graphk;
+  long long single_steps = 0;      // steps replayed from graph1
   long long graph_rebuild_launches = 0;   // kernel launches of a conditional rebuild chain (run on rebuild steps only)
 
   // timing
@@ -671,12 +672,11 @@ nep_status compute_internal(nep_handle *h, float *qout, double *Fout = nullptr) 
   return NEP_OK;
 }
 
-// Steps that a replayed graph holds at most: of plain kernels, and with a conditional rebuild chain per step.  A
-// chain costs its capture and instantiation 30 us, and more than two per replay gain nothing: ten steps of 55,296
-// student atoms from graphs of 1 / 2 / 4 / 8 / 16 steps 830 / 821 / 820 / 825 / 816 us, the call that builds the graph
-// 917 (one step) / 906 / 969 / 1,096 / 1,143; 23,328 teacher atoms 775 / 764 / 769 / 772 / 764, built in 850 / 848 /
-// 907 / 1,019 / 1,073.
-constexpr int GRAPH_STEPS = 16, GRAPH_COND_STEPS = 2;
+// Steps that a replayed graph holds at most.
+constexpr int GRAPH_STEPS = 16;
+// A conditional rebuild chain costs its capture and instantiation 30 us, a replay 5: a graph of K steps with chains is
+// built when 8 K steps of its length have been replayed one by one, or are about to be.
+constexpr int GRAPH_EARNED = 8;
 
 // Captures `steps` MD steps: with the rebuild chain behind a conditional node, or (small systems, whose chain is
 // two kernels that take the decision themselves) as plain kernels.
@@ -1056,16 +1056,21 @@ nep_status md_verlet_step(nep_handle *h, double dt_fs, int n_steps) {
   const long long rebuilds_before = h->h_rep->ctrl.rebuilds;
   int left = n_steps;
   if (!h->timing) {
-    // A graph of several steps saves the 5 us between replays and, for small systems, the 2 us between launches: ten
-    // steps of 256 atoms take 212 us from a graph, 230 launch by launch.  Small systems' graphs hold as many steps as
-    // the first call that builds one has (up to GRAPH_STEPS); one from a short call is replaced when a call comes that
-    // is long enough to repay it (a graph of 4 steps costs 64 steps of 256 atoms 37 us of 1,254 against one of 16, which
-    // is built in 130).  Larger systems, whose graphs hold a conditional chain per step, get theirs in a second call.
+    // A graph of several steps (as many as the call that builds it has, at most GRAPH_STEPS) saves the 5 us between
+    // replays and, for small systems, the 2 us between launches: ten steps of 256 atoms take 212 us from a graph, 230
+    // launch by launch, and a first call builds it.  Larger systems' graphs hold a conditional chain per step and are
+    // built when they pay (GRAPH_EARNED): ten steps of 56,000 student atoms, with their state and sums read, take 902 us
+    // from a graph of ten, 916 in fours and 923 in twos, but building the ten takes 300 us, where the one-step graph of
+    // the first calls takes 80.  A graph from a short call is replaced when a call comes that is long enough to repay it
+    // (four steps per graph cost 64 steps of 256 atoms 37 us of 1,254 against sixteen, built in 130).
     const bool conditional = !cell_sort_decides(h->n, h->ncell);
     const bool fresh = h->graphk.exec && h->graphk.dt == dt_fs;
-    const bool replace = fresh && !conditional && h->graphk.steps < GRAPH_STEPS && left >= 16 * GRAPH_STEPS;
-    if (left >= 4 && (!fresh || replace) && (!conditional || (h->graph1.exec && h->graph1.dt == dt_fs))) {
-      nep_status s = build_graph(h, h->graphk, dt_fs, std::min(left, conditional ? GRAPH_COND_STEPS : GRAPH_STEPS));
+    const int K = std::min(left, GRAPH_STEPS);
+    const long long single = h->graph1.exec && h->graph1.dt == dt_fs ? h->single_steps : 0;
+    const bool build = fresh ? h->graphk.steps < GRAPH_STEPS && left >= 16 * GRAPH_STEPS
+                             : !conditional || single + left >= GRAPH_EARNED * K;
+    if (left >= 4 && build) {
+      nep_status s = build_graph(h, h->graphk, dt_fs, K);
       if (s != NEP_OK) return s;
     }
     const bool several = h->graphk.exec && h->graphk.dt == dt_fs;
@@ -1078,7 +1083,9 @@ nep_status md_verlet_step(nep_handle *h, double dt_fs, int n_steps) {
       if (!h->graph1.exec || h->graph1.dt != dt_fs) {
         nep_status s = build_graph(h, h->graph1, dt_fs, 1);
         if (s != NEP_OK) return s;
+        h->single_steps = 0;
       }
+      h->single_steps += left;
       for (; left > 0; --left) {
         NEP_CUDA(h, cudaGraphLaunch(h->graph1.exec, h->stream));
         h->launch_total += h->graph1.launches;

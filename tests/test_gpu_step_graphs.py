@@ -1,5 +1,5 @@
 """MD steps from replayed graphs above the sizes whose cell sort is one kernel: every step's rebuild chain sits behind a
-conditional node, one step per graph in a first call and several from the second call on.  Any grouping of the steps
+conditional node, one step per graph at first and several when enough steps have been asked for.  Any grouping of the steps
 into calls gives the bits, rebuilds, evaluations and flagged atoms of single steps and of launches one by one."""
 import numpy as np
 import pytest
@@ -20,8 +20,9 @@ def api():
     return pkg
 
 
-# (dt, steps) of the calls: the one-step graph, then the longer one, whole and with remainders, another dt and back
-CALLS = [(1.0, 10), (1.0, 10), (1.0, 10), (1.0, 25), (1.0, 3), (0.5, 7), (0.5, 10), (1.0, 5)]
+# (dt, steps) of the calls: one step per graph until 80 steps have been asked for, then ten (8 times their own length),
+# with a remainder and a call too short for them; another dt, and a call long enough to get its graph of 16 at once; back
+CALLS = [(1.0, 10)] * 10 + [(1.0, 25), (1.0, 3), (0.5, 7), (0.5, 150), (1.0, 5)]
 SINGLE = [(dt, 1) for dt, k in CALLS for _ in range(k)]
 # lanes per atom and a cell sort in a chain of kernels; the fused kernels; the two-kernel form
 CASES = {
