@@ -309,8 +309,8 @@ def _takes_fused_loss(E, F, cells, s0, s1, w_E, w_F) -> bool:
 def loss_fn(E, F, cells: CellSet, s0: int, s1: int, w_E: float = 1.0, w_F: float = 10.0):
     """w_E * mean_s ((E_s - E*_s) / n_s)^2 + w_F * mean over force components (F - F*)^2.
 
-    One fused pass forward and one backward (st_loss, st_loss_grad) instead of 27 operations; a training step is
-    bound by its launches: 423 us for 40 cells, of which the device is busy for 87, against 796 us with the plain form
+    One fused pass forward and one backward (st_loss_keep, st_loss_kept_grad) instead of 27 operations; a training step
+    is bound by its launches: 433 us for 40 cells, of which the device is busy for 87, against 839 with the plain form
     and whole-set buffers for each batch."""
     global _LOSS
     if not _takes_fused_loss(E, F, cells, s0, s1, w_E, w_F):
