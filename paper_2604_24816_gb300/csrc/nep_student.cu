@@ -602,7 +602,9 @@ k_st_jvp(int a0, int a1, int n, const int *__restrict__ nbr, const float4 *__res
 // W0, 4 of cR, 2 of b0 and of w1, b1) in registers over the atoms of its group, and only the block's totals go
 // through shared memory, in a fixed order.  (Records of 289 floats per atom in shared memory, read back for every
 // product, held 6 warps per SM and took 34 us for 21,000 atoms.)  Block rows are summed by k_st_grad_reduce in
-// float64 in a fixed order, and there are enough of them that no float32 sum runs over more than GRAD_SERIAL atoms.
+// float64 in a fixed order, and there are enough of them that no float32 sum runs over more than
+// GRAD_SERIAL atoms: equal atoms are off by 1.8e-7 for 21,000 and 5.6e-7 for a million or twelve (9.7e-7 with one record
+// per atom and rows of 64; 9.1e-6 for twelve million with never more than four rows per SM).
 constexpr int GRAD_BLOCK = 256;
 constexpr int GRAD_WARPS = GRAD_BLOCK / 32;
 
